@@ -182,6 +182,15 @@ __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // 32 consecutive columns of this thread's tensor-memory lane (lane field of taddr = first lane of the warp's quarter)
 __device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t (&r)[32])
@@ -302,15 +311,15 @@ __device__ __forceinline__ uint32_t hif8_to_bf16_bits(uint32_t c)
 }
 
 // Fills the decode table: entry (code c, lane l) at word c * ROW_WORDS + l holds the BF16 bits of code c (one copy per
-// lane, so that a warp's lookups never meet in a bank).  A warp takes 32 codes: each lane works out one code's value
-// once and the warp hands the 32 values round.
+// lane, so that a warp's lookups never meet in a bank).  A warp writes four rows per step, eight lanes with 16 bytes each to
+// a row, every lane working out its row's value itself: all the warps of a block take part and none of them shuffles (with
+// 32 codes per warp, handed round by shuffles, eight warps worked 1300 cycles at the head of every kernel).
 template <int ROW_WORDS>
 __device__ __forceinline__ void fill_decode_table(uint32_t* table, int warp, int lane, int n_warps)
 {
-    for (int c0 = warp * 32; c0 < 256; c0 += n_warps * 32) {
-        const uint32_t v = hif8_to_bf16_bits((uint32_t)(c0 + lane));
-#pragma unroll 8
-        for (int k = 0; k < 32; k++) table[(c0 + k) * ROW_WORDS + lane] = __shfl_sync(0xFFFFFFFFu, v, k);
+    for (int i = warp; i < 64; i += n_warps) {
+        const uint32_t code = (uint32_t)(4 * i + (lane >> 3)), v = hif8_to_bf16_bits(code);
+        *reinterpret_cast<uint4*>(table + code * ROW_WORDS + (lane & 7) * 4) = make_uint4(v, v, v, v);
     }
 }
 
@@ -1023,17 +1032,28 @@ static_assert(kTmemAccN + kNwTmemStages * (BK / 2) <= kTmemColsN, "weight stages
 static_assert(2 * kNwMaxIssuers * 32 <= kTmemAccN, "four issuers x two buffers x 32 rows");
 
 // Work split of the narrow kernel.  The unit is a pair block (two k-blocks; the second one of a slab's last pair may lie
-// beyond K, where the copies fill zeros).  The (slab, pair block) units are numbered slab-major, total = slabs * pair
-// blocks, and CTA c of G takes the contiguous range [total c / G, total (c + 1) / G): every SM streams the same number of
-// weight bytes whatever the number of slabs.  A range cuts slabs into segments.  A segment that covers its whole slab is finished by
+// beyond K, where the copies fill zeros).  The (slab, pair block) units are numbered slab-major, and CTA c of G takes a
+// contiguous range of q or q + 1 of them (the first `rem` CTAs one more): every SM streams the same number of weight bytes
+// whatever the number of slabs.  A range cuts slabs into segments.  A segment that covers its whole slab is finished by
 // its CTA; otherwise the CTA stores its FP32 partial sums as slice (slab, its position among the slab's contributors),
 // and the last contributor to arrive (one ticket per slab and epilogue warp) adds the slices in position order - so the
 // result does not depend on arrival order - and writes C.
+// (Everything in 32 bits, q and rem from the host: N K < 2^45 bytes, so slabs * pair blocks < 2^31.  What a call costs
+// beyond its weight bytes is latency: with 64-bit products and divisions in the kernel, exponents loaded after the sums
+// were complete, one accumulator read per wait and the first copies issued behind the table set-up, 16 x 512 x 512 took
+// 10.2 us a call, 14.1 us with room for the status word only; now 7.5 and 10.3 us.  16 x 28672 x 8192: 67.7 -> 65.5 us.)
 struct NarrowPlan {
-    long long total;     // slabs * pair blocks
+    int q, rem;          // units per CTA; the first rem CTAs take one more
     float* part;         // [slab][pmax][mp][128] partial sums, or nullptr when every range is made of whole slabs
     unsigned* tickets;   // [slab][4], zero at launch
     int pmax;            // slices per slab
+
+    __device__ int first(int c) const { return c * q + (c < rem ? c : rem); }  // first unit of CTA c
+    __device__ int owner(int x) const                                          // the CTA that takes unit x
+    {
+        const int cut = rem * (q + 1);
+        return x < cut ? x / (q + 1) : rem + (x - cut) / q;
+    }
 };
 
 // In front of the narrow kernel when the workspace has room: the activations [M,K] (contiguous bytes) expanded to BF16, and
@@ -1100,10 +1120,9 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     uint32_t* lut_all = reinterpret_cast<uint32_t*>(sm + lay.lut);
     const uint32_t lut = lay.lut + 4u * lane;
     const int num_pb = (p.K + BK2 - 1) / BK2, num_kb = 2 * num_pb;  // per slab
-    const long long G = gridDim.x;
-    const long long pair0 = plan.total * blockIdx.x / G, pair1 = plan.total * (blockIdx.x + 1) / G;  // this CTA's (slab, pair block) range
-    const long long lin0 = 2 * pair0, lin1 = 2 * pair1;  // the same in k-blocks
-    const int n_pairs = (int)(pair1 - pair0), n_it = 2 * n_pairs;
+    const int pair0 = plan.first((int)blockIdx.x), pair1 = plan.first((int)blockIdx.x + 1);  // this CTA's (slab, pair block) range
+    const int n_pairs = pair1 - pair0, n_it = 2 * n_pairs;
+    const int slab0 = pair0 / num_pb, pb0 = pair0 - slab0 * num_pb;  // where the range starts
     const uint32_t act_bytes = (uint32_t)mp * BK2;
     // Up to 32 activation rows: four issuers with two accumulators each (the epilogue of one segment overlaps the next
     // segment's MMAs).  Above that issuers x buffers x rows must stay within 256 columns: four issuers with one accumulator
@@ -1112,15 +1131,35 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     const int bufs = (mp <= 32 || issuers == 2) ? 2 : 1;
     auto acc_col = [&](int q, int buf) { return (uint32_t)((q * bufs + buf) * mp); };  // accumulator of issuer q, buffer buf
 
-    fill_decode_table<(1 << (kLutShiftN - 2))>(lut_all, warp, lane, kThreadsN / 32);  // rows of 1 << kLutShiftN bytes
-    if (threadIdx.x == 0) {
+    // copies of unit i of the range: its weight bytes (and, as bytes, its activations) into stage i % S8
+    int cp_slab = slab0, cp_pb = pb0;
+    auto copy_bytes = [&](int i) {
+        const int s = i % S8;
+        const uint32_t dst_w = lay.u8(s), dst_a = dst_w + kU8Act;
+        const uint64_t w_policy = l2_policy_evict_first();
+        mbar_arrive_expect_tx(bar_u8_full(s), 2 * kNwW8 + (ACT_BF16 ? 0u : act_bytes));
+        // (the weight is read once: its lines are the first to leave L2 again, so that the expanded activations, which
+        // every CTA reads, and the slices of the slabs that two CTAs share stay there)
+        if (W_IS_NK) tma_load_2d_hint(dst_w, &map_w, cp_pb * BK2, cp_slab * BM, bar_u8_full(s), w_policy);
+        else tma_load_2d_hint(dst_w, &map_w, cp_slab * BM, cp_pb * BK2, bar_u8_full(s), w_policy);
+        if (!ACT_BF16) tma_load_2d(dst_a, &map_act, cp_pb * BK2, 0, bar_u8_full(s));
+        if (++cp_pb == num_pb) { cp_pb = 0; cp_slab++; }
+    };
+    const int n_early = min(S8, n_pairs);
+    if (threadIdx.x == kTmaWarp * 32) {
         for (int s = 0; s < S8; s++) { mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), 2 * kGroupWarps); }  // both halves' groups
         // operands ready: the group's warps, plus (ACT_BF16) the announcement of the activation tile's bytes
         for (int s = 0; s < S; s++) { mbar_init(bar_bf_full(s), kGroupWarps + (ACT_BF16 ? 1 : 0)); mbar_init(bar_bf_empty(s), 1); }
         for (int b = 0; b < 2; b++) { mbar_init(bar_acc_full(b), issuers); mbar_init(bar_acc_empty(b), kEpiWarps); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        // The first round of byte copies starts here, under the table set-up: nothing in front of this kernel writes the
+        // operands (the launch before it writes the expanded activations and the cleared words only, and that launch itself
+        // waits for everything before it).
+        for (int i = 0; i < n_early; i++) copy_bytes(i);
     }
+    fill_decode_table<(1 << (kLutShiftN - 2))>(lut_all, warp, lane, kThreadsN / 32);  // rows of 1 << kLutShiftN bytes
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(lay.tmem_slot()), "r"(kTmemColsN) : "memory");
@@ -1136,22 +1175,16 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
 
     if (warp == kTmaWarp) {
         if (lane == 0) {
-            int issued = 0, issued_act = 0;
+            int issued = n_early, issued_act = 0;
             bool aborted = false;
-            const uint64_t w_policy = l2_policy_evict_first();
-            int j = (int)(pair0 / num_pb), pb = (int)(pair0 % num_pb);
+            int pb = pb0;
             for (int it = 0; it < n_pairs; it++) {
-                const int s = it % S8, round = it / S8;
-                if (round > 0 && !mbar_wait(bar_u8_empty(s), (round - 1) & 1, abort_flag, p.status, 31)) break;
-                if (*abort_flag) break;
-                const uint32_t dst_w = lay.u8(s), dst_a = dst_w + kU8Act;
-                mbar_arrive_expect_tx(bar_u8_full(s), 2 * kNwW8 + (ACT_BF16 ? 0u : act_bytes));
-                // (the weight is read once: its lines are the first to leave L2 again, so that the expanded activations, which
-                // every CTA reads, and the slices of the slabs that two CTAs share stay there)
-                if (W_IS_NK) tma_load_2d_hint(dst_w, &map_w, pb * BK2, j * BM, bar_u8_full(s), w_policy);
-                else tma_load_2d_hint(dst_w, &map_w, j * BM, pb * BK2, bar_u8_full(s), w_policy);
-                if (!ACT_BF16) tma_load_2d(dst_a, &map_act, pb * BK2, 0, bar_u8_full(s));
-                issued = it + 1;
+                if (it >= S8) {
+                    if (!mbar_wait(bar_u8_empty(it % S8), (it / S8 - 1) & 1, abort_flag, p.status, 31)) break;
+                    if (*abort_flag) break;
+                    copy_bytes(it);
+                    issued = it + 1;
+                }
                 if (ACT_BF16) {
                     // Activations expanded to BF16 beforehand (map_act is then the map of that copy): the tiles of the pair's
                     // two k-blocks go straight into their operand stages, in the 128-byte-swizzled layout the MMA reads, once
@@ -1167,7 +1200,7 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                     }
                     if (aborted) break;
                 }
-                if (++pb == num_pb) { pb = 0; j++; }
+                if (++pb == num_pb) pb = 0;
             }
             if (*abort_flag) {  // let the copies already issued land before this CTA's shared memory goes away
                 for (int it = max(0, issued - S8); it < issued; it++) {
@@ -1189,7 +1222,7 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             // descriptor of stage 0; a stage or a 16-k step further on adds to the address field only
             const uint64_t da0 = make_smem_desc(lay.bf(0), 16, 1024);
             bool ok = true, first = true;
-            int kb = (int)(lin0 % num_kb), seg = 0;
+            int kb = 2 * pb0, seg = 0;
             for (int it = 0; it < n_it && ok; it++) {
                 const int buf = bufs == 2 ? seg & 1 : 0, use = bufs == 2 ? seg >> 1 : seg;  // use: how often the buffer was filled before
                 if ((it & (issuers - 1)) == q) {
@@ -1290,110 +1323,121 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             if (lane == 0) mbar_arrive(bar_bf_full(s));
         }
     } else {
-        // epilogue warps 0-3: TMEM lane = weight column n, TMEM column = activation row m
-        const int sa = p.d_sa ? *p.d_sa : 0;
-        long long lin = lin0;
-        for (int seg = 0; lin < lin1; seg++) {
-            const int j = (int)(lin / num_kb), kb_a = (int)(lin % num_kb), buf = bufs == 2 ? seg & 1 : 0, use = bufs == 2 ? seg >> 1 : seg;
-            const long long slab_end = (long long)(j + 1) * num_kb, seg_end = slab_end < lin1 ? slab_end : lin1;
-            const bool whole = kb_a == 0 && seg_end == slab_end;
-            if (!mbar_wait(bar_acc_full(buf), use & 1, abort_flag, p.status, 35)) break;
-            tc_fence_after();
-            const int n = j * BM + warp * 32 + lane;
-            const int sw = p.d_sw_channel ? (n < p.N ? p.d_sw_channel[n] : 0) : (p.d_sw ? *p.d_sw : 0);
-            const int sc = -(sa + sw), s1 = sc / 2, s2 = sc - s1;
+        // epilogue warps 0-3: TMEM lane = weight column n, TMEM column = activation row m.  Whatever does not need the sums
+        // (exponents, the slab's contributors) is worked out before the wait for them: after it, it cost every segment
+        // several thousand cycles of load latency and divisions.
+        const int sa = p.d_sa ? *p.d_sa : 0, sw_all = (p.d_sw && !p.d_sw_channel) ? *p.d_sw : 0;
+        const uint32_t tlane = tmem_base + ((uint32_t)(warp * 32) << 16);
+        int slab = slab0, pb_a = pb0, done = 0;  // the segment: units [done, done + len) of the range, from pair block pb_a of the slab
+        for (int seg = 0; done < n_pairs; seg++) {
+            const int buf = bufs == 2 ? seg & 1 : 0, use = bufs == 2 ? seg >> 1 : seg;
+            const int len = min(num_pb - pb_a, n_pairs - done);
+            const bool whole = len == num_pb;
+            const int n = slab * BM + warp * 32 + lane;
+            const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = sc / 2, s2 = sc - s1;
             const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
-            auto finish = [&](int m, float acc) {  // C[m][n] from the complete sum
-                float v = acc * f1 * f2;
-                if (p.c_is_f32) {
-                    float* out = reinterpret_cast<float*>(p.C) + (long long)m * p.ldc + n;
-                    *out = p.accumulate ? v + *out : v;
-                } else {
-                    unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + (long long)m * p.ldc + n;
-                    if (p.accumulate) v += __uint_as_float((uint32_t)*out << 16);
-                    unsigned short b;
-                    asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b) : "f"(v));  // round to nearest even; a NaN stays a NaN
-                    *out = b;
-                }
-            };
-            // contributors of slab j are the CTAs owner(first pair block) .. owner(last pair block);
-            // owner(x) = the largest c with total c / G <= x
-            const long long c_first = (((long long)j * num_pb + 1) * G - 1) / plan.total, c_last = ((long long)(j + 1) * num_pb * G - 1) / plan.total;
-            const int pos = (int)(blockIdx.x - c_first), count = (int)(c_last - c_first + 1);
-            float* slab_part = whole ? nullptr : plan.part + (size_t)j * plan.pmax * mp * BM + warp * 32 + lane;
+            // contributors of the slab: the CTAs from the owner of its first pair block to that of its last one
+            const int c_first = whole ? 0 : plan.owner(slab * num_pb), c_last = whole ? 0 : plan.owner((slab + 1) * num_pb - 1);
+            const int pos = (int)blockIdx.x - c_first, count = c_last - c_first + 1;
+            float* slab_part = whole ? nullptr : plan.part + (size_t)slab * plan.pmax * mp * BM + warp * 32 + lane;
             float* mine = whole ? nullptr : slab_part + (size_t)pos * mp * BM;
-            const uint32_t tlane = tmem_base + ((uint32_t)(warp * 32) << 16);
-            const int it_a = (int)(lin - lin0), it_n = (int)(seg_end - lin);  // the segment's k-blocks, counted within this CTA's range
-            for (int c = 0; c < mp; c += 32) {
-                float r[32];  // this lane's row of the segment's sum, columns c .. c + 31: the issuers' accumulators added in order
+            const int it_a = 2 * done, it_n = 2 * len;  // the segment's k-blocks, counted within this CTA's range
+            // C[m0 .. m0 + 15][n] from complete sums
+            auto finish16 = [&](int m0, const float (&acc)[16]) {
+                if (n >= p.N) return;
+                if (p.c_is_f32) {
+                    float* out = reinterpret_cast<float*>(p.C) + (long long)m0 * p.ldc + n;
 #pragma unroll
-                for (int i = 0; i < 32; i++) r[i] = 0.f;
-                for (int q = 0; q < issuers; q++) {
-                    // issuer q took the k-blocks it = q (mod issuers): none of them in a short segment leaves its accumulator stale
-                    if (it_n < issuers && ((q - it_a) & (issuers - 1)) >= it_n) continue;
-                    uint32_t t[32];
-                    tmem_ld_32x32b_x32(tlane + acc_col(q, buf) + c, t);
-                    tmem_ld_wait();
+                    for (int h = 0; h < 16; h += 8) {
+                        float old[8];
 #pragma unroll
-                    for (int i = 0; i < 32; i++) r[i] += __uint_as_float(t[i]);
-                }
-                if (whole) {
-                    if (n < p.N) {
+                        for (int u = 0; u < 8; u++) old[u] = (p.accumulate && m0 + h + u < p.M) ? out[(h + u) * p.ldc] : 0.f;
 #pragma unroll
-                        for (int i = 0; i < 32; i++)
-                            if (c + i < p.M) finish(c + i, r[i]);
+                        for (int u = 0; u < 8; u++)
+                            if (m0 + h + u < p.M) out[(h + u) * p.ldc] = p.accumulate ? acc[h + u] * f1 * f2 + old[u] : acc[h + u] * f1 * f2;
                     }
                 } else {
+                    unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + (long long)m0 * p.ldc + n;
 #pragma unroll
-                    for (int i = 0; i < 32; i++)
-                        if (c + i < mp) __stcg(mine + (c + i) * BM, r[i]);
+                    for (int h = 0; h < 16; h += 8) {
+                        uint32_t old[8];
+#pragma unroll
+                        for (int u = 0; u < 8; u++) old[u] = (p.accumulate && m0 + h + u < p.M) ? (uint32_t)out[(h + u) * p.ldc] << 16 : 0u;
+#pragma unroll
+                        for (int u = 0; u < 8; u++) {
+                            float v = acc[h + u] * f1 * f2;
+                            if (p.accumulate) v += __uint_as_float(old[u]);
+                            unsigned short b;
+                            asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b) : "f"(v));  // round to nearest even; a NaN stays a NaN
+                            if (m0 + h + u < p.M) out[(h + u) * p.ldc] = b;
+                        }
+                    }
+                }
+            };
+            if (!mbar_wait(bar_acc_full(buf), use & 1, abort_flag, p.status, 35)) break;
+            tc_fence_after();
+#pragma unroll 1
+            for (int c = 0; c < mp; c += 16) {
+                float r[16];  // this lane's row of the segment's sum, columns c .. c + 15: the issuers' accumulators added in order
+#pragma unroll
+                for (int i = 0; i < 16; i++) r[i] = 0.f;
+#pragma unroll 1
+                for (int q = 0; q < issuers; q += 2) {
+                    // issuer q took the k-blocks it = q (mod issuers): none of them in a short segment leaves its accumulator stale
+                    const bool live0 = it_n >= issuers || ((q - it_a) & (issuers - 1)) < it_n;
+                    const bool live1 = it_n >= issuers || ((q + 1 - it_a) & (issuers - 1)) < it_n;
+                    uint32_t t0[16], t1[16];
+                    tmem_ld_32x32b_x16(tlane + acc_col(q, buf) + c, t0);
+                    tmem_ld_32x32b_x16(tlane + acc_col(q + 1, buf) + c, t1);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 16; i++) {
+                        if (live0) r[i] += __uint_as_float(t0[i]);
+                        if (live1) r[i] += __uint_as_float(t1[i]);
+                    }
+                }
+                if (whole) finish16(c, r);
+                else {
+#pragma unroll
+                    for (int i = 0; i < 16; i++) __stcg(mine + (c + i) * BM, r[i]);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty(buf));  // the accumulator has been read: it may be overwritten
             if (!whole) {
-                __threadfence();
-                __syncwarp();
+                // the warp's slice is complete; lane 0's release covers what the other lanes stored before the barrier
                 unsigned prior = 0;
-                if (lane == 0) prior = atomicAdd(plan.tickets + j * kEpiWarps + warp, 1u);
+                if (lane == 0)
+                    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prior) : "l"(plan.tickets + slab * kEpiWarps + warp) : "memory");
                 prior = __shfl_sync(0xFFFFFFFFu, prior, 0);
                 if (prior == (unsigned)(count - 1)) {  // every slice of this quarter slab is complete
                     __threadfence();
-                    if (n < p.N) {
-                        // sixteen rows at a time: their loads are independent, so the L2 latency is paid once per slice
-                        for (int m0 = 0; m0 < p.M; m0 += 16) {
-                            float acc[16];
-                            if (count == 2) {
-                                // two contributors (the usual case): both slices' loads in flight together, same order of addition
-                                float v0[16], v1[16];
+                    // sixteen rows at a time: their loads are independent, so the L2 latency is paid once per two slices
+#pragma unroll 1
+                    for (int m0 = 0; m0 < mp; m0 += 16) {
+                        const float* sl = slab_part + (size_t)m0 * BM;  // m0 + 15 < mp: mp is a multiple of 16
+                        float acc[16], v[16];
 #pragma unroll
-                                for (int u = 0; u < 16; u++) v0[u] = __ldcg(slab_part + (size_t)m0 * BM + u * BM);
+                        for (int u = 0; u < 16; u++) acc[u] = __ldcg(sl + u * BM);
+                        sl += (size_t)mp * BM;  // (a slab that is not whole has two contributors at least)
 #pragma unroll
-                                for (int u = 0; u < 16; u++) v1[u] = __ldcg(slab_part + ((size_t)mp + m0) * BM + u * BM);
+                        for (int u = 0; u < 16; u++) v[u] = __ldcg(sl + u * BM);
 #pragma unroll
-                                for (int u = 0; u < 16; u++)
-                                    if (m0 + u < p.M) finish(m0 + u, (0.f + v0[u]) + v1[u]);
-                                continue;
-                            }
+                        for (int u = 0; u < 16; u++) acc[u] = (0.f + acc[u]) + v[u];
+#pragma unroll 1
+                        for (int i = 2; i < count; i++) {
+                            sl += (size_t)mp * BM;
 #pragma unroll
-                            for (int u = 0; u < 16; u++) acc[u] = 0.f;
-                            for (int i = 0; i < count; i++) {
-                                const float* sl = slab_part + ((size_t)i * mp + m0) * BM;  // m0 + 15 < mp: mp is a multiple of 16
-                                float v[16];
+                            for (int u = 0; u < 16; u++) v[u] = __ldcg(sl + u * BM);
 #pragma unroll
-                                for (int u = 0; u < 16; u++) v[u] = __ldcg(sl + u * BM);
-#pragma unroll
-                                for (int u = 0; u < 16; u++) acc[u] += v[u];
-                            }
-#pragma unroll
-                            for (int u = 0; u < 16; u++)
-                                if (m0 + u < p.M) finish(m0 + u, acc[u]);
+                            for (int u = 0; u < 16; u++) acc[u] += v[u];
                         }
+                        finish16(m0, acc);
                     }
                 }
             }
-            lin = seg_end;
+            done += len; pb_a = 0; slab++;
         }
     }
 
@@ -1880,16 +1924,17 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         if (!okn) return HIF8_ERR_CUDA;
         const long long slabs = (N + BM - 1) / BM, num_pb = (K + BK2 - 1) / BK2;  // pair blocks: two k-blocks
         NarrowPlan plan{};
-        plan.total = slabs * num_pb;
+        const long long total = slabs * num_pb;
+        if (total > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
         // One CTA per SM, equal k-block ranges, when the workspace holds the partial sums of the slabs that a range
         // boundary cuts; otherwise one CTA per slab.
         long long grid = slabs;
         {
             // aim at four or more pair blocks per CTA, but never fewer CTAs than the per-slab grid would keep busy
-            long long g = plan.total / 4 < sm_count ? plan.total / 4 : sm_count;
+            long long g = total / 4 < sm_count ? total / 4 : sm_count;
             const long long floor_g = slabs < sm_count ? slabs : sm_count;
             if (g < floor_g) g = floor_g;
-            const long long per = plan.total / g;
+            const long long per = total / g;
             const long long pmax = (num_pb + per - 1) / per + 1;
             const size_t ticket_bytes = (((size_t)slabs * kEpiWarps * 4) + 255) & ~(size_t)255;
             const size_t part_bytes = (size_t)slabs * pmax * mp * BM * 4;
@@ -1903,6 +1948,7 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
             }
         }
         if (grid > 0x7FFFFFFFll) return HIF8_ERR_SHAPE;
+        plan.q = (int)(total / grid); plan.rem = (int)(total % grid);
         // With room left for the activations as BF16 (2 M K bytes behind the partial sums) they are expanded once, here,
         // and their tiles are copied straight into the operand stages: otherwise every CTA decodes the activation tile of
         // every k-block again for each of its slabs, a seventh (16 rows) to a third (64 rows) of the kernel's table lookups.
