@@ -205,6 +205,17 @@ __device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_
           "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
 }
+// 16 lanes x 32 columns (lane field of taddr = the first of the sixteen): thread t holds, for column octet j, columns
+// 8 j + 2 (t % 4) and + 1 of lane t / 4 in r[4 j], r[4 j + 1] and of lane t / 4 + 8 in r[4 j + 2], r[4 j + 3]
+__device__ __forceinline__ void tmem_st_16x256b_x4(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // ---- CTA pairs (cluster of two CTAs, cta_group::2)
@@ -339,10 +350,14 @@ __device__ __forceinline__ uint2 lds_v2(uint32_t addr)
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
     return v;
 }
-__device__ __forceinline__ uint32_t lds_u8(uint32_t addr)
+// Two 16 x 16 byte matrices, transposed: lane l gives the address of row l % 16 of matrix l / 16 (16 bytes); thread t gets
+// bytes 4 (t % 4) .. + 3 of the first matrix's column t / 4 in v.x and of its column t / 4 + 8 in v.y, the second one's in
+// v.z and v.w.
+__device__ __forceinline__ uint4 ldmatrix_trans_bytes_x2(uint32_t addr)
 {
-    uint32_t v;
-    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(addr));
+    uint4 v;
+    asm volatile("ldmatrix.sync.aligned.m16n16.x2.trans.shared.b8 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ uint4 lds_v4(uint32_t addr)
@@ -969,53 +984,61 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 // consecutive lanes on consecutive n.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kNarrowMaxM = 64;
-constexpr uint32_t kNwW8 = BM * BK, kNwA8 = kNarrowMaxM * BK;          // byte tiles per stage: 8 KiB weights, 4 KiB activations
-constexpr uint32_t kNwABf = kNarrowMaxM * BK * 2;  // activation operand tile per stage: 8 KiB (the weights go to tensor memory)
+constexpr uint32_t kNwW8 = BM * BK;  // weight bytes of a k-block: 8 KiB
 // A copy brings two k-blocks (a "pair block": 128 bytes of k) of weights and of activations: issuing a tile copy costs
 // its thread a few hundred cycles whatever the size, and with one copy of each kind per k-block that thread set the pace.
-// Four stages of 16 KiB + 8 KiB: 64 KiB of weights in flight per SM (a fifth stage changed nothing).
-constexpr int kNwByteStages = 4, BK2 = 2 * BK;
-// Operand stages (32 tensor-memory columns of weights + 8 KiB of activations in shared memory each): two per group, so
+constexpr int BK2 = 2 * BK;
+// Byte stages (one pair block of weights each, and of activations when they are bytes).  The weight stream needs about
+// 64 KiB per SM in flight for the rate of HBM, so six stages of 16 KiB where they fit: with four, and with the
+// activation tiles issued by the thread that issues the weight copies (which then waited for MMAs before it asked for the next weights), a kernel without any lookups still took 54 of 63 us at 16 x 28672 x 8192; now 59 us with them (64 rows:
+// 72 -> 67 us).  The number is even: each decode group then meets the same stages in every round.
+constexpr int kNwMaxByteStages = 6, kNwMinByteStages = 4;
+// Operand stages (32 tensor-memory columns of weights + mp rows of activations in shared memory each): two per group, so
 // that a group starts its next k-block without waiting for the MMAs of its previous one
 constexpr int kNwTmemStages = 2 * kDecodeGroups;
-struct SmemLayoutN {
-    static constexpr uint32_t bf = 0;
-    static constexpr uint32_t u8 = bf + kNwTmemStages * kNwABf;
-    static constexpr uint32_t lut = u8 + kNwByteStages * 2 * (kNwW8 + kNwA8);
-    static constexpr uint32_t bars = lut + 256 * 32 * 4;
-    static constexpr uint32_t n_bars = 2 * kNwByteStages + 2 * kNwTmemStages + 4;
-    static constexpr uint32_t tmem_slot = bars + n_bars * 8;
-    static constexpr uint32_t abort_flag = tmem_slot + 4;
-    static constexpr uint32_t total = abort_flag + 4;
-};
-constexpr uint32_t kSmemBytesN = SmemLayoutN::total + 1024;
-// Where the narrow kernel keeps what.  WIDE = false: the fixed layout above.  WIDE = true ([N,K] weights with the activations
-// expanded beforehand: the byte stages hold weights only, 16 KiB each): the decode table has rows of 256 bytes and starts on a 64 KiB boundary
-// of the shared window, so that one byte permute makes a lookup's address (see decode8); as many operand stages (8 KiB) as
-// fit lie in front of it, the other operand stages, the byte stages and the barriers behind it.
-template <bool WIDE>
+constexpr uint32_t kNwBars = 2 * kNwMaxByteStages + 2 * kNwTmemStages + 4;
+constexpr uint32_t kSmemBytesN = 227 * 1024;  // the whole opt-in maximum; the kernel checks that its layout fits
+// Where the narrow kernel keeps what (mp activation rows).  WIDE ([N,K] weights with the activations expanded beforehand):
+// the decode table has rows of 256 bytes and starts on a 64 KiB boundary of the shared window, so that one byte permute makes
+// a lookup's address (see decode8); operand stages and then byte stages as they fit in front of it, the rest behind it.
+// Otherwise: operand stages, byte stages and the 32 KiB table in a row.
+template <bool WIDE, bool ACT_BF16>
 struct NarrowSmem {
     uint32_t base, lut, bars, end;  // shared-window addresses; base is 1024-byte aligned
-    uint32_t behind, u8_0;
-    int n_front;
-    __device__ explicit NarrowSmem(uint32_t raw)
+    uint32_t behind_act, behind_u8, front_u8, act_bytes, u8_bytes;
+    int act_front, u8_front, stages8;
+    __device__ NarrowSmem(uint32_t raw, uint32_t limit, int mp)
     {
         base = (raw + 1023u) & ~1023u;
+        act_bytes = ((uint32_t)mp * BK * 2u + 1023u) & ~1023u;
+        u8_bytes = 2 * kNwW8 + (ACT_BF16 ? 0u : ((uint32_t)mp * BK2 + 1023u) & ~1023u);
+        stages8 = kNwMaxByteStages;
+        place();
+        if (end > limit) { stages8 = kNwMinByteStages; place(); }
+    }
+    __device__ void place()
+    {
         if (!WIDE) {
-            lut = base + SmemLayoutN::lut; bars = base + SmemLayoutN::bars; end = base + SmemLayoutN::total;
-            behind = 0; u8_0 = base + SmemLayoutN::u8; n_front = kNwTmemStages;
+            act_front = kNwTmemStages; u8_front = stages8; behind_act = behind_u8 = 0;
+            front_u8 = base + kNwTmemStages * act_bytes;
+            lut = front_u8 + (uint32_t)stages8 * u8_bytes;
+            bars = lut + kLutBytesNarrow;
         } else {
             lut = (base + kLutBytesWide - 1) & ~(kLutBytesWide - 1);
-            n_front = (int)min((lut - base) / kNwABf, (uint32_t)kNwTmemStages);
-            behind = lut + kLutBytesWide;
-            u8_0 = behind + (uint32_t)(kNwTmemStages - n_front) * kNwABf;
-            bars = u8_0 + kNwByteStages * 2 * kNwW8;
-            end = bars + SmemLayoutN::n_bars * 8 + 8;
+            const uint32_t front = lut - base;
+            act_front = kNwTmemStages;
+            while ((uint32_t)act_front * act_bytes > front) act_front--;
+            front_u8 = base + (uint32_t)act_front * act_bytes;
+            u8_front = (int)min((lut - front_u8) / (2 * kNwW8), (uint32_t)stages8);  // (WIDE: weights only)
+            behind_act = lut + kLutBytesWide;
+            behind_u8 = behind_act + (uint32_t)(kNwTmemStages - act_front) * act_bytes;
+            bars = behind_u8 + (uint32_t)(stages8 - u8_front) * u8_bytes;
         }
+        end = bars + kNwBars * 8 + 8;
     }
-    __device__ uint32_t bf(int s) const { return s < n_front ? base + (uint32_t)s * kNwABf : behind + (uint32_t)(s - n_front) * kNwABf; }
-    __device__ uint32_t u8(int s) const { return u8_0 + (uint32_t)s * (WIDE ? 2 * kNwW8 : 2 * (kNwW8 + kNwA8)); }
-    __device__ uint32_t tmem_slot() const { return bars + SmemLayoutN::n_bars * 8; }
+    __device__ uint32_t bf(int s) const { return s < act_front ? base + (uint32_t)s * act_bytes : behind_act + (uint32_t)(s - act_front) * act_bytes; }
+    __device__ uint32_t u8(int s) const { return s < u8_front ? front_u8 + (uint32_t)s * u8_bytes : behind_u8 + (uint32_t)(s - u8_front) * u8_bytes; }
+    __device__ uint32_t tmem_slot() const { return bars + kNwBars * 8; }
     __device__ uint32_t abort_flag() const { return tmem_slot() + 4; }
 };
 // Tensor memory: the accumulators (two per issuer: the epilogue of one segment overlaps the next segment's MMAs), then
@@ -1023,10 +1046,10 @@ struct NarrowSmem {
 // MMA issuers.  One thread that waits for a stage, issues its four MMAs and commits spends about a thousand cycles per
 // k-block, more than the decode groups or the copies need; so up to four threads (one per warp) share the k-blocks,
 // issuer q taking the k-blocks it = q (mod issuers) into accumulators of its own, which the epilogue adds.  Up to 32
-// activation rows every issuer has two accumulators; above that either four issuers with one accumulator each or two with
-// two (the kernel says which): issuers x buffers x rows stays within 256 columns.
+// activation rows every issuer has two accumulators, above that one: issuers x buffers x rows stays within 256 columns.
 constexpr int kNwMaxIssuers = 4;
-constexpr int kThreadsN = kThreads + (kNwMaxIssuers - 1) * 32;  // 800: the first issuer is the MMA warp of the other kernels
+// the first issuer is the MMA warp of the other kernels; the warp behind the others copies expanded activations
+constexpr int kNwActWarp = kThreads / 32 + kNwMaxIssuers - 1, kThreadsN = (kNwActWarp + 1) * 32;  // 832
 constexpr uint32_t kTmemAccN = 2 * 2 * kNarrowMaxM, kTmemColsN = 512;
 static_assert(kTmemAccN + kNwTmemStages * (BK / 2) <= kTmemColsN, "weight stages fit beside the accumulators");
 static_assert(2 * kNwMaxIssuers * 32 <= kTmemAccN, "four issuers x two buffers x 32 rows");
@@ -1047,6 +1070,7 @@ struct NarrowPlan {
     float* part;         // [slab][pmax][mp][128] partial sums, or nullptr when every range is made of whole slabs
     unsigned* tickets;   // [slab][4], zero at launch
     int pmax;            // slices per slab
+    int clear_status;    // nonzero: no launch in front of this one clears the status word
 
     __device__ int first(int c) const { return c * q + (c < rem ? c : rem); }  // first unit of CTA c
     __device__ int owner(int x) const                                          // the CTA that takes unit x
@@ -1088,15 +1112,16 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                         const NarrowPlan plan)
 {
     extern __shared__ unsigned char smem_raw[];
-    // the 64 KiB table pays for [N,K] weights, whose bytes are extracted from registers (76 against 85 us at 16 x 28672 x 8192);
-    // [K,N] weights arrive a byte per load and ran slower with it (84 against 81 us)
-    constexpr bool kWideN = ACT_BF16 && W_IS_NK;
+    // the 64 KiB table fits once no activations are decoded here (76 against 85 us at 16 x 28672 x 8192, [N,K])
+    constexpr bool kWideN = ACT_BF16;
     constexpr int kLutShiftN = kWideN ? 8 : 7;
-    const NarrowSmem<kWideN> lay(smem_u32(smem_raw));
+    uint32_t dyn_bytes;
+    asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
+    // (a wait that gives up does so two seconds into the kernel, long after this; a separate launch cost 2 us)
+    if (!ACT_BF16 && plan.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile int*>(p.status) = 0;
+    const NarrowSmem<kWideN, ACT_BF16> lay(smem_u32(smem_raw), smem_u32(smem_raw) + dyn_bytes, mp);
     unsigned char* sm = smem_raw - smem_u32(smem_raw);  // generic pointer of shared-window address 0
     {
-        uint32_t dyn_bytes;
-        asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
         if (lay.end > smem_u32(smem_raw) + dyn_bytes) {  // the layout does not fit (the same answer in every thread)
             if (ACT_BF16) asm volatile("griddepcontrol.wait;" ::: "memory");  // (the launch in front clears the status word)
             if (threadIdx.x == 0) atomicCAS(p.status, 0, 7);
@@ -1106,15 +1131,16 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int S = kNwTmemStages;  // operand ring: the it-th k-block uses stage it % S
     static_assert(S % kDecodeGroups == 0, "an operand stage is always written by the same group");
-    constexpr int S8 = kNwByteStages;   // byte ring: the i-th pair block of this CTA lands in stage i % S8
+    const int S8 = lay.stages8;         // byte ring: the i-th pair block of this CTA lands in stage i % S8
+    constexpr int kS8 = kNwMaxByteStages;
     constexpr uint32_t kU8Act = 2 * kNwW8;  // byte stage: 128 weight columns x 128 k, then (activations as bytes) act rows x 128 k
     const uint32_t bars = lay.bars;
     auto bar_u8_full = [&](int s) { return bars + 8u * s; };
-    auto bar_u8_empty = [&](int s) { return bars + 8u * (S8 + s); };
-    auto bar_bf_full = [&](int s) { return bars + 8u * (2 * S8 + s); };
-    auto bar_bf_empty = [&](int s) { return bars + 8u * (2 * S8 + S + s); };
-    auto bar_acc_full = [&](int b) { return bars + 8u * (2 * S8 + 2 * S + b); };
-    auto bar_acc_empty = [&](int b) { return bars + 8u * (2 * S8 + 2 * S + 2 + b); };
+    auto bar_u8_empty = [&](int s) { return bars + 8u * (kS8 + s); };
+    auto bar_bf_full = [&](int s) { return bars + 8u * (2 * kS8 + s); };
+    auto bar_bf_empty = [&](int s) { return bars + 8u * (2 * kS8 + S + s); };
+    auto bar_acc_full = [&](int b) { return bars + 8u * (2 * kS8 + 2 * S + b); };
+    auto bar_acc_empty = [&](int b) { return bars + 8u * (2 * kS8 + 2 * S + 2 + b); };
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + lay.abort_flag());
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + lay.tmem_slot());
     uint32_t* lut_all = reinterpret_cast<uint32_t*>(sm + lay.lut);
@@ -1124,17 +1150,16 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     const int n_pairs = pair1 - pair0, n_it = 2 * n_pairs;
     const int slab0 = pair0 / num_pb, pb0 = pair0 - slab0 * num_pb;  // where the range starts
     const uint32_t act_bytes = (uint32_t)mp * BK2;
-    // Up to 32 activation rows: four issuers with two accumulators each (the epilogue of one segment overlaps the next
-    // segment's MMAs).  Above that issuers x buffers x rows must stay within 256 columns: four issuers with one accumulator
-    // for [N,K] weights (91 against 94 us at 64 x 28672 x 8192), two with two for [K,N] weights (92 against 95 us).
-    const int issuers = (mp <= 32 || W_IS_NK) ? kNwMaxIssuers : 2;
-    const int bufs = (mp <= 32 || issuers == 2) ? 2 : 1;
+    // Up to 32 activation rows every issuer has two accumulators (the epilogue of one segment overlaps the next segment's
+    // MMAs).  Above that issuers x buffers x rows must stay within 256 columns, and four issuers with one accumulator each
+    // are faster than two with two (91 against 94 us at 64 x 28672 x 8192 when that was the whole call).
+    constexpr int issuers = kNwMaxIssuers;
+    const int bufs = mp <= 32 ? 2 : 1;
     auto acc_col = [&](int q, int buf) { return (uint32_t)((q * bufs + buf) * mp); };  // accumulator of issuer q, buffer buf
 
-    // copies of unit i of the range: its weight bytes (and, as bytes, its activations) into stage i % S8
+    // copies of the range's next unit: its weight bytes (and, as bytes, its activations) into stage s
     int cp_slab = slab0, cp_pb = pb0;
-    auto copy_bytes = [&](int i) {
-        const int s = i % S8;
+    auto copy_bytes = [&](int s) {
         const uint32_t dst_w = lay.u8(s), dst_a = dst_w + kU8Act;
         const uint64_t w_policy = l2_policy_evict_first();
         mbar_arrive_expect_tx(bar_u8_full(s), 2 * kNwW8 + (ACT_BF16 ? 0u : act_bytes));
@@ -1145,7 +1170,7 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
         if (!ACT_BF16) tma_load_2d(dst_a, &map_act, cp_pb * BK2, 0, bar_u8_full(s));
         if (++cp_pb == num_pb) { cp_pb = 0; cp_slab++; }
     };
-    const int n_early = min(S8, n_pairs);
+    const int n_early = min(2, n_pairs);
     if (threadIdx.x == kTmaWarp * 32) {
         for (int s = 0; s < S8; s++) { mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), 2 * kGroupWarps); }  // both halves' groups
         // operands ready: the group's warps, plus (ACT_BF16) the announcement of the activation tile's bytes
@@ -1154,7 +1179,8 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        // The first round of byte copies starts here, under the table set-up: nothing in front of this kernel writes the
+        // The first byte copies start here, under the table set-up (two of them: each takes this thread a few hundred cycles,
+        // and the block waits for it): nothing in front of this kernel writes the
         // operands (the launch before it writes the expanded activations and the cleared words only, and that launch itself
         // waits for everything before it).
         for (int i = 0; i < n_early; i++) copy_bytes(i);
@@ -1171,45 +1197,46 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     const uint32_t tmem_base = *tmem_slot;
     // The launch in front of this kernel expands the activations and clears the status word and the tickets; this kernel was
     // started while that one ran, so that the set-up above overlaps it.  From here on its results are complete.
-    if (ACT_BF16) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (Not the weight producer: it reads none of them.)
+    if (ACT_BF16 && warp != kTmaWarp) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp == kTmaWarp) {
         if (lane == 0) {
-            int issued = n_early, issued_act = 0;
-            bool aborted = false;
-            int pb = pb0;
-            for (int it = 0; it < n_pairs; it++) {
-                if (it >= S8) {
-                    if (!mbar_wait(bar_u8_empty(it % S8), (it / S8 - 1) & 1, abort_flag, p.status, 31)) break;
-                    if (*abort_flag) break;
-                    copy_bytes(it);
-                    issued = it + 1;
-                }
-                if (ACT_BF16) {
-                    // Activations expanded to BF16 beforehand (map_act is then the map of that copy): the tiles of the pair's
-                    // two k-blocks go straight into their operand stages, in the 128-byte-swizzled layout the MMA reads, once
-                    // the MMAs of each stage's previous use have read it.  (The byte copy above is needed eight k-blocks later;
-                    // these are needed by the end of their k-block's decode, and their waits end about when the next byte
-                    // stage falls free, so one thread keeps both streams going.)
-                    for (int h = 0; h < 2 && !aborted; h++) {
-                        const int ik = 2 * it + h, sb = ik % S, rb = ik / S;
-                        if (rb > 0 && !mbar_wait(bar_bf_empty(sb), (rb - 1) & 1, abort_flag, p.status, 37)) { aborted = true; break; }
-                        mbar_arrive_expect_tx(bar_bf_full(sb), (uint32_t)mp * BK * 2u);
-                        tma_load_2d(lay.bf(sb), &map_act, (2 * pb + h) * BK, 0, bar_bf_full(sb));
-                        issued_act = ik + 1;
-                    }
-                    if (aborted) break;
-                }
-                if (++pb == num_pb) pb = 0;
+            int issued = n_early, s = n_early;
+            uint32_t ph = 1;  // parity of the round before the one that fills stage s next
+            for (int it = n_early; it < n_pairs; it++) {
+                if (it >= S8 && !mbar_wait(bar_u8_empty(s), ph, abort_flag, p.status, 31)) break;
+                if (*abort_flag) break;
+                copy_bytes(s);
+                issued = it + 1;
+                if (++s == S8) { s = 0; ph ^= 1u; }
             }
             if (*abort_flag) {  // let the copies already issued land before this CTA's shared memory goes away
                 for (int it = max(0, issued - S8); it < issued; it++) {
                     const unsigned long long t0 = global_ns();
                     while (!mbar_try_wait(bar_u8_full(it % S8), (it / S8) & 1) && global_ns() - t0 < kWaitLimitNs) {}
                 }
-                for (int ik = max(0, issued_act - S); ik < issued_act; ik++) {
+            }
+        }
+    } else if (warp == kNwActWarp) {
+        // Activations expanded to BF16 beforehand (map_act is then the map of that copy): the tile of every k-block goes
+        // straight into its operand stage, in the 128-byte-swizzled layout the MMA reads, once the MMAs of the stage's
+        // previous use have read it.
+        if (ACT_BF16 && lane == 0) {
+            int issued = 0, kb = 2 * pb0;
+            for (int it = 0; it < n_it; it++) {
+                const int sb = it % S, rb = it / S;
+                if (rb > 0 && !mbar_wait(bar_bf_empty(sb), (rb - 1) & 1, abort_flag, p.status, 37)) break;
+                if (*abort_flag) break;
+                mbar_arrive_expect_tx(bar_bf_full(sb), (uint32_t)mp * BK * 2u);
+                tma_load_2d(lay.bf(sb), &map_act, kb * BK, 0, bar_bf_full(sb));
+                issued = it + 1;
+                if (++kb == num_kb) kb = 0;
+            }
+            if (*abort_flag) {
+                for (int it = max(0, issued - S); it < issued; it++) {
                     const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(bar_bf_full(ik % S), (ik / S) & 1) && global_ns() - t0 < kWaitLimitNs) {}
+                    while (!mbar_try_wait(bar_bf_full(it % S), (it / S) & 1) && global_ns() - t0 < kWaitLimitNs) {}
                 }
             }
         }
@@ -1258,23 +1285,38 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
         const int dt = threadIdx.x - (kFirstDecodeWarp + group * kGroupWarps) * 32;
         const int act_chunks = mp * (BK / 8);  // 8-byte chunks of the activation tile
         bool ok = true;
+        int s8 = group >> 1;  // byte stage of the group's next k-block, and the parity of its round
+        uint32_t ph8 = 0;
+        const int h = group & 1;  // which k-block of its pair block
         for (int it = group; it < n_it && ok; it += kDecodeGroups) {
-            const int s = it % S, r = it / S, s8 = (it >> 1) % S8, h = it & 1;  // h: which k-block of its pair block
-            ok = mbar_wait(bar_u8_full(s8), ((it >> 1) / S8) & 1, abort_flag, p.status, 33);
+            const int s = it % S, r = it / S;
+            ok = mbar_wait(bar_u8_full(s8), ph8, abort_flag, p.status, 33);
             if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 34);
             if (!ok) break;
             const uint32_t w8 = lay.u8(s8), a8 = w8 + kU8Act + (uint32_t)h * BK;
             const uint32_t abf = lay.bf(s);
             uint2 va[kNarrowMaxM * (BK / 8) / kGroupThreads];
             uint4 vr[BK / 16];
-            // this thread owns weight column (operand row, tensor-memory lane) quarter * 32 + lane of the slab
-            const int wr = (warp & 3) * 32 + lane;
+            // this warp's 32 weight columns (operand rows, tensor-memory lanes): quarter * 32 ..
+            const int quarter = warp & 3;
             if (W_IS_NK) {
-                // [N,K] weights: the byte tile (rows of 128 k) arrives with the 128-byte TMA swizzle (chunk j of row r at chunk
-                // j ^ (r & 7)): conflict-free row reads
+                // [N,K] weights, a thread per column: the byte tile (rows of 128 k) arrives with the 128-byte TMA swizzle (chunk
+                // j of row r at chunk j ^ (r & 7)): conflict-free row reads
+                const int wr = quarter * 32 + lane;
                 const uint32_t w_row = w8 + (uint32_t)wr * BK2, sw = (uint32_t)wr & 7u;
 #pragma unroll
                 for (int jj = 0; jj < BK / 16; jj++) vr[jj] = lds_v4(w_row + (((uint32_t)(4 * h + jj) ^ sw) << 4));
+            } else {
+                // [K,N] weights: the rows of the tile are k, 128 columns each, with the same swizzle.  16 x 16 byte matrices
+                // are read transposed, so that a thread holds four consecutive k of a column: vr[2 i + c] = k 32 i .. 32 i + 31
+                // of the quarter's columns 16 c .. 16 c + 15.  (Read a byte per load, a k-block took 256 more shared-memory
+                // wavefronts, as many as its lookups.)
+                const int k = h * BK + lane;
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+#pragma unroll
+                    for (int c = 0; c < 2; c++)
+                        vr[2 * i + c] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(k + 32 * i) * BM + ((uint32_t)((2 * quarter + c) ^ (lane & 7)) << 4));
             }
             if (!ACT_BF16) {
 #pragma unroll
@@ -1283,32 +1325,31 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                     if (q < act_chunks) va[i] = lds_v2(a8 + (q >> 3) * BK2 + (q & 7) * 8);
                 }
             }
-            uint32_t o[BK / 2];  // 64 BF16 of this weight column, two per tensor-memory column
+            __syncwarp();  // the byte stage has been read: the producer may refill it during the decode
+            if (lane == 0) mbar_arrive(bar_u8_empty(s8));
+            uint32_t o[BK / 2];  // two BF16 per tensor-memory column
+            const uint32_t st_base = tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemAccN + (uint32_t)(s * (BK / 2));
             if (W_IS_NK) {
-                __syncwarp();  // the byte stage has been read: the producer may refill it during the decode
-                if (lane == 0) mbar_arrive(bar_u8_empty(s8));
 #pragma unroll
                 for (int jj = 0; jj < BK / 16; jj++) {
                     const uint4 lo = decode8<kLutShiftN>(make_uint2(vr[jj].x, vr[jj].y), lut), hi = decode8<kLutShiftN>(make_uint2(vr[jj].z, vr[jj].w), lut);
                     o[8 * jj + 0] = lo.x; o[8 * jj + 1] = lo.y; o[8 * jj + 2] = lo.z; o[8 * jj + 3] = lo.w;
                     o[8 * jj + 4] = hi.x; o[8 * jj + 5] = hi.y; o[8 * jj + 6] = hi.z; o[8 * jj + 7] = hi.w;
                 }
+                tmem_st_32x32b_x32(st_base, o);
             } else {
-                // [K,N] weights: row k of the pair's tile holds the 128 columns of the slab (the pair's second k-block is its
-                // rows 64-127), so the column is read a byte per k: the 32 lanes of a warp read 32 consecutive bytes, one
-                // wavefront, and the byte is the table row without any extraction
-                const uint32_t w_col = w8 + (uint32_t)h * kNwW8 + (uint32_t)wr;
 #pragma unroll
-                for (int j = 0; j < BK / 2; j++) {
-                    const uint32_t c0 = lds_u8(w_col + (uint32_t)(2 * j) * BM), c1 = lds_u8(w_col + (uint32_t)(2 * j + 1) * BM);
-                    // (rows of 256 bytes: the byte replaces byte 1 of the lane's table address, one permute)
-                    if (kLutShiftN == 8) o[j] = __byte_perm(lds_u32(__byte_perm(c0, lut, 0x7604)), lds_u32(__byte_perm(c1, lut, 0x7604)), 0x5410);
-                    else o[j] = __byte_perm(lds_u32(lut + (c0 << 7)), lds_u32(lut + (c1 << 7)), 0x5410);
+                for (int c = 0; c < 2; c++) {
+#pragma unroll
+                    for (int i = 0; i < 2; i++) {
+                        const uint4 v = vr[2 * i + c];
+                        const uint4 lo = decode8<kLutShiftN>(make_uint2(v.x, v.y), lut), hi = decode8<kLutShiftN>(make_uint2(v.z, v.w), lut);
+                        uint32_t* d = o + 16 * c + 8 * i;
+                        d[0] = lo.x; d[1] = lo.y; d[2] = lo.z; d[3] = lo.w; d[4] = hi.x; d[5] = hi.y; d[6] = hi.z; d[7] = hi.w;
+                    }
+                    tmem_st_16x256b_x4(st_base + ((uint32_t)(16 * c) << 16), o + 16 * c);
                 }
-                __syncwarp();  // the byte stage has been read
-                if (lane == 0) mbar_arrive(bar_u8_empty(s8));
             }
-            tmem_st_32x32b_x32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + kTmemAccN + (uint32_t)(s * (BK / 2)), o);
             if (!ACT_BF16) {
 #pragma unroll
                 for (int i = 0; i < kNarrowMaxM * (BK / 8) / kGroupThreads; i++) {
@@ -1321,6 +1362,8 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_bf_full(s));
+            s8 += 2;
+            if (s8 >= S8) { s8 -= S8; ph8 ^= 1u; }
         }
     } else {
         // epilogue warps 0-3: TMEM lane = weight column n, TMEM column = activation row m.  Whatever does not need the sums
@@ -1785,7 +1828,7 @@ bool gemm_kernels_ready(int dev, int* sm_count_out)
         const void* narrow[4] = {(const void*)hif8_gemm_narrow_kernel<false, false>, (const void*)hif8_gemm_narrow_kernel<false, true>,
                                  (const void*)hif8_gemm_narrow_kernel<true, false>, (const void*)hif8_gemm_narrow_kernel<true, true>};
         for (int i = 0; i < 4 && out->rc == cudaSuccess; i++)
-            out->rc = cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, i == 3 ? kSmemBytesWide : kSmemBytesN);  // (the last one: wide table)
+            out->rc = cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesN);
         if (out->rc == cudaSuccess) out->rc = cudaDeviceGetAttribute(&out->sm_count, cudaDevAttrMultiProcessorCount, d);
     });
     if (!s) return false;
@@ -1918,9 +1961,9 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         const int mp = (M + 15) & ~15;
         CUtensorMap map_act, map_ws;
         if (!make_map(&map_act, Aq, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK2, (uint32_t)mp)) return HIF8_ERR_CUDA;
-        // ([N,K] weights: 64-byte rows with the 64-byte swizzle, read row-wise and decoded into tensor memory)
+        // (weight tiles: 128-byte rows with the 128-byte swizzle, of 128 k or of 128 columns)
         const bool okn = w_is_nk ? make_map(&map_ws, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, BK2, BM, false, 128)
-                                 : make_map(&map_ws, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, BK2);
+                                 : make_map(&map_ws, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, BK2, false, 128);
         if (!okn) return HIF8_ERR_CUDA;
         const long long slabs = (N + BM - 1) / BM, num_pb = (K + BK2 - 1) / BK2;  // pair blocks: two k-blocks
         NarrowPlan plan{};
@@ -1969,11 +2012,12 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
                 act_bf16 = true;
             }
         }
-        if (!act_bf16 && cudaMemsetAsync(workspace, 0, clear_bytes, st) != cudaSuccess) return HIF8_ERR_CUDA;
+        plan.clear_status = !act_bf16 && !plan.tickets;
+        if (!act_bf16 && plan.tickets && cudaMemsetAsync(workspace, 0, clear_bytes, st) != cudaSuccess) return HIF8_ERR_CUDA;
         cudaLaunchConfig_t cn{};
         cn.gridDim = dim3((unsigned)grid);
         cn.blockDim = dim3(kThreadsN);
-        cn.dynamicSmemBytes = (act_bf16 && w_is_nk) ? kSmemBytesWide : kSmemBytesN;
+        cn.dynamicSmemBytes = kSmemBytesN;
         cn.stream = st;
         // with the preparing kernel right in front: programmatic stream serialization (that kernel lets its dependents start
         // at once; this one waits for its completion once its own set-up is done)
