@@ -45,7 +45,7 @@ namespace {
 constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int kStages8 = 4;    // staging ring of HiF8 byte tiles
 constexpr int kStagesBf = 4;   // ring of decoded BF16 operand tiles
-constexpr int kStagesBfSwapped = 4, kMaxStagesBf = 8;  // the swapped form (see hif8_gemm_kernel): stages of 128 k, twice the size
+constexpr int kMaxStagesBf = 8;
 constexpr int kEpiWarps = 4, kDecodeWarps = 16;
 // The decode warps work in groups, group g on the k-blocks kb = g (mod kDecodeGroups): several k-blocks are in the
 // decode stage at once, which covers the latency of each one's lookups, proxy fence and barrier hand-over.  Group g
@@ -267,10 +267,10 @@ __device__ __forceinline__ void tc_mma_bf16_cta_a_tmem(uint32_t d_tmem, uint32_t
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar)  // arrives on `bar` in both CTAs of the pair
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint32_t lead = 0)  // arrives on `bar` in both CTAs of the pair lead, lead + 1
 {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(bar), "h"((unsigned short)3) : "memory");
+                 ::"r"(bar), "h"((unsigned short)(3u << lead)) : "memory");
 }
 __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
 {
@@ -365,10 +365,6 @@ __device__ __forceinline__ uint4 lds_v4(uint32_t addr)
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
     return v;
-}
-__device__ __forceinline__ void sts_u16(uint32_t addr, unsigned short v)
-{
-    asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
 }
 __device__ __forceinline__ void sts_v4(uint32_t addr, uint4 v)
 {
@@ -550,13 +546,9 @@ constexpr uint32_t kSlotBytes = 16384, kLutBytesWide = 65536, kLutBytesNarrow = 
 static_assert(kBBfBytes == kSlotBytes && kA8Bytes + kB8Bytes == kSlotBytes, "one stage per slot");
 constexpr uint32_t kSmemBytesWide = 227 * 1024;  // the whole opt-in maximum; the kernel checks that its plan fits
 
-// PLAN 0: slots around the 64 KiB table.  1: the layout of SmemLayout (A operand tiles in shared memory).  2: the swapped
-// form -- eight operand stages of 16 KiB, four byte stages of 8 KiB, the 32 KiB table, barriers, one after the other.
-constexpr int kStages8Swapped = 4;  // byte stages of the swapped form (A bytes only, 128 k: 16 KiB each)
-constexpr uint32_t kSmemBytesSwapped = kStagesBfSwapped * 2 * kBBfBytes + kStages8Swapped * 2 * kA8Bytes + 256 * 32 * 4 + kBarsBytes + 1024;
-template <int PLAN>
+// FIXED: the layout of SmemLayout (A operand tiles in shared memory).
+template <bool FIXED>
 struct FusedSmem {
-    static constexpr bool FIXED = PLAN == 1;
     uint32_t base, lut, bars, behind;  // shared-window addresses; base is 1024-byte aligned
     int n_front;                       // slots in front of the table
     uint32_t end;                      // first byte behind everything
@@ -566,9 +558,6 @@ struct FusedSmem {
         base = (raw + 1023u) & ~1023u;
         if (FIXED) {
             lut = base + SmemLayout::lut; bars = base + SmemLayout::bars; behind = 0; n_front = 0; end = base + SmemLayout::total;
-        } else if (PLAN == 2) {
-            behind = 0; n_front = 2 * kStagesBfSwapped;
-            lut = base + kStagesBfSwapped * 2 * kBBfBytes + kStages8Swapped * 2 * kA8Bytes; bars = lut + kLutBytesNarrow; end = bars + kBarsBytes;
         } else if (!kWideLut) {
             // table with rows of 128 bytes: no alignment to honour, everything in a row: slots, table, barriers
             n_front = (int)kFusedSlots; behind = 0;
@@ -586,12 +575,8 @@ struct FusedSmem {
     }
     __device__ uint32_t slot(int i) const { return i < n_front ? base + (uint32_t)i * kSlotBytes : behind + (uint32_t)(i - n_front) * kSlotBytes; }
     __device__ uint32_t a_bf(int s) const { return base + SmemLayout::bf + s * (kABfBytes + kBBfBytes); }                       // FIXED only
-    __device__ uint32_t w_bf(int s) const { return PLAN == 2 ? base + (uint32_t)s * 2 * kBBfBytes : (FIXED ? a_bf(s) + kABfBytes : slot(s)); }
-    __device__ uint32_t a_u8(int s) const
-    {
-        if (PLAN == 2) return base + kStagesBfSwapped * 2 * kBBfBytes + (uint32_t)s * 2 * kA8Bytes;
-        return FIXED ? base + SmemLayout::u8 + s * (kA8Bytes + kB8Bytes) : slot(kStagesBf + s);
-    }
+    __device__ uint32_t w_bf(int s) const { return FIXED ? a_bf(s) + kABfBytes : slot(s); }
+    __device__ uint32_t a_u8(int s) const { return FIXED ? base + SmemLayout::u8 + s * (kA8Bytes + kB8Bytes) : slot(kStagesBf + s); }
     // staging box j (16 KiB) of the result tile: the operand stages, idle once the accumulator is complete
     __device__ uint32_t box(int j) const { return FIXED ? base + SmemLayout::bf + (uint32_t)j * kSlotBytes : slot(j); }
     __device__ uint32_t w_u8(int s) const { return a_u8(s) + kA8Bytes; }
@@ -599,27 +584,18 @@ struct FusedSmem {
     __device__ uint32_t abort_flag() const { return tmem_slot() + 4; }
 };
 
-// A_MODE 0: A given as [M,K] bytes, decoded into tensor memory.  1: A given as [K,M] bytes, decoded into shared memory
-// (MN-major operand).  2: A already expanded to BF16 [M,K] in the caller's workspace (only W is decoded here): its tiles
-// come by TMA straight into the K-major operand stages, completing on the leader's "operands ready" barrier.
-// SWAPPED (with A_MODE 0 and W_IS_NK): the kernel computes C^T = W^T A^T.  Its byte operand -- rows decoded into tensor
-// memory -- is the caller's [N,K] weight, its shared-memory operand the caller's activations, already expanded to BF16
-// [M,K] and brought by TMA; nothing decoded here is stored to shared memory or read back from it by the tensor core.  The
-// kernel's "M" is the caller's N and vice versa, and the epilogue writes the accumulator transposed.
-template <int A_MODE, bool W_IS_NK, bool SWAPPED = false>
+// A_IS_KM = false: A given as [M,K] bytes, decoded into tensor memory.  true: A given as [K,M] bytes, decoded into shared
+// memory (MN-major operand).
+template <bool A_IS_KM, bool W_IS_NK>
 __global__ void __launch_bounds__(kThreads, 1)
 hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                  const __grid_constant__ CUtensorMap map_c, const GemmParams p)
 {
     extern __shared__ unsigned char smem_raw[];
-    constexpr bool A_IS_KM = A_MODE == 1, A_BF16 = A_MODE == 2, kFixed = A_MODE != 0;
-    static_assert(!SWAPPED || (A_MODE == 0 && W_IS_NK), "the swapped form reads both operands K-major");
-    constexpr int kLutShift = (kFixed || SWAPPED || !kWideLut) ? 7 : 8;
-    constexpr int kS8 = SWAPPED ? kStages8Swapped : (kFixed ? kStages8 : kStages8Deep);  // depth of the byte ring
-    // operand stages: one per decode group, or (SWAPPED: nothing decoded goes to shared memory, which leaves the room) two, so
-    // that a group starts its next k-block while the MMAs of its last one are still queued behind the other groups'
-    constexpr int kSB = SWAPPED ? kStagesBfSwapped : kStagesBf;
-    const FusedSmem<SWAPPED ? 2 : (kFixed ? 1 : 0)> plan(smem_u32(smem_raw));
+    constexpr int kLutShift = (A_IS_KM || !kWideLut) ? 7 : 8;
+    constexpr int kS8 = A_IS_KM ? kStages8 : kStages8Deep;  // depth of the byte ring
+    constexpr int kSB = kStagesBf;  // operand stages: one per decode group
+    const FusedSmem<A_IS_KM> plan(smem_u32(smem_raw));
     const uint32_t base = plan.base;
     unsigned char* sm = smem_raw - smem_u32(smem_raw);  // generic pointer of shared-window address 0
     {
@@ -649,16 +625,13 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     int tile_m, tile_n;
     tile_coords((int)(blockIdx.x >> 1), (p.M + 2 * BM - 1) / (2 * BM), p.tiles_n, tile_m, tile_n);
     const int m0 = tile_m * 2 * BM + (int)rank * BM, n0 = tile_n * BN, nh = n0 + (int)rank * (BN / 2);
-    // k per operand stage: 64, or (SWAPPED) 128 -- one hand-over, one commit and one probe by the MMA thread per 128 k
-    constexpr int KB = SWAPPED ? 2 * BK : BK;
-    const int num_kb = (p.K + KB - 1) / KB;
+    const int num_kb = (p.K + BK - 1) / BK;
 
     // ---- set-up
     fill_decode_table<(1 << (kLutShift - 2))>(lut_all, warp, lane, kThreads / 32);  // rows of 1 << kLutShift bytes
     if (threadIdx.x == 0) {
         for (int s = 0; s < kS8; s++) { mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps); }
-        // operands ready: both CTAs' decode group, plus (A_BF16) the leader's announcement of the A tile bytes
-        for (int s = 0; s < kSB; s++) { mbar_init(bar_bf_full(s), 2 * kGroupWarps + ((A_BF16 || SWAPPED) ? 1 : 0)); mbar_init(bar_bf_empty(s), 1); }
+        for (int s = 0; s < kSB; s++) { mbar_init(bar_bf_full(s), 2 * kGroupWarps); mbar_init(bar_bf_empty(s), 1); }  // full: both CTAs' decode group
         mbar_init(bar_acc_full, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -674,26 +647,6 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    if ((A_BF16 || SWAPPED) && warp == 0) {
-        // ------------------------------------------------------------------ second producer (an epilogue warp, idle until the
-        // accumulator is complete): the BF16 tiles of the operand that was expanded beforehand.  Issuing a tile copy costs its
-        // thread a few hundred cycles, and with both kinds of copy on one thread that thread set the pace.  The tile of k-block
-        // kb goes straight into operand stage sb (this CTA's 128 rows) once the MMAs of its previous use have read it; both
-        // CTAs' copies complete on the leader's "operands ready" barrier, which the leader arms with the bytes of both.
-        if (lane == 0) {
-            for (int kb = 0; kb < num_kb; kb++) {
-                const int sb = kb % kSB, rb = kb / kSB;
-                if (rb > 0 && !mbar_wait(bar_bf_empty(sb), (rb - 1) & 1, abort_flag, p.status, 6)) break;
-                if (*abort_flag) break;
-                if (leader) mbar_arrive_expect_tx(bar_bf_full(sb), SWAPPED ? 4 * kBBfBytes : 2 * kABfBytes);
-                if (SWAPPED) {  // 128 k of BF16 are two boxes of 64 (the swizzle span), into the two halves of the stage
-                    tma_load_3d_pair(plan.w_bf(sb), &map_w, kb * KB, nh, 0, map_to_cta(bar_bf_full(sb), 0));
-                    tma_load_3d_pair(plan.w_bf(sb) + kBBfBytes, &map_w, kb * KB + BK, nh, 0, map_to_cta(bar_bf_full(sb), 0));
-                } else tma_load_3d_pair(plan.a_bf(sb), &map_a, kb * BK, m0, 0, map_to_cta(bar_bf_full(sb), 0));
-            }
-        }
-        __syncwarp();
-    }
     if (warp == kTmaWarp) {
         // ------------------------------------------------------------------ TMA producer (each CTA feeds itself)
         if (lane == 0) {
@@ -703,11 +656,10 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 if (round > 0 && !mbar_wait(bar_u8_empty(s), (round - 1) & 1, abort_flag, p.status, 1)) break;
                 if (*abort_flag) break;
                 const uint32_t dst_a = plan.a_u8(s), dst_b = plan.w_u8(s);
-                mbar_arrive_expect_tx(bar_u8_full(s), (A_BF16 ? 0u : (SWAPPED ? 2 * kA8Bytes : kA8Bytes)) + (SWAPPED ? 0u : kB8Bytes));
+                mbar_arrive_expect_tx(bar_u8_full(s), kA8Bytes + kB8Bytes);
                 if (A_IS_KM) tma_load_2d(dst_a, &map_a, m0, kb * BK, bar_u8_full(s));
-                else if (!A_BF16) tma_load_2d(dst_a, &map_a, kb * KB, m0, bar_u8_full(s));  // (SWAPPED: one box of 128 k)
-                if (SWAPPED) {}
-                else if (W_IS_NK) tma_load_2d(dst_b, &map_w, kb * BK, nh, bar_u8_full(s));
+                else tma_load_2d(dst_a, &map_a, kb * BK, m0, bar_u8_full(s));
+                if (W_IS_NK) tma_load_2d(dst_b, &map_w, kb * BK, nh, bar_u8_full(s));
                 else tma_load_2d(dst_b, &map_w, nh, kb * BK, bar_u8_full(s));
                 issued = kb + 1;
             }
@@ -717,11 +669,6 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     const int s = kb % kS8;
                     const unsigned long long t0 = global_ns();
                     while (!mbar_try_wait(bar_u8_full(s), (kb / kS8) & 1) && global_ns() - t0 < kWaitLimitNs) {}
-                }
-                if (A_BF16 || SWAPPED) {  // (the BF16 tiles complete on a barrier that also counts the decode groups, which have given up:
-                               // their copies get a fixed 50 us instead)
-                    const unsigned long long t0 = global_ns();
-                    while (global_ns() - t0 < 50000ull) {}
                 }
             }
         }
@@ -742,21 +689,18 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 bool next_ready = true;
                 uint32_t a_next = 0, b_next = 0, t_next = 0;
 #pragma unroll
-                for (int kk = 0; kk < KB / 16; kk++) {
-                    if (kk == KB / 16 - 1 && kb + 1 < num_kb) {
+                for (int kk = 0; kk < BK / 16; kk++) {
+                    if (kk == BK / 16 - 1 && kb + 1 < num_kb) {
                         const int sn = (kb + 1) % kSB;
                         next_ready = mbar_try_wait(bar_bf_full(sn), (uint32_t)(((kb + 1) / kSB) & 1));
                         a_next = plan.a_bf(sn); b_next = plan.w_bf(sn);
-                        t_next = tmem_base + kTmemColsAcc + (uint32_t)(sn * (KB / 2));
+                        t_next = tmem_base + kTmemColsAcc + (uint32_t)(sn * kTmemAStageCols);
                     }
-                    // K-major: 16 k = 32 bytes inside the 128-byte row (SWAPPED: the second 64 k are the stage's second half);
-                    // MN-major: 16 k = two 1024-byte atoms
-                    const uint64_t db = W_IS_NK ? make_smem_desc(b_addr + (kk >> 2) * kBBfBytes + (kk & 3) * 32, 16, 1024)
+                    // K-major: 16 k = 32 bytes inside the 128-byte row; MN-major: 16 k = two 1024-byte atoms
+                    const uint64_t db = W_IS_NK ? make_smem_desc(b_addr + kk * 32, 16, 1024)
                                                 : make_smem_desc(b_addr + kk * 2048, 8192, 1024);
                     if (A_IS_KM) {
                         tc_mma_bf16_pair(tmem_base, make_smem_desc(a_addr + kk * 2048, 8192, 1024), db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-                    } else if (A_BF16) {
-                        tc_mma_bf16_pair(tmem_base, make_smem_desc(a_addr + kk * 32, 16, 1024), db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                     } else {
                         // A from tensor memory: stage s, 16 k = 8 columns
                         tc_mma_bf16_pair_a_tmem(tmem_base, a_tmem + (uint32_t)(kk * 8), db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
@@ -790,33 +734,6 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 __syncwarp();  // every lane's reads of the byte stage are done: the producer may refill it during the decode
                 if (lane == 0) mbar_arrive(bar_u8_empty(s8));
                 decode_tile_chunks<true, kLutShift>(va, abf, dt, lut);
-            } else if (A_BF16) {
-                // A was expanded beforehand and arrives by TMA: only the W tile is decoded here
-                load_tile_chunks<!W_IS_NK>(b8, dt, vw);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_u8_empty(s8));
-            } else if (SWAPPED) {
-                // As below, with rows of 128 k: the byte tile arrives with the 128-byte TMA swizzle (chunk j of row r at chunk
-                // j ^ (r & 7)), the row is decoded in two halves of 64 into the two halves of the 64-column stage.
-                const int quarter = warp & 3, r = quarter * 32 + lane;
-                const uint32_t a_row = a8 + (uint32_t)r * KB, sw = (uint32_t)r & 7u;
-                uint4 va[KB / 16];
-#pragma unroll
-                for (int j = 0; j < KB / 16; j++) va[j] = lds_v4(a_row + (((uint32_t)j ^ sw) << 4));
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_u8_empty(s8));
-#pragma unroll
-                for (int half = 0; half < 2; half++) {
-                    uint32_t o[BK / 2];
-#pragma unroll
-                    for (int j = 0; j < BK / 16; j++) {
-                        const uint4 v = va[half * (BK / 16) + j];
-                        const uint4 lo = decode8<kLutShift>(make_uint2(v.x, v.y), lut), hi = decode8<kLutShift>(make_uint2(v.z, v.w), lut);
-                        o[8 * j + 0] = lo.x; o[8 * j + 1] = lo.y; o[8 * j + 2] = lo.z; o[8 * j + 3] = lo.w;
-                        o[8 * j + 4] = hi.x; o[8 * j + 5] = hi.y; o[8 * j + 6] = hi.z; o[8 * j + 7] = hi.w;
-                    }
-                    tmem_st_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemColsAcc + (uint32_t)(sb * (KB / 2) + half * (BK / 2)), o);
-                }
             } else {
                 // A [M,K]: this thread owns row (its warp's quarter of the 128 tensor-memory lanes) * 32 + lane.  The byte
                 // tile arrives with the 64-byte TMA swizzle (16-byte chunk j of row r sits at chunk j ^ ((r >> 1) & 3)), so
@@ -838,8 +755,8 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 }
                 tmem_st_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemColsAcc + (uint32_t)(sb * kTmemAStageCols), o);
             }
-            if (!SWAPPED) decode_tile_chunks<!W_IS_NK, kLutShift>(vw, bbf, dt, lut);
-            if (A_MODE == 0) tmem_st_wait();  // the row is in tensor memory
+            decode_tile_chunks<!W_IS_NK, kLutShift>(vw, bbf, dt, lut);
+            if (!A_IS_KM) tmem_st_wait();  // the row is in tensor memory
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // make the stores visible to the tensor core
             tc_fence_before();
             __syncwarp();
@@ -864,59 +781,7 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
             const int row = m0 + quarter * 32 + lane;
             // (separate loops rather than branches inside one: the register allocation of each stays that of its own path)
-            if (SWAPPED) {
-                // accumulator row = the caller's column n (one weight exponent per thread), accumulator column = the caller's
-                // row m: for every m the warp writes 32 consecutive n
-                const int sw = p.d_sw_channel ? (row < p.M ? __ldg(p.d_sw_channel + row) : 0) : (p.d_sw ? *p.d_sw : 0);
-                const int sc = -(sa + sw), t1 = sc / 2, t2 = sc - t1;
-                const float g1 = __uint_as_float((uint32_t)(t1 + 127) << 23), g2 = __uint_as_float((uint32_t)(t2 + 127) << 23);
-                if (p.c_by_tma) {
-                    // BF16 result that replaces C: into the staging boxes of the tile stores (64 of the caller's columns x 128
-                    // of its rows each, 128-byte-swizzled; box = column half + 2 * row half of this CTA's 256 x 128 piece).  For
-                    // one row m the 32 lanes write 32 consecutive columns: 64 contiguous bytes of one line.
-                    const int nl = quarter * 32 + lane;
-                    const uint32_t piece = (uint32_t)((nl & 63) >> 3), within = (uint32_t)(nl & 7) * 2u;
-#pragma unroll 1
-                    for (int c = share * 32; c < BN; c += 5 * 32) {
-                        uint32_t r[32];
-                        tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + c, r);
-                        tmem_ld_wait();
-                        const uint32_t box = plan.box((nl >> 6) + 2 * (c >> 7));
-#pragma unroll
-                        for (int i = 0; i < 32; i++) {
-                            const uint32_t rr = (uint32_t)((c + i) & 127);
-                            unsigned short b;
-                            asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b) : "f"(__uint_as_float(r[i]) * g1 * g2));
-                            sts_u16(box + (rr >> 3) * 1024u + (rr & 7u) * 128u + ((piece ^ (rr & 7u)) << 4) + within, b);
-                        }
-                    }
-                } else
-#pragma unroll 1
-                for (int c = share * 32; c < BN; c += 5 * 32) {
-                    uint32_t r[32];
-                    tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + c, r);
-                    tmem_ld_wait();
-                    if (row < p.M) {
-#pragma unroll
-                        for (int i = 0; i < 32; i++) {
-                            const int m = n0 + c + i;
-                            if (m < p.N) {
-                                float v = __uint_as_float(r[i]) * g1 * g2;
-                                if (p.c_is_f32) {
-                                    float* out = reinterpret_cast<float*>(p.C) + (long long)m * p.ldc + row;
-                                    *out = p.accumulate ? v + *out : v;
-                                } else {
-                                    unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + (long long)m * p.ldc + row;
-                                    if (p.accumulate) v += __uint_as_float((uint32_t)*out << 16);
-                                    unsigned short b;
-                                    asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b) : "f"(v));
-                                    *out = b;
-                                }
-                            }
-                        }
-                    }
-                }
-            } else if (!A_IS_KM && p.c_by_tma) {
+            if (!A_IS_KM && p.c_by_tma) {
 #pragma unroll 1
                 for (int c = share * 32; c < BN; c += 5 * 32) {
                     uint32_t r[32];
@@ -944,13 +809,8 @@ hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("bar.sync 1, %0;" ::"n"((kEpiWarps + kDecodeWarps) * 32) : "memory");
             if (threadIdx.x == 0 && ok && !*abort_flag) {
-                if (SWAPPED) {  // x = the caller's column (this CTA's 128, two boxes), y = its row (256, two boxes)
 #pragma unroll
-                    for (int j = 0; j < 4; j++) tma_store_2d(&map_c, plan.box(j), m0 + (j & 1) * 64, n0 + (j >> 1) * 128);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < BN / 64; j++) tma_store_2d(&map_c, plan.box(j), n0 + j * 64, m0);
-                }
+                for (int j = 0; j < BN / 64; j++) tma_store_2d(&map_c, plan.box(j), n0 + j * 64, m0);
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             }
@@ -1080,16 +940,18 @@ struct NarrowPlan {
     }
 };
 
-// In front of the narrow kernel when the workspace has room: the activations [M,K] (contiguous bytes) expanded to BF16, and
-// the status word and the tickets cleared, in one launch.  Its dependents may start at once (the narrow kernel builds its
-// table meanwhile and waits for this grid's completion before it reads any of this).
-__global__ void __launch_bounds__(256) narrow_prepare_kernel(const uint4* __restrict__ a, uint4* __restrict__ a_bf, unsigned long long n_vec,
-                                                             uint32_t* __restrict__ clear, unsigned clear_words)
+// In front of the kernels that read expanded activations: the activations [M,K] (contiguous bytes) to BF16, and the status
+// word (and the narrow kernel's tickets) cleared, in one launch.  It may itself start while the launch before it drains; its
+// dependents may start once that one is complete (they read weights and exponents at once, and wait for this grid's
+// completion before they read what it writes).
+__global__ void __launch_bounds__(256) expand_activations_kernel(const uint4* __restrict__ a, uint4* __restrict__ a_bf, unsigned long long n_vec,
+                                                                 uint32_t* __restrict__ clear, unsigned clear_words)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ uint32_t lut[256];
     lut[threadIdx.x] = hif8_to_bf16_bits(threadIdx.x);
     __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x == 0)
         for (unsigned i = threadIdx.x; i < clear_words; i += 256) clear[i] = 0u;
     for (unsigned long long u = (unsigned long long)blockIdx.x * 256 + threadIdx.x; u < n_vec; u += (unsigned long long)gridDim.x * 256) {
@@ -1493,6 +1355,363 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
 }
 
 // ---------------------------------------------------------------------------------------------------------
+// Weights decoded into tensor memory, activations expanded to BF16 beforehand (in the caller's workspace): C^T = W^T A^T.
+// A pair of CTAs computes 256 weight columns x bn activation rows: each CTA decodes 128 weight columns straight into its
+// tensor memory (the 128-row A operand of the MMA; nothing decoded touches shared memory) and brings bn / 2 activation
+// rows by TMA (the B operand).  A k-block here is 128 k.  Warp roles per CTA:
+//   warps 0-3   epilogue: accumulator column = activation row m, lane = weight column n
+//   warp  4     copies of weight bytes, four stages of 16 KiB       warp 22  copies of the activation tiles, four stages
+//   warp  5     MMA issuer (even CTA)                               warps 6-21  four decode groups, group g on it = g (mod 4)
+// Two forms, one kernel:
+//   split = 1   persistent: pair p of P takes tiles p, p + P, ..; copies and decode of a tile run on under the epilogue of
+//               the one before (only its MMAs wait for the accumulator).
+//   split > 1   a cluster of `split` pairs per tile, each pair a part of K; the pairs exchange their partial sums through
+//               distributed shared memory, every pair finishes a part of the activation rows, adding in pair order.  For
+//               products with too few tiles for the device and for the last, incomplete round of the persistent form.
+// What bounds it: per k-block and SM 256 x 2 lookup wavefronts (one per 32 bytes), the byte tile in and out and the
+// activation tile in and out, about 1100 cycles of shared memory against 1024 of the tensor pipe at bn = 256.
+// ---------------------------------------------------------------------------------------------------------
+constexpr int kWdStages = 4, kWdActWarp = kThreads / 32, kThreadsWd = kThreads + 32;  // 736
+constexpr int kWdMaxSplit = 4;
+constexpr uint32_t kWdActBytes = 2 * (BN / 2) * BK * 2, kWdW8Bytes = BM * 2 * BK;  // 32 KiB, 16 KiB per stage
+struct SmemLayoutWd {
+    static constexpr uint32_t act = 0;
+    static constexpr uint32_t u8 = act + kWdStages * kWdActBytes;
+    static constexpr uint32_t lut = u8 + kWdStages * kWdW8Bytes;
+    static constexpr uint32_t bars = lut + kLutBytesNarrow;
+    static constexpr uint32_t n_bars = 4 * kWdStages + 2;
+    static constexpr uint32_t tmem_slot = bars + n_bars * 8;
+    static constexpr uint32_t abort_flag = tmem_slot + 4;
+    static constexpr uint32_t total = abort_flag + 4;
+};
+constexpr uint32_t kSmemBytesWd = SmemLayoutWd::total + 1024;
+static_assert(kSmemBytesWd <= 227 * 1024, "shared memory of one CTA");
+static_assert((kWdMaxSplit - 1) * (BN / kWdMaxSplit) * BM * 4 <= SmemLayoutWd::lut && (2 - 1) * (BN / 2) * BM * 4 <= SmemLayoutWd::lut,
+              "the partial sums received fit in the idle stages");
+
+struct TilePlan {
+    int first, count;  // tiles [first, first + count) of the product
+    int chunks, bn;    // activation rows in `chunks` pieces of bn (a multiple of 32); tile t = weight slab t / chunks, piece t % chunks
+    int split;
+};
+
+__device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ float lds_f32(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+// 32 finished sums of this thread's weight column n, activation rows m0 .. m0 + 31, of which `rows` exist.  For one m a warp
+// writes 32 consecutive columns.
+__device__ __forceinline__ void store_columns(const GemmParams& p, int n, int m0, int rows, const float (&v)[32])
+{
+    if (p.c_is_f32) {
+        float* out = reinterpret_cast<float*>(p.C) + (long long)m0 * p.ldc + n;
+#pragma unroll
+        for (int h = 0; h < 32; h += 8) {
+            float old[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) old[i] = (p.accumulate && h + i < rows) ? __ldcs(out + (h + i) * p.ldc) : 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+                if (h + i < rows) __stcs(out + (h + i) * p.ldc, p.accumulate ? v[h + i] + old[i] : v[h + i]);
+        }
+    } else {
+        unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + (long long)m0 * p.ldc + n;
+#pragma unroll
+        for (int h = 0; h < 32; h += 8) {
+            uint32_t old[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) old[i] = (p.accumulate && h + i < rows) ? (uint32_t)out[(h + i) * p.ldc] << 16 : 0u;
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                unsigned short b;
+                asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b) : "f"(p.accumulate ? v[h + i] + __uint_as_float(old[i]) : v[h + i]));
+                if (h + i < rows) out[(h + i) * p.ldc] = b;
+            }
+        }
+    }
+}
+
+template <bool W_IS_NK>
+__global__ void __launch_bounds__(kThreadsWd, 1)
+hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_act, const GemmParams p, const TilePlan tp)
+{
+    extern __shared__ unsigned char smem_raw[];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    unsigned char* sm = smem_raw + (base - smem_u32(smem_raw));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank(), half = rank & 1u, lead = rank & ~1u;  // half 0: leader of its pair (issues the MMAs)
+    const bool leader = half == 0;
+    const uint32_t bars = base + SmemLayoutWd::bars;
+    auto bar_u8_full = [&](int s) { return bars + 8u * s; };                       // per CTA
+    auto bar_u8_empty = [&](int s) { return bars + 8u * (kWdStages + s); };        // per CTA
+    auto bar_bf_full = [&](int s) { return bars + 8u * (2 * kWdStages + s); };     // leader: both CTAs' decode warps and activation tiles
+    auto bar_bf_empty = [&](int s) { return bars + 8u * (3 * kWdStages + s); };    // per CTA, leader's commits
+    const uint32_t bar_acc_full = bars + 8u * (4 * kWdStages);                     // per CTA, leader's commit
+    const uint32_t bar_acc_empty = bars + 8u * (4 * kWdStages + 1);                // leader: both CTAs' epilogue warps
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + SmemLayoutWd::abort_flag);
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + SmemLayoutWd::tmem_slot);
+    const uint32_t lut = base + SmemLayoutWd::lut + 4u * lane;
+    auto act_stage = [&](int s) { return base + SmemLayoutWd::act + (uint32_t)s * kWdActBytes; };
+    auto u8_stage = [&](int s) { return base + SmemLayoutWd::u8 + (uint32_t)s * kWdW8Bytes; };
+
+    constexpr int KB = 2 * BK;
+    const int num_kb = (p.K + KB - 1) / KB, split = tp.split, part = split > 1 ? (int)(rank >> 1) : 0;
+    const int kb0 = split > 1 ? num_kb * part / split : 0, kb1 = split > 1 ? num_kb * (part + 1) / split : num_kb;
+    const int t0 = tp.first + (int)(split > 1 ? blockIdx.x / (2 * split) : blockIdx.x >> 1);
+    const int t_end = tp.first + tp.count, t_step = split > 1 ? tp.count : (int)(gridDim.x >> 1);
+
+    // ---- set-up
+    if (threadIdx.x == kTmaWarp * 32) {
+        for (int s = 0; s < kWdStages; s++) {
+            mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps);
+            mbar_init(bar_bf_full(s), 2 * kGroupWarps + 1); mbar_init(bar_bf_empty(s), 1);  // (+ 1: the leader's announcement of the tile bytes)
+        }
+        mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * kEpiWarps);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    fill_decode_table<32>(reinterpret_cast<uint32_t*>(sm + SmemLayoutWd::lut), warp, lane, kThreadsWd / 32);
+    if (warp == kMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(base + SmemLayoutWd::tmem_slot), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();  // barriers of all CTAs exist before anyone signals across
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == kTmaWarp) {
+        // ------------------------------------------------------------------ weight bytes (each CTA feeds itself).  Nothing the
+        // launch in front of this one writes is read here, and what came before that is complete.
+        if (lane == 0) {
+            int it = 0;
+            bool ok = true;
+            for (int t = t0; t < t_end && ok; t += t_step) {
+                const int n0 = t / tp.chunks * 2 * BM + (int)half * BM;
+                for (int kb = kb0; kb < kb1; kb++, it++) {
+                    const int s = it % kWdStages;
+                    if (it >= kWdStages) ok = mbar_wait(bar_u8_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 41);
+                    if (!ok || *abort_flag) { ok = false; break; }
+                    mbar_arrive_expect_tx(bar_u8_full(s), kWdW8Bytes);
+                    if (W_IS_NK) tma_load_2d(u8_stage(s), &map_w, kb * KB, n0, bar_u8_full(s));
+                    else tma_load_2d(u8_stage(s), &map_w, n0, kb * KB, bar_u8_full(s));
+                }
+            }
+            if (*abort_flag) {
+                for (int i = max(0, it - kWdStages); i < it; i++) {  // let the copies already issued land
+                    const unsigned long long c0 = global_ns();
+                    while (!mbar_try_wait(bar_u8_full(i % kWdStages), (i / kWdStages) & 1) && global_ns() - c0 < kWaitLimitNs) {}
+                }
+            }
+        }
+    } else if (warp == kWdActWarp) {
+        // ------------------------------------------------------------------ activation tiles: this CTA's bn / 2 rows, two boxes of
+        // 64 k (the swizzle span); both CTAs' copies complete on the leader's "operands ready" barrier
+        if (lane == 0) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            int it = 0;
+            bool ok = true;
+            for (int t = t0; t < t_end && ok; t += t_step) {
+                const int m0 = t % tp.chunks * tp.bn + (int)half * (tp.bn / 2);
+                for (int kb = kb0; kb < kb1; kb++, it++) {
+                    const int s = it % kWdStages;
+                    if (it >= kWdStages) ok = mbar_wait(bar_bf_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 46);
+                    if (!ok || *abort_flag) { ok = false; break; }
+                    if (leader) mbar_arrive_expect_tx(bar_bf_full(s), (uint32_t)tp.bn * KB * 2u);
+                    const uint32_t full = map_to_cta(bar_bf_full(s), lead);
+                    tma_load_3d_pair(act_stage(s), &map_act, kb * KB, m0, 0, full);
+                    tma_load_3d_pair(act_stage(s) + kWdActBytes / 2, &map_act, kb * KB + BK, m0, 0, full);
+                }
+            }
+            if (*abort_flag) {  // (their barrier also counts the decode groups, which have given up: a fixed 50 us instead)
+                const unsigned long long c0 = global_ns();
+                while (global_ns() - c0 < 50000ull) {}
+            }
+        }
+    } else if (warp == kMmaWarp) {
+        // ------------------------------------------------------------------ MMA issuer (leader CTA only)
+        if (lane == 0 && leader) {
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(tp.bn >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
+            const uint64_t db0 = make_smem_desc(act_stage(0), 16, 1024);
+            int it = 0, local = 0;
+            bool ok = true;
+            for (int t = t0; t < t_end && ok; t += t_step, local++) {
+                if (local > 0) ok = mbar_wait(bar_acc_empty, (local - 1) & 1, abort_flag, p.status, 45);
+                for (int kb = kb0; kb < kb1 && ok; kb++, it++) {
+                    const int s = it % kWdStages;
+                    ok = mbar_wait(bar_bf_full(s), (it / kWdStages) & 1, abort_flag, p.status, 42);
+                    if (!ok) break;
+                    tc_fence_after();
+#pragma unroll
+                    for (int kk = 0; kk < KB / 16; kk++) {
+                        const uint32_t off = (uint32_t)s * kWdActBytes + (kk >> 2) * (kWdActBytes / 2) + (kk & 3) * 32;
+                        tc_mma_bf16_pair_a_tmem(tmem_base, tmem_base + kTmemColsAcc + (uint32_t)(s * (KB / 2) + kk * 8), db0 + (uint64_t)(off >> 4), idesc,
+                                                (kb > kb0 || kk > 0) ? 1u : 0u);
+                    }
+                    tc_commit_pair(bar_bf_empty(s), lead);
+                }
+                if (ok) tc_commit_pair(bar_acc_full, lead);
+            }
+        }
+    } else if (warp >= kFirstDecodeWarp) {
+        // ------------------------------------------------------------------ decode warps
+        const int group = (warp - kFirstDecodeWarp) / kGroupWarps, quarter = warp & 3;
+        const int n_it = ((t_end - t0 + t_step - 1) / t_step) * (kb1 - kb0);
+        const uint32_t tlane = tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemColsAcc;
+        bool ok = true;
+        for (int it = group; it < n_it && ok; it += kDecodeGroups) {
+            const int s = it % kWdStages, r = it / kWdStages;
+            ok = mbar_wait(bar_u8_full(s), r & 1, abort_flag, p.status, 43);
+            if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 44);
+            if (!ok) break;
+            const uint32_t w8 = u8_stage(s);
+            uint4 v[KB / 16];
+            if (W_IS_NK) {
+                // a thread per weight column: rows of 128 k with the 128-byte swizzle (chunk j of row r at chunk j ^ (r & 7))
+                const uint32_t row = (uint32_t)(quarter * 32 + lane), w_row = w8 + row * KB, sw = row & 7u;
+#pragma unroll
+                for (int j = 0; j < KB / 16; j++) v[j] = lds_v4(w_row + (((uint32_t)j ^ sw) << 4));
+            } else {
+                // rows of 128 columns, one per k: read transposed; v[2 i + c] = k 32 i .. of the quarter's columns 16 c .. (see
+                // the narrow kernel)
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+#pragma unroll
+                    for (int c = 0; c < 2; c++)
+                        v[2 * i + c] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(32 * i + lane) * BM + ((uint32_t)((2 * quarter + c) ^ (lane & 7)) << 4));
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_u8_empty(s));
+            const uint32_t dst = tlane + (uint32_t)(s * (KB / 2));
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                uint32_t o[32];
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    // [N,K]: 64 k of the column per half; [K,N]: all 128 k of the sixteen columns of half h
+                    const uint4 w = W_IS_NK ? v[4 * h + j] : v[2 * j + h];
+                    const uint4 lo = decode8<7>(make_uint2(w.x, w.y), lut), hi = decode8<7>(make_uint2(w.z, w.w), lut);
+                    o[8 * j + 0] = lo.x; o[8 * j + 1] = lo.y; o[8 * j + 2] = lo.z; o[8 * j + 3] = lo.w;
+                    o[8 * j + 4] = hi.x; o[8 * j + 5] = hi.y; o[8 * j + 6] = hi.z; o[8 * j + 7] = hi.w;
+                }
+                if (W_IS_NK) tmem_st_32x32b_x32(dst + (uint32_t)(h * (BK / 2)), o);
+                else {
+                    tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16), o);
+                    tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16) + BK / 2, o + 16);
+                }
+            }
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(map_to_cta(bar_bf_full(s), lead));
+        }
+    } else if (split == 1) {
+        // ------------------------------------------------------------------ epilogue of the persistent form
+        const int sa = p.d_sa ? *p.d_sa : 0, sw_all = (p.d_sw && !p.d_sw_channel) ? *p.d_sw : 0;
+        int local = 0;
+        for (int t = t0; t < t_end; t += t_step, local++) {
+            const int slab = t / tp.chunks, m0 = (t - slab * tp.chunks) * tp.bn, n = slab * 2 * BM + (int)half * BM + warp * 32 + lane;
+            const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = sc / 2, s2 = sc - s1;
+            const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
+            if (!mbar_wait(bar_acc_full, local & 1, abort_flag, p.status, 47)) break;
+            tc_fence_after();
+            const int cols = min(tp.bn, p.M - m0);
+#pragma unroll 1
+            for (int c = 0; c < cols; c += 32) {
+                uint32_t r[32];
+                float v[32];
+                tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(warp * 32) << 16) + c, r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]) * f1 * f2;
+                if (n < p.N) store_columns(p, n, m0 + c, cols - c, v);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(map_to_cta(bar_acc_empty, lead));
+        }
+    }
+    if (split > 1) {
+        // ------------------------------------------------------------------ exchange and epilogue of the split form: all warps, a
+        // warp on lanes (warp % 4) * 32 .. of every sixth (fifth) 32-column piece.  Columns are dealt to the pairs in pieces.
+        __syncwarp();
+        const int quarter = warp & 3, shares = quarter < 3 ? 6 : 5, share = warp >> 2;
+        static_assert(kThreadsWd / 32 == 23, "six warps on the lanes of quarters 0 to 2, five on those of quarter 3");
+        const int slab = t0 / tp.chunks, m0 = (t0 - slab * tp.chunks) * tp.bn, row = quarter * 32 + lane, n = slab * 2 * BM + (int)half * BM + row;
+        const int cols = min(tp.bn, p.M - m0), pieces = (cols + 31) / 32, per = (pieces + split - 1) / split;
+        const int sa = p.d_sa ? *p.d_sa : 0, sw = p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : (p.d_sw ? *p.d_sw : 0);
+        const int sc = -(sa + sw), s1 = sc / 2, s2 = sc - s1;
+        const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
+        const uint32_t tl = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const bool ok = mbar_wait(bar_acc_full, 0, abort_flag, p.status, 48);
+        tc_fence_after();
+        __syncwarp();
+        cluster_sync_all();  // every pair's MMAs and copies are done: the stages of all CTAs are free
+        if (ok) {
+#pragma unroll 1
+            for (int j = share; j < pieces; j += shares) {
+                const int owner = j / per;
+                if (owner == part) continue;
+                uint32_t r[32];
+                tmem_ld_32x32b_x32(tl + j * 32, r);
+                tmem_ld_wait();
+                const int slot = part < owner ? part : part - 1;
+                const uint32_t to = map_to_cta(base + (uint32_t)(((slot * per + (j - owner * per)) * 32) * BM + row) * 4u, 2u * owner + half);
+#pragma unroll
+                for (int i = 0; i < 32; i++) st_cluster_f32(to + i * BM * 4, __uint_as_float(r[i]));
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();
+        if (ok) {
+#pragma unroll 1
+            for (int j = part * per + (share - part * per % shares + shares) % shares; j < min(pieces, (part + 1) * per); j += shares) {
+                uint32_t r[32];
+                float v[32];
+                tmem_ld_32x32b_x32(tl + j * 32, r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; i++) v[i] = 0.f;
+#pragma unroll 1
+                for (int q = 0; q < split; q++) {  // in pair order
+                    const uint32_t from = base + (uint32_t)((((q < part ? q : q - 1) * per + (j - part * per)) * 32) * BM + row) * 4u;
+                    if (q == part) {
+#pragma unroll
+                        for (int i = 0; i < 32; i++) v[i] += __uint_as_float(r[i]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; i++) v[i] += lds_f32(from + i * BM * 4);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 32; i++) v[i] = v[i] * f1 * f2;
+                if (n < p.N) store_columns(p, n, m0 + j * 32, cols - j * 32, v);
+            }
+        }
+    }
+
+    // ---- teardown: all waits are bounded, so everybody arrives; nobody leaves while the peer may still read this
+    // CTA's operands or signal its barriers; then the allocating warps free TMEM
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == kMmaWarp) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------------------------------------
 // Decode-once path: operands already decoded to BF16 (by the conversion kernels of this library, into the caller's
 // workspace).  Persistent kernel on CTA pairs (cta_group::2), 64-wide k-blocks.
 //   warps 0-3  epilogue (TMEM -> global), overlapped with the next tile through two TMEM accumulators
@@ -1724,6 +1943,23 @@ __global__ void wait_selftest_kernel(int* status, unsigned long long limit_ns)
 // ---------------------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------------------
+cudaError_t launch_expand_activations(const uint8_t* a, void* a_bf, unsigned long long n, void* clear, size_t clear_bytes, int sm_count, cudaStream_t st)
+{
+    const unsigned long long n_vec = n / 16;  // K is a multiple of 16
+    const unsigned long long want = (n_vec + 255) / 256, cap = (unsigned long long)sm_count * 32;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(want < cap ? want : cap));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return cudaLaunchKernelEx(&cfg, expand_activations_kernel, reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a_bf), n_vec,
+                              reinterpret_cast<uint32_t*>(clear), (unsigned)(clear_bytes / 4));
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1807,24 +2043,36 @@ bool make_map3(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t rows,
 struct GemmDeviceSetup {
     cudaError_t rc;
     int sm_count;
+    int wd_clusters[kWdMaxSplit + 1];  // clusters of s pairs of hif8_gemm_weights_kernel that fit on the device at once, s = 1, 2, 4
 };
 PerDevice<GemmDeviceSetup> g_gemm_setup;
 
-bool gemm_kernels_ready(int dev, int* sm_count_out)
+bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nullptr)
 {
     const GemmDeviceSetup* s = g_gemm_setup.get(dev, [](int d, GemmDeviceSetup* out) {
         out->rc = cudaSuccess;
         out->sm_count = 0;
-        if (out->rc == cudaSuccess)
-            out->rc = cudaFuncSetAttribute(hif8_gemm_kernel<0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesSwapped);
-        const void* fused[6] = {(const void*)hif8_gemm_kernel<0, false>, (const void*)hif8_gemm_kernel<0, true>,
-                                (const void*)hif8_gemm_kernel<1, false>, (const void*)hif8_gemm_kernel<1, true>,
-                                (const void*)hif8_gemm_kernel<2, false>, (const void*)hif8_gemm_kernel<2, true>};
+        std::memset(out->wd_clusters, 0, sizeof out->wd_clusters);
+        // [M,K] activations (the first two): the wide-table plan
+        const void* fused[4] = {(const void*)hif8_gemm_kernel<false, false>, (const void*)hif8_gemm_kernel<false, true>,
+                                (const void*)hif8_gemm_kernel<true, false>, (const void*)hif8_gemm_kernel<true, true>};
         const void* pair[2] = {(const void*)bf16_gemm_pair_kernel<false>, (const void*)bf16_gemm_pair_kernel<true>};
-        for (int i = 0; i < 6 && out->rc == cudaSuccess; i++)  // [M,K] byte activations (the first two): the wide-table plan
+        const void* wd[2] = {(const void*)hif8_gemm_weights_kernel<false>, (const void*)hif8_gemm_weights_kernel<true>};
+        for (int i = 0; i < 4 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(fused[i], cudaFuncAttributeMaxDynamicSharedMemorySize, i < 2 ? kSmemBytesWide : kSmemBytes);
         for (int i = 0; i < 2 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(pair[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2);
+        for (int i = 0; i < 2 && out->rc == cudaSuccess; i++)
+            out->rc = cudaFuncSetAttribute(wd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesWd);
+        for (int s = 1; s <= kWdMaxSplit && out->rc == cudaSuccess; s *= 2) {
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 2 * s; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            cfg.gridDim = dim3(2 * s); cfg.blockDim = dim3(kThreadsWd); cfg.dynamicSmemBytes = kSmemBytesWd;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            out->rc = cudaOccupancyMaxActiveClusters(&out->wd_clusters[s], wd[1], &cfg);
+        }
         const void* narrow[4] = {(const void*)hif8_gemm_narrow_kernel<false, false>, (const void*)hif8_gemm_narrow_kernel<false, true>,
                                  (const void*)hif8_gemm_narrow_kernel<true, false>, (const void*)hif8_gemm_narrow_kernel<true, true>};
         for (int i = 0; i < 4 && out->rc == cudaSuccess; i++)
@@ -1833,7 +2081,8 @@ bool gemm_kernels_ready(int dev, int* sm_count_out)
     });
     if (!s) return false;
     *sm_count_out = s->sm_count;
-    return s->rc == cudaSuccess && s->sm_count > 0;
+    if (wd_clusters) *wd_clusters = s->wd_clusters;
+    return s->rc == cudaSuccess && s->sm_count > 0 && s->wd_clusters[1] > 0;
 }
 
 // The status word of the most recent GEMM-class call per stream, for hif8_last_device_status.
@@ -1899,6 +2148,63 @@ int launch_bf16_pair_gemm(const void* a_bf, const void* w_bf, int w_is_nk, GemmP
 
 using namespace hif8;
 
+// C = A W^T-or-W with the weights decoded inside the kernel and the activations given as BF16 [M,K] by the launch in front
+// of this one.  `clusters[s]`: how many clusters of s pairs the device holds.
+static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, const void* a_bf, const GemmParams& p, const int* clusters, cudaStream_t st)
+{
+    const int M = p.M, N = p.N, K = p.K, chunks = (M + BN - 1) / BN, bn = ((M + chunks - 1) / chunks + 31) & ~31;
+    const long long slabs = (N + 2 * BM - 1) / (2 * BM), tiles_ll = slabs * chunks;
+    if (tiles_ll > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
+    const int tiles = (int)tiles_ll, num_kb = (K + 2 * BK - 1) / (2 * BK);
+    CUtensorMap map_w, map_act;
+    const bool okw = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, 2 * BK, BM, false, 128)
+                             : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, 2 * BK, false, 128);
+    if (!okw || !make_map3(&map_act, a_bf, (uint64_t)K, (uint64_t)M, 1, 0, BK, (uint32_t)bn / 2)) return HIF8_ERR_CUDA;
+    // Time in k-blocks: a round of `n` tiles takes num_kb / split of them, and the exchange of a split one about as long as
+    // three.  A launch of its own for the last round costs about four (set-up, first copies).
+    auto cost = [&](int n, int s) {
+        if (s > num_kb || clusters[s] <= 0) return 1 << 30;
+        return (n + clusters[s] - 1) / clusters[s] * ((num_kb + s - 1) / s + (s > 1 ? 3 : 0));
+    };
+    auto best_split = [&](int n) {
+        int best = 1;
+        for (int s = 2; s <= kWdMaxSplit; s *= 2)
+            if (cost(n, s) < cost(n, best)) best = s;
+        return best;
+    };
+    const int pairs = clusters[1];
+    TilePlan launch[2];
+    int launches = 1;
+    launch[0] = TilePlan{0, tiles, chunks, bn, tiles <= pairs ? best_split(tiles) : 1};
+    if (tiles > pairs && tiles % pairs) {
+        const int rem = tiles % pairs, s = best_split(rem);
+        if (s > 1 && cost(rem, s) + 4 < num_kb) {
+            launch[0].count = tiles - rem;
+            launch[1] = TilePlan{tiles - rem, rem, chunks, bn, s};
+            launches = 2;
+        }
+    }
+    for (int i = 0; i < launches; i++) {
+        const TilePlan& tp = launch[i];
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(2u * (unsigned)(tp.split > 1 ? tp.count * tp.split : (tp.count < pairs ? tp.count : pairs)));
+        cfg.blockDim = dim3(kThreadsWd);
+        cfg.dynamicSmemBytes = kSmemBytesWd;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2u * (unsigned)tp.split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr; cfg.numAttrs = 2;
+        const cudaError_t rc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true>, map_w, map_act, p, tp)
+                                       : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false>, map_w, map_act, p, tp);
+        if (rc != cudaSuccess) return HIF8_ERR_CUDA;
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+    }
+    return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+}
+
 static std::atomic<int> g_path_policy{HIF8_GEMM_PATH_AUTO};
 
 extern "C" int hif8_gemm_path_policy(int policy)
@@ -1952,7 +2258,8 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     note_status_word(st, reinterpret_cast<const int*>(workspace));
 
     int sm_count = 0;
-    if (!gemm_kernels_ready(dev, &sm_count)) return HIF8_ERR_CUDA;
+    const int* wd_clusters = nullptr;
+    if (!gemm_kernels_ready(dev, &sm_count, &wd_clusters)) return HIF8_ERR_CUDA;
     // the status word is cleared on the stream before the kernels; the narrow path clears its tickets in the same operation
     size_t clear_bytes = 4;
 
@@ -2002,13 +2309,7 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
             if (lda == K && workspace_bytes >= off + bytes_act && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
                 unsigned char* a_bf = reinterpret_cast<unsigned char*>(workspace) + off;
                 if (!make_map(&map_act, a_bf, (uint64_t)K, (uint64_t)M, (uint64_t)K, BK, (uint32_t)mp, true)) return HIF8_ERR_CUDA;
-                const unsigned long long n_vec = (unsigned long long)M * K / 16;  // K is a multiple of 16
-                const unsigned long long want = (n_vec + 255) / 256, cap = (unsigned long long)sm_count * 4;
-                narrow_prepare_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
-                    reinterpret_cast<const uint4*>(Aq), reinterpret_cast<uint4*>(a_bf), n_vec, reinterpret_cast<uint32_t*>(workspace),
-                    (unsigned)(clear_bytes / 4));
-                if (cudaGetLastError() != cudaSuccess) return HIF8_ERR_CUDA;
-                g_launches.fetch_add(1, std::memory_order_relaxed);
+                if (launch_expand_activations(Aq, a_bf, (unsigned long long)M * K, workspace, clear_bytes, sm_count, st) != cudaSuccess) return HIF8_ERR_CUDA;
                 act_bf16 = true;
             }
         }
@@ -2035,12 +2336,11 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
     }
 
-    if (cudaMemsetAsync(workspace, 0, clear_bytes, st) != cudaSuccess) return HIF8_ERR_CUDA;
     // Decode-once path: with room for both operands as BF16 in the workspace (and contiguous operands), each HiF8
     // byte is decoded exactly once by the conversion kernel and the tensor-core kernel reads BF16 tiles through TMA.
-    // Otherwise the fused kernel decodes the byte tiles of every CTA in shared memory.
+    // Otherwise the weights are decoded inside the tensor-core kernel, and the activations too when there is no room for them.
     const size_t bytes_a = (((size_t)M * K * 2) + 255) & ~(size_t)255, bytes_w = (((size_t)K * N * 2) + 255) & ~(size_t)255;
-    const bool contiguous = lda == (a_is_km ? M : K) && ldw == (w_is_nk ? K : N);
+    const bool a_contiguous = lda == (a_is_km ? M : K), w_contiguous = ldw == (w_is_nk ? K : N);
     // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element
     // moved) at the higher rate of the decode-once kernel: with about 268 flops per byte of copy bandwidth for that kernel,
     // 233 for the swapped A-expanded form ([N,K] weights) and 210 for the other (their measured rates against the copy rate)
@@ -2048,59 +2348,26 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     const double mk = (double)M * K, kn = (double)K * N, flops = 2.0 * mk * N;
     const bool w_expansion_pays = g_path_policy.load(std::memory_order_relaxed) == HIF8_GEMM_PATH_EXPAND_BOTH ||
                                   3.0 * kn + flops / 268.0 < flops / (w_is_nk ? 233.0 : 210.0);
-    if (contiguous && w_expansion_pays && workspace_bytes >= kGemmWorkspaceBytes + bytes_a + bytes_w &&
-        !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
+    if (a_contiguous && workspace_bytes >= kGemmWorkspaceBytes + bytes_a && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
         unsigned char* a_bf = reinterpret_cast<unsigned char*>(workspace) + kGemmWorkspaceBytes;
-        unsigned char* w_bf = a_bf + bytes_a;
-        // an A given as [K,M] is written as [M,K] while it is expanded: the tensor-core kernel streams a K-major A fastest
-        int rc = a_is_km ? decode_transpose_bf16(Aq, a_bf, K, M, st) : hif8_decode(Aq, a_bf, HIF8_BF16, (size_t)M * K, 0, stream);
-        if (rc == HIF8_OK) rc = hif8_decode(Wq, w_bf, HIF8_BF16, (size_t)K * N, 0, stream);
+        // (an A given as [K,M] is written as [M,K] while it is expanded; either launch clears the status word)
+        int rc = HIF8_OK;
+        if (a_is_km) rc = decode_transpose_bf16(Aq, a_bf, K, M, reinterpret_cast<uint32_t*>(workspace), st);
+        else if (launch_expand_activations(Aq, a_bf, (unsigned long long)M * K, workspace, 4, sm_count, st) != cudaSuccess) rc = HIF8_ERR_CUDA;
         if (rc != HIF8_OK) return rc;
-        return launch_bf16_pair_gemm(a_bf, w_bf, w_is_nk, p, st);
-    }
-    // In between: room for A alone as BF16 (2 M K bytes; W, usually the larger operand, stays bytes).  A is expanded once
-    // (as [M,K] whichever way it was given) and the fused kernel decodes only its W tiles; W may have any leading dimension.
-    int a_mode = a_is_km ? 1 : 0;
-    if (lda == (a_is_km ? M : K) && workspace_bytes >= kGemmWorkspaceBytes + bytes_a && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
-        unsigned char* a_bf = reinterpret_cast<unsigned char*>(workspace) + kGemmWorkspaceBytes;
-        const int rc = a_is_km ? decode_transpose_bf16(Aq, a_bf, K, M, st) : hif8_decode(Aq, a_bf, HIF8_BF16, (size_t)M * K, 0, stream);
-        if (rc != HIF8_OK) return rc;
-        // boxes of 64 k x 128 rows in the 128-byte-swizzled operand layout (a stack of one matrix: the pair form of the copy)
-        if (!make_map3(&map_a, a_bf, (uint64_t)K, (uint64_t)M, 1, 0, BK, BM)) return HIF8_ERR_CUDA;
-        a_mode = 2;
-        if (w_is_nk) {
-            // [N,K] weights: the swapped form, C^T = W^T A^T.  The weight rows are the operand that is decoded into tensor
-            // memory, the expanded activations the one in shared memory; the kernel's M is N and its N is M.
-            GemmParams q = p;
-            q.M = N; q.N = M;
-            q.c_by_tma = (c_dtype == HIF8_BF16 && !accumulate) ? 1 : 0;
-            CUtensorMap map_cs;
-            if (q.c_by_tma && !make_map(&map_cs, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 64, BM, true)) return HIF8_ERR_CUDA;
-            q.tiles_m = (N + BM - 1) / BM; q.tiles_n = (M + BN - 1) / BN;
-            const long long tiles2s = (long long)((N + 2 * BM - 1) / (2 * BM)) * q.tiles_n;
-            if (tiles2s > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
-            CUtensorMap map_wb, map_ab;
-            if (!make_map(&map_wb, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, 2 * BK, BM, false, 128)) return HIF8_ERR_CUDA;  // rows of 128 k
-            if (!make_map3(&map_ab, a_bf, (uint64_t)K, (uint64_t)M, 1, 0, BK, BN / 2)) return HIF8_ERR_CUDA;
-            cudaLaunchConfig_t cs{};
-            cs.gridDim = dim3(2u * (unsigned)tiles2s);
-            cs.blockDim = dim3(kThreads);
-            cs.dynamicSmemBytes = kSmemBytesSwapped;
-            cs.stream = st;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-            cs.attrs = at; cs.numAttrs = 1;
-            const cudaError_t src = cudaLaunchKernelEx(&cs, hif8_gemm_kernel<0, true, true>, map_wb, map_ab, q.c_by_tma ? map_cs : map_ab, q);
-            g_launches.fetch_add(1, std::memory_order_relaxed);
-            return (src == cudaSuccess && cudaGetLastError() == cudaSuccess) ? HIF8_OK : HIF8_ERR_CUDA;
+        if (w_contiguous && w_expansion_pays && workspace_bytes >= kGemmWorkspaceBytes + bytes_a + bytes_w) {
+            unsigned char* w_bf = a_bf + bytes_a;
+            rc = hif8_decode(Wq, w_bf, HIF8_BF16, (size_t)K * N, 0, stream);
+            return rc != HIF8_OK ? rc : launch_bf16_pair_gemm(a_bf, w_bf, w_is_nk, p, st);
         }
+        return launch_weights_gemm(Wq, ldw, w_is_nk, a_bf, p, wd_clusters, st);
     }
+    if (cudaMemsetAsync(workspace, 0, 4, st) != cudaSuccess) return HIF8_ERR_CUDA;
 
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2u * (unsigned)tiles2);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = a_mode == 0 ? kSmemBytesWide : kSmemBytes;
+    cfg.dynamicSmemBytes = a_is_km ? kSmemBytes : kSmemBytesWide;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2109,14 +2376,12 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     cudaError_t lrc;
     // BF16 results that replace C leave the [M,K]-activation kernel through tile stores (boxes of 64 columns x 128 rows)
     CUtensorMap map_c = map_a;  // (a valid map in any case; only read when c_by_tma is set)
-    p.c_by_tma = (a_mode != 1 && c_dtype == HIF8_BF16 && !accumulate) ? 1 : 0;
+    p.c_by_tma = (!a_is_km && c_dtype == HIF8_BF16 && !accumulate) ? 1 : 0;
     if (p.c_by_tma && !make_map(&map_c, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 64, BM, true)) return HIF8_ERR_CUDA;
-    if (a_mode == 1) lrc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<1, true>, map_a, map_w, map_c, p)
-                                   : cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<1, false>, map_a, map_w, map_c, p);
-    else if (a_mode == 2) lrc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<2, true>, map_a, map_w, map_c, p)
-                                        : cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<2, false>, map_a, map_w, map_c, p);
-    else lrc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<0, true>, map_a, map_w, map_c, p)
-                       : cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<0, false>, map_a, map_w, map_c, p);
+    if (a_is_km) lrc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<true, true>, map_a, map_w, map_c, p)
+                               : cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<true, false>, map_a, map_w, map_c, p);
+    else lrc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<false, true>, map_a, map_w, map_c, p)
+                       : cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<false, false>, map_a, map_w, map_c, p);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return (lrc == cudaSuccess && cudaGetLastError() == cudaSuccess) ? HIF8_OK : HIF8_ERR_CUDA;
 }

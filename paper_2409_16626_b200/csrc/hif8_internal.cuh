@@ -34,8 +34,8 @@ int launch_bf16_pair_gemm(const void* a_bf, const void* w_bf, int w_is_nk, GemmP
                           long long a_stack_stride = 0, long long w_stack_stride = 0);
 
 // dst[c][r] = BF16 value of the HiF8 byte src[r][c]; src [rows, cols] contiguous (rows a multiple of 8, cols of 16), both
-// pointers 16-byte aligned
-int decode_transpose_bf16(const uint8_t* src, void* dst, long long rows, long long cols, cudaStream_t st);
+// pointers 16-byte aligned.  The launch also clears the device word `clear_word` (may be null).
+int decode_transpose_bf16(const uint8_t* src, void* dst, long long rows, long long cols, uint32_t* clear_word, cudaStream_t st);
 
 // Remembers `word` (a device int that a kernel sets when one of its bounded waits gives up) as the status word of the
 // latest GEMM-class call on stream `st` of the current device; hif8_last_device_status reads it back.

@@ -191,13 +191,17 @@ __global__ void __launch_bounds__(kThreads) encode_transpose_scalar_kernel(const
 constexpr int kDtRows = 64, kDtCols = 256, kDtStride = kDtCols + 4;
 
 __global__ void __launch_bounds__(kThreads) decode_transpose_bf16_kernel(const uint8_t* __restrict__ src, unsigned short* __restrict__ dst,
-                                                                         long long rows, long long cols)
+                                                                         long long rows, long long cols, uint32_t* clear_word)
 {
     __shared__ uint32_t tile[kDtRows * kDtStride / 4];
     __shared__ unsigned short lut[256];
     lut[threadIdx.x] = (unsigned short)(decode_bits_f32(threadIdx.x) >> 16);  // every HiF8 value is exact in BF16
     const long long tiles_c = (cols + kDtCols - 1) / kDtCols, tiles_r = (rows + kDtRows - 1) / kDtRows;
     const uint8_t* tb = reinterpret_cast<const uint8_t*>(tile);
+    // (dependents only once everything before this launch is complete: they read operands of it at once)
+    pdl_wait_prior_grid();
+    pdl_launch_dependents();
+    if (clear_word && blockIdx.x == 0 && threadIdx.x == 0) *clear_word = 0u;
     for (long long tix = blockIdx.x; tix < tiles_c * tiles_r; tix += gridDim.x) {
         const long long tc = tix / tiles_r, tr = tix % tiles_r;
         const long long r0 = tr * kDtRows, c0 = tc * kDtCols;
@@ -270,13 +274,13 @@ int launch_mode(int rnd, const TrParams& p, bool vec, int sms, cudaStream_t st)
 
 }  // namespace
 
-int decode_transpose_bf16(const uint8_t* src, void* dst, long long rows, long long cols, cudaStream_t st)
+int decode_transpose_bf16(const uint8_t* src, void* dst, long long rows, long long cols, uint32_t* clear_word, cudaStream_t st)
 {
     if (rows <= 0 || cols <= 0 || (rows & 7) || (cols & 15)) return HIF8_ERR_SHAPE;
     if ((reinterpret_cast<uintptr_t>(src) & 15u) || (reinterpret_cast<uintptr_t>(dst) & 15u)) return HIF8_ERR_ALIGN;
     const long long tiles = ((cols + kDtCols - 1) / kDtCols) * ((rows + kDtRows - 1) / kDtRows);
-    decode_transpose_bf16_kernel<<<(unsigned)(tiles < 0x7FFFFFFFll ? tiles : 0x7FFFFFFFll), kThreads, 0, st>>>(
-        src, reinterpret_cast<unsigned short*>(dst), rows, cols);
+    launch_pdl(decode_transpose_bf16_kernel, (unsigned)(tiles < 0x7FFFFFFFll ? tiles : 0x7FFFFFFFll), st, src,
+               reinterpret_cast<unsigned short*>(dst), rows, cols, clear_word);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
 }
