@@ -191,6 +191,11 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld_32x32b_x8(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // 32 consecutive columns of this thread's tensor-memory lane (lane field of taddr = first lane of the warp's quarter)
 __device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t (&r)[32])
@@ -241,6 +246,8 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -306,13 +313,13 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_
 }
 
 // BF16 bits of one HiF8 byte (Eq. 1, Eq. 2, specials); used to fill the shared lookup table
-__device__ __forceinline__ uint32_t hif8_to_bf16_bits(uint32_t c)
+__host__ __device__ constexpr uint32_t hif8_to_bf16_bits(uint32_t c)
 {
     uint32_t sign = (c & 0x80u) << 8, m = c & 0x7Fu;
     if (m == 0) return sign ? 0x7FC0u : 0u;
     if (m == 0x6F) return sign | 0x7F80u;
     if (m < 8) return sign | ((m + 104u) << 7);
-    int E; uint32_t M, w;
+    int E = 0; uint32_t M = 0, w = 0;
     if (m < 0x10)      { E = 0; M = m & 7; w = 3; }
     else if (m < 0x20) { E = 1; M = m & 7; w = 3; if (m & 0x08) E = -E; }
     else if (m < 0x40) { E = 2 | ((m >> 3) & 1); M = m & 7; w = 3; if (m & 0x10) E = -E; }
@@ -321,18 +328,36 @@ __device__ __forceinline__ uint32_t hif8_to_bf16_bits(uint32_t c)
     return sign | ((uint32_t)(E + 127) << 7) | (M << (7 - w));
 }
 
+struct Bf16OfCode { uint16_t v[256]; };
+constexpr Bf16OfCode make_bf16_of_code()
+{
+    Bf16OfCode t{};
+    for (uint32_t c = 0; c < 256; c++) t.v[c] = (uint16_t)hif8_to_bf16_bits(c);
+    return t;
+}
+__device__ const Bf16OfCode g_bf16_of_code = make_bf16_of_code();
+
 // Fills the decode table: entry (code c, lane l) at word c * ROW_WORDS + l holds the BF16 bits of code c (one copy per
 // lane, so that a warp's lookups never meet in a bank).  A warp writes four rows per step, eight lanes with 16 bytes each to
-// a row, every lane working out its row's value itself: all the warps of a block take part and none of them shuffles (with
-// 32 codes per warp, handed round by shuffles, eight warps worked 1300 cycles at the head of every kernel).
+// a row; at most three steps for the 22 warps or more of a block, their values loaded together.  (What runs once at the head
+// of a kernel costs its instruction fetches above all, so the values come from a table in global memory and not from the
+// field definitions: 1050 -> 600 cycles; eight warps with 32 codes each, handed round by shuffles, took 1300.)
 template <int ROW_WORDS>
 __device__ __forceinline__ void fill_decode_table(uint32_t* table, int warp, int lane, int n_warps)
 {
-    for (int i = warp; i < 64; i += n_warps) {
-        const uint32_t code = (uint32_t)(4 * i + (lane >> 3)), v = hif8_to_bf16_bits(code);
-        *reinterpret_cast<uint4*>(table + code * ROW_WORDS + (lane & 7) * 4) = make_uint4(v, v, v, v);
+    uint32_t v[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int i = warp + k * n_warps;
+        v[k] = i < 64 ? __ldg(g_bf16_of_code.v + 4 * i + (lane >> 3)) : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int i = warp + k * n_warps;
+        if (i < 64) *reinterpret_cast<uint4*>(table + (4 * i + (lane >> 3)) * ROW_WORDS + (lane & 7) * 4) = make_uint4(v[k], v[k], v[k], v[k]);
     }
 }
+static_assert(3 * (kThreads / 32) >= 64, "three steps fill the table");
 
 // Shared-memory accesses by 32-bit shared-window address: the operand ring lives at a run-time offset inside the dynamic
 // allocation, and spelling the state space out keeps every one of these an LDS / STS (never a generic access).
@@ -1395,45 +1420,47 @@ struct TilePlan {
     int split;
 };
 
-__device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v)
+__device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ float lds_f32(uint32_t addr)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
-// 32 finished sums of this thread's weight column n, activation rows m0 .. m0 + 31, of which `rows` exist.  For one m a warp
-// writes 32 consecutive columns.
-__device__ __forceinline__ void store_columns(const GemmParams& p, int n, int m0, int rows, const float (&v)[32])
+// Eight finished sums of this thread's weight column, activation rows m .. m + 7 of which `rows` exist, to C: `out` is the
+// place of the first, `pitch` the bytes from row to row (below 2^32: more than 64 rows fit in memory).  For one row a warp
+// writes 32 consecutive columns.  Issue slots bound this: with two scale factors, 64-bit row addresses and a test per row
+// the epilogue of a 256 x 256 tile took 5300 cycles, 19 instructions a store.
+__device__ __forceinline__ void store_columns(unsigned char* out, uint32_t pitch, int is_f32, int accumulate, int rows, float (&v)[8])
 {
-    if (p.c_is_f32) {
-        float* out = reinterpret_cast<float*>(p.C) + (long long)m0 * p.ldc + n;
+    auto at = [&](int i) { return out + (unsigned long long)pitch * (uint32_t)i; };
+    if (accumulate) {
+        if (is_f32) {
 #pragma unroll
-        for (int h = 0; h < 32; h += 8) {
-            float old[8];
+            for (int i = 0; i < 8; i++) v[i] += i < rows ? __ldcs(reinterpret_cast<const float*>(at(i))) : 0.f;
+        } else {
 #pragma unroll
-            for (int i = 0; i < 8; i++) old[i] = (p.accumulate && h + i < rows) ? __ldcs(out + (h + i) * p.ldc) : 0.f;
+            for (int i = 0; i < 8; i++) v[i] += i < rows ? __uint_as_float((uint32_t)*reinterpret_cast<const unsigned short*>(at(i)) << 16) : 0.f;
+        }
+    }
+    if (is_f32) {
+        if (rows >= 8) {
+#pragma unroll
+            for (int i = 0; i < 8; i++) __stcs(reinterpret_cast<float*>(at(i)), v[i]);
+        } else {
 #pragma unroll
             for (int i = 0; i < 8; i++)
-                if (h + i < rows) __stcs(out + (h + i) * p.ldc, p.accumulate ? v[h + i] + old[i] : v[h + i]);
+                if (i < rows) __stcs(reinterpret_cast<float*>(at(i)), v[i]);
         }
     } else {
-        unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + (long long)m0 * p.ldc + n;
+        unsigned short b[8];
 #pragma unroll
-        for (int h = 0; h < 32; h += 8) {
-            uint32_t old[8];
+        for (int i = 0; i < 8; i++) asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b[i]) : "f"(v[i]));  // round to nearest even; a NaN stays a NaN
+        if (rows >= 8) {
 #pragma unroll
-            for (int i = 0; i < 8; i++) old[i] = (p.accumulate && h + i < rows) ? (uint32_t)out[(h + i) * p.ldc] << 16 : 0u;
+            for (int i = 0; i < 8; i++) *reinterpret_cast<unsigned short*>(at(i)) = b[i];
+        } else {
 #pragma unroll
-            for (int i = 0; i < 8; i++) {
-                unsigned short b;
-                asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b) : "f"(p.accumulate ? v[h + i] + __uint_as_float(old[i]) : v[h + i]));
-                if (h + i < rows) out[(h + i) * p.ldc] = b;
-            }
+            for (int i = 0; i < 8; i++)
+                if (i < rows) *reinterpret_cast<unsigned short*>(at(i)) = b[i];
         }
     }
 }
@@ -1467,7 +1494,16 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     const int t0 = tp.first + (int)(split > 1 ? blockIdx.x / (2 * split) : blockIdx.x >> 1);
     const int t_end = tp.first + tp.count, t_step = split > 1 ? tp.count : (int)(gridDim.x >> 1);
 
-    // ---- set-up
+    // ---- set-up.  A call of a small product is mostly latency: the first weight copies go out under the table set-up, and only
+    // what touches the other CTAs waits for the cluster (its barrier takes 1400 to 1900 cycles from the start of the kernel,
+    // in which a first k-block is copied and decoded).
+    auto copy_weights = [&](int it, int n0, int kb) {  // stage it % kWdStages, free
+        const int s = it % kWdStages;
+        mbar_arrive_expect_tx(bar_u8_full(s), kWdW8Bytes);
+        if (W_IS_NK) tma_load_2d(u8_stage(s), &map_w, kb * KB, n0, bar_u8_full(s));
+        else tma_load_2d(u8_stage(s), &map_w, n0, kb * KB, bar_u8_full(s));
+    };
+    const int n_first = t0 / tp.chunks * 2 * BM + (int)half * BM;  // weight columns of the first tile
     if (threadIdx.x == kTmaWarp * 32) {
         for (int s = 0; s < kWdStages; s++) {
             mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps);
@@ -1476,6 +1512,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * kEpiWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        copy_weights(0, n_first, kb0);
     }
     fill_decode_table<32>(reinterpret_cast<uint32_t*>(sm + SmemLayoutWd::lut), warp, lane, kThreadsWd / 32);
     if (warp == kMmaWarp) {
@@ -1485,25 +1523,28 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     }
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();  // barriers of all CTAs exist before anyone signals across
+    cluster_arrive();  // barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == kTmaWarp) {
         // ------------------------------------------------------------------ weight bytes (each CTA feeds itself).  Nothing the
         // launch in front of this one writes is read here, and what came before that is complete.
+        const int n_early = min(kWdStages, kb1 - kb0);  // of the first tile, without waiting for anybody
+        if (lane == 0)
+            for (int i = 1; i < n_early; i++) copy_weights(i, n_first, kb0 + i);
+        __syncwarp();
+        cluster_wait();
         if (lane == 0) {
             int it = 0;
             bool ok = true;
             for (int t = t0; t < t_end && ok; t += t_step) {
                 const int n0 = t / tp.chunks * 2 * BM + (int)half * BM;
                 for (int kb = kb0; kb < kb1; kb++, it++) {
-                    const int s = it % kWdStages;
-                    if (it >= kWdStages) ok = mbar_wait(bar_u8_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 41);
+                    if (it < n_early) continue;
+                    if (it >= kWdStages) ok = mbar_wait(bar_u8_empty(it % kWdStages), (it / kWdStages - 1) & 1, abort_flag, p.status, 41);
                     if (!ok || *abort_flag) { ok = false; break; }
-                    mbar_arrive_expect_tx(bar_u8_full(s), kWdW8Bytes);
-                    if (W_IS_NK) tma_load_2d(u8_stage(s), &map_w, kb * KB, n0, bar_u8_full(s));
-                    else tma_load_2d(u8_stage(s), &map_w, n0, kb * KB, bar_u8_full(s));
+                    copy_weights(it, n0, kb);
                 }
             }
             if (*abort_flag) {
@@ -1516,6 +1557,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     } else if (warp == kWdActWarp) {
         // ------------------------------------------------------------------ activation tiles: this CTA's bn / 2 rows, two boxes of
         // 64 k (the swizzle span); both CTAs' copies complete on the leader's "operands ready" barrier
+        cluster_wait();
         if (lane == 0) {
             asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1540,6 +1582,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         }
     } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
+        cluster_wait();
         if (lane == 0 && leader) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(tp.bn >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
             const uint64_t db0 = make_smem_desc(act_stage(0), 16, 1024);
@@ -1568,39 +1611,37 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         const int group = (warp - kFirstDecodeWarp) / kGroupWarps, quarter = warp & 3;
         const int n_it = ((t_end - t0 + t_step - 1) / t_step) * (kb1 - kb0);
         const uint32_t tlane = tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemColsAcc;
-        bool ok = true;
+        bool ok = true, joined = false;
         for (int it = group; it < n_it && ok; it += kDecodeGroups) {
             const int s = it % kWdStages, r = it / kWdStages;
             ok = mbar_wait(bar_u8_full(s), r & 1, abort_flag, p.status, 43);
             if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 44);
             if (!ok) break;
-            const uint32_t w8 = u8_stage(s);
-            uint4 v[KB / 16];
-            if (W_IS_NK) {
-                // a thread per weight column: rows of 128 k with the 128-byte swizzle (chunk j of row r at chunk j ^ (r & 7))
-                const uint32_t row = (uint32_t)(quarter * 32 + lane), w_row = w8 + row * KB, sw = row & 7u;
-#pragma unroll
-                for (int j = 0; j < KB / 16; j++) v[j] = lds_v4(w_row + (((uint32_t)j ^ sw) << 4));
-            } else {
-                // rows of 128 columns, one per k: read transposed; v[2 i + c] = k 32 i .. of the quarter's columns 16 c .. (see
-                // the narrow kernel)
-#pragma unroll
-                for (int i = 0; i < 4; i++)
-#pragma unroll
-                    for (int c = 0; c < 2; c++)
-                        v[2 * i + c] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(32 * i + lane) * BM + ((uint32_t)((2 * quarter + c) ^ (lane & 7)) << 4));
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_u8_empty(s));
-            const uint32_t dst = tlane + (uint32_t)(s * (KB / 2));
-#pragma unroll
+            const uint32_t w8 = u8_stage(s), dst = tlane + (uint32_t)(s * (KB / 2));
+            // in two halves, one piece of code for both (unrolled, the first pass over it cost every group a thousand cycles of
+            // instruction fetches): [N,K] 64 k of the thread's column, [K,N] all 128 k of sixteen of the quarter's columns
+#pragma unroll 1
             for (int h = 0; h < 2; h++) {
+                uint4 v[4];
+                if (W_IS_NK) {
+                    // rows of 128 k with the 128-byte swizzle (chunk j of row r at chunk j ^ (r & 7))
+                    const uint32_t row = (uint32_t)(quarter * 32 + lane), w_row = w8 + row * KB, sw = row & 7u;
+#pragma unroll
+                    for (int j = 0; j < 4; j++) v[j] = lds_v4(w_row + (((uint32_t)(4 * h + j) ^ sw) << 4));
+                } else {
+                    // rows of 128 columns, one per k, read transposed (see the narrow kernel)
+#pragma unroll
+                    for (int j = 0; j < 4; j++)
+                        v[j] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(32 * j + lane) * BM + ((uint32_t)((2 * quarter + h) ^ (lane & 7)) << 4));
+                }
+                if (h == 1) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_u8_empty(s));
+                }
                 uint32_t o[32];
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    // [N,K]: 64 k of the column per half; [K,N]: all 128 k of the sixteen columns of half h
-                    const uint4 w = W_IS_NK ? v[4 * h + j] : v[2 * j + h];
-                    const uint4 lo = decode8<7>(make_uint2(w.x, w.y), lut), hi = decode8<7>(make_uint2(w.z, w.w), lut);
+                    const uint4 lo = decode8<7>(make_uint2(v[j].x, v[j].y), lut), hi = decode8<7>(make_uint2(v[j].z, v[j].w), lut);
                     o[8 * j + 0] = lo.x; o[8 * j + 1] = lo.y; o[8 * j + 2] = lo.z; o[8 * j + 3] = lo.w;
                     o[8 * j + 4] = hi.x; o[8 * j + 5] = hi.y; o[8 * j + 6] = hi.z; o[8 * j + 7] = hi.w;
                 }
@@ -1613,90 +1654,89 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
+            if (!joined) { cluster_wait(); joined = true; }  // before the first signal to another CTA
             if (lane == 0) mbar_arrive_remote(map_to_cta(bar_bf_full(s), lead));
         }
-    } else if (split == 1) {
-        // ------------------------------------------------------------------ epilogue of the persistent form
-        const int sa = p.d_sa ? *p.d_sa : 0, sw_all = (p.d_sw && !p.d_sw_channel) ? *p.d_sw : 0;
+        if (!joined) { __syncwarp(); cluster_wait(); }
+    } else cluster_wait();
+
+    const bool one_tile = tp.count <= t_step;  // per pair: all warps are free for its epilogue
+    if (one_tile || warp < kEpiWarps) {
+        // ------------------------------------------------------------------ epilogue, in pieces of eight columns.  With several
+        // tiles per pair warps 0-3, one per quarter of the lanes; with one all warps, six (five) to a quarter.  In the split form
+        // the pairs exchange first: each finishes `per` of the pieces.
+        __syncwarp();
+        const int quarter = warp & 3, shares = !one_tile ? 1 : (quarter < 3 ? 6 : 5), share = !one_tile ? 0 : warp >> 2;
+        static_assert(kThreadsWd / 32 == 23, "six warps on the lanes of quarters 0 to 2, five on those of quarter 3");
+        const int row = quarter * 32 + lane, sa = p.d_sa ? *p.d_sa : 0, sw_all = (p.d_sw && !p.d_sw_channel) ? *p.d_sw : 0;
+        const int c_size = p.c_is_f32 ? 4 : 2;
+        const long long pitch = p.ldc * c_size;
+        const uint32_t tl = tmem_base + ((uint32_t)(quarter * 32) << 16), mine = base + (uint32_t)row * 16u;
         int local = 0;
         for (int t = t0; t < t_end; t += t_step, local++) {
-            const int slab = t / tp.chunks, m0 = (t - slab * tp.chunks) * tp.bn, n = slab * 2 * BM + (int)half * BM + warp * 32 + lane;
-            const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = sc / 2, s2 = sc - s1;
-            const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
-            if (!mbar_wait(bar_acc_full, local & 1, abort_flag, p.status, 47)) break;
+            const int slab = t / tp.chunks, m0 = (t - slab * tp.chunks) * tp.bn, n = slab * 2 * BM + (int)half * BM + row;
+            // 2^sc as one factor, and a second one for the few scales that need it
+            const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = max(-126, min(126, sc));
+            const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(sc - s1 + 127) << 23);
+            const int cols = min(tp.bn, p.M - m0), pieces = (cols + 7) / 8, per = split == 1 ? pieces : (pieces + split - 1) / split;
+            unsigned char* out = reinterpret_cast<unsigned char*>(p.C) + (long long)m0 * pitch + (long long)n * c_size;
+            const bool ok = mbar_wait(bar_acc_full, local & 1, abort_flag, p.status, 47);
+            if (!ok && split == 1) break;
             tc_fence_after();
-            const int cols = min(tp.bn, p.M - m0);
+            if (split > 1) {
+                __syncwarp();
+                cluster_sync_all();  // every pair's MMAs and copies are done: the stages of all CTAs are free
+                if (ok) {
 #pragma unroll 1
-            for (int c = 0; c < cols; c += 32) {
-                uint32_t r[32];
-                float v[32];
-                tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(warp * 32) << 16) + c, r);
+                    for (int j = share; j < pieces; j += shares) {
+                        const int owner = j / per;
+                        if (owner == part) continue;
+                        uint32_t r[8];
+                        tmem_ld_32x32b_x8(tl + j * 8, r);
+                        tmem_ld_wait();
+                        const int slot = part < owner ? part : part - 1;
+                        const uint32_t to = map_to_cta(mine + (uint32_t)((slot * per + (j - owner * per)) * 8 * BM) * 4u, 2u * owner + half);
+                        st_cluster_v4(to, r[0], r[1], r[2], r[3]);
+                        st_cluster_v4(to + BM * 16, r[4], r[5], r[6], r[7]);
+                    }
+                }
+                __syncwarp();
+                cluster_sync_all();
+                if (!ok) break;
+            }
+            const int j0 = part * per, j1 = min(pieces, j0 + per);
+#pragma unroll 1
+            for (int j = j0 + share; j < j1; j += shares) {
+                uint32_t r[8];
+                float v[8];
+                tmem_ld_32x32b_x8(tl + j * 8, r);
                 tmem_ld_wait();
+                if (split > 1) {  // the pairs' sums in pair order
 #pragma unroll
-                for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]) * f1 * f2;
-                if (n < p.N) store_columns(p, n, m0 + c, cols - c, v);
+                    for (int i = 0; i < 8; i++) v[i] = 0.f;
+#pragma unroll 1
+                    for (int q = 0; q < split; q++) {
+                        const uint32_t from = mine + (uint32_t)(((q < part ? q : q - 1) * per + (j - j0)) * 8 * BM) * 4u;
+                        uint4 lo = make_uint4(r[0], r[1], r[2], r[3]), hi = make_uint4(r[4], r[5], r[6], r[7]);
+                        if (q != part) { lo = lds_v4(from); hi = lds_v4(from + BM * 16); }
+                        v[0] += __uint_as_float(lo.x); v[1] += __uint_as_float(lo.y); v[2] += __uint_as_float(lo.z); v[3] += __uint_as_float(lo.w);
+                        v[4] += __uint_as_float(hi.x); v[5] += __uint_as_float(hi.y); v[6] += __uint_as_float(hi.z); v[7] += __uint_as_float(hi.w);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; i++) v[i] *= f1;
+                if (sc != s1) {
+#pragma unroll
+                    for (int i = 0; i < 8; i++) v[i] *= f2;
+                }
+                if (n < p.N) store_columns(out + j * 8 * pitch, (uint32_t)pitch, p.c_is_f32, p.accumulate, cols - j * 8, v);
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_remote(map_to_cta(bar_acc_empty, lead));
-        }
-    }
-    if (split > 1) {
-        // ------------------------------------------------------------------ exchange and epilogue of the split form: all warps, a
-        // warp on lanes (warp % 4) * 32 .. of every sixth (fifth) 32-column piece.  Columns are dealt to the pairs in pieces.
-        __syncwarp();
-        const int quarter = warp & 3, shares = quarter < 3 ? 6 : 5, share = warp >> 2;
-        static_assert(kThreadsWd / 32 == 23, "six warps on the lanes of quarters 0 to 2, five on those of quarter 3");
-        const int slab = t0 / tp.chunks, m0 = (t0 - slab * tp.chunks) * tp.bn, row = quarter * 32 + lane, n = slab * 2 * BM + (int)half * BM + row;
-        const int cols = min(tp.bn, p.M - m0), pieces = (cols + 31) / 32, per = (pieces + split - 1) / split;
-        const int sa = p.d_sa ? *p.d_sa : 0, sw = p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : (p.d_sw ? *p.d_sw : 0);
-        const int sc = -(sa + sw), s1 = sc / 2, s2 = sc - s1;
-        const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
-        const uint32_t tl = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        const bool ok = mbar_wait(bar_acc_full, 0, abort_flag, p.status, 48);
-        tc_fence_after();
-        __syncwarp();
-        cluster_sync_all();  // every pair's MMAs and copies are done: the stages of all CTAs are free
-        if (ok) {
-#pragma unroll 1
-            for (int j = share; j < pieces; j += shares) {
-                const int owner = j / per;
-                if (owner == part) continue;
-                uint32_t r[32];
-                tmem_ld_32x32b_x32(tl + j * 32, r);
-                tmem_ld_wait();
-                const int slot = part < owner ? part : part - 1;
-                const uint32_t to = map_to_cta(base + (uint32_t)(((slot * per + (j - owner * per)) * 32) * BM + row) * 4u, 2u * owner + half);
-#pragma unroll
-                for (int i = 0; i < 32; i++) st_cluster_f32(to + i * BM * 4, __uint_as_float(r[i]));
-            }
-        }
-        __syncwarp();
-        cluster_sync_all();
-        if (ok) {
-#pragma unroll 1
-            for (int j = part * per + (share - part * per % shares + shares) % shares; j < min(pieces, (part + 1) * per); j += shares) {
-                uint32_t r[32];
-                float v[32];
-                tmem_ld_32x32b_x32(tl + j * 32, r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int i = 0; i < 32; i++) v[i] = 0.f;
-#pragma unroll 1
-                for (int q = 0; q < split; q++) {  // in pair order
-                    const uint32_t from = base + (uint32_t)((((q < part ? q : q - 1) * per + (j - part * per)) * 32) * BM + row) * 4u;
-                    if (q == part) {
-#pragma unroll
-                        for (int i = 0; i < 32; i++) v[i] += __uint_as_float(r[i]);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 32; i++) v[i] += lds_f32(from + i * BM * 4);
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < 32; i++) v[i] = v[i] * f1 * f2;
-                if (n < p.N) store_columns(p, n, m0 + j * 32, cols - j * 32, v);
-            }
+            if (!one_tile && lane == 0) mbar_arrive_remote(map_to_cta(bar_acc_empty, lead));
         }
     }
 
@@ -2160,11 +2200,15 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
     const bool okw = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, 2 * BK, BM, false, 128)
                              : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, 2 * BK, false, 128);
     if (!okw || !make_map3(&map_act, a_bf, (uint64_t)K, (uint64_t)M, 1, 0, BK, (uint32_t)bn / 2)) return HIF8_ERR_CUDA;
-    // Time in k-blocks: a round of `n` tiles takes num_kb / split of them, and the exchange of a split one about as long as
-    // three.  A launch of its own for the last round costs about four (set-up, first copies).
+    // Time in k-blocks (of 128 k, about 1050 cycles): a round of tiles takes num_kb / split of them.  The exchange of a split one
+    // (two cluster barriers, the sums at 20 bytes a cycle, less what the shared epilogue saves) measured 3.1 for two pairs and
+    // 7 for four at bn = 256, about half of that at 128.  A launch of its own for the last round costs about four (set-up,
+    // first copies).
+    const double f = bn / 256.0;
     auto cost = [&](int n, int s) {
-        if (s > num_kb || clusters[s] <= 0) return 1 << 30;
-        return (n + clusters[s] - 1) / clusters[s] * ((num_kb + s - 1) / s + (s > 1 ? 3 : 0));
+        if (s > num_kb || clusters[s] <= 0) return 1e30;
+        const double exchange = s == 1 ? 0.0 : (s == 2 ? 1.2 + 1.9 * f : 2.0 + 5.0 * f);
+        return (n + clusters[s] - 1) / clusters[s] * ((num_kb + s - 1) / s + exchange);
     };
     auto best_split = [&](int n) {
         int best = 1;
