@@ -13,6 +13,9 @@ def __getattr__(name):
         return importlib.import_module("." + name, __name__)
     binding = importlib.import_module(".binding", __name__)
     try:
-        return getattr(binding, name)
+        value = getattr(binding, name)
     except AttributeError:
         raise AttributeError(f"module {__name__!r} has no attribute {name!r}") from None
+    if name in binding.PUBLIC:  # an ordinary attribute from now on: this lookup costs about a microsecond
+        globals()[name] = value
+    return value

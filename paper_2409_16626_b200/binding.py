@@ -3,6 +3,9 @@
 Functions carry the C names and argument order of include/hif8.h.  Tensors are torch CUDA tensors (used for
 device memory and streams only); pointers may also be given as plain ints.  A missing or unloadable library
 is an error: there is no fallback path.
+
+The conversions and products go through csrc/hif8_call.cpp (a few hundred nanoseconds a call); what it does not take
+(arguments of other types, the first call before CUDA is initialised) goes through ctypes, which also reports the errors.
 """
 import ctypes as C
 import os
@@ -27,6 +30,10 @@ EXPORTS = ["hif8_encode", "hif8_decode", "hif8_amax", "hif8_amax_scale_encode", 
 if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: run `python -m paper_2409_16626_b200.build` (needs nvcc)")
 lib = C.CDLL(LIB_PATH)
+from . import _hif8_call as _c  # noqa: E402  (linked against the library above)
+
+_c.set_up(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+os.register_at_fork(after_in_child=lambda: _c.set_cuda_ready(False))
 
 _vp, _sz, _i, _u, _u64, _i64 = C.c_void_p, C.c_size_t, C.c_int, C.c_uint, C.c_uint64, C.c_int64
 lib.hif8_encode.argtypes = [_vp, _i, _vp, _sz, _i, _i, _u, _u64, _vp]
@@ -107,6 +114,15 @@ def _stream(stream):
     return stream.cuda_stream
 
 
+def _via_ctypes(name, args):
+    """The same call through ctypes: pointers by _ptr, the last argument is the stream."""
+    fn = getattr(lib, name)
+    converted = [_ptr(a) if t is _vp else a for a, t in zip(args[:-1], fn.argtypes)]
+    rc = fn(*converted, _stream(args[-1]))
+    _c.set_cuda_ready(torch.cuda.is_initialized())
+    return rc
+
+
 def _check(rc, check):
     if check and rc != OK:
         raise Hif8Error(rc)
@@ -126,7 +142,9 @@ def hif8_launch_count():
 
 
 def hif8_encode(src, src_dtype, dst, n, scale_exp=0, rnd=RND_TA, flags=0, seed=0, stream=None, check=True):
-    return _check(lib.hif8_encode(_ptr(src), src_dtype, _ptr(dst), n, scale_exp, rnd, flags, seed, _stream(stream)), check)
+    args = (src, src_dtype, dst, n, scale_exp, rnd, flags, seed, stream)
+    rc = _c.hif8_encode(*args)
+    return _check(_via_ctypes("hif8_encode", args) if rc is None else rc, check)
 
 
 def hif8_encode_f32_patterns(first_pattern, dst, n, scale_exp=0, rnd=RND_TA, flags=0, seed=0, stream=None, check=True):
@@ -135,42 +153,50 @@ def hif8_encode_f32_patterns(first_pattern, dst, n, scale_exp=0, rnd=RND_TA, fla
 
 
 def hif8_decode(src, dst, dst_dtype, n, scale_exp=0, stream=None, check=True):
-    return _check(lib.hif8_decode(_ptr(src), _ptr(dst), dst_dtype, n, scale_exp, _stream(stream)), check)
+    args = (src, dst, dst_dtype, n, scale_exp, stream)
+    rc = _c.hif8_decode(*args)
+    return _check(_via_ctypes("hif8_decode", args) if rc is None else rc, check)
 
 
 def hif8_amax_scale_encode(src, src_dtype, dst, n, target_exp=14, rnd=RND_TA, flags=0, seed=0, d_scale_exp_in=None,
                            d_amax_out=None, d_scale_exp_out=None, d_scale_out=None, workspace=None,
                            workspace_bytes=0, stream=None, check=True):
-    return _check(lib.hif8_amax_scale_encode(_ptr(src), src_dtype, _ptr(dst), n, target_exp, rnd, flags, seed,
-                                             _ptr(d_scale_exp_in), _ptr(d_amax_out), _ptr(d_scale_exp_out),
-                                             _ptr(d_scale_out), _ptr(workspace), workspace_bytes, _stream(stream)), check)
+    args = (src, src_dtype, dst, n, target_exp, rnd, flags, seed, d_scale_exp_in, d_amax_out, d_scale_exp_out, d_scale_out,
+            workspace, workspace_bytes, stream)
+    rc = _c.hif8_amax_scale_encode(*args)
+    return _check(_via_ctypes("hif8_amax_scale_encode", args) if rc is None else rc, check)
 
 
 def hif8_amax(src, src_dtype, n, d_amax_out, workspace, workspace_bytes, stream=None, check=True):
-    return _check(lib.hif8_amax(_ptr(src), src_dtype, n, _ptr(d_amax_out), _ptr(workspace), workspace_bytes, _stream(stream)), check)
+    args = (src, src_dtype, n, d_amax_out, workspace, workspace_bytes, stream)
+    rc = _c.hif8_amax(*args)
+    return _check(_via_ctypes("hif8_amax", args) if rc is None else rc, check)
 
 
 def hif8_amax_scale_encode_static(src, src_dtype, dst, n, target_exp=14, rnd=RND_TA, flags=0, seed=0,
                                   d_scale_exp_in=None, d_amax_out=None, d_scale_exp_out=None, d_scale_out=None,
                                   stream=None, check=True):
     """hif8_amax_scale_encode for callers that cannot hand over a workspace (scratch lives inside the library)."""
-    return _check(lib.hif8_amax_scale_encode_static(_ptr(src), src_dtype, _ptr(dst), n, target_exp, rnd, flags, seed,
-                                                    _ptr(d_scale_exp_in), _ptr(d_amax_out), _ptr(d_scale_exp_out),
-                                                    _ptr(d_scale_out), _stream(stream)), check)
+    args = (src, src_dtype, dst, n, target_exp, rnd, flags, seed, d_scale_exp_in, d_amax_out, d_scale_exp_out, d_scale_out,
+            stream)
+    rc = _c.hif8_amax_scale_encode_static(*args)
+    return _check(_via_ctypes("hif8_amax_scale_encode_static", args) if rc is None else rc, check)
 
 
 def hif8_fake_quant(src, dst, dtype, n, use_amax=0, scale_or_target_exp=0, rnd=RND_TA, flags=0, seed=0,
                     d_amax_out=None, d_scale_exp_out=None, workspace=None, workspace_bytes=0, stream=None, check=True):
-    return _check(lib.hif8_fake_quant(_ptr(src), _ptr(dst), dtype, n, use_amax, scale_or_target_exp, rnd, flags, seed,
-                                      _ptr(d_amax_out), _ptr(d_scale_exp_out), _ptr(workspace), workspace_bytes,
-                                      _stream(stream)), check)
+    args = (src, dst, dtype, n, use_amax, scale_or_target_exp, rnd, flags, seed, d_amax_out, d_scale_exp_out, workspace,
+            workspace_bytes, stream)
+    rc = _c.hif8_fake_quant(*args)
+    return _check(_via_ctypes("hif8_fake_quant", args) if rc is None else rc, check)
 
 
 def hif8_gemm(Aq, lda, Wq, ldw, w_is_nk, Cmat, ldc, c_dtype, M, N, K, d_scale_exp_a=None, d_scale_exp_w=None,
               workspace=None, workspace_bytes=0, stream=None, check=True):
-    return _check(lib.hif8_gemm(_ptr(Aq), lda, _ptr(Wq), ldw, w_is_nk, _ptr(Cmat), ldc, c_dtype, M, N, K,
-                                _ptr(d_scale_exp_a), _ptr(d_scale_exp_w), _ptr(workspace), workspace_bytes,
-                                _stream(stream)), check)
+    args = (Aq, lda, Wq, ldw, w_is_nk, Cmat, ldc, c_dtype, M, N, K, d_scale_exp_a, d_scale_exp_w, workspace,
+            workspace_bytes, stream)
+    rc = _c.hif8_gemm(*args)
+    return _check(_via_ctypes("hif8_gemm", args) if rc is None else rc, check)
 
 
 def hif8_gemm_status(workspace, stream=None):
@@ -216,16 +242,18 @@ def hif8_selftest_wait_timeout(workspace, limit_ms, stream=None, check=True):
 
 def hif8_channel_amax_scale_encode(W, src_dtype, dst, rows, cols, channel_axis, target_exp=14, rnd=RND_TA, flags=0, seed=0,
                                    d_scale_exp_in=None, d_amax=None, d_scale_exp_out=None, stream=None, check=True):
-    return _check(lib.hif8_channel_amax_scale_encode(_ptr(W), src_dtype, _ptr(dst), rows, cols, channel_axis, target_exp, rnd,
-                                                     flags, seed, _ptr(d_scale_exp_in), _ptr(d_amax), _ptr(d_scale_exp_out),
-                                                     _stream(stream)), check)
+    args = (W, src_dtype, dst, rows, cols, channel_axis, target_exp, rnd, flags, seed, d_scale_exp_in, d_amax,
+            d_scale_exp_out, stream)
+    rc = _c.hif8_channel_amax_scale_encode(*args)
+    return _check(_via_ctypes("hif8_channel_amax_scale_encode", args) if rc is None else rc, check)
 
 
 def hif8_gemm_channel_scaled(Aq, lda, Wq, ldw, w_is_nk, Cmat, ldc, c_dtype, M, N, K, d_scale_exp_a=None,
                              d_scale_exp_w_channel=None, workspace=None, workspace_bytes=0, stream=None, check=True):
-    return _check(lib.hif8_gemm_channel_scaled(_ptr(Aq), lda, _ptr(Wq), ldw, w_is_nk, _ptr(Cmat), ldc, c_dtype, M, N, K,
-                                               _ptr(d_scale_exp_a), _ptr(d_scale_exp_w_channel), _ptr(workspace),
-                                               workspace_bytes, _stream(stream)), check)
+    args = (Aq, lda, Wq, ldw, w_is_nk, Cmat, ldc, c_dtype, M, N, K, d_scale_exp_a, d_scale_exp_w_channel, workspace,
+            workspace_bytes, stream)
+    rc = _c.hif8_gemm_channel_scaled(*args)
+    return _check(_via_ctypes("hif8_gemm_channel_scaled", args) if rc is None else rc, check)
 
 
 def hif8_scale_state_init(d_state, hist_len, stream=None, check=True):
@@ -234,21 +262,24 @@ def hif8_scale_state_init(d_state, hist_len, stream=None, check=True):
 
 def hif8_delayed_scale_encode(src, src_dtype, dst, n, rnd, flags, seed, d_state, measure, target_exp=14, stream=None,
                               check=True):
-    return _check(lib.hif8_delayed_scale_encode(_ptr(src), src_dtype, _ptr(dst), n, rnd, flags, seed, _ptr(d_state),
-                                                int(measure), target_exp, _stream(stream)), check)
+    args = (src, src_dtype, dst, n, rnd, flags, seed, d_state, int(measure), target_exp, stream)
+    rc = _c.hif8_delayed_scale_encode(*args)
+    return _check(_via_ctypes("hif8_delayed_scale_encode", args) if rc is None else rc, check)
 
 
 def hif8_gemm_ex(Aq, lda, a_is_km, Wq, ldw, w_is_nk, Cmat, ldc, c_dtype, M, N, K, d_scale_exp_a=None, d_scale_exp_w=None,
                  d_scale_exp_w_channel=None, accumulate=0, workspace=None, workspace_bytes=0, stream=None, check=True):
-    return _check(lib.hif8_gemm_ex(_ptr(Aq), lda, int(a_is_km), _ptr(Wq), ldw, int(w_is_nk), _ptr(Cmat), ldc, c_dtype, M, N, K,
-                                   _ptr(d_scale_exp_a), _ptr(d_scale_exp_w), _ptr(d_scale_exp_w_channel), int(accumulate),
-                                   _ptr(workspace), workspace_bytes, _stream(stream)), check)
+    args = (Aq, lda, int(a_is_km), Wq, ldw, int(w_is_nk), Cmat, ldc, c_dtype, M, N, K, d_scale_exp_a, d_scale_exp_w,
+            d_scale_exp_w_channel, int(accumulate), workspace, workspace_bytes, stream)
+    rc = _c.hif8_gemm_ex(*args)
+    return _check(_via_ctypes("hif8_gemm_ex", args) if rc is None else rc, check)
 
 
 def hif8_encode_transpose(src, src_dtype, dst, rows, cols, scale_exp=0, d_scale_exp=None, rnd=RND_TA, flags=0, seed=0,
                           stream=None, check=True):
-    return _check(lib.hif8_encode_transpose(_ptr(src), src_dtype, _ptr(dst), rows, cols, scale_exp, _ptr(d_scale_exp), rnd,
-                                            flags, seed, _stream(stream)), check)
+    args = (src, src_dtype, dst, rows, cols, scale_exp, d_scale_exp, rnd, flags, seed, stream)
+    rc = _c.hif8_encode_transpose(*args)
+    return _check(_via_ctypes("hif8_encode_transpose", args) if rc is None else rc, check)
 
 
 def hif8_als_state_init(d_state, init_scale_exp=32, init_window_index=1, stream=None, check=True):
@@ -256,14 +287,23 @@ def hif8_als_state_init(d_state, init_scale_exp=32, init_window_index=1, stream=
 
 
 def hif8_als_update(d_state, d_found_inf, stream=None, check=True):
-    return _check(lib.hif8_als_update(_ptr(d_state), _ptr(d_found_inf), _stream(stream)), check)
+    args = (d_state, d_found_inf, stream)
+    rc = _c.hif8_als_update(*args)
+    return _check(_via_ctypes("hif8_als_update", args) if rc is None else rc, check)
 
 
 def hif8_check_finite(src, dtype, n, d_found_inf, stream=None, check=True):
-    return _check(lib.hif8_check_finite(_ptr(src), dtype, n, _ptr(d_found_inf), _stream(stream)), check)
+    args = (src, dtype, n, d_found_inf, stream)
+    rc = _c.hif8_check_finite(*args)
+    return _check(_via_ctypes("hif8_check_finite", args) if rc is None else rc, check)
 
 
 def hif8_encode_from_amax(src, src_dtype, dst, n, target_exp, rnd, flags, seed, d_amax, d_scale_exp_out=None, d_scale_out=None,
                           stream=None, check=True):
-    return _check(lib.hif8_encode_from_amax(_ptr(src), src_dtype, _ptr(dst), n, target_exp, rnd, flags, seed, _ptr(d_amax),
-                                            _ptr(d_scale_exp_out), _ptr(d_scale_out), _stream(stream)), check)
+    args = (src, src_dtype, dst, n, target_exp, rnd, flags, seed, d_amax, d_scale_exp_out, d_scale_out, stream)
+    rc = _c.hif8_encode_from_amax(*args)
+    return _check(_via_ctypes("hif8_encode_from_amax", args) if rc is None else rc, check)
+
+
+# the names that the package itself offers (see the package's __getattr__)
+PUBLIC = frozenset(n for n in globals() if not n.startswith("_") and n not in ("C", "lib", "os", "torch"))

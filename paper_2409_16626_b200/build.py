@@ -1,13 +1,16 @@
-"""Build libhif8.so (sm_100a) in-tree with nvcc.  `python -m paper_2409_16626_b200.build [--force]`."""
+"""Build libhif8.so (sm_100a) and the CPython entry to it in-tree.  `python -m paper_2409_16626_b200.build [--force]`."""
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhif8.so")
+CALL_SRC, CALL = os.path.join(CSRC, "hif8_call.cpp"), os.path.join(HERE, "_hif8_call.so")
+CXX = os.environ.get("CXX", "g++")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
@@ -18,10 +21,10 @@ def sources():
 
 
 def _stale():
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
+    deps = sources() + [CALL_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -40,6 +43,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if p.wait() != 0:
             raise RuntimeError("nvcc failed: " + " ".join(cmd))
     subprocess.check_call([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB] + objs + ["-lcudart"])
+    subprocess.check_call([CXX, "-O2", "-std=c++17", "-Wall", "-fPIC", "-shared", "-I" + os.path.join(ROOT, "include"),
+                           "-I" + sysconfig.get_paths()["include"], CALL_SRC, "-o", CALL, "-L" + HERE, "-l:libhif8.so", "-Wl,-rpath,$ORIGIN"])
     return LIB
 
 

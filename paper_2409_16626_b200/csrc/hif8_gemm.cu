@@ -2279,16 +2279,6 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
     if (major != 10) return HIF8_ERR_CUDA;
 
-    CUtensorMap map_a, map_w;
-    // ([M,K] activations: 64-byte rows with the 64-byte swizzle, read row-wise by the decode warps of the fused kernel)
-    const bool ok_a = a_is_km ? make_map(&map_a, Aq, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BM, BK)
-                              : make_map(&map_a, Aq, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM, false, 64);
-    if (!ok_a) return HIF8_ERR_CUDA;
-    // byte tiles of one CTA of a pair: 128 rows of A, 128 of the 256 columns of W
-    const bool ok_w = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, BK, BN / 2)
-                              : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BN / 2, BK);
-    if (!ok_w) return HIF8_ERR_CUDA;
-
     GemmParams p{};
     p.C = C; p.ldc = ldc; p.c_is_f32 = c_dtype == HIF8_F32; p.M = M; p.N = N; p.K = K;
     p.d_sa = d_scale_exp_a; p.d_sw = d_scale_exp_w; p.d_sw_channel = d_scale_exp_w_channel;
@@ -2406,8 +2396,18 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         }
         return launch_weights_gemm(Wq, ldw, w_is_nk, a_bf, p, wd_clusters, st);
     }
-    if (cudaMemsetAsync(workspace, 0, 4, st) != cudaSuccess) return HIF8_ERR_CUDA;
+    // No room for the activations: both operands are decoded in the kernel.
+    CUtensorMap map_a, map_w;
+    // ([M,K] activations: 64-byte rows with the 64-byte swizzle, read row-wise by the decode warps of the fused kernel)
+    const bool ok_a = a_is_km ? make_map(&map_a, Aq, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BM, BK)
+                              : make_map(&map_a, Aq, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM, false, 64);
+    if (!ok_a) return HIF8_ERR_CUDA;
+    // byte tiles of one CTA of a pair: 128 rows of A, 128 of the 256 columns of W
+    const bool ok_w = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, BK, BN / 2)
+                              : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BN / 2, BK);
+    if (!ok_w) return HIF8_ERR_CUDA;
 
+    if (cudaMemsetAsync(workspace, 0, 4, st) != cudaSuccess) return HIF8_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2u * (unsigned)tiles2);
     cfg.blockDim = dim3(kThreads);
