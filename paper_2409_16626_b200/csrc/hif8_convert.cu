@@ -37,6 +37,122 @@ std::atomic<uint64_t> g_launches{0};
 
 namespace {
 
+// One source vector (16 bytes, vector index u of the tensor) converted and stored.
+template <int SRC, int MODE, bool FQ, bool AMAX, bool PATTERN>
+__device__ __forceinline__ void convert_vector(const ConvParams& p, const SmemTables& sm, const uint4& v, unsigned long long u, float scale,
+                                               float d1, float d2, uint32_t k0, uint32_t k1, float& amax)
+{
+    constexpr int PV = SrcTraits<SRC>::kPerVec;
+    if constexpr (SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ) {
+        // two elements per word (see encode_sum16)
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w}, ns2 = neg_scale_bf16x2(scale);
+        uint32_t y[4], c[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (AMAX) {
+                amax = amax_step(amax, __uint_as_float(w[k] << 16));
+                amax = amax_step(amax, __uint_as_float(w[k] & 0xFFFF0000u));
+            }
+            y[k] = mul_bf16x2(w[k], ns2);
+            c[k] = encode_sum16(w[k], y[k], sm.ta, sm.thr);
+        }
+        // gather the codes and the sign bytes of four elements; a set (inverted) sign clears bit 7
+        const uint32_t c0 = __byte_perm(c[0], c[1], 0x5410), c1 = __byte_perm(c[2], c[3], 0x5410);
+        const uint32_t s0 = __byte_perm(y[0], y[1], 0x7531), s1 = __byte_perm(y[2], y[3], 0x7531);
+        __stcs(reinterpret_cast<uint2*>(p.dst) + u, make_uint2(c0 & (~s0 | 0x7F7F7F7Fu), c1 & (~s1 | 0x7F7F7F7Fu)));
+        return;
+    }
+    if constexpr (SRC == HIF8_F32 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ) {
+        // four elements: neighbour-pair words, the comparisons pick the bytes pairwise, one sign step for all four
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        uint32_t y[4], ent[4], sel[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const float x = __uint_as_float(w[k]);
+            if (AMAX) amax = amax_step(amax, x);
+            const float ys = x * -scale;
+            y[k] = __float_as_uint(ys);
+            sel[k] = pair32_lookup<MODE>(ys, w[k], reinterpret_cast<const uint32_t*>(sm.ta), ent[k]) ? 1u : 0u;
+        }
+        const uint32_t c01 = __byte_perm(ent[0], ent[1], 0x4051u + sel[0] + (sel[1] << 4));
+        const uint32_t c23 = __byte_perm(ent[2], ent[3], 0x4051u + sel[2] + (sel[3] << 4));
+        const uint32_t s01 = __byte_perm(y[0], y[1], 0x7373), s23 = __byte_perm(y[2], y[3], 0x7373);
+        const uint32_t c = __byte_perm(c01, c23, 0x5410), s = __byte_perm(s01, s23, 0x5410);
+        __stcs(reinterpret_cast<uint32_t*>(p.dst) + u, c & (~s | 0x7F7F7F7Fu));  // a set (inverted) sign clears bit 7
+        return;
+    }
+    if constexpr (MODE == HIF8_RND_TA && !FQ && !PATTERN) {  // (a pattern sweep has neighbouring lanes in one table word anyway)
+        // the code table is read sign-free, the signs go back onto the packed words (see ta_magnitude_code)
+        uint32_t c[8];
+#pragma unroll
+        for (int k = 0; k < PV; k++) {
+            float x; uint32_t raw;
+            unpack<SRC>(v, k, x, raw);
+            if (AMAX) amax = amax_step(amax, x);
+            c[k] = ta_magnitude_code(x, scale, sm.ta);
+        }
+        uint32_t w0 = c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24), w1 = 0;
+        if (PV == 8) w1 = c[4] | (c[5] << 8) | (c[6] << 16) | (c[7] << 24);
+        put_signs<SRC>(v, w0, w1);
+        if (PV == 4) __stcs(reinterpret_cast<uint32_t*>(p.dst) + u, w0);
+        else __stcs(reinterpret_cast<uint2*>(p.dst) + u, make_uint2(w0, w1));
+        return;
+    }
+    uint32_t codes[PV];
+    uint4 r0 = make_uint4(0, 0, 0, 0), r1 = r0;
+    if (MODE == HIF8_RND_SR) {
+        r0 = philox4x32_10((uint32_t)(u * (PV / 4)), (uint32_t)((u * (PV / 4)) >> 32), k0, k1);
+        if (PV == 8) r1 = philox4x32_10((uint32_t)(u * 2 + 1), (uint32_t)((u * 2 + 1) >> 32), k0, k1);
+    }
+    const uint32_t rw[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+#pragma unroll
+    for (int k = 0; k < PV; k++) {
+        float x; uint32_t raw;
+        unpack<SRC>(v, k, x, raw);
+        if (AMAX) amax = amax_step(amax, x);
+        codes[k] = encode_one<MODE, SRC>(x, raw, scale, sm.ta, sm.thr, rw[k]);
+    }
+    if (!FQ) {
+        uint32_t w0 = codes[0] | (codes[1] << 8) | (codes[2] << 16) | (codes[3] << 24);
+        if (PV == 4) __stcs(reinterpret_cast<uint32_t*>(p.dst) + u, w0);
+        else {
+            uint32_t w1 = codes[4] | (codes[5] << 8) | (codes[6] << 16) | (codes[7] << 24);
+            __stcs(reinterpret_cast<uint2*>(p.dst) + u, make_uint2(w0, w1));
+        }
+    } else {
+        uint32_t o[PV];
+#pragma unroll
+        for (int k = 0; k < PV; k++) o[k] = to_bits<SRC>(sm.dec[codes[k]] * d1 * d2);
+        uint4 out;
+        if (PV == 4) out = make_uint4(o[0], o[1], o[2], o[3]);
+        else out = make_uint4(o[0] | (o[1] << 16), o[2] | (o[3] << 16), o[4] | (o[5] << 16), o[6] | (o[7] << 16));
+        __stcs(reinterpret_cast<uint4*>(p.dst) + u, out);
+    }
+}
+
+// element i on its own (what whole vectors do not cover)
+template <int SRC, int MODE, bool FQ>
+__device__ __forceinline__ void convert_element(const ConvParams& p, const SmemTables& sm, float x, uint32_t raw, unsigned long long i, float scale,
+                                                float d1, float d2, uint32_t k0, uint32_t k1)
+{
+    uint32_t word = 0;
+    if (MODE == HIF8_RND_SR) {
+        uint4 r = philox4x32_10((uint32_t)(i >> 2), (uint32_t)(i >> 34), k0, k1);
+        word = philox_word(r, (unsigned)i & 3u);
+    }
+    uint32_t c;
+    if constexpr (SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ) {
+        const uint32_t y = mul_bf16x2(raw, neg_scale_bf16x2(scale));  // the element as the low half of a word
+        c = encode_sum16(raw, y, sm.ta, sm.thr) & (~(y >> 8) | 0x7Fu) & 0xFFu;
+    } else c = encode_one<MODE, SRC>(x, raw, scale, sm.ta, sm.thr, word);
+    if (!FQ) reinterpret_cast<uint8_t*>(p.dst)[i] = (uint8_t)c;
+    else {
+        uint32_t o = to_bits<SRC>(sm.dec[c] * d1 * d2);
+        if (SRC == HIF8_F32) reinterpret_cast<uint32_t*>(p.dst)[i] = o;
+        else reinterpret_cast<unsigned short*>(p.dst)[i] = (unsigned short)o;
+    }
+}
+
 // One group of kUnroll vectors per thread starting at vector index `base`.  FULL: the whole group lies inside the
 // tensor, so no bounds are checked.
 // PATTERN (FP32 only): the source is not read; element i is the FP32 value with encoding p.pattern_first + i.
@@ -44,7 +160,6 @@ template <int SRC, int MODE, bool FQ, bool AMAX, bool FULL, bool PATTERN = false
 __device__ __forceinline__ void convert_group(const ConvParams& p, const SmemTables& sm, unsigned long long base, unsigned long long n_vec,
                                               float scale, float d1, float d2, uint32_t k0, uint32_t k1, float& amax)
 {
-    constexpr int PV = SrcTraits<SRC>::kPerVec;
     const uint4* src = reinterpret_cast<const uint4*>(p.src);
     uint4 v[kUnroll];
 #pragma unroll
@@ -60,91 +175,7 @@ __device__ __forceinline__ void convert_group(const ConvParams& p, const SmemTab
     for (int j = 0; j < kUnroll; j++) {
         unsigned long long u = base + (unsigned long long)j * kThreads + threadIdx.x;
         if (!FULL && u >= n_vec) continue;
-        if constexpr (SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ) {
-            // two elements per word (see encode_sum16)
-            const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w}, ns2 = neg_scale_bf16x2(scale);
-            uint32_t y[4], c[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                if (AMAX) {
-                    amax = amax_step(amax, __uint_as_float(w[k] << 16));
-                    amax = amax_step(amax, __uint_as_float(w[k] & 0xFFFF0000u));
-                }
-                y[k] = mul_bf16x2(w[k], ns2);
-                c[k] = encode_sum16(w[k], y[k], sm.ta, sm.thr);
-            }
-            // gather the codes and the sign bytes of four elements; a set (inverted) sign clears bit 7
-            const uint32_t c0 = __byte_perm(c[0], c[1], 0x5410), c1 = __byte_perm(c[2], c[3], 0x5410);
-            const uint32_t s0 = __byte_perm(y[0], y[1], 0x7531), s1 = __byte_perm(y[2], y[3], 0x7531);
-            __stcs(reinterpret_cast<uint2*>(p.dst) + u, make_uint2(c0 & (~s0 | 0x7F7F7F7Fu), c1 & (~s1 | 0x7F7F7F7Fu)));
-            continue;
-        }
-        if constexpr (SRC == HIF8_F32 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ) {
-            // four elements: neighbour-pair words, the comparisons pick the bytes pairwise, one sign step for all four
-            const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
-            uint32_t y[4], ent[4], sel[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const float x = __uint_as_float(w[k]);
-                if (AMAX) amax = amax_step(amax, x);
-                const float ys = x * -scale;
-                y[k] = __float_as_uint(ys);
-                sel[k] = pair32_lookup<MODE>(ys, w[k], reinterpret_cast<const uint32_t*>(sm.ta), ent[k]) ? 1u : 0u;
-            }
-            const uint32_t c01 = __byte_perm(ent[0], ent[1], 0x4051u + sel[0] + (sel[1] << 4));
-            const uint32_t c23 = __byte_perm(ent[2], ent[3], 0x4051u + sel[2] + (sel[3] << 4));
-            const uint32_t s01 = __byte_perm(y[0], y[1], 0x7373), s23 = __byte_perm(y[2], y[3], 0x7373);
-            const uint32_t c = __byte_perm(c01, c23, 0x5410), s = __byte_perm(s01, s23, 0x5410);
-            __stcs(reinterpret_cast<uint32_t*>(p.dst) + u, c & (~s | 0x7F7F7F7Fu));  // a set (inverted) sign clears bit 7
-            continue;
-        }
-        if constexpr (MODE == HIF8_RND_TA && !FQ && !PATTERN) {  // (a pattern sweep has neighbouring lanes in one table word anyway)
-            // the code table is read sign-free, the signs go back onto the packed words (see ta_magnitude_code)
-            uint32_t c[8];
-#pragma unroll
-            for (int k = 0; k < PV; k++) {
-                float x; uint32_t raw;
-                unpack<SRC>(v[j], k, x, raw);
-                if (AMAX) amax = amax_step(amax, x);
-                c[k] = ta_magnitude_code(x, scale, sm.ta);
-            }
-            uint32_t w0 = c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24), w1 = 0;
-            if (PV == 8) w1 = c[4] | (c[5] << 8) | (c[6] << 16) | (c[7] << 24);
-            put_signs<SRC>(v[j], w0, w1);
-            if (PV == 4) __stcs(reinterpret_cast<uint32_t*>(p.dst) + u, w0);
-            else __stcs(reinterpret_cast<uint2*>(p.dst) + u, make_uint2(w0, w1));
-            continue;
-        }
-        uint32_t codes[PV];
-        uint4 r0 = make_uint4(0, 0, 0, 0), r1 = r0;
-        if (MODE == HIF8_RND_SR) {
-            r0 = philox4x32_10((uint32_t)(u * (PV / 4)), (uint32_t)((u * (PV / 4)) >> 32), k0, k1);
-            if (PV == 8) r1 = philox4x32_10((uint32_t)(u * 2 + 1), (uint32_t)((u * 2 + 1) >> 32), k0, k1);
-        }
-        const uint32_t rw[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-#pragma unroll
-        for (int k = 0; k < PV; k++) {
-            float x; uint32_t raw;
-            unpack<SRC>(v[j], k, x, raw);
-            if (AMAX) amax = amax_step(amax, x);
-            codes[k] = encode_one<MODE, SRC>(x, raw, scale, sm.ta, sm.thr, rw[k]);
-        }
-        if (!FQ) {
-            uint32_t w0 = codes[0] | (codes[1] << 8) | (codes[2] << 16) | (codes[3] << 24);
-            if (PV == 4) __stcs(reinterpret_cast<uint32_t*>(p.dst) + u, w0);
-            else {
-                uint32_t w1 = codes[4] | (codes[5] << 8) | (codes[6] << 16) | (codes[7] << 24);
-                __stcs(reinterpret_cast<uint2*>(p.dst) + u, make_uint2(w0, w1));
-            }
-        } else {
-            uint32_t o[PV];
-#pragma unroll
-            for (int k = 0; k < PV; k++) o[k] = to_bits<SRC>(sm.dec[codes[k]] * d1 * d2);
-            uint4 out;
-            if (PV == 4) out = make_uint4(o[0], o[1], o[2], o[3]);
-            else out = make_uint4(o[0] | (o[1] << 16), o[2] | (o[3] << 16), o[4] | (o[5] << 16), o[6] | (o[7] << 16));
-            __stcs(reinterpret_cast<uint4*>(p.dst) + u, out);
-        }
+        convert_vector<SRC, MODE, FQ, AMAX, PATTERN>(p, sm, v[j], u, scale, d1, d2, k0, k1, amax);
     }
 }
 
@@ -190,22 +221,7 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const ConvParams p, u
             if (PATTERN) { raw = p.pattern_first + (uint32_t)i; x = __uint_as_float(raw); }
             else load_scalar<SRC>(p.src, i, x, raw);
             if (AMAX) amax = amax_step(amax, x);
-            uint32_t word = 0;
-            if (MODE == HIF8_RND_SR) {
-                uint4 r = philox4x32_10((uint32_t)(i >> 2), (uint32_t)(i >> 34), k0, k1);
-                word = philox_word(r, (unsigned)i & 3u);
-            }
-            uint32_t c;
-            if constexpr (kPair16) {
-                const uint32_t y = mul_bf16x2(raw, neg_scale_bf16x2(scale));  // the element as the low half of a word
-                c = encode_sum16(raw, y, sm.ta, sm.thr) & (~(y >> 8) | 0x7Fu) & 0xFFu;
-            } else c = encode_one<MODE, SRC>(x, raw, scale, sm.ta, sm.thr, word);
-            if (!FQ) reinterpret_cast<uint8_t*>(p.dst)[i] = (uint8_t)c;
-            else {
-                uint32_t o = to_bits<SRC>(sm.dec[c] * d1 * d2);
-                if (SRC == HIF8_F32) reinterpret_cast<uint32_t*>(p.dst)[i] = o;
-                else reinterpret_cast<unsigned short*>(p.dst)[i] = (unsigned short)o;
-            }
+            convert_element<SRC, MODE, FQ>(p, sm, x, raw, i, scale, d1, d2, k0, k1);
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -231,6 +247,84 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const ConvParams p, u
                 }
             }
         }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Just-in-time scaling of a small tensor in one launch: a cluster of up to eight blocks holds the source in shared memory,
+// reduces its amax (each block tells the others its own through distributed shared memory, one cluster barrier), and converts
+// from there.  No accumulator in the workspace, so nothing to clear.  Latency and launches bound it: the three launches of the
+// general path (clear, amax, convert) take 3.3 us on the device and 8 us from the host, this 2.3 us and 4 us (512 BF16
+// elements, round half away); 3.9 against 3.1 us at 131072.  The limits are where eight blocks take as long on the device as
+// three launches over all SMs: 256 KiB of source, half of that for dequantized results, which carry more arithmetic
+// (131072 BF16 elements under hybrid rounding: 4.5 us by three launches, 5.0 us by one).
+// ------------------------------------------------------------------------------------------------
+constexpr int kOneThreads = 512, kOneVecs = 4, kOneBlocks = 8;  // 32 KiB of source per block
+constexpr unsigned long long kOneMaxVecs = (unsigned long long)kOneThreads * kOneVecs * kOneBlocks, kOneMaxVecsFq = kOneMaxVecs / 2;
+
+template <int SRC, int MODE, bool FQ>
+__global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParams p, unsigned n_vec)
+{
+    extern __shared__ __align__(16) uint4 s_src[];
+    __shared__ SmemTables sm;
+    __shared__ uint32_t s_part[kOneThreads / 32], s_block[kOneBlocks];
+    constexpr int PV = SrcTraits<SRC>::kPerVec;
+    constexpr bool kPair16 = SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ;
+    pdl_launch_dependents();
+    const unsigned first = blockIdx.x * kOneThreads + threadIdx.x, step = gridDim.x * kOneThreads;  // vectors first, first + step, ..
+    pdl_wait_prior_grid();
+    const uint4* src = reinterpret_cast<const uint4*>(p.src);
+    uint4 v[kOneVecs];
+#pragma unroll
+    for (int j = 0; j < kOneVecs; j++) v[j] = first + j * step < n_vec ? __ldcs(src + first + j * step) : make_uint4(0, 0, 0, 0);
+    // what whole vectors do not cover: at most PV - 1 elements, one per thread of the first block
+    const unsigned long long i_tail = (unsigned long long)n_vec * PV + threadIdx.x;
+    const bool tail = blockIdx.x == 0 && i_tail < p.n;
+    float x_tail = 0.f;
+    uint32_t raw_tail = 0u;
+    if (tail) load_scalar<SRC>(p.src, i_tail, x_tail, raw_tail);
+    // (tables under the loads' latency)
+    if (kPair16) setup_sum16<MODE, kOneThreads>(sm.ta, sm.thr, p.flags);
+    else setup_tables<true, MODE != HIF8_RND_TA, FQ, MODE, SRC, kOneThreads>(sm, p.flags);
+    float amax = amax_step(0.f, x_tail);
+#pragma unroll
+    for (int j = 0; j < kOneVecs; j++) {
+        if (first + j * step < n_vec) s_src[j * kOneThreads + threadIdx.x] = v[j];
+#pragma unroll
+        for (int k = 0; k < PV; k++) {
+            float x; uint32_t raw;
+            unpack<SRC>(v[j], k, x, raw);
+            amax = amax_step(amax, x);
+        }
+    }
+    uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));  // non-negative floats order as integers
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kOneThreads / 32 ? s_part[threadIdx.x] : 0u);
+        if (threadIdx.x < gridDim.x) {
+            uint32_t to;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(s_block + blockIdx.x)), "r"(threadIdx.x));
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to), "r"(m) : "memory");
+        }
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    uint32_t ab = 0u;
+    for (unsigned b = 0; b < gridDim.x; b++) ab = max(ab, s_block[b]);
+
+    const int se = scale_exp_from_amax(ab, p.target_exp), da = (-se) / 2, db = -se - da;
+    const float scale = pow2f(se), d1 = pow2f(da), d2 = pow2f(db);
+    const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
+    float unused = 0.f;
+#pragma unroll 1
+    for (unsigned u = first, j = threadIdx.x; u < n_vec; u += step, j += kOneThreads)
+        convert_vector<SRC, MODE, FQ, false, false>(p, sm, s_src[j], u, scale, d1, d2, k0, k1, unused);
+    if (tail) convert_element<SRC, MODE, FQ>(p, sm, x_tail, raw_tail, i_tail, scale, d1, d2, k0, k1);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (p.d_scale_exp_out) *p.d_scale_exp_out = se;
+        if (p.d_scale_out) *p.d_scale_out = scale;
+        if (p.d_amax_out) *p.d_amax_out = __uint_as_float(ab);
     }
 }
 
@@ -685,6 +779,53 @@ int dispatch_convert(int dtype, int rnd, const ConvParams& p, bool vec_ok, int s
     }
 }
 
+template <int SRC, int MODE, bool FQ>
+int launch_one(const ConvParams& p, cudaStream_t st)
+{
+    static_assert(sizeof(SmemTables) + kOneThreads * kOneVecs * 16 + 256 <= 48 * 1024, "no opt-in to more shared memory");
+    const unsigned n_vec = (unsigned)(p.n / SrcTraits<SRC>::kPerVec);
+    // two vectors per thread while there are blocks to add
+    unsigned blocks = 1;
+    while (blocks < (unsigned)kOneBlocks && blocks * kOneThreads * 2 < n_vec) blocks *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kOneThreads);
+    cfg.dynamicSmemBytes = (size_t)((n_vec + blocks * kOneThreads - 1) / (blocks * kOneThreads)) * kOneThreads * 16;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = blocks; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t lrc = cudaLaunchKernelEx(&cfg, one_launch_kernel<SRC, MODE, FQ>, p, n_vec);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return lrc == cudaSuccess && cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+}
+
+template <int SRC, bool FQ>
+int dispatch_one_mode(int rnd, const ConvParams& p, cudaStream_t st)
+{
+    switch (rnd) {
+        case HIF8_RND_TA: return launch_one<SRC, HIF8_RND_TA, FQ>(p, st);
+        case HIF8_RND_HR: return launch_one<SRC, HIF8_RND_HR, FQ>(p, st);
+        case HIF8_RND_SSR: return launch_one<SRC, HIF8_RND_SSR, FQ>(p, st);
+        case HIF8_RND_TE: return launch_one<SRC, HIF8_RND_TE, FQ>(p, st);
+        default: return launch_one<SRC, HIF8_RND_SR, FQ>(p, st);
+    }
+}
+
+template <bool FQ>
+int dispatch_one(int dtype, int rnd, const ConvParams& p, cudaStream_t st)
+{
+    switch (dtype) {
+        case HIF8_F32: return dispatch_one_mode<HIF8_F32, FQ>(rnd, p, st);
+        case HIF8_BF16: return dispatch_one_mode<HIF8_BF16, FQ>(rnd, p, st);
+        default: return dispatch_one_mode<HIF8_F16, FQ>(rnd, p, st);
+    }
+}
+
 int launch_fq_ta(int dtype, int rnd, const ConvParams& p, bool vec_ok, int sms, cudaStream_t st)
 {
     const unsigned long long pv = dtype == HIF8_F32 ? 4 : 8;
@@ -822,6 +963,9 @@ static int scaled_convert(bool fq, const void* src, void* dst, int dtype, size_t
     bool vec_ok = aligned16(src) && (reinterpret_cast<uintptr_t>(dst) % out_align) == 0;
     if (jit || want_amax) {
         if (!ws || workspace_bytes < kConvWorkspaceBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return HIF8_ERR_WORKSPACE;
+        // a tensor that one cluster holds: one launch (what is not 16-byte aligned: the general path)
+        if (jit && vec_ok && n / (dtype == HIF8_F32 ? 4 : 8) <= (fq ? kOneMaxVecsFq : kOneMaxVecs))
+            return fq ? dispatch_one<true>(dtype, rnd, p, st) : dispatch_one<false>(dtype, rnd, p, st);
         // (a delayed-scaling state keeps its two words at zero between passes itself)
         if (!scale_state) {
             if (launch_pdl(clear_accum_kernel, 1u, st, ws) != cudaSuccess) return HIF8_ERR_CUDA;

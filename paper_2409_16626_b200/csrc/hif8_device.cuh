@@ -390,10 +390,10 @@ __device__ __forceinline__ uint32_t encode_one(float x, uint32_t raw, float scal
 //   reach 2^-22 exactly when floor(4 F) >= T2; smaller values add nothing.  Anything that ends below 2^-22 reads zero.
 //   code8[(e, top three mantissa bits)] is the truncated magnitude with bit 7 = "takes the sign" (see pair_entry).
 // ------------------------------------------------------------------------------------------------
-template <int MODE>
+template <int MODE, int NT = kThreads>
 __device__ __forceinline__ void setup_sum16(uint8_t* code8, uint32_t* inck, unsigned flags)
 {
-    for (int i = threadIdx.x; i < 512; i += kThreads) {  // four codes per word
+    for (int i = threadIdx.x; i < 512; i += NT) {  // four codes per word
         uint32_t word = 0;
 #pragma unroll
         for (int b = 0; b < 4; b++) {
@@ -407,7 +407,7 @@ __device__ __forceinline__ void setup_sum16(uint8_t* code8, uint32_t* inck, unsi
         }
         reinterpret_cast<uint32_t*>(code8)[i] = word;
     }
-    {
+    if (threadIdx.x < kThreads) {
         const int e = threadIdx.x, E = e - 127;  // kThreads == 256 biased exponents
         uint32_t v = 0u;
         if (E >= -24 && E <= 15) {
@@ -460,7 +460,8 @@ struct __align__(16) SmemTables {
     float dec[256];
 };
 
-template <bool NEED_TA, bool NEED_SH, bool NEED_DEC, int MODE = HIF8_RND_TA, int SRC = HIF8_F32>
+// NT threads (kThreads or more) take part
+template <bool NEED_TA, bool NEED_SH, bool NEED_DEC, int MODE = HIF8_RND_TA, int SRC = HIF8_F32, int NT = kThreads>
 __device__ __forceinline__ void setup_tables(SmemTables& s, unsigned flags)
 {
     constexpr bool kPair = (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && SRC == HIF8_F32;  // neighbour-pair words instead of code bytes
@@ -468,7 +469,7 @@ __device__ __forceinline__ void setup_tables(SmemTables& s, unsigned flags)
         // 2048 words indexed by (exponent, top three mantissa bits).  The magnitudes that reach the lookup lie in
         // 2^-23 .. Inf / NaN; 2^-23 .. 2^15 come from the compile-time table, everything above is Inf.
         uint32_t* d = reinterpret_cast<uint32_t*>(s.ta);
-        for (int i = threadIdx.x; i < 2048; i += kThreads) {
+        for (int i = threadIdx.x; i < 2048; i += NT) {
             const int e = i >> 3, E = e - 127;
             uint32_t v = 0u;
             if (e >= 104 && e <= 142) v = g_pair_table.v[i];
@@ -497,7 +498,7 @@ __device__ __forceinline__ void setup_tables(SmemTables& s, unsigned flags)
         constexpr bool kTrunc = MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR || MODE == HIF8_RND_TE;  // modes that round before the lookup
         const uint4* g = reinterpret_cast<const uint4*>(kTrunc ? g_trunc_table.v : g_ta_table.v);
         uint4* d = reinterpret_cast<uint4*>(s.ta);
-        for (int i = threadIdx.x; i < 512; i += kThreads) {
+        for (int i = threadIdx.x; i < 512; i += NT) {
             const uint32_t e = i & 255, inf = ((uint32_t)(i >> 8) << 7) | 0x6Fu;
             uint4 v;
             if (e < 103) v = make_uint4(0, 0, 0, 0);
@@ -524,7 +525,7 @@ __device__ __forceinline__ void setup_tables(SmemTables& s, unsigned flags)
             d[i] = v;
         }
     }
-    if (NEED_SH && !kPair) {
+    if (NEED_SH && !kPair && threadIdx.x < kThreads) {
         const int e = threadIdx.x, E = e - 127;  // kThreads == 256 biased exponents
         constexpr bool kThreshold = MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR;
         // TE / SR: thr[e] = e0.  Threshold modes (16-bit sources): thr[2e] = e0 (source LSB 0), thr[2e + 1] = e1 (LSB 1).
@@ -546,7 +547,7 @@ __device__ __forceinline__ void setup_tables(SmemTables& s, unsigned flags)
         if (kThreshold) { s.thr[2 * e] = e0; s.thr[2 * e + 1] = e1; }
         else s.thr[e] = e0;
     }
-    if (NEED_DEC) s.dec[threadIdx.x] = __uint_as_float(decode_bits_f32(threadIdx.x));
+    if (NEED_DEC && threadIdx.x < kThreads) s.dec[threadIdx.x] = __uint_as_float(decode_bits_f32(threadIdx.x));
     __syncthreads();
 }
 

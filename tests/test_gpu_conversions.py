@@ -203,6 +203,44 @@ def test_amax_scale_encode_jit_and_delayed(dtype):
     assert_same(rb(), O.encode(src, dtype, 5, O.TA, 0, quick=True), src)
 
 
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
+@pytest.mark.parametrize("mode", MODES)
+def test_scaled_conversions_of_small_tensors(dtype, mode):
+    """The one-launch form: no, one and several vectors per thread, 1 to 8 blocks, tails; its limit and the first size above;
+    a source that is not 16-byte aligned takes the general path and gives the same."""
+    pv = 4 if dtype == H.F32 else 8
+    ws, wsb = workspace()
+    outs = torch.zeros(4, dtype=torch.int32, device="cuda")
+    for i, n in enumerate([1, pv - 1, pv, 511 * pv + 3, 1024 * pv, 1024 * pv + 1, 1025 * pv, 4096 * pv + 2, 8192 * pv + pv - 1,
+                           8193 * pv, 16384 * pv - 1, 16384 * pv + pv - 1, 16385 * pv]):
+        if dtype == H.F32:
+            src = W.loguniform_f32(n, seed=i, lo_exp=-30, hi_exp=20).view(np.uint32).copy()
+        else:
+            src = (W.normal_bf16(n, seed=i) if dtype == H.BF16 else W.normal_f32(n, seed=i).astype(np.float16).view(np.uint16)).copy()
+        specials = {H.F32: [0x7F800000, 0xFFC00001], H.BF16: [0x7F80, 0xFFC1], H.F16: [0xFC00, 0x7E01]}[dtype]
+        if n > 100:
+            src[[3, n - 1]] = specials                       # Inf / NaN do not take part in amax
+        flags = FLAGSETS[i % 4]
+        amax, se = O.amax_scale(src, dtype, 14)
+        want, want_fq = O.encode(src, dtype, se, mode, flags, seed=9, quick=True), O.fake_quant(src, dtype, se, mode, flags, seed=9, quick=True)
+        d_src = to_dev(src)
+        shifted = torch.empty(n * src.itemsize + 16, dtype=torch.uint8, device="cuda")
+        shifted[4:4 + n * src.itemsize] = torch.from_numpy(src.view(np.uint8)).cuda()
+        for source in (d_src, shifted.data_ptr() + 4):
+            _, dptr, rb = dev_empty(n, np.uint8)
+            H.hif8_amax_scale_encode(source, dtype, dptr, n, 14, mode, flags, 9, None, outs[0:1], outs[1:2], outs[2:3], ws, wsb)
+            torch.cuda.synchronize()
+            o = outs.cpu().numpy()
+            assert o[0:1].view(np.float32)[0] == np.float32(amax) and o[1] == se and o[2:3].view(np.float32)[0] == np.float32(2.0) ** se
+            assert_same(rb(), want, src)
+        buf = d_src.clone()
+        H.hif8_fake_quant(buf, buf, dtype, n, 1, 14, mode, flags, 9, outs[0:1], outs[1:2], ws, wsb)
+        torch.cuda.synchronize()
+        o = outs.cpu().numpy()
+        assert o[0:1].view(np.float32)[0] == np.float32(amax) and o[1] == se
+        assert_same(buf.cpu().numpy().view(NP_OF[dtype]), want_fq, src)
+
+
 def test_amax_alone():
     ws, wsb = workspace()
     out = torch.zeros(1, dtype=torch.float32, device="cuda")
