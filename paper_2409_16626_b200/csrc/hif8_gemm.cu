@@ -1386,10 +1386,12 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
 // rows by TMA (the B operand).  A k-block here is 128 k.  Warp roles per CTA:
 //   warps 0-3   epilogue: accumulator column = activation row m, lane = weight column n
 //   warp  4     copies of weight bytes, four stages of 16 KiB       warp 22  copies of the activation tiles, four stages
-//   warp  5     MMA issuer (even CTA)                               warps 6-21  four decode groups, group g on it = g (mod 4)
+//   warp  5     MMA issuer (even CTA)                               warps 6-21  four decode groups, group g on it = g (mod 4),
+//                                                                              and the epilogue
 // Two forms, one kernel:
-//   split = 1   persistent: pair p of P takes tiles p, p + P, ..; copies and decode of a tile run on under the epilogue of
-//               the one before (only its MMAs wait for the accumulator).
+//   split = 1   persistent: pair p of P takes tiles p, p + P, ..  A decode group that is through with a tile decodes one k-block
+//               of the next (which fills the four stages) and then joins the epilogue: with warps 0-3 alone the accumulator was
+//               occupied for 13400 cycles (against 64000 for the k-blocks at K = 7168), now 5000.
 //   split > 1   a cluster of `split` pairs per tile, each pair a part of K; the pairs exchange their partial sums through
 //               distributed shared memory, every pair finishes a part of the activation rows, adding in pair order.  For
 //               products with too few tiles for the device and for the last, incomplete round of the persistent form.
@@ -1509,7 +1511,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps);
             mbar_init(bar_bf_full(s), 2 * kGroupWarps + 1); mbar_init(bar_bf_empty(s), 1);  // (+ 1: the leader's announcement of the tile bytes)
         }
-        mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * kEpiWarps);
+        mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps));
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1606,74 +1608,77 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                 if (ok) tc_commit_pair(bar_acc_full, lead);
             }
         }
-    } else if (warp >= kFirstDecodeWarp) {
-        // ------------------------------------------------------------------ decode warps
-        const int group = (warp - kFirstDecodeWarp) / kGroupWarps, quarter = warp & 3;
-        const int n_it = ((t_end - t0 + t_step - 1) / t_step) * (kb1 - kb0);
-        const uint32_t tlane = tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemColsAcc;
-        bool ok = true, joined = false;
-        for (int it = group; it < n_it && ok; it += kDecodeGroups) {
-            const int s = it % kWdStages, r = it / kWdStages;
-            ok = mbar_wait(bar_u8_full(s), r & 1, abort_flag, p.status, 43);
-            if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 44);
-            if (!ok) break;
-            const uint32_t w8 = u8_stage(s), dst = tlane + (uint32_t)(s * (KB / 2));
-            // in two halves, one piece of code for both (unrolled, the first pass over it cost every group a thousand cycles of
-            // instruction fetches): [N,K] 64 k of the thread's column, [K,N] all 128 k of sixteen of the quarter's columns
-#pragma unroll 1
-            for (int h = 0; h < 2; h++) {
-                uint4 v[4];
-                if (W_IS_NK) {
-                    // rows of 128 k with the 128-byte swizzle (chunk j of row r at chunk j ^ (r & 7))
-                    const uint32_t row = (uint32_t)(quarter * 32 + lane), w_row = w8 + row * KB, sw = row & 7u;
-#pragma unroll
-                    for (int j = 0; j < 4; j++) v[j] = lds_v4(w_row + (((uint32_t)(4 * h + j) ^ sw) << 4));
-                } else {
-                    // rows of 128 columns, one per k, read transposed (see the narrow kernel)
-#pragma unroll
-                    for (int j = 0; j < 4; j++)
-                        v[j] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(32 * j + lane) * BM + ((uint32_t)((2 * quarter + h) ^ (lane & 7)) << 4));
-                }
-                if (h == 1) {
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_u8_empty(s));
-                }
-                uint32_t o[32];
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint4 lo = decode8<7>(make_uint2(v[j].x, v[j].y), lut), hi = decode8<7>(make_uint2(v[j].z, v[j].w), lut);
-                    o[8 * j + 0] = lo.x; o[8 * j + 1] = lo.y; o[8 * j + 2] = lo.z; o[8 * j + 3] = lo.w;
-                    o[8 * j + 4] = hi.x; o[8 * j + 5] = hi.y; o[8 * j + 6] = hi.z; o[8 * j + 7] = hi.w;
-                }
-                if (W_IS_NK) tmem_st_32x32b_x32(dst + (uint32_t)(h * (BK / 2)), o);
-                else {
-                    tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16), o);
-                    tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16) + BK / 2, o + 16);
-                }
-            }
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (!joined) { cluster_wait(); joined = true; }  // before the first signal to another CTA
-            if (lane == 0) mbar_arrive_remote(map_to_cta(bar_bf_full(s), lead));
-        }
-        if (!joined) { __syncwarp(); cluster_wait(); }
-    } else cluster_wait();
+    } else if (warp < kFirstDecodeWarp) cluster_wait();  // warps 0-3
 
-    const bool one_tile = tp.count <= t_step;  // per pair: all warps are free for its epilogue
-    if (one_tile || warp < kEpiWarps) {
-        // ------------------------------------------------------------------ epilogue, in pieces of eight columns.  With several
-        // tiles per pair warps 0-3, one per quarter of the lanes; with one all warps, six (five) to a quarter.  In the split form
-        // the pairs exchange first: each finishes `per` of the pieces.
+    const bool one_tile = tp.count <= t_step, decodes = warp >= kFirstDecodeWarp && warp < kFirstDecodeWarp + kDecodeWarps;
+    if (one_tile || warp < kEpiWarps || decodes) {
+        // ------------------------------------------------------------------ decode and epilogue.  An epilogue is done in pieces of
+        // eight columns by five warps per quarter of the lanes; with one tile per pair all warps take part, six (five) to a
+        // quarter.  In the split form the pairs exchange first: each finishes `per` of the pieces.
         __syncwarp();
-        const int quarter = warp & 3, shares = !one_tile ? 1 : (quarter < 3 ? 6 : 5), share = !one_tile ? 0 : warp >> 2;
-        static_assert(kThreadsWd / 32 == 23, "six warps on the lanes of quarters 0 to 2, five on those of quarter 3");
+        const int group = (warp - kFirstDecodeWarp) / kGroupWarps, quarter = warp & 3;
+        const int shares = one_tile && quarter < 3 ? 6 : 5;
+        const int share = one_tile ? warp >> 2 : (decodes ? (warp - quarter) / 4 - (quarter < 2 ? 1 : 0) : 0);
+        static_assert(kThreadsWd / 32 == 23 && kFirstDecodeWarp == 6 && kDecodeWarps == 16,
+                      "six warps on the lanes of quarters 0 to 2, five on those of quarter 3; five each without warps 4, 5 and 22");
         const int row = quarter * 32 + lane, sa = p.d_sa ? *p.d_sa : 0, sw_all = (p.d_sw && !p.d_sw_channel) ? *p.d_sw : 0;
         const int c_size = p.c_is_f32 ? 4 : 2;
         const long long pitch = p.ldc * c_size;
-        const uint32_t tl = tmem_base + ((uint32_t)(quarter * 32) << 16), mine = base + (uint32_t)row * 16u;
-        int local = 0;
-        for (int t = t0; t < t_end; t += t_step, local++) {
+        const uint32_t tl = tmem_base + ((uint32_t)(quarter * 32) << 16), mine = base + (uint32_t)row * 16u, tlane = tl + kTmemColsAcc;
+        const int n_kb = kb1 - kb0;
+        int it = decodes ? group : 0x7FFFFFFF, tile_it = 0, local = 0;  // next k-block of the group; first k-block of the tile to finish next
+        bool joined = !decodes;
+        for (int t = t0; t < t_end;) {
+            // the group's k-blocks of this tile, and one of the next
+            const int n_it_known = t + t_step < t_end ? tile_it + 2 * n_kb : tile_it + n_kb;
+            if (it < tile_it + n_kb || (it < n_it_known && it - kDecodeGroups < tile_it + n_kb)) {
+                const int s = it % kWdStages, r = it / kWdStages;
+                bool ok = mbar_wait(bar_u8_full(s), r & 1, abort_flag, p.status, 43);
+                if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 44);
+                if (!ok) { it = 0x7FFFFFFF; continue; }  // (gives up at the next wait)
+                const uint32_t w8 = u8_stage(s), dst = tlane + (uint32_t)(s * (KB / 2));
+                // in two halves, one piece of code for both (unrolled, the first pass over it cost every group a thousand cycles of
+                // instruction fetches): [N,K] 64 k of the thread's column, [K,N] all 128 k of sixteen of the quarter's columns
+#pragma unroll 1
+                for (int h = 0; h < 2; h++) {
+                    uint4 v[4];
+                    if (W_IS_NK) {
+                        // rows of 128 k with the 128-byte swizzle (chunk j of row r at chunk j ^ (r & 7))
+                        const uint32_t row = (uint32_t)(quarter * 32 + lane), w_row = w8 + row * KB, sw = row & 7u;
+#pragma unroll
+                        for (int j = 0; j < 4; j++) v[j] = lds_v4(w_row + (((uint32_t)(4 * h + j) ^ sw) << 4));
+                    } else {
+                        // rows of 128 columns, one per k, read transposed (see the narrow kernel)
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            v[j] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(32 * j + lane) * BM + ((uint32_t)((2 * quarter + h) ^ (lane & 7)) << 4));
+                    }
+                    if (h == 1) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar_u8_empty(s));
+                    }
+                    uint32_t o[32];
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const uint4 lo = decode8<7>(make_uint2(v[j].x, v[j].y), lut), hi = decode8<7>(make_uint2(v[j].z, v[j].w), lut);
+                        o[8 * j + 0] = lo.x; o[8 * j + 1] = lo.y; o[8 * j + 2] = lo.z; o[8 * j + 3] = lo.w;
+                        o[8 * j + 4] = hi.x; o[8 * j + 5] = hi.y; o[8 * j + 6] = hi.z; o[8 * j + 7] = hi.w;
+                    }
+                    if (W_IS_NK) tmem_st_32x32b_x32(dst + (uint32_t)(h * (BK / 2)), o);
+                    else {
+                        tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16), o);
+                        tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16) + BK / 2, o + 16);
+                    }
+                }
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (!joined) { cluster_wait(); joined = true; }  // before the first signal to another CTA
+                if (lane == 0) mbar_arrive_remote(map_to_cta(bar_bf_full(s), lead));
+                it += kDecodeGroups;
+                continue;
+            }
+            if (!joined) { __syncwarp(); cluster_wait(); joined = true; }
             const int slab = t / tp.chunks, m0 = (t - slab * tp.chunks) * tp.bn, n = slab * 2 * BM + (int)half * BM + row;
             // 2^sc as one factor, and a second one for the few scales that need it
             const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = max(-126, min(126, sc));
@@ -1737,7 +1742,9 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             tc_fence_before();
             __syncwarp();
             if (!one_tile && lane == 0) mbar_arrive_remote(map_to_cta(bar_acc_empty, lead));
+            t += t_step; tile_it += n_kb; local++;
         }
+        if (!joined) { __syncwarp(); cluster_wait(); }
     }
 
     // ---- teardown: all waits are bounded, so everybody arrives; nobody leaves while the peer may still read this
