@@ -2,26 +2,18 @@
 //
 //   C[m,n] = 2^-(sa+sw) * sum_k value(Aq[m,k]) * value(Wq[k,n])       (Algorithm 1, "MatMul & Restore")
 //
-// Two paths behind one entry point.  The fused kernel (described next) needs no memory beyond its operands and
-// decodes the byte tiles of every CTA in shared memory; because every operand element is then decoded once per
-// tile that uses it, it is bound by the decode rate.  With a workspace large enough for both operands in BF16 the
-// call decodes each byte once (conversion kernel) and runs the BF16 CTA-pair tensor-core kernel further down.
+// Three kernels behind one entry point, chosen by the sizes and by what fits in the caller's workspace:
+//   narrow   up to 64 activation rows: bound by reading the weight bytes once
+//   weights  weights decoded into tensor memory by the tensor-core kernel; the activations come expanded to BF16 from the
+//            workspace, or, with no room there, as bytes that are decoded in the kernel too
+//   pair     both operands expanded to BF16 in the workspace (large products)
 //
 // Every HiF8 value has at most 4 significant bits and an exponent in [-22, 15], so it is exact in BF16 and every
 // product of two of them is exact in the FP32 accumulator of the tensor core.
 //
-// A pair of CTAs (cluster of two, cta_group::2) computes one 256 x 256 tile of C: each CTA stages and decodes its
-// own 128 rows of A and 128 columns of W, the even CTA issues the MMAs for both.  Warp roles per CTA:
-//   warps 0-3  epilogue: TMEM -> registers -> descale -> BF16 / FP32 -> global
-//   warp  4    TMA producer: HiF8 byte tiles (A: 128 x 64, W: 128 x 64 or 64 x 128) into a 4-stage staging ring
-//   warp  5    MMA issuer: one elected thread of the even CTA issues tcgen05.mma (256 x 256 x 16 over the pair,
-//              BF16 x BF16 -> FP32 in the TMEM of both CTAs)
-//   warps 6-21 decode: staging bytes -> BF16; W goes into the canonical 128-byte-swizzled shared-memory operand layout,
-//              A ([M,K] form) goes straight into tensor memory (tcgen05.st, one thread per row), from where the MMA
-//              reads it as its A operand: the decoded A tile costs neither a shared-memory store nor an operand read
 // The operand layout follows the shared-memory matrix descriptor of tcgen05: K-major operands are rows of 64 BF16
 // (128 bytes), eight rows form a 1024-byte swizzle atom, 16-byte chunk j of row r is stored at chunk j ^ (r % 8).
-// W given as [K, N] is decoded in place as an MN-major operand (atoms of 8 k-rows x 64 n), so no transpose is needed.
+// MN-major operands have atoms of 8 k-rows x 64 columns.
 //
 // Every wait on an mbarrier is bounded; a wait that runs out records a status word, makes all roles leave their
 // loops, lets outstanding TMA copies land, frees TMEM and returns.
@@ -43,55 +35,20 @@ extern std::atomic<uint64_t> g_launches;
 namespace {
 
 constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int kStages8 = 4;    // staging ring of HiF8 byte tiles
-constexpr int kStagesBf = 4;   // ring of decoded BF16 operand tiles
-constexpr int kMaxStagesBf = 8;
 constexpr int kEpiWarps = 4, kDecodeWarps = 16;
 // The decode warps work in groups, group g on the k-blocks kb = g (mod kDecodeGroups): several k-blocks are in the
 // decode stage at once, which covers the latency of each one's lookups, proxy fence and barrier hand-over.  Group g
 // owns byte stage g and operand stage g, so every barrier is waited on by one party in program order (a waiter is never
 // more than one phase ahead of the barrier, which a parity wait could not tell apart).
 constexpr int kDecodeGroups = 4, kGroupWarps = kDecodeWarps / kDecodeGroups, kGroupThreads = kGroupWarps * 32;
-static_assert(kStages8 == kDecodeGroups && kStagesBf == kDecodeGroups, "group g owns byte stage g and operand stage g");
-// With A decoded into tensor memory the shared memory freed by the A operand tiles can hold either a deeper byte ring
-// (8 stages, table with 128-byte rows) or the 64 KiB table whose addresses cost one instruction (4 stages).  Measured at
-// 8192 x 28672 x 8192: 4.84 ms against 4.71 ms -- the TMA latency is already covered by four stages, so the wide table is
-// the default.
-#ifndef HIF8_FUSED_BYTE_STAGES
-#define HIF8_FUSED_BYTE_STAGES 4
-#endif
-#ifndef HIF8_FUSED_WIDE_LUT
-#define HIF8_FUSED_WIDE_LUT 1
-#endif
-constexpr int kStages8Deep = HIF8_FUSED_BYTE_STAGES, kMaxStages8 = 8;  // (barrier slots for up to eight byte stages)
-static_assert(kStages8Deep <= kMaxStages8 && kStages8 <= kMaxStages8, "barrier slots");
-constexpr bool kWideLut = HIF8_FUSED_WIDE_LUT != 0;
-static_assert(kStages8Deep % kDecodeGroups == 0, "a byte stage is always read by the same group");
-static_assert(!kWideLut || kStages8Deep == 4, "the 64 KiB table leaves room for four byte stages only");
 constexpr int kThreads = (kEpiWarps + 2 + kDecodeWarps) * 32;  // 704
 constexpr int kTmaWarp = 4, kMmaWarp = 5, kFirstDecodeWarp = 6;
-// per CTA of a pair: 128 rows of A and 128 of the 256 columns of W
-constexpr uint32_t kA8Bytes = BM * BK, kB8Bytes = (BN / 2) * BK;            // 8 KiB + 8 KiB
-constexpr uint32_t kABfBytes = BM * BK * 2, kBBfBytes = (BN / 2) * BK * 2;  // 16 KiB + 16 KiB
-// tensor memory of the fused kernel: columns 0-255 the 128 x 256 FP32 accumulator, then one A operand stage (128 rows x
-// 64 BF16 = 32 columns) per operand stage; allocations are powers of two
-constexpr uint32_t kTmemColsAcc = 256, kTmemAStageCols = BK / 2, kTmemCols = 512;
-static_assert(kTmemColsAcc + kMaxStagesBf * kTmemAStageCols <= kTmemCols, "A operand stages must fit beside the accumulator");
+constexpr uint32_t kABfBytes = BM * BK * 2, kBBfBytes = (BN / 2) * BK * 2;  // BF16 tiles of one CTA of a pair: 16 KiB + 16 KiB
+// tensor memory beside the accumulator: decoded operand stages
+constexpr uint32_t kTmemColsAcc = 256, kTmemCols = 512;
+constexpr uint32_t kSlotBytes = 16384, kLutBytesWide = 65536, kLutBytesNarrow = 256 * 32 * 4;  // decode tables with rows of 256 and 128 bytes
+constexpr uint32_t kSmemBytesMax = 227 * 1024;  // the whole opt-in maximum; kernels that take it check that their layout fits
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
-
-struct SmemLayout {
-    static constexpr uint32_t bf = 0;                                                  // 1024-byte aligned atoms
-    static constexpr uint32_t u8 = bf + kStagesBf * (kABfBytes + kBBfBytes);           // 96 KiB
-    static constexpr uint32_t lut = u8 + kStages8 * (kA8Bytes + kB8Bytes);             // + 64 KiB
-    static constexpr uint32_t bars = lut + 256 * 32 * 4;                                // lane-replicated table, 32 KiB
-    static constexpr uint32_t n_bars = 2 * kMaxStages8 + 2 * kMaxStagesBf + 1;
-    static constexpr uint32_t tmem_slot = bars + n_bars * 8;
-    static constexpr uint32_t abort_flag = tmem_slot + 4;
-    static constexpr uint32_t total = abort_flag + 4;
-};
-constexpr uint32_t kSmemBytes = SmemLayout::total + 1024;  // slack for manual 1024-byte alignment
-constexpr uint32_t kBarsBytes = 320;                       // barriers, tensor-memory slot, abort flag
-static_assert(SmemLayout::n_bars * 8 + 8 <= kBarsBytes, "barrier block");
 
 // ---------------------------------------------------------------------------------------------------------
 // PTX wrappers
@@ -531,328 +488,6 @@ __device__ __forceinline__ void apply_channel_scale(const GemmParams& p, int col
     }
 }
 
-// Fused kernel, decode warps: one 128 x 64 tile of HiF8 bytes -> BF16 in the 128-byte-swizzled operand layout, in two
-// steps so that the byte tile can be handed back to the TMA producer as soon as it has been read: first a thread's
-// eight 8-byte chunks into registers, then lookups and swizzled stores.
-constexpr int kChunksPerThread = (BM * BK / 8) / kGroupThreads;  // 8
-// K-major source tile [128 rows][64 k]: chunk j (8 codes) of row r -> atom r/8, row r%8, chunk j ^ (r%8).
-// MN-major source tile [64 k][128 mn]: chunk (k, mn/8) -> atom (mn/64) * 8 + k/8, row k%8, chunk (mn/8)%8 ^ (k%8).
-template <bool MN_MAJOR>
-__device__ __forceinline__ void load_tile_chunks(uint32_t src8, int dt, uint2 (&v)[kChunksPerThread])
-{
-#pragma unroll
-    for (int it = 0; it < kChunksPerThread; it++) {
-        const int q = it * kGroupThreads + dt;
-        v[it] = MN_MAJOR ? lds_v2(src8 + (q >> 4) * BM + (q & 15) * 8) : lds_v2(src8 + (q >> 3) * BK + (q & 7) * 8);
-    }
-}
-template <bool MN_MAJOR, int ROW_SHIFT = 7>
-__device__ __forceinline__ void decode_tile_chunks(const uint2 (&v)[kChunksPerThread], uint32_t dst, int dt, uint32_t lut)
-{
-#pragma unroll
-    for (int it = 0; it < kChunksPerThread; it++) {
-        const int q = it * kGroupThreads + dt;
-        if (MN_MAJOR) {
-            const int k = q >> 4, jn = q & 15, atom = (jn >> 3) * 8 + (k >> 3);
-            sts_v4(dst + atom * 1024 + (k & 7) * 128 + (((jn & 7) ^ (k & 7)) << 4), decode8<ROW_SHIFT>(v[it], lut));
-        } else {
-            const int r = q >> 3, j = q & 7;
-            sts_v4(dst + (r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4), decode8<ROW_SHIFT>(v[it], lut));
-        }
-    }
-}
-
-// Shared memory of the fused kernel.
-// A given as [K,M] (decoded into shared memory): the fixed layout of SmemLayout.
-// A given as [M,K] (decoded into tensor memory): no A operand tiles, and the lookup table has rows of 256 bytes and starts on
-// a 64 KiB boundary of the shared window (see decode8).  Everything else is dealt out in 16 KiB slots around the table: as
-// many as fit in front of it, the rest behind it.  Slots 0-3: W operand stages, slots 4-7: byte stages (A 8 KiB + W 8 KiB).
-constexpr uint32_t kSlotBytes = 16384, kLutBytesWide = 65536, kLutBytesNarrow = 256 * 32 * 4, kFusedSlots = kStagesBf + kStages8Deep;
-static_assert(kBBfBytes == kSlotBytes && kA8Bytes + kB8Bytes == kSlotBytes, "one stage per slot");
-constexpr uint32_t kSmemBytesWide = 227 * 1024;  // the whole opt-in maximum; the kernel checks that its plan fits
-
-// FIXED: the layout of SmemLayout (A operand tiles in shared memory).
-template <bool FIXED>
-struct FusedSmem {
-    uint32_t base, lut, bars, behind;  // shared-window addresses; base is 1024-byte aligned
-    int n_front;                       // slots in front of the table
-    uint32_t end;                      // first byte behind everything
-
-    __device__ explicit FusedSmem(uint32_t raw)
-    {
-        base = (raw + 1023u) & ~1023u;
-        if (FIXED) {
-            lut = base + SmemLayout::lut; bars = base + SmemLayout::bars; behind = 0; n_front = 0; end = base + SmemLayout::total;
-        } else if (!kWideLut) {
-            // table with rows of 128 bytes: no alignment to honour, everything in a row: slots, table, barriers
-            n_front = (int)kFusedSlots; behind = 0;
-            lut = base + kFusedSlots * kSlotBytes; bars = lut + kLutBytesNarrow; end = bars + kBarsBytes;
-        } else {
-            lut = (base + kLutBytesWide - 1) & ~(kLutBytesWide - 1);
-            const uint32_t front = lut - base;
-            n_front = (int)min(front / kSlotBytes, kFusedSlots);
-            behind = lut + kLutBytesWide;
-            const uint32_t after_slots = behind + (kFusedSlots - n_front) * kSlotBytes;
-            // barriers, tensor-memory slot and abort flag (256 bytes): in the gap in front of the table if there is one
-            bars = (front - n_front * kSlotBytes >= kBarsBytes) ? base + n_front * kSlotBytes : after_slots;
-            end = bars >= after_slots ? bars + kBarsBytes : after_slots;
-        }
-    }
-    __device__ uint32_t slot(int i) const { return i < n_front ? base + (uint32_t)i * kSlotBytes : behind + (uint32_t)(i - n_front) * kSlotBytes; }
-    __device__ uint32_t a_bf(int s) const { return base + SmemLayout::bf + s * (kABfBytes + kBBfBytes); }                       // FIXED only
-    __device__ uint32_t w_bf(int s) const { return FIXED ? a_bf(s) + kABfBytes : slot(s); }
-    __device__ uint32_t a_u8(int s) const { return FIXED ? base + SmemLayout::u8 + s * (kA8Bytes + kB8Bytes) : slot(kStagesBf + s); }
-    // staging box j (16 KiB) of the result tile: the operand stages, idle once the accumulator is complete
-    __device__ uint32_t box(int j) const { return FIXED ? base + SmemLayout::bf + (uint32_t)j * kSlotBytes : slot(j); }
-    __device__ uint32_t w_u8(int s) const { return a_u8(s) + kA8Bytes; }
-    __device__ uint32_t tmem_slot() const { return bars + SmemLayout::n_bars * 8; }
-    __device__ uint32_t abort_flag() const { return tmem_slot() + 4; }
-};
-
-// A_IS_KM = false: A given as [M,K] bytes, decoded into tensor memory.  true: A given as [K,M] bytes, decoded into shared
-// memory (MN-major operand).
-template <bool A_IS_KM, bool W_IS_NK>
-__global__ void __launch_bounds__(kThreads, 1)
-hif8_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
-                 const __grid_constant__ CUtensorMap map_c, const GemmParams p)
-{
-    extern __shared__ unsigned char smem_raw[];
-    constexpr int kLutShift = (A_IS_KM || !kWideLut) ? 7 : 8;
-    constexpr int kS8 = A_IS_KM ? kStages8 : kStages8Deep;  // depth of the byte ring
-    constexpr int kSB = kStagesBf;  // operand stages: one per decode group
-    const FusedSmem<A_IS_KM> plan(smem_u32(smem_raw));
-    const uint32_t base = plan.base;
-    unsigned char* sm = smem_raw - smem_u32(smem_raw);  // generic pointer of shared-window address 0
-    {
-        uint32_t dyn_bytes;
-        asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
-        if (plan.end > smem_u32(smem_raw) + dyn_bytes) {  // the plan does not fit (the same answer in every thread of the pair)
-            if (threadIdx.x == 0) atomicCAS(p.status, 0, 7);
-            return;
-        }
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank();  // 0: leader of the pair (issues the MMAs), 1: peer
-    const bool leader = rank == 0;
-
-    const uint32_t bars = plan.bars;
-    auto bar_u8_full = [&](int s) { return bars + 8u * s; };                                   // per CTA
-    auto bar_u8_empty = [&](int s) { return bars + 8u * (kMaxStages8 + s); };                     // per CTA
-    auto bar_bf_full = [&](int s) { return bars + 8u * (2 * kMaxStages8 + s); };                  // leader: both CTAs' decode warps
-    auto bar_bf_empty = [&](int s) { return bars + 8u * (2 * kMaxStages8 + kMaxStagesBf + s); };  // per CTA, leader's commits
-    const uint32_t bar_acc_full = bars + 8u * (2 * kMaxStages8 + 2 * kMaxStagesBf);                  // per CTA, leader's commit
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + plan.abort_flag());
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + plan.tmem_slot());
-    uint32_t* lut_all = reinterpret_cast<uint32_t*>(sm + plan.lut);
-    const uint32_t lut = plan.lut + 4u * lane;  // this lane's column of the table
-
-    // 256 x 256 tile of this pair (groups of 8 tile-rows share their W tiles in L2); this CTA: 128 rows, 128 columns of W
-    int tile_m, tile_n;
-    tile_coords((int)(blockIdx.x >> 1), (p.M + 2 * BM - 1) / (2 * BM), p.tiles_n, tile_m, tile_n);
-    const int m0 = tile_m * 2 * BM + (int)rank * BM, n0 = tile_n * BN, nh = n0 + (int)rank * (BN / 2);
-    const int num_kb = (p.K + BK - 1) / BK;
-
-    // ---- set-up
-    fill_decode_table<(1 << (kLutShift - 2))>(lut_all, warp, lane, kThreads / 32);  // rows of 1 << kLutShift bytes
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kS8; s++) { mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps); }
-        for (int s = 0; s < kSB; s++) { mbar_init(bar_bf_full(s), 2 * kGroupWarps); mbar_init(bar_bf_empty(s), 1); }  // full: both CTAs' decode group
-        mbar_init(bar_acc_full, 1);
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == kMmaWarp) {  // this warp owns the TMEM allocation (both CTAs of the pair take part)
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(plan.tmem_slot()), "r"(kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync_all();  // barriers of both CTAs exist before anyone signals across
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-
-    if (warp == kTmaWarp) {
-        // ------------------------------------------------------------------ TMA producer (each CTA feeds itself)
-        if (lane == 0) {
-            int issued = 0;
-            for (int kb = 0; kb < num_kb; kb++) {
-                const int s = kb % kS8, round = kb / kS8;
-                if (round > 0 && !mbar_wait(bar_u8_empty(s), (round - 1) & 1, abort_flag, p.status, 1)) break;
-                if (*abort_flag) break;
-                const uint32_t dst_a = plan.a_u8(s), dst_b = plan.w_u8(s);
-                mbar_arrive_expect_tx(bar_u8_full(s), kA8Bytes + kB8Bytes);
-                if (A_IS_KM) tma_load_2d(dst_a, &map_a, m0, kb * BK, bar_u8_full(s));
-                else tma_load_2d(dst_a, &map_a, kb * BK, m0, bar_u8_full(s));
-                if (W_IS_NK) tma_load_2d(dst_b, &map_w, kb * BK, nh, bar_u8_full(s));
-                else tma_load_2d(dst_b, &map_w, nh, kb * BK, bar_u8_full(s));
-                issued = kb + 1;
-            }
-            if (*abort_flag) {
-                // let the copies already issued land before this CTA's shared memory goes away
-                for (int kb = max(0, issued - kS8); kb < issued; kb++) {
-                    const int s = kb % kS8;
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(bar_u8_full(s), (kb / kS8) & 1) && global_ns() - t0 < kWaitLimitNs) {}
-                }
-            }
-        }
-    } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (lane == 0 && leader) {
-            // instruction descriptor: FP32 accumulator, BF16 A and B, A K-major, B K- or MN-major, N = 256, M = 256 (pair)
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_IS_KM ? 1u : 0u) << 15) | ((W_IS_NK ? 0u : 1u) << 16) |
-                                   ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
-            // An MMA is accepted only when the tensor pipe has room, so whatever this thread does between two of them leaves
-            // the pipe idle: the barrier of the next k-block is probed, and its addresses are formed, between the third and
-            // the fourth MMA of the current one (while the third runs), not after the commit.
-            bool ok = mbar_wait(bar_bf_full(0), 0, abort_flag, p.status, 2);
-            uint32_t a_addr = plan.a_bf(0), b_addr = plan.w_bf(0), a_tmem = tmem_base + kTmemColsAcc;
-            for (int kb = 0; kb < num_kb && ok; kb++) {
-                const int s = kb % kSB;
-                tc_fence_after();
-                bool next_ready = true;
-                uint32_t a_next = 0, b_next = 0, t_next = 0;
-#pragma unroll
-                for (int kk = 0; kk < BK / 16; kk++) {
-                    if (kk == BK / 16 - 1 && kb + 1 < num_kb) {
-                        const int sn = (kb + 1) % kSB;
-                        next_ready = mbar_try_wait(bar_bf_full(sn), (uint32_t)(((kb + 1) / kSB) & 1));
-                        a_next = plan.a_bf(sn); b_next = plan.w_bf(sn);
-                        t_next = tmem_base + kTmemColsAcc + (uint32_t)(sn * kTmemAStageCols);
-                    }
-                    // K-major: 16 k = 32 bytes inside the 128-byte row; MN-major: 16 k = two 1024-byte atoms
-                    const uint64_t db = W_IS_NK ? make_smem_desc(b_addr + kk * 32, 16, 1024)
-                                                : make_smem_desc(b_addr + kk * 2048, 8192, 1024);
-                    if (A_IS_KM) {
-                        tc_mma_bf16_pair(tmem_base, make_smem_desc(a_addr + kk * 2048, 8192, 1024), db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-                    } else {
-                        // A from tensor memory: stage s, 16 k = 8 columns
-                        tc_mma_bf16_pair_a_tmem(tmem_base, a_tmem + (uint32_t)(kk * 8), db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-                    }
-                }
-                tc_commit_pair(bar_bf_empty(s));  // frees this operand stage in both CTAs once the MMAs have read it
-                if (kb + 1 < num_kb) {
-                    if (!next_ready) ok = mbar_wait(bar_bf_full((kb + 1) % kSB), (uint32_t)(((kb + 1) / kSB) & 1), abort_flag, p.status, 2);
-                    a_addr = a_next; b_addr = b_next; a_tmem = t_next;
-                }
-            }
-            if (ok) tc_commit_pair(bar_acc_full);
-        }
-    } else if (warp >= kFirstDecodeWarp) {
-        // ------------------------------------------------------------------ decode warps
-        const int group = (warp - kFirstDecodeWarp) / kGroupWarps;
-        const int dt = threadIdx.x - (kFirstDecodeWarp + group * kGroupWarps) * 32;  // 0..kGroupThreads-1
-        bool ok = true;
-        for (int kb = group; kb < num_kb && ok; kb += kDecodeGroups) {
-            const int s8 = kb % kS8, r8 = kb / kS8, sb = kb % kSB, rb = kb / kSB;
-            ok = mbar_wait(bar_u8_full(s8), r8 & 1, abort_flag, p.status, 3);
-            if (ok && rb > 0) ok = mbar_wait(bar_bf_empty(sb), (rb - 1) & 1, abort_flag, p.status, 4);
-            if (!ok) break;
-            const uint32_t a8 = plan.a_u8(s8), b8 = plan.w_u8(s8);
-            const uint32_t abf = plan.a_bf(sb), bbf = plan.w_bf(sb);
-            uint2 vw[kChunksPerThread];
-            if (A_IS_KM) {
-                uint2 va[kChunksPerThread];
-                load_tile_chunks<true>(a8, dt, va);
-                load_tile_chunks<!W_IS_NK>(b8, dt, vw);
-                __syncwarp();  // every lane's reads of the byte stage are done: the producer may refill it during the decode
-                if (lane == 0) mbar_arrive(bar_u8_empty(s8));
-                decode_tile_chunks<true, kLutShift>(va, abf, dt, lut);
-            } else {
-                // A [M,K]: this thread owns row (its warp's quarter of the 128 tensor-memory lanes) * 32 + lane.  The byte
-                // tile arrives with the 64-byte TMA swizzle (16-byte chunk j of row r sits at chunk j ^ ((r >> 1) & 3)), so
-                // the lanes of a warp, 64 bytes apart, read their chunk j from different banks.
-                const int quarter = warp & 3, r = quarter * 32 + lane;
-                const uint32_t a_row = a8 + (uint32_t)r * BK, sw = (uint32_t)(r >> 1) & 3u;
-                uint4 va[BK / 16];
-#pragma unroll
-                for (int j = 0; j < BK / 16; j++) va[j] = lds_v4(a_row + (((uint32_t)j ^ sw) << 4));
-                load_tile_chunks<!W_IS_NK>(b8, dt, vw);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_u8_empty(s8));
-                uint32_t o[BK / 2];  // 64 BF16 of this row, two per column
-#pragma unroll
-                for (int j = 0; j < BK / 16; j++) {
-                    const uint4 lo = decode8<kLutShift>(make_uint2(va[j].x, va[j].y), lut), hi = decode8<kLutShift>(make_uint2(va[j].z, va[j].w), lut);
-                    o[8 * j + 0] = lo.x; o[8 * j + 1] = lo.y; o[8 * j + 2] = lo.z; o[8 * j + 3] = lo.w;
-                    o[8 * j + 4] = hi.x; o[8 * j + 5] = hi.y; o[8 * j + 6] = hi.z; o[8 * j + 7] = hi.w;
-                }
-                tmem_st_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemColsAcc + (uint32_t)(sb * kTmemAStageCols), o);
-            }
-            decode_tile_chunks<!W_IS_NK, kLutShift>(vw, bbf, dt, lut);
-            if (!A_IS_KM) tmem_st_wait();  // the row is in tensor memory
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // make the stores visible to the tensor core
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_remote(map_to_cta(bar_bf_full(sb), 0));  // the leader's MMAs read both CTAs' operands
-        }
-    }
-    if (warp != kTmaWarp && warp != kMmaWarp) {
-        // ------------------------------------------------------------------ epilogue (each CTA drains its rows)
-        // Warps 0-3 and, once their k-blocks are done, the sixteen decode warps: a warp reaches the quarter (warp % 4) of
-        // the tensor-memory lanes, so every quarter has five warps, which share its eight 32-column chunks (the drain is
-        // not overlapped with anything: with four warps it took a tenth of the tile's time).
-        const int quarter = warp & 3;
-        const int share = warp < kEpiWarps ? 0 : (warp - quarter) / 4 - (quarter < 2 ? 1 : 0);  // 0..4 within the quarter
-        static_assert(kEpiWarps == 4 && kTmaWarp == 4 && kMmaWarp == 5 && kFirstDecodeWarp == 6 && kDecodeWarps == 16,
-                      "five warps per lane quarter: w, and w + 4k without the two single-thread warps");
-        const bool ok = mbar_wait(bar_acc_full, 0, abort_flag, p.status, 5);
-        if (ok) {
-            tc_fence_after();
-            const int sa = p.d_sa ? *p.d_sa : 0;
-            const int s = p.d_sw_channel ? 0 : -(sa + (p.d_sw ? *p.d_sw : 0));
-            const int s1 = s / 2, s2 = s - s1;  // |s1|, |s2| <= 126: two exact power-of-two factors
-            const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
-            const int row = m0 + quarter * 32 + lane;
-            // (separate loops rather than branches inside one: the register allocation of each stays that of its own path)
-            if (!A_IS_KM && p.c_by_tma) {
-#pragma unroll 1
-                for (int c = share * 32; c < BN; c += 5 * 32) {
-                    uint32_t r[32];
-                    tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + c, r);
-                    tmem_ld_wait();
-                    if (p.d_sw_channel) apply_channel_scale(p, n0 + c, lane, sa, r);
-                    // the operand stages are idle once the accumulator is complete: box c / 64 of the result tile goes there
-                    stage_chunk_bf16(plan.box(c >> 6), quarter * 32 + lane, (c & 63) >> 3, r, f1, f2);
-                }
-            } else {
-#pragma unroll 1
-                for (int c = share * 32; c < BN; c += 5 * 32) {
-                    uint32_t r[32];
-                    tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + c, r);
-                    tmem_ld_wait();
-                    if (p.d_sw_channel) apply_channel_scale(p, n0 + c, lane, sa, r);
-                    store_chunk(p, row, n0 + c, r, f1, f2);
-                }
-            }
-        }
-        if (!A_IS_KM && p.c_by_tma) {
-            // Stores of 16 bytes per lane to 32 different rows made the drain as slow as one L2 transaction per clock allows
-            // (4096 of them per CTA); four tile stores write whole lines instead.  All twenty warps meet (named barrier 1),
-            // then one thread issues the stores and waits until shared memory has been read.
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("bar.sync 1, %0;" ::"n"((kEpiWarps + kDecodeWarps) * 32) : "memory");
-            if (threadIdx.x == 0 && ok && !*abort_flag) {
-#pragma unroll
-                for (int j = 0; j < BN / 64; j++) tma_store_2d(&map_c, plan.box(j), n0 + j * 64, m0);
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            }
-        }
-    }
-
-    // ---- teardown: all waits are bounded, so everybody arrives; nobody leaves while the peer may still read this
-    // CTA's operands or signal its barriers; then the allocating warps free TMEM
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync_all();
-    if (warp == kMmaWarp) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
-    }
-}
-
 // ---------------------------------------------------------------------------------------------------------
 // Narrow products (M <= 64 rows of activations: the decode phase of inference).  The product is bound by reading the
 // weight bytes once, so the roles are swapped: a CTA streams a slab of 128 weight columns as the 128-row MMA operand and
@@ -882,7 +517,6 @@ constexpr int kNwMaxByteStages = 6, kNwMinByteStages = 4;
 // that a group starts its next k-block without waiting for the MMAs of its previous one
 constexpr int kNwTmemStages = 2 * kDecodeGroups;
 constexpr uint32_t kNwBars = 2 * kNwMaxByteStages + 2 * kNwTmemStages + 4;
-constexpr uint32_t kSmemBytesN = 227 * 1024;  // the whole opt-in maximum; the kernel checks that its layout fits
 // Where the narrow kernel keeps what (mp activation rows).  WIDE ([N,K] weights with the activations expanded beforehand):
 // the decode table has rows of 256 bytes and starts on a 64 KiB boundary of the shared window, so that one byte permute makes
 // a lookup's address (see decode8); operand stages and then byte stages as they fit in front of it, the rest behind it.
@@ -1380,10 +1014,12 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// Weights decoded into tensor memory, activations expanded to BF16 beforehand (in the caller's workspace): C^T = W^T A^T.
+// Weights decoded into tensor memory: C^T = W^T A^T.
 // A pair of CTAs computes 256 weight columns x bn activation rows: each CTA decodes 128 weight columns straight into its
-// tensor memory (the 128-row A operand of the MMA; nothing decoded touches shared memory) and brings bn / 2 activation
-// rows by TMA (the B operand).  A k-block here is 128 k.  Warp roles per CTA:
+// tensor memory (the 128-row A operand of the MMA; nothing decoded there touches shared memory) and provides bn / 2 activation
+// rows (the B operand): expanded to BF16 beforehand in the caller's workspace and brought by TMA (a k-block is 128 k then), or,
+// when there is no room for them, as bytes [M,K] or [K,M] that the decode groups decode into shared memory as well (64 k).
+// Warp roles per CTA:
 //   warps 0-3   epilogue: accumulator column = activation row m, lane = weight column n
 //   warp  4     copies of weight bytes, four stages of 16 KiB       warp 22  copies of the activation tiles, four stages
 //   warp  5     MMA issuer (even CTA)                               warps 6-21  four decode groups, group g on it = g (mod 4),
@@ -1400,26 +1036,47 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kWdStages = 4, kWdActWarp = kThreads / 32, kThreadsWd = kThreads + 32;  // 736
 constexpr int kWdMaxSplit = 4;
-constexpr uint32_t kWdActBytes = 2 * (BN / 2) * BK * 2, kWdW8Bytes = BM * 2 * BK;  // 32 KiB, 16 KiB per stage
-struct SmemLayoutWd {
-    static constexpr uint32_t act = 0;
-    static constexpr uint32_t u8 = act + kWdStages * kWdActBytes;
-    static constexpr uint32_t lut = u8 + kWdStages * kWdW8Bytes;
-    static constexpr uint32_t bars = lut + kLutBytesNarrow;
+static_assert(kWdStages == kDecodeGroups, "group g owns stage g, so every barrier is waited on in program order");
+enum Activations { kActExpanded, kActRows, kActColumns };  // BF16 [M,K], bytes [M,K], bytes [K,M]
+
+// Shared memory.  Expanded activations: four operand stages of 32 KiB, four stages of weight bytes of 16 KiB, the 32 KiB table.
+// Activations as bytes: eight slots of 16 KiB (four operand stages; four byte stages, weights then activations) around the 64 KiB
+// table, which starts on a 64 KiB boundary of the shared window (see decode8).  The partial sums that a pair receives in the
+// split form go to `base` and up, over stages and table: nothing there is needed any more.
+template <int ACT>
+struct WdSmem {
+    static constexpr int KB = ACT == kActExpanded ? 2 * BK : BK;  // k per k-block
+    static constexpr uint32_t kActStage = (BN / 2) * KB * 2, kW8 = BM * KB;
     static constexpr uint32_t n_bars = 4 * kWdStages + 2;
-    static constexpr uint32_t tmem_slot = bars + n_bars * 8;
-    static constexpr uint32_t abort_flag = tmem_slot + 4;
-    static constexpr uint32_t total = abort_flag + 4;
+    uint32_t base, lut, bars, end;
+    int front;
+    __device__ explicit WdSmem(uint32_t raw)
+    {
+        base = (raw + 1023u) & ~1023u;
+        if (ACT == kActExpanded) {
+            lut = base + kWdStages * (kActStage + kW8); bars = lut + kLutBytesNarrow; front = 0;
+        } else {
+            lut = (base + kLutBytesWide - 1) & ~(kLutBytesWide - 1);
+            front = min((int)((lut - base) / kSlotBytes), 2 * kWdStages);
+            bars = lut + kLutBytesWide + (uint32_t)(2 * kWdStages - front) * kSlotBytes;
+        }
+        end = bars + n_bars * 8 + 8;
+    }
+    __device__ uint32_t slot(int i) const { return i < front ? base + (uint32_t)i * kSlotBytes : lut + kLutBytesWide + (uint32_t)(i - front) * kSlotBytes; }
+    __device__ uint32_t act(int s) const { return ACT == kActExpanded ? base + (uint32_t)s * kActStage : slot(s); }
+    __device__ uint32_t u8(int s) const { return ACT == kActExpanded ? base + kWdStages * kActStage + (uint32_t)s * kW8 : slot(kWdStages + s); }
+    __device__ uint32_t tmem_slot() const { return bars + n_bars * 8; }
+    __device__ uint32_t abort_flag() const { return tmem_slot() + 4; }
 };
-constexpr uint32_t kSmemBytesWd = SmemLayoutWd::total + 1024;
-static_assert(kSmemBytesWd <= 227 * 1024, "shared memory of one CTA");
-static_assert((kWdMaxSplit - 1) * (BN / kWdMaxSplit) * BM * 4 <= SmemLayoutWd::lut && (2 - 1) * (BN / 2) * BM * 4 <= SmemLayoutWd::lut,
-              "the partial sums received fit in the idle stages");
+static_assert(WdSmem<kActRows>::kActStage == kSlotBytes && 2 * WdSmem<kActRows>::kW8 == kSlotBytes, "one stage per slot");
+static_assert((kWdMaxSplit - 1) * (BN / kWdMaxSplit) * BM * 4 <= 2 * kWdStages * kSlotBytes && (2 - 1) * (BN / 2) * BM * 4 <= 2 * kWdStages * kSlotBytes,
+              "the partial sums received stay below the barriers");
 
 struct TilePlan {
     int first, count;  // tiles [first, first + count) of the product
     int chunks, bn;    // activation rows in `chunks` pieces of bn (a multiple of 32); tile t = weight slab t / chunks, piece t % chunks
     int split;
+    int clear_status;  // nonzero: no launch in front of this one clears the status word
 };
 
 __device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
@@ -1467,30 +1124,39 @@ __device__ __forceinline__ void store_columns(unsigned char* out, uint32_t pitch
     }
 }
 
-template <bool W_IS_NK>
+template <bool W_IS_NK, int ACT>
 __global__ void __launch_bounds__(kThreadsWd, 1)
 hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_act, const GemmParams p, const TilePlan tp)
 {
     extern __shared__ unsigned char smem_raw[];
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    unsigned char* sm = smem_raw + (base - smem_u32(smem_raw));
+    using Smem = WdSmem<ACT>;
+    constexpr int KB = Smem::KB, kLutShift = ACT == kActExpanded ? 7 : 8;
+    const Smem lay(smem_u32(smem_raw));
+    const uint32_t base = lay.base;
+    unsigned char* sm = smem_raw - smem_u32(smem_raw);  // generic pointer of shared-window address 0
+    if (ACT != kActExpanded) {
+        uint32_t dyn_bytes;
+        asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
+        if (lay.end > smem_u32(smem_raw) + dyn_bytes) {  // the layout does not fit (the same answer in every thread of the grid)
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile int*>(p.status) = 7;
+            return;
+        }
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank(), half = rank & 1u, lead = rank & ~1u;  // half 0: leader of its pair (issues the MMAs)
     const bool leader = half == 0;
-    const uint32_t bars = base + SmemLayoutWd::bars;
+    const uint32_t bars = lay.bars;
     auto bar_u8_full = [&](int s) { return bars + 8u * s; };                       // per CTA
     auto bar_u8_empty = [&](int s) { return bars + 8u * (kWdStages + s); };        // per CTA
     auto bar_bf_full = [&](int s) { return bars + 8u * (2 * kWdStages + s); };     // leader: both CTAs' decode warps and activation tiles
     auto bar_bf_empty = [&](int s) { return bars + 8u * (3 * kWdStages + s); };    // per CTA, leader's commits
     const uint32_t bar_acc_full = bars + 8u * (4 * kWdStages);                     // per CTA, leader's commit
     const uint32_t bar_acc_empty = bars + 8u * (4 * kWdStages + 1);                // leader: both CTAs' epilogue warps
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + SmemLayoutWd::abort_flag);
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + SmemLayoutWd::tmem_slot);
-    const uint32_t lut = base + SmemLayoutWd::lut + 4u * lane;
-    auto act_stage = [&](int s) { return base + SmemLayoutWd::act + (uint32_t)s * kWdActBytes; };
-    auto u8_stage = [&](int s) { return base + SmemLayoutWd::u8 + (uint32_t)s * kWdW8Bytes; };
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + lay.abort_flag());
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + lay.tmem_slot());
+    const uint32_t lut = lay.lut + 4u * lane;
 
-    constexpr int KB = 2 * BK;
     const int num_kb = (p.K + KB - 1) / KB, split = tp.split, part = split > 1 ? (int)(rank >> 1) : 0;
     const int kb0 = split > 1 ? num_kb * part / split : 0, kb1 = split > 1 ? num_kb * (part + 1) / split : num_kb;
     const int t0 = tp.first + (int)(split > 1 ? blockIdx.x / (2 * split) : blockIdx.x >> 1);
@@ -1499,28 +1165,34 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     // ---- set-up.  A call of a small product is mostly latency: the first weight copies go out under the table set-up, and only
     // what touches the other CTAs waits for the cluster (its barrier takes 1400 to 1900 cycles from the start of the kernel,
     // in which a first k-block is copied and decoded).
-    auto copy_weights = [&](int it, int n0, int kb) {  // stage it % kWdStages, free
-        const int s = it % kWdStages;
-        mbar_arrive_expect_tx(bar_u8_full(s), kWdW8Bytes);
-        if (W_IS_NK) tma_load_2d(u8_stage(s), &map_w, kb * KB, n0, bar_u8_full(s));
-        else tma_load_2d(u8_stage(s), &map_w, n0, kb * KB, bar_u8_full(s));
+    auto copy_bytes = [&](int it, int t, int kb) {  // tile t's bytes of k-block kb into stage it % kWdStages, which is free
+        const int s = it % kWdStages, slab = t / tp.chunks, n0 = slab * 2 * BM + (int)half * BM;
+        const uint32_t dst = lay.u8(s), bar = bar_u8_full(s);
+        mbar_arrive_expect_tx(bar, Smem::kW8 + (ACT == kActExpanded ? 0u : (uint32_t)(tp.bn / 2) * KB));
+        if (W_IS_NK) tma_load_2d(dst, &map_w, kb * KB, n0, bar);
+        else tma_load_2d(dst, &map_w, n0, kb * KB, bar);
+        if (ACT != kActExpanded) {
+            const int m0 = (t - slab * tp.chunks) * tp.bn + (int)half * (tp.bn / 2);
+            if (ACT == kActRows) tma_load_2d(dst + Smem::kW8, &map_act, kb * KB, m0, bar);
+            else tma_load_2d(dst + Smem::kW8, &map_act, m0, kb * KB, bar);
+        }
     };
-    const int n_first = t0 / tp.chunks * 2 * BM + (int)half * BM;  // weight columns of the first tile
     if (threadIdx.x == kTmaWarp * 32) {
         for (int s = 0; s < kWdStages; s++) {
             mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps);
-            mbar_init(bar_bf_full(s), 2 * kGroupWarps + 1); mbar_init(bar_bf_empty(s), 1);  // (+ 1: the leader's announcement of the tile bytes)
+            // operands ready: both CTAs' groups, plus (expanded activations) the leader's announcement of the tile bytes
+            mbar_init(bar_bf_full(s), 2 * kGroupWarps + (ACT == kActExpanded ? 1 : 0)); mbar_init(bar_bf_empty(s), 1);
         }
         mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps));
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        copy_weights(0, n_first, kb0);
+        if (ACT == kActExpanded) copy_bytes(0, t0, kb0);
     }
-    fill_decode_table<32>(reinterpret_cast<uint32_t*>(sm + SmemLayoutWd::lut), warp, lane, kThreadsWd / 32);
+    fill_decode_table<(1 << (kLutShift - 2))>(reinterpret_cast<uint32_t*>(sm + lay.lut), warp, lane, kThreadsWd / 32);
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(base + SmemLayoutWd::tmem_slot), "r"(kTmemCols) : "memory");
+                     ::"r"(lay.tmem_slot()), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -1528,25 +1200,29 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     cluster_arrive();  // barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    if (ACT != kActExpanded) {
+        // Nothing was launched in front of this kernel to order it behind what produces its operands.
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (tp.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile int*>(p.status) = 0;  // (a wait gives up seconds later)
+    }
 
     if (warp == kTmaWarp) {
-        // ------------------------------------------------------------------ weight bytes (each CTA feeds itself).  Nothing the
-        // launch in front of this one writes is read here, and what came before that is complete.
+        // ------------------------------------------------------------------ bytes (each CTA feeds itself).  Beside expanded
+        // activations nothing is read here that the launch in front of this one writes, and what came before that is complete.
         const int n_early = min(kWdStages, kb1 - kb0);  // of the first tile, without waiting for anybody
         if (lane == 0)
-            for (int i = 1; i < n_early; i++) copy_weights(i, n_first, kb0 + i);
+            for (int i = ACT == kActExpanded ? 1 : 0; i < n_early; i++) copy_bytes(i, t0, kb0 + i);
         __syncwarp();
         cluster_wait();
         if (lane == 0) {
             int it = 0;
             bool ok = true;
             for (int t = t0; t < t_end && ok; t += t_step) {
-                const int n0 = t / tp.chunks * 2 * BM + (int)half * BM;
                 for (int kb = kb0; kb < kb1; kb++, it++) {
                     if (it < n_early) continue;
                     if (it >= kWdStages) ok = mbar_wait(bar_u8_empty(it % kWdStages), (it / kWdStages - 1) & 1, abort_flag, p.status, 41);
                     if (!ok || *abort_flag) { ok = false; break; }
-                    copy_weights(it, n0, kb);
+                    copy_bytes(it, t, kb);
                 }
             }
             if (*abort_flag) {
@@ -1557,14 +1233,14 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             }
         }
     } else if (warp == kWdActWarp) {
-        // ------------------------------------------------------------------ activation tiles: this CTA's bn / 2 rows, two boxes of
+        // ------------------------------------------------------------------ expanded activations: this CTA's bn / 2 rows, two boxes of
         // 64 k (the swizzle span); both CTAs' copies complete on the leader's "operands ready" barrier
         cluster_wait();
         if (lane == 0) {
             asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             int it = 0;
-            bool ok = true;
+            bool ok = ACT == kActExpanded;
             for (int t = t0; t < t_end && ok; t += t_step) {
                 const int m0 = t % tp.chunks * tp.bn + (int)half * (tp.bn / 2);
                 for (int kb = kb0; kb < kb1; kb++, it++) {
@@ -1573,11 +1249,11 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                     if (!ok || *abort_flag) { ok = false; break; }
                     if (leader) mbar_arrive_expect_tx(bar_bf_full(s), (uint32_t)tp.bn * KB * 2u);
                     const uint32_t full = map_to_cta(bar_bf_full(s), lead);
-                    tma_load_3d_pair(act_stage(s), &map_act, kb * KB, m0, 0, full);
-                    tma_load_3d_pair(act_stage(s) + kWdActBytes / 2, &map_act, kb * KB + BK, m0, 0, full);
+                    tma_load_3d_pair(lay.act(s), &map_act, kb * KB, m0, 0, full);
+                    tma_load_3d_pair(lay.act(s) + Smem::kActStage / 2, &map_act, kb * KB + BK, m0, 0, full);
                 }
             }
-            if (*abort_flag) {  // (their barrier also counts the decode groups, which have given up: a fixed 50 us instead)
+            if (ACT == kActExpanded && *abort_flag) {  // (their barrier also counts the decode groups, which have given up: a fixed 50 us instead)
                 const unsigned long long c0 = global_ns();
                 while (global_ns() - c0 < 50000ull) {}
             }
@@ -1586,8 +1262,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
         cluster_wait();
         if (lane == 0 && leader) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(tp.bn >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
-            const uint64_t db0 = make_smem_desc(act_stage(0), 16, 1024);
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((ACT == kActColumns ? 1u : 0u) << 16) | ((uint32_t)(tp.bn >> 3) << 17) |
+                                   ((uint32_t)((2 * BM) >> 4) << 24);
             int it = 0, local = 0;
             bool ok = true;
             for (int t = t0; t < t_end && ok; t += t_step, local++) {
@@ -1597,10 +1273,13 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                     ok = mbar_wait(bar_bf_full(s), (it / kWdStages) & 1, abort_flag, p.status, 42);
                     if (!ok) break;
                     tc_fence_after();
+                    // [M,K]: 16 k = 32 bytes inside the 128-byte rows (the second 64 k of an expanded block are the stage's second
+                    // half); [K,M]: 16 k = two 1024-byte atoms
+                    const uint64_t db = ACT == kActColumns ? make_smem_desc(lay.act(s), 8192, 1024) : make_smem_desc(lay.act(s), 16, 1024);
 #pragma unroll
                     for (int kk = 0; kk < KB / 16; kk++) {
-                        const uint32_t off = (uint32_t)s * kWdActBytes + (kk >> 2) * (kWdActBytes / 2) + (kk & 3) * 32;
-                        tc_mma_bf16_pair_a_tmem(tmem_base, tmem_base + kTmemColsAcc + (uint32_t)(s * (KB / 2) + kk * 8), db0 + (uint64_t)(off >> 4), idesc,
+                        const uint32_t off = ACT == kActColumns ? kk * 2048 : (kk >> 2) * (Smem::kActStage / 2) + (kk & 3) * 32;
+                        tc_mma_bf16_pair_a_tmem(tmem_base, tmem_base + kTmemColsAcc + (uint32_t)(s * (KB / 2) + kk * 8), db + (uint64_t)(off >> 4), idesc,
                                                 (kb > kb0 || kk > 0) ? 1u : 0u);
                     }
                     tc_commit_pair(bar_bf_empty(s), lead);
@@ -1636,39 +1315,70 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                 bool ok = mbar_wait(bar_u8_full(s), r & 1, abort_flag, p.status, 43);
                 if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 44);
                 if (!ok) { it = 0x7FFFFFFF; continue; }  // (gives up at the next wait)
-                const uint32_t w8 = u8_stage(s), dst = tlane + (uint32_t)(s * (KB / 2));
-                // in two halves, one piece of code for both (unrolled, the first pass over it cost every group a thousand cycles of
-                // instruction fetches): [N,K] 64 k of the thread's column, [K,N] all 128 k of sixteen of the quarter's columns
+                const uint32_t w8 = lay.u8(s), dst = tlane + (uint32_t)(s * (KB / 2));
+                // activations as bytes: eight 8-byte chunks of the tile per thread at most (it lies in a row, [M,K] or [K,M])
+                const int dt = threadIdx.x - (kFirstDecodeWarp + group * kGroupWarps) * 32, n_chunks = tp.bn / 2 * (BK / 8);
+                uint2 va[ACT == kActExpanded ? 1 : (BN / 2) * (BK / 8) / kGroupThreads];
+                if (ACT != kActExpanded) {
+#pragma unroll
+                    for (int i = 0; i < (int)(sizeof(va) / sizeof(va[0])); i++)
+                        if (i * kGroupThreads + dt < n_chunks) va[i] = lds_v2(w8 + Smem::kW8 + (uint32_t)(i * kGroupThreads + dt) * 8u);
+                }
+                // 64 bytes of weights per thread and pass, one piece of code for both passes of an expanded block (unrolled, the first
+                // time through cost every group a thousand cycles of instruction fetches)
 #pragma unroll 1
-                for (int h = 0; h < 2; h++) {
+                for (int h = 0; h < KB / BK; h++) {
                     uint4 v[4];
                     if (W_IS_NK) {
-                        // rows of 128 k with the 128-byte swizzle (chunk j of row r at chunk j ^ (r & 7))
-                        const uint32_t row = (uint32_t)(quarter * 32 + lane), w_row = w8 + row * KB, sw = row & 7u;
+                        // a thread per weight column; rows of KB k with the swizzle of that span: chunk j of row r at j ^ (r & 7), or
+                        // with 64 bytes at j ^ ((r >> 1) & 3)
+                        const uint32_t w_row = w8 + (uint32_t)row * KB, sw = KB == 2 * BK ? (uint32_t)row & 7u : (uint32_t)(row >> 1) & 3u;
 #pragma unroll
                         for (int j = 0; j < 4; j++) v[j] = lds_v4(w_row + (((uint32_t)(4 * h + j) ^ sw) << 4));
                     } else {
-                        // rows of 128 columns, one per k, read transposed (see the narrow kernel)
+                        // rows of 128 columns, one per k, read transposed (see the narrow kernel): 128 k of sixteen columns a pass, or
+                        // 64 k of sixteen columns in v[0], v[1] and of the next sixteen in v[2], v[3]
 #pragma unroll
-                        for (int j = 0; j < 4; j++)
-                            v[j] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(32 * j + lane) * BM + ((uint32_t)((2 * quarter + h) ^ (lane & 7)) << 4));
+                        for (int j = 0; j < 4; j++) {
+                            const int i = KB == 2 * BK ? j : j & 1, c = KB == 2 * BK ? h : j >> 1;
+                            v[j] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(32 * i + lane) * BM + ((uint32_t)((2 * quarter + c) ^ (lane & 7)) << 4));
+                        }
                     }
-                    if (h == 1) {
+                    if (h == KB / BK - 1) {
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar_u8_empty(s));
                     }
                     uint32_t o[32];
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
-                        const uint4 lo = decode8<7>(make_uint2(v[j].x, v[j].y), lut), hi = decode8<7>(make_uint2(v[j].z, v[j].w), lut);
+                        const uint4 lo = decode8<kLutShift>(make_uint2(v[j].x, v[j].y), lut), hi = decode8<kLutShift>(make_uint2(v[j].z, v[j].w), lut);
                         o[8 * j + 0] = lo.x; o[8 * j + 1] = lo.y; o[8 * j + 2] = lo.z; o[8 * j + 3] = lo.w;
                         o[8 * j + 4] = hi.x; o[8 * j + 5] = hi.y; o[8 * j + 6] = hi.z; o[8 * j + 7] = hi.w;
                     }
                     if (W_IS_NK) tmem_st_32x32b_x32(dst + (uint32_t)(h * (BK / 2)), o);
-                    else {
+                    else if (KB == 2 * BK) {
                         tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16), o);
                         tmem_st_16x256b_x4(dst + ((uint32_t)(16 * h) << 16) + BK / 2, o + 16);
+                    } else {
+                        tmem_st_16x256b_x4(dst, o);
+                        tmem_st_16x256b_x4(dst + (16u << 16), o + 16);
                     }
+                }
+                if (ACT != kActExpanded) {
+                    const uint32_t abf = lay.act(s);
+                    const int per_row = tp.bn >> 4;  // [K,M]: 8-byte chunks per k (8 or 16)
+#pragma unroll
+                    for (int i = 0; i < (int)(sizeof(va) / sizeof(va[0])); i++) {
+                        const int q = i * kGroupThreads + dt;
+                        uint32_t at;
+                        if (ACT == kActRows) at = abf + (q >> 6) * 1024 + ((q >> 3) & 7) * 128 + (((q ^ (q >> 3)) & 7) << 4);
+                        else {
+                            const int kr = per_row == 16 ? q >> 4 : q >> 3, jn = q & (per_row - 1);
+                            at = abf + ((jn >> 3) * 8 + (kr >> 3)) * 1024 + (kr & 7) * 128 + (((jn ^ kr) & 7) << 4);
+                        }
+                        if (q < n_chunks) sts_v4(at, decode8<kLutShift>(va[i], lut));
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core
                 }
                 tmem_st_wait();
                 tc_fence_before();
@@ -2199,30 +1909,27 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
         out->rc = cudaSuccess;
         out->sm_count = 0;
         std::memset(out->wd_clusters, 0, sizeof out->wd_clusters);
-        // [M,K] activations (the first two): the wide-table plan
-        const void* fused[4] = {(const void*)hif8_gemm_kernel<false, false>, (const void*)hif8_gemm_kernel<false, true>,
-                                (const void*)hif8_gemm_kernel<true, false>, (const void*)hif8_gemm_kernel<true, true>};
         const void* pair[2] = {(const void*)bf16_gemm_pair_kernel<false>, (const void*)bf16_gemm_pair_kernel<true>};
-        const void* wd[2] = {(const void*)hif8_gemm_weights_kernel<false>, (const void*)hif8_gemm_weights_kernel<true>};
-        for (int i = 0; i < 4 && out->rc == cudaSuccess; i++)
-            out->rc = cudaFuncSetAttribute(fused[i], cudaFuncAttributeMaxDynamicSharedMemorySize, i < 2 ? kSmemBytesWide : kSmemBytes);
+        const void* wd[6] = {(const void*)hif8_gemm_weights_kernel<false, kActExpanded>, (const void*)hif8_gemm_weights_kernel<true, kActExpanded>,
+                             (const void*)hif8_gemm_weights_kernel<false, kActRows>, (const void*)hif8_gemm_weights_kernel<true, kActRows>,
+                             (const void*)hif8_gemm_weights_kernel<false, kActColumns>, (const void*)hif8_gemm_weights_kernel<true, kActColumns>};
         for (int i = 0; i < 2 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(pair[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2);
-        for (int i = 0; i < 2 && out->rc == cudaSuccess; i++)
-            out->rc = cudaFuncSetAttribute(wd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesWd);
+        for (int i = 0; i < 6 && out->rc == cudaSuccess; i++)
+            out->rc = cudaFuncSetAttribute(wd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
         for (int s = 1; s <= kWdMaxSplit && out->rc == cudaSuccess; s *= 2) {
             cudaLaunchConfig_t cfg{};
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = 2 * s; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-            cfg.gridDim = dim3(2 * s); cfg.blockDim = dim3(kThreadsWd); cfg.dynamicSmemBytes = kSmemBytesWd;
+            cfg.gridDim = dim3(2 * s); cfg.blockDim = dim3(kThreadsWd); cfg.dynamicSmemBytes = kSmemBytesMax;
             cfg.attrs = attr; cfg.numAttrs = 1;
             out->rc = cudaOccupancyMaxActiveClusters(&out->wd_clusters[s], wd[1], &cfg);
         }
         const void* narrow[4] = {(const void*)hif8_gemm_narrow_kernel<false, false>, (const void*)hif8_gemm_narrow_kernel<false, true>,
                                  (const void*)hif8_gemm_narrow_kernel<true, false>, (const void*)hif8_gemm_narrow_kernel<true, true>};
         for (int i = 0; i < 4 && out->rc == cudaSuccess; i++)
-            out->rc = cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesN);
+            out->rc = cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
         if (out->rc == cudaSuccess) out->rc = cudaDeviceGetAttribute(&out->sm_count, cudaDevAttrMultiProcessorCount, d);
     });
     if (!s) return false;
@@ -2304,52 +2011,91 @@ int launch_bf16_pair_gemm(const void* a_bf, const void* w_bf, int w_is_nk, GemmP
 
 using namespace hif8;
 
-// C = A W^T-or-W with the weights decoded inside the kernel and the activations given as BF16 [M,K] by the launch in front
-// of this one.  `clusters[s]`: how many clusters of s pairs the device holds.
-static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, const void* a_bf, const GemmParams& p, const int* clusters, cudaStream_t st)
-{
-    const int M = p.M, N = p.N, K = p.K, chunks = (M + BN - 1) / BN, bn = ((M + chunks - 1) / chunks + 31) & ~31;
-    const long long slabs = (N + 2 * BM - 1) / (2 * BM), tiles_ll = slabs * chunks;
-    if (tiles_ll > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
-    const int tiles = (int)tiles_ll, num_kb = (K + 2 * BK - 1) / (2 * BK);
-    CUtensorMap map_w, map_act;
-    const bool okw = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, 2 * BK, BM, false, 128)
-                             : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, 2 * BK, false, 128);
-    if (!okw || !make_map3(&map_act, a_bf, (uint64_t)K, (uint64_t)M, 1, 0, BK, (uint32_t)bn / 2)) return HIF8_ERR_CUDA;
-    // Time in k-blocks (of 128 k, about 1050 cycles): a round of tiles takes num_kb / split of them.  The exchange of a split one
-    // (two cluster barriers, the sums at 20 bytes a cycle, less what the shared epilogue saves) measured 3.1 for two pairs and
-    // 7 for four at bn = 256, about half of that at 128.  A launch of its own for the last round costs about four (set-up,
-    // first copies).
-    const double f = bn / 256.0;
-    auto cost = [&](int n, int s) {
-        if (s > num_kb || clusters[s] <= 0) return 1e30;
-        const double exchange = s == 1 ? 0.0 : (s == 2 ? 1.2 + 1.9 * f : 2.0 + 5.0 * f);
-        return (n + clusters[s] - 1) / clusters[s] * ((num_kb + s - 1) / s + exchange);
-    };
-    auto best_split = [&](int n) {
+// Time of the weights kernel in cycles, from measurements: a k-block (64 k with activations as bytes, 128 k otherwise) and a
+// tile's drain; what the exchange of a split tile costs beyond that (two cluster barriers, the sums at 20 bytes a cycle, less
+// what the shared epilogue saves) at bn = 256, about half of it at 128; a launch of its own for the last round (set-up, first
+// copies).
+struct WeightsCost {
+    int num_kb, bn;
+    const int* clusters;  // clusters of s pairs that the device holds
+    static constexpr double kblock = 1150.0;
+    double tiles(long long n, int split) const
+    {
+        if (split > num_kb || clusters[split] <= 0) return 1e30;
+        const double f = bn / 256.0, exchange = split == 1 ? 0.0 : (split == 2 ? 1300.0 + 2000.0 * f : 2100.0 + 5300.0 * f);
+        return (double)((n + clusters[split] - 1) / clusters[split]) * ((num_kb + split - 1) / split * kblock + 5000.0 * f + exchange);
+    }
+    int best_split(long long n) const
+    {
         int best = 1;
         for (int s = 2; s <= kWdMaxSplit; s *= 2)
-            if (cost(n, s) < cost(n, best)) best = s;
+            if (tiles(n, s) < tiles(n, best)) best = s;
         return best;
-    };
-    const int pairs = clusters[1];
-    TilePlan launch[2];
-    int launches = 1;
-    launch[0] = TilePlan{0, tiles, chunks, bn, tiles <= pairs ? best_split(tiles) : 1};
-    if (tiles > pairs && tiles % pairs) {
-        const int rem = tiles % pairs, s = best_split(rem);
-        if (s > 1 && cost(rem, s) + 4 < num_kb) {
-            launch[0].count = tiles - rem;
-            launch[1] = TilePlan{tiles - rem, rem, chunks, bn, s};
-            launches = 2;
-        }
     }
-    for (int i = 0; i < launches; i++) {
+    // tiles of the last round that a launch of their own, split, finishes earlier (0: none)
+    long long remainder(long long n) const
+    {
+        const long long rem = n > clusters[1] ? n % clusters[1] : 0;
+        if (!rem) return 0;
+        const int s = best_split(rem);
+        return s > 1 && tiles(rem, s) + 4200.0 < tiles(rem, 1) ? rem : 0;
+    }
+    double all(long long n) const
+    {
+        const long long rem = remainder(n);
+        return n <= clusters[1] ? tiles(n, best_split(n)) : (rem ? tiles(n - rem, 1) + tiles(rem, best_split(rem)) + 4200.0 : tiles(n, 1));
+    }
+};
+
+struct WeightsTiling {
+    int chunks, bn;
+    long long tiles;
+    WeightsCost cost;
+    WeightsTiling(int M, int N, int K, int act, const int* clusters)
+    {
+        // activation rows in pieces of at most 256, a multiple of 32 (of 128 as bytes [K,M]: whole 64-column atoms per CTA)
+        const int unit = act == kActColumns ? 128 : 32, kb = act == kActExpanded ? 2 * BK : BK;
+        chunks = (M + BN - 1) / BN;
+        bn = ((M + chunks - 1) / chunks + unit - 1) / unit * unit;
+        tiles = (long long)((N + 2 * BM - 1) / (2 * BM)) * chunks;
+        cost = WeightsCost{(K + kb - 1) / kb, bn, clusters};
+    }
+};
+
+template <int ACT>
+static cudaError_t launch_weights_kernel(const cudaLaunchConfig_t& cfg, int w_is_nk, const CUtensorMap& map_w, const CUtensorMap& map_act, const GemmParams& p,
+                                         const TilePlan& tp)
+{
+    return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true, ACT>, map_w, map_act, p, tp)
+                   : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false, ACT>, map_w, map_act, p, tp);
+}
+
+// C = A W with the weights decoded inside the kernel.  act = kActExpanded: `a` is BF16 [M,K], written by the launch in front of
+// this one, which also clears the status word; otherwise the caller's bytes.
+static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, int act, const void* a, int64_t lda, const GemmParams& p, const int* clusters,
+                               cudaStream_t st)
+{
+    const int M = p.M, N = p.N, K = p.K, kb = act == kActExpanded ? 2 * BK : BK;
+    const WeightsTiling tl(M, N, K, act, clusters);
+    if (tl.tiles > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
+    const int tiles = (int)tl.tiles, pairs = clusters[1];
+    CUtensorMap map_w, map_act;
+    const bool okw = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, (uint32_t)kb, BM, false, (uint32_t)kb)
+                             : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, (uint32_t)kb, false, 128);
+    const bool oka = act == kActExpanded ? make_map3(&map_act, a, (uint64_t)K, (uint64_t)M, 1, 0, BK, (uint32_t)tl.bn / 2)
+                     : act == kActRows   ? make_map(&map_act, a, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, (uint32_t)tl.bn / 2)
+                                         : make_map(&map_act, a, (uint64_t)M, (uint64_t)K, (uint64_t)lda, (uint32_t)tl.bn / 2, BK);
+    if (!okw || !oka) return HIF8_ERR_CUDA;
+    const int rem = (int)tl.cost.remainder(tiles), clear = act != kActExpanded;
+    TilePlan launch[2];
+    launch[0] = TilePlan{0, tiles - rem, tl.chunks, tl.bn, tiles <= pairs ? tl.cost.best_split(tiles) : 1, clear};
+    launch[1] = TilePlan{tiles - rem, rem, tl.chunks, tl.bn, rem ? tl.cost.best_split(rem) : 1, 0};
+    for (int i = 0; i < (rem ? 2 : 1); i++) {
         const TilePlan& tp = launch[i];
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(2u * (unsigned)(tp.split > 1 ? tp.count * tp.split : (tp.count < pairs ? tp.count : pairs)));
         cfg.blockDim = dim3(kThreadsWd);
-        cfg.dynamicSmemBytes = kSmemBytesWd;
+        cfg.dynamicSmemBytes = kSmemBytesMax;
         cfg.stream = st;
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2357,8 +2103,9 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = 2;
-        const cudaError_t rc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true>, map_w, map_act, p, tp)
-                                       : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false>, map_w, map_act, p, tp);
+        const cudaError_t rc = act == kActExpanded ? launch_weights_kernel<kActExpanded>(cfg, w_is_nk, map_w, map_act, p, tp)
+                               : act == kActRows   ? launch_weights_kernel<kActRows>(cfg, w_is_nk, map_w, map_act, p, tp)
+                                                   : launch_weights_kernel<kActColumns>(cfg, w_is_nk, map_w, map_act, p, tp);
         if (rc != cudaSuccess) return HIF8_ERR_CUDA;
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
@@ -2400,10 +2147,6 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     p.d_sa = d_scale_exp_a; p.d_sw = d_scale_exp_w; p.d_sw_channel = d_scale_exp_w_channel;
     p.accumulate = accumulate ? 1 : 0;
     p.status = reinterpret_cast<int*>(workspace);
-    p.tiles_m = (M + BM - 1) / BM; p.tiles_n = (N + BN - 1) / BN;
-    // both kernels work on 256 x 256 tiles, one per pair of CTAs
-    const long long tiles2 = (long long)((M + 2 * BM - 1) / (2 * BM)) * p.tiles_n;
-    if (tiles2 > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
     cudaStream_t st = (cudaStream_t)stream;
     note_status_word(st, reinterpret_cast<const int*>(workspace));
 
@@ -2468,7 +2211,7 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         cudaLaunchConfig_t cn{};
         cn.gridDim = dim3((unsigned)grid);
         cn.blockDim = dim3(kThreadsN);
-        cn.dynamicSmemBytes = kSmemBytesN;
+        cn.dynamicSmemBytes = kSmemBytesMax;
         cn.stream = st;
         // with the preparing kernel right in front: programmatic stream serialization (that kernel lets its dependents start
         // at once; this one waits for its completion once its own set-up is done)
@@ -2491,13 +2234,16 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     // Otherwise the weights are decoded inside the tensor-core kernel, and the activations too when there is no room for them.
     const size_t bytes_a = (((size_t)M * K * 2) + 255) & ~(size_t)255, bytes_w = (((size_t)K * N * 2) + 255) & ~(size_t)255;
     const bool a_contiguous = lda == (a_is_km ? M : K), w_contiguous = ldw == (w_is_nk ? K : N);
-    // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element
-    // moved) at the higher rate of the decode-once kernel: with about 268 flops per byte of copy bandwidth for that kernel,
-    // 233 for the swapped A-expanded form ([N,K] weights) and 210 for the other (their measured rates against the copy rate)
-    // they meet near M = 4800 and M = 1450, whatever N and K.
-    const double mk = (double)M * K, kn = (double)K * N, flops = 2.0 * mk * N;
+    // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element moved, at
+    // 3300 bytes a cycle, and a launch) by the cheaper k-blocks and tiles of the pair kernel: 545 cycles per
+    // 64 k and nothing between tiles, against the weights kernel's cost above.  Measured (us, both expanded / weights decoded in
+    // the kernel): 2048 x 7168 x 4096 105 / 98, 3072 rows 130 / 133, 4096 rows 172 / 176; 1536 x 8192 x 1024 28.5 / 33;
+    // 2048 x 16384 x 8192 381 / 357, 4096 rows 702 / 732.
+    const WeightsTiling tl(M, N, K, kActExpanded, wd_clusters);
+    const long long pair_rounds = ((long long)((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN) + sm_count / 2 - 1) / (sm_count / 2);
+    const double expand_w = 6000.0 + 3.0 * (double)K * N / 3300.0, pair_cycles = (double)pair_rounds * ((K + BK - 1) / BK * 545.0 + 500.0);
     const bool w_expansion_pays = g_path_policy.load(std::memory_order_relaxed) == HIF8_GEMM_PATH_EXPAND_BOTH ||
-                                  3.0 * kn + flops / 268.0 < flops / (w_is_nk ? 233.0 : 210.0);
+                                  expand_w + pair_cycles < 1.03 * tl.cost.all(tl.tiles);  // (equal at 1.03: the lookups also cost clock under the power limit)
     if (a_contiguous && workspace_bytes >= kGemmWorkspaceBytes + bytes_a && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
         unsigned char* a_bf = reinterpret_cast<unsigned char*>(workspace) + kGemmWorkspaceBytes;
         // (an A given as [K,M] is written as [M,K] while it is expanded; either launch clears the status word)
@@ -2510,40 +2256,10 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
             rc = hif8_decode(Wq, w_bf, HIF8_BF16, (size_t)K * N, 0, stream);
             return rc != HIF8_OK ? rc : launch_bf16_pair_gemm(a_bf, w_bf, w_is_nk, p, st);
         }
-        return launch_weights_gemm(Wq, ldw, w_is_nk, a_bf, p, wd_clusters, st);
+        return launch_weights_gemm(Wq, ldw, w_is_nk, kActExpanded, a_bf, K, p, wd_clusters, st);
     }
     // No room for the activations: both operands are decoded in the kernel.
-    CUtensorMap map_a, map_w;
-    // ([M,K] activations: 64-byte rows with the 64-byte swizzle, read row-wise by the decode warps of the fused kernel)
-    const bool ok_a = a_is_km ? make_map(&map_a, Aq, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BM, BK)
-                              : make_map(&map_a, Aq, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM, false, 64);
-    if (!ok_a) return HIF8_ERR_CUDA;
-    // byte tiles of one CTA of a pair: 128 rows of A, 128 of the 256 columns of W
-    const bool ok_w = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, BK, BN / 2)
-                              : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BN / 2, BK);
-    if (!ok_w) return HIF8_ERR_CUDA;
-
-    if (cudaMemsetAsync(workspace, 0, 4, st) != cudaSuccess) return HIF8_ERR_CUDA;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(2u * (unsigned)tiles2);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = a_is_km ? kSmemBytes : kSmemBytesWide;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    cudaError_t lrc;
-    // BF16 results that replace C leave the [M,K]-activation kernel through tile stores (boxes of 64 columns x 128 rows)
-    CUtensorMap map_c = map_a;  // (a valid map in any case; only read when c_by_tma is set)
-    p.c_by_tma = (!a_is_km && c_dtype == HIF8_BF16 && !accumulate) ? 1 : 0;
-    if (p.c_by_tma && !make_map(&map_c, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 64, BM, true)) return HIF8_ERR_CUDA;
-    if (a_is_km) lrc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<true, true>, map_a, map_w, map_c, p)
-                               : cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<true, false>, map_a, map_w, map_c, p);
-    else lrc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<false, true>, map_a, map_w, map_c, p)
-                       : cudaLaunchKernelEx(&cfg, hif8_gemm_kernel<false, false>, map_a, map_w, map_c, p);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return (lrc == cudaSuccess && cudaGetLastError() == cudaSuccess) ? HIF8_OK : HIF8_ERR_CUDA;
+    return launch_weights_gemm(Wq, ldw, w_is_nk, a_is_km ? kActColumns : kActRows, Aq, lda, p, wd_clusters, st);
 }
 
 extern "C" int hif8_gemm(const uint8_t* Aq, int64_t lda, const uint8_t* Wq, int64_t ldw, int w_is_nk, void* C, int64_t ldc,

@@ -348,3 +348,50 @@ def test_gemm_repeated_runs_are_bit_identical(mode):
     for _ in range(8):
         again = run_gemm(Aq, Wq, w_is_nk, H.F32, sa=2, sw=-3, staged=staged)
         assert np.array_equal(first, again)
+
+
+@pytest.mark.parametrize("accumulate", [0, 1])
+@pytest.mark.parametrize("c_dtype", [H.F32, H.BF16])
+@pytest.mark.parametrize("w_is_nk", [0, 1])
+@pytest.mark.parametrize("form", ["rows", "columns", "rows_expanded", "columns_expanded"])
+@pytest.mark.parametrize("shape", [(65, 272, 128), (96, 512, 16), (208, 1008, 2064), (128, 512, 4096), (512, 1040, 1168), (304, 10000, 1040), (512, 20000, 144)])
+def test_gemm_weights_decoded_in_the_kernel(shape, form, w_is_nk, c_dtype, accumulate):
+    # One tile per pair without and with a split along K (parts of unequal length, K that ends within a k-block), 80 tiles on
+    # 74 pairs (the last ones split, in a launch of their own) and 160 (several tiles per pair, fewer k-blocks than decode groups);
+    # activation rows in one and two pieces, ending within a piece of eight; activations as bytes and expanded, from both layouts.
+    M, N, K = shape
+    columns, expanded = form.startswith("columns"), form.endswith("expanded")
+    lda = (M + 15) // 16 * 16 if columns else K
+    if columns and expanded and lda != M:
+        M = lda                                               # (a padded [K,M] operand is not expanded)
+    Aq, Wkn = W.random_codes((M, K), seed=M + K), W.random_codes((K, N), seed=N + K + 1)
+    for t in (Aq, Wkn):
+        t[(t == 0x80) | ((t & 0x7F) == 0x6F)] = 0x33
+    if columns:
+        A = np.full((K, lda), 0x7B, dtype=np.uint8)
+        A[:, :M] = Aq.T
+    else:
+        A = Aq
+    Wq = np.ascontiguousarray(Wkn.T) if w_is_nk else Wkn
+    rng = np.random.default_rng(M)
+    ldc = N + 8
+    c0 = (rng.standard_normal((M, ldc)) * 50).astype(np.float32)
+    C = torch.from_numpy(c0.copy()).cuda()
+    if c_dtype == H.BF16:
+        C = C.bfloat16()
+        c0 = C.float().cpu().numpy()
+    wsb = 256 + (2 * M * K + 255) // 256 * 256 if expanded else 256
+    ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")
+    H.hif8_gemm_ex(to_dev(A), lda, columns, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
+                   torch.tensor([3], dtype=torch.int32, device="cuda"), torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    assert H.hif8_gemm_status(ws) == 0
+    out = C.float().cpu().numpy().astype(np.float64)
+    assert np.array_equal(out[:, N:], c0[:, N:].astype(np.float64))
+    rows = np.concatenate([rng.integers(0, M, 20000), np.repeat(np.arange(M), 8), rng.integers(0, M, 2048)])
+    cols = np.concatenate([rng.integers(0, N, 20000), np.tile(np.arange(N - 8, N), M), np.arange(2048) % N])
+    P, S = O.gemm_entries(Aq, Wkn, False, 3, -4, rows, cols)
+    want = P + c0[rows, cols] if accumulate else P
+    tol = 1e-5 * S + 2.0 ** -24 * np.abs(want)
+    if c_dtype == H.BF16:
+        tol = tol + bf16_half_ulp(np.abs(want) + tol)
+    assert np.all(np.abs(out[rows, cols] - want) <= tol)
