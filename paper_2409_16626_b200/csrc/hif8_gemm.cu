@@ -203,6 +203,11 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+__device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all()
@@ -567,6 +572,7 @@ struct NarrowSmem {
 // issuer q taking the k-blocks it = q (mod issuers) into accumulators of its own, which the epilogue adds.  Up to 32
 // activation rows every issuer has two accumulators, above that one: issuers x buffers x rows stays within 256 columns.
 constexpr int kNwMaxIssuers = 4;
+constexpr int kNwMaxSplit = 8;
 // the first issuer is the MMA warp of the other kernels; the warp behind the others copies expanded activations
 constexpr int kNwActWarp = kThreads / 32 + kNwMaxIssuers - 1, kThreadsN = (kNwActWarp + 1) * 32;  // 832
 constexpr uint32_t kTmemAccN = 2 * 2 * kNarrowMaxM, kTmemColsN = 512;
@@ -580,6 +586,10 @@ static_assert(2 * kNwMaxIssuers * 32 <= kTmemAccN, "four issuers x two buffers x
 // its CTA; otherwise the CTA stores its FP32 partial sums as slice (slab, its position among the slab's contributors),
 // and the last contributor to arrive (one ticket per slab and epilogue warp) adds the slices in position order - so the
 // result does not depend on arrival order - and writes C.
+// Few slabs go another way: a cluster of CTAs per slab, each an equal part of its pair blocks; the partial sums are exchanged
+// through distributed shared memory and added in rank order.  Nothing of that is in the workspace, and after the last MMA it
+// takes 4000 cycles where slices, tickets and a reduction by one warp take 8000 (16 rows) to 22000 (64 rows).  us a call: 64 x
+// 4096 x 4096 21.2 -> 12.8, 16 rows 12.9 -> 11.4; with room for the status word only, where a slab had one CTA: 26.8 -> 12.4.
 // (Everything in 32 bits, q and rem from the host: N K < 2^45 bytes, so slabs * pair blocks < 2^31.  What a call costs
 // beyond its weight bytes is latency: with 64-bit products and divisions in the kernel, exponents loaded after the sums
 // were complete, one accumulator read per wait and the first copies issued behind the table set-up, 16 x 512 x 512 took
@@ -590,6 +600,7 @@ struct NarrowPlan {
     unsigned* tickets;   // [slab][4], zero at launch
     int pmax;            // slices per slab
     int clear_status;    // nonzero: no launch in front of this one clears the status word
+    int split;           // above 1: a cluster of `split` CTAs per slab, each a part of its pair blocks (see below)
 
     __device__ int first(int c) const { return c * q + (c < rem ? c : rem); }  // first unit of CTA c
     __device__ int owner(int x) const                                          // the CTA that takes unit x
@@ -627,7 +638,7 @@ __global__ void __launch_bounds__(256) expand_activations_kernel(const uint4* __
     }
 }
 
-template <bool W_IS_NK, bool ACT_BF16>
+template <bool W_IS_NK, bool ACT_BF16, bool CLUSTER>
 __global__ void __launch_bounds__(kThreadsN, 1)
 hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_constant__ CUtensorMap map_w, const GemmParams p, int mp,
                         const NarrowPlan plan)
@@ -667,9 +678,19 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     uint32_t* lut_all = reinterpret_cast<uint32_t*>(sm + lay.lut);
     const uint32_t lut = lay.lut + 4u * lane;
     const int num_pb = (p.K + BK2 - 1) / BK2, num_kb = 2 * num_pb;  // per slab
-    const int pair0 = plan.first((int)blockIdx.x), pair1 = plan.first((int)blockIdx.x + 1);  // this CTA's (slab, pair block) range
-    const int n_pairs = pair1 - pair0, n_it = 2 * n_pairs;
-    const int slab0 = pair0 / num_pb, pb0 = pair0 - slab0 * num_pb;  // where the range starts
+    // this CTA's (slab, pair block) range: where it starts, and its length
+    const int split = CLUSTER ? plan.split : 1, part = CLUSTER ? (int)cluster_ctarank() : 0;
+    int slab0, pb0, n_pairs;
+    if (CLUSTER) {
+        slab0 = (int)blockIdx.x / split;
+        pb0 = num_pb * part / split;
+        n_pairs = num_pb * (part + 1) / split - pb0;
+    } else {
+        const int pair0 = plan.first((int)blockIdx.x);
+        slab0 = pair0 / num_pb; pb0 = pair0 - slab0 * num_pb;
+        n_pairs = plan.first((int)blockIdx.x + 1) - pair0;
+    }
+    const int n_it = 2 * n_pairs;
     const uint32_t act_bytes = (uint32_t)mp * BK2;
     // Up to 32 activation rows every issuer has two accumulators (the epilogue of one segment overlaps the next segment's
     // MMAs).  Above that issuers x buffers x rows must stay within 256 columns, and four issuers with one accumulator each
@@ -886,7 +907,7 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             s8 += 2;
             if (s8 >= S8) { s8 -= S8; ph8 ^= 1u; }
         }
-    } else {
+    } else if (!CLUSTER) {
         // epilogue warps 0-3: TMEM lane = weight column n, TMEM column = activation row m.  Whatever does not need the sums
         // (exponents, the slab's contributors) is worked out before the wait for them: after it, it cost every segment
         // several thousand cycles of load latency and divisions.
@@ -1004,6 +1025,72 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             done += len; pb_a = 0; slab++;
         }
     }
+    if (CLUSTER) {
+        // Exchange and epilogue of a slab shared by a cluster: pieces of eight activation rows, dealt to the CTAs in runs of `per`.
+        // Every CTA sends its sums of a piece to the owner (itself included), which adds them in rank order.
+        __syncwarp();
+        const int quarter = warp & 3, shares = quarter < 2 ? 7 : 6, pieces = mp / 8, per = (pieces + split - 1) / split;
+        static_assert(kThreadsN / 32 == 26, "seven warps on the lanes of quarters 0 and 1, six on the others");
+        const int sa = p.d_sa ? *p.d_sa : 0, sw_all = (p.d_sw && !p.d_sw_channel) ? *p.d_sw : 0;
+        const bool ok = mbar_wait(bar_acc_full(0), 0, abort_flag, p.status, 38);
+        tc_fence_after();
+        __syncwarp();
+        cluster_sync_all();  // all CTAs are done with their stages
+        if (ok) {
+#pragma unroll 1
+            for (int j = warp >> 2; j < pieces; j += shares) {
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; i++) v[i] = 0.f;
+#pragma unroll 1
+                for (int q = 0; q < issuers; q++) {
+                    if (q >= n_it) break;  // (an issuer without a k-block left its accumulator as it was)
+                    uint32_t r[8];
+                    tmem_ld_32x32b_x8(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc_col(q, 0) + j * 8, r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 8; i++) v[i] += __uint_as_float(r[i]);
+                }
+                const int owner = j / per;
+                const uint32_t to = map_to_cta(lay.base + (uint32_t)(((part * per + j - owner * per) * 2 * BM + quarter * 32 + lane) * 16), (uint32_t)owner);
+                st_cluster_v4(to, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
+                st_cluster_v4(to + BM * 16, __float_as_uint(v[4]), __float_as_uint(v[5]), __float_as_uint(v[6]), __float_as_uint(v[7]));
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();
+        // four activation rows of a quarter's columns per warp and step
+        const int items = max(0, min(pieces - part * per, per)) * 8;
+#pragma unroll 1
+        for (int u = warp; ok && u < items; u += kThreadsN / 32) {
+            const int nl = (u & 3) * 32 + lane, n = slab0 * BM + nl, m = (part * per + (u >> 3)) * 8 + ((u >> 2) & 1) * 4;
+            const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = sc / 2, s2 = sc - s1;
+            const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(s2 + 127) << 23);
+            float v[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int q = 0; q < split; q++) {
+                const uint4 w = lds_v4(lay.base + (uint32_t)((((q * per + (u >> 3)) * 2 + ((u >> 2) & 1)) * BM + nl) * 16));
+                v[0] += __uint_as_float(w.x); v[1] += __uint_as_float(w.y); v[2] += __uint_as_float(w.z); v[3] += __uint_as_float(w.w);
+            }
+            if (n < p.N) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    if (m + i >= p.M) continue;
+                    float x = v[i] * f1 * f2;
+                    const long long at = (long long)(m + i) * p.ldc + n;
+                    if (p.c_is_f32) {
+                        float* out = reinterpret_cast<float*>(p.C) + at;
+                        *out = p.accumulate ? x + *out : x;
+                    } else {
+                        unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + at;
+                        if (p.accumulate) x += __uint_as_float((uint32_t)*out << 16);
+                        unsigned short b;
+                        asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(b) : "f"(x));  // round to nearest even; a NaN stays a NaN
+                        *out = b;
+                    }
+                }
+            }
+        }
+    }
 
     tc_fence_before();
     __syncthreads();
@@ -1078,11 +1165,6 @@ struct TilePlan {
     int split;
     int clear_status;  // nonzero: no launch in front of this one clears the status word
 };
-
-__device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
 
 // Eight finished sums of this thread's weight column, activation rows m .. m + 7 of which `rows` exist, to C: `out` is the
 // place of the first, `pitch` the bytes from row to row (below 2^32: more than 64 rows fit in memory).  For one row a warp
@@ -1899,16 +1981,18 @@ bool make_map3(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t rows,
 struct GemmDeviceSetup {
     cudaError_t rc;
     int sm_count;
+    int nw_clusters[kNwMaxSplit + 1];  // clusters of s CTAs of the narrow kernel, s = 1, 2, 4, 8
     int wd_clusters[kWdMaxSplit + 1];  // clusters of s pairs of hif8_gemm_weights_kernel that fit on the device at once, s = 1, 2, 4
 };
 PerDevice<GemmDeviceSetup> g_gemm_setup;
 
-bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nullptr)
+bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nullptr, const int** nw_clusters = nullptr)
 {
     const GemmDeviceSetup* s = g_gemm_setup.get(dev, [](int d, GemmDeviceSetup* out) {
         out->rc = cudaSuccess;
         out->sm_count = 0;
         std::memset(out->wd_clusters, 0, sizeof out->wd_clusters);
+        std::memset(out->nw_clusters, 0, sizeof out->nw_clusters);
         const void* pair[2] = {(const void*)bf16_gemm_pair_kernel<false>, (const void*)bf16_gemm_pair_kernel<true>};
         const void* wd[6] = {(const void*)hif8_gemm_weights_kernel<false, kActExpanded>, (const void*)hif8_gemm_weights_kernel<true, kActExpanded>,
                              (const void*)hif8_gemm_weights_kernel<false, kActRows>, (const void*)hif8_gemm_weights_kernel<true, kActRows>,
@@ -1926,15 +2010,27 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
             cfg.attrs = attr; cfg.numAttrs = 1;
             out->rc = cudaOccupancyMaxActiveClusters(&out->wd_clusters[s], wd[1], &cfg);
         }
-        const void* narrow[4] = {(const void*)hif8_gemm_narrow_kernel<false, false>, (const void*)hif8_gemm_narrow_kernel<false, true>,
-                                 (const void*)hif8_gemm_narrow_kernel<true, false>, (const void*)hif8_gemm_narrow_kernel<true, true>};
-        for (int i = 0; i < 4 && out->rc == cudaSuccess; i++)
+        const void* narrow[8] = {(const void*)hif8_gemm_narrow_kernel<false, false, false>, (const void*)hif8_gemm_narrow_kernel<false, true, false>,
+                                 (const void*)hif8_gemm_narrow_kernel<true, false, false>, (const void*)hif8_gemm_narrow_kernel<true, true, false>,
+                                 (const void*)hif8_gemm_narrow_kernel<false, false, true>, (const void*)hif8_gemm_narrow_kernel<false, true, true>,
+                                 (const void*)hif8_gemm_narrow_kernel<true, false, true>, (const void*)hif8_gemm_narrow_kernel<true, true, true>};
+        for (int i = 0; i < 8 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
+        for (int s = 1; s <= kNwMaxSplit && out->rc == cudaSuccess; s *= 2) {
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = s; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            cfg.gridDim = dim3(s); cfg.blockDim = dim3(kThreadsN); cfg.dynamicSmemBytes = kSmemBytesMax;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            out->rc = cudaOccupancyMaxActiveClusters(&out->nw_clusters[s], narrow[7], &cfg);
+        }
         if (out->rc == cudaSuccess) out->rc = cudaDeviceGetAttribute(&out->sm_count, cudaDevAttrMultiProcessorCount, d);
     });
     if (!s) return false;
     *sm_count_out = s->sm_count;
     if (wd_clusters) *wd_clusters = s->wd_clusters;
+    if (nw_clusters) *nw_clusters = s->nw_clusters;
     return s->rc == cudaSuccess && s->sm_count > 0 && s->wd_clusters[1] > 0;
 }
 
@@ -2112,6 +2208,14 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, int 
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
 }
 
+template <bool W_IS_NK, bool ACT_BF16>
+static cudaError_t launch_narrow_kernel(const cudaLaunchConfig_t& cfg, bool cluster, const CUtensorMap& map_act, const CUtensorMap& map_w, const GemmParams& p,
+                                        int mp, const NarrowPlan& plan)
+{
+    return cluster ? cudaLaunchKernelEx(&cfg, hif8_gemm_narrow_kernel<W_IS_NK, ACT_BF16, true>, map_act, map_w, p, mp, plan)
+                   : cudaLaunchKernelEx(&cfg, hif8_gemm_narrow_kernel<W_IS_NK, ACT_BF16, false>, map_act, map_w, p, mp, plan);
+}
+
 static std::atomic<int> g_path_policy{HIF8_GEMM_PATH_AUTO};
 
 extern "C" int hif8_gemm_path_policy(int policy)
@@ -2151,8 +2255,8 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     note_status_word(st, reinterpret_cast<const int*>(workspace));
 
     int sm_count = 0;
-    const int* wd_clusters = nullptr;
-    if (!gemm_kernels_ready(dev, &sm_count, &wd_clusters)) return HIF8_ERR_CUDA;
+    const int *wd_clusters = nullptr, *nw_clusters = nullptr;
+    if (!gemm_kernels_ready(dev, &sm_count, &wd_clusters, &nw_clusters)) return HIF8_ERR_CUDA;
     // the status word is cleared on the stream before the kernels; the narrow path clears its tickets in the same operation
     size_t clear_bytes = 4;
 
@@ -2169,11 +2273,21 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         NarrowPlan plan{};
         const long long total = slabs * num_pb;
         if (total > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
-        // One CTA per SM, equal k-block ranges, when the workspace holds the partial sums of the slabs that a range
-        // boundary cuts; otherwise one CTA per slab.
-        long long grid = slabs;
+        // Cycles: a k-block takes about 500 (mp = 16) to 590 (64); a cluster's exchange 4000, and clusters of eight start later;
+        // ranges of slabs end in a reduction of 2500 + 290 mp.  A cluster per slab (or one CTA: split 1), or, when the workspace
+        // holds the partial sums of the slabs that a range boundary cuts, one CTA per SM with equal ranges: for many slabs that do
+        // not divide among the SMs, and few rows.
+        const double c_pb = 2.0 * (470.0 + 1.9 * mp);
+        double best = 1e30;
+        for (int s = 1; s <= kNwMaxSplit && s <= num_pb; s *= 2) {
+            if (nw_clusters[s] <= 0) continue;
+            const long long rounds = (slabs + nw_clusters[s] - 1) / nw_clusters[s];
+            const double c = (double)rounds * ((double)((num_pb + s - 1) / s) * c_pb + 4500.0 + (s == 1 ? 0.0 : (s < 8 ? 4000.0 : 6000.0)));
+            if (c < best) { best = c; plan.split = s; }
+        }
+        long long grid = slabs * plan.split;
         {
-            // aim at four or more pair blocks per CTA, but never fewer CTAs than the per-slab grid would keep busy
+            // four or more pair blocks per CTA, but never fewer CTAs than slabs
             long long g = total / 4 < sm_count ? total / 4 : sm_count;
             const long long floor_g = slabs < sm_count ? slabs : sm_count;
             if (g < floor_g) g = floor_g;
@@ -2181,11 +2295,13 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
             const long long pmax = (num_pb + per - 1) / per + 1;
             const size_t ticket_bytes = (((size_t)slabs * kEpiWarps * 4) + 255) & ~(size_t)255;
             const size_t part_bytes = (size_t)slabs * pmax * mp * BM * 4;
-            if (g != slabs && workspace_bytes >= kGemmWorkspaceBytes + ticket_bytes + part_bytes && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
+            const double c = (double)(per + 1) * c_pb + 4500.0 + 2500.0 + 290.0 * mp;
+            if (c < best && workspace_bytes >= kGemmWorkspaceBytes + ticket_bytes + part_bytes && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
                 unsigned char* wsb = reinterpret_cast<unsigned char*>(workspace) + kGemmWorkspaceBytes;
                 plan.tickets = reinterpret_cast<unsigned*>(wsb);
                 plan.part = reinterpret_cast<float*>(wsb + ticket_bytes);
                 plan.pmax = (int)pmax;
+                plan.split = 0;
                 grid = g;
                 clear_bytes = kGemmWorkspaceBytes + ticket_bytes;  // the tickets follow the status block
             }
@@ -2215,15 +2331,23 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         cn.stream = st;
         // with the preparing kernel right in front: programmatic stream serialization (that kernel lets its dependents start
         // at once; this one waits for its completion once its own set-up is done)
-        cudaLaunchAttribute an[1];
-        an[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        an[0].val.programmaticStreamSerializationAllowed = 1;
-        cn.attrs = an; cn.numAttrs = act_bf16 ? 1 : 0;
+        cudaLaunchAttribute an[2];
+        int n_an = 0;
+        if (act_bf16) {
+            an[n_an].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            an[n_an++].val.programmaticStreamSerializationAllowed = 1;
+        }
+        if (plan.split > 1) {
+            an[n_an].id = cudaLaunchAttributeClusterDimension;
+            an[n_an].val.clusterDim.x = (unsigned)plan.split; an[n_an].val.clusterDim.y = 1; an[n_an++].val.clusterDim.z = 1;
+        }
+        cn.attrs = an; cn.numAttrs = (unsigned)n_an;
         cudaError_t nrc;
-        if (w_is_nk) nrc = act_bf16 ? cudaLaunchKernelEx(&cn, hif8_gemm_narrow_kernel<true, true>, map_act, map_ws, p, mp, plan)
-                                    : cudaLaunchKernelEx(&cn, hif8_gemm_narrow_kernel<true, false>, map_act, map_ws, p, mp, plan);
-        else nrc = act_bf16 ? cudaLaunchKernelEx(&cn, hif8_gemm_narrow_kernel<false, true>, map_act, map_ws, p, mp, plan)
-                            : cudaLaunchKernelEx(&cn, hif8_gemm_narrow_kernel<false, false>, map_act, map_ws, p, mp, plan);
+        const bool cluster = plan.split > 1;
+        if (w_is_nk) nrc = act_bf16 ? launch_narrow_kernel<true, true>(cn, cluster, map_act, map_ws, p, mp, plan)
+                                    : launch_narrow_kernel<true, false>(cn, cluster, map_act, map_ws, p, mp, plan);
+        else nrc = act_bf16 ? launch_narrow_kernel<false, true>(cn, cluster, map_act, map_ws, p, mp, plan)
+                            : launch_narrow_kernel<false, false>(cn, cluster, map_act, map_ws, p, mp, plan);
         if (nrc != cudaSuccess) return HIF8_ERR_CUDA;
         g_launches.fetch_add(1, std::memory_order_relaxed);
         return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;

@@ -395,3 +395,42 @@ def test_gemm_weights_decoded_in_the_kernel(shape, form, w_is_nk, c_dtype, accum
     if c_dtype == H.BF16:
         tol = tol + bf16_half_ulp(np.abs(want) + tol)
     assert np.all(np.abs(out[rows, cols] - want) <= tol)
+
+
+@pytest.mark.parametrize("accumulate", [0, 1])
+@pytest.mark.parametrize("c_dtype", [H.F32, H.BF16])
+@pytest.mark.parametrize("w_is_nk", [0, 1])
+@pytest.mark.parametrize("staged", [False, True])
+@pytest.mark.parametrize("shape", [(1, 1000, 4112), (40, 1000, 4112), (24, 4000, 2064), (64, 4000, 2064), (16, 9008, 2064), (64, 9008, 2064), (16, 20000, 1040),
+                                   (48, 20000, 2064)])
+def test_gemm_narrow_splits(shape, staged, w_is_nk, c_dtype, accumulate):
+    # Slabs shared by clusters of 8, 4 and 2 CTAs in parts of unequal length (2, 4, 6 and 8 pieces of eight rows dealt to them, so
+    # that some CTAs finish none), with the activations as bytes and expanded; and (last two, with the workspace) equal ranges of
+    # 157 slabs on 148 SMs.
+    M, N, K = shape
+    Aq, Wkn = W.random_codes((M, K), seed=M + K), W.random_codes((K, N), seed=N + K + 1)
+    for t in (Aq, Wkn):
+        t[(t == 0x80) | ((t & 0x7F) == 0x6F)] = 0x33
+    Wq = np.ascontiguousarray(Wkn.T) if w_is_nk else np.pad(Wkn, ((0, 0), (0, -N % 16)))
+    rng = np.random.default_rng(M + N)
+    ldc = N + 8
+    c0 = (rng.standard_normal((M, ldc)) * 50).astype(np.float32)
+    C = torch.from_numpy(c0.copy()).cuda()
+    if c_dtype == H.BF16:
+        C = C.bfloat16()
+        c0 = C.float().cpu().numpy()
+    wsb = H.hif8_workspace_bytes(H.WS_GEMM, M * K + K * N) if staged else 256
+    ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")
+    H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
+                   torch.tensor([3], dtype=torch.int32, device="cuda"), torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    assert H.hif8_gemm_status(ws) == 0
+    out = C.float().cpu().numpy().astype(np.float64)
+    assert np.array_equal(out[:, N:], c0[:, N:].astype(np.float64))
+    rows = np.concatenate([rng.integers(0, M, 20000), np.repeat(np.arange(M), 130)])
+    cols = np.concatenate([rng.integers(0, N, 20000), np.tile(np.arange(N - 130, N), M)])
+    P, S = O.gemm_entries(Aq, Wkn, False, 3, -4, rows, cols)
+    want = P + c0[rows, cols] if accumulate else P
+    tol = 1e-5 * S + 2.0 ** -24 * np.abs(want)
+    if c_dtype == H.BF16:
+        tol = tol + bf16_half_ulp(np.abs(want) + tol)
+    assert np.all(np.abs(out[rows, cols] - want) <= tol)
