@@ -258,8 +258,7 @@ int hif8_fake_quant(const void* src, void* dst, int dtype, size_t n, int use_ama
  * multiple of 16 (HIF8_ERR_SHAPE).  NaN / Inf codes propagate as in IEEE arithmetic.
  * workspace: at least hif8_workspace_bytes(HIF8_WS_GEMM, 0) = 256 bytes, 16-byte aligned; its first int is a device
  * status word that the call clears and the kernel sets if one of its bounded waits ever gives up (see
- * hif8_gemm_status).  With only that, the fused kernel decodes the HiF8 byte tiles of every CTA pair inside the
- * tensor-core kernel (W into shared memory, an A given as [M,K] straight into tensor memory).
+ * hif8_gemm_status).  With only that, the tensor-core kernel decodes both byte operands itself.
  * With hif8_workspace_bytes(HIF8_WS_GEMM, M*K + K*N) bytes, 256-byte aligned, and contiguous operands (lda = K,
  * ldw = row length of Wq), each operand byte is instead decoded once into the workspace (BF16, exact) and the
  * tensor-core kernel streams BF16 tiles: several times faster for compute-bound shapes, same results.
@@ -268,9 +267,9 @@ int hif8_fake_quant(const void* src, void* dst, int dtype, size_t n, int use_ama
  * not fit but the activation's does; same results.  A workspace with room for both operands takes this form too while
  * the product is too small to win the pass over W back (see hif8_gemm_path_policy).
  * Products with at most 64 rows of A (and A given as [M,K]) take a weight-streaming kernel whatever the workspace;
- * with the workspace size above it spreads the weight bytes evenly over all SMs (partial sums of a column slab that
- * two SMs share go through the workspace and are added in a fixed order: results are reproducible run to run) and,
- * with A contiguous, first expands the few rows of A to BF16 there (one small launch more, same results).
+ * with the workspace size above it first expands the few rows of A to BF16 there (one small launch more, A contiguous).
+ * Where several SMs share the sum of an output (K split among them), the parts are added in a fixed order: results are
+ * reproducible run to run; how K is split depends on the sizes, the device and the workspace.
  */
 int hif8_gemm(const uint8_t* Aq, int64_t lda, const uint8_t* Wq, int64_t ldw, int w_is_nk, void* C,
               int64_t ldc, int c_dtype, int M, int N, int K, const int* d_scale_exp_a,
