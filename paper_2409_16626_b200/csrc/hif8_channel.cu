@@ -52,6 +52,12 @@ template <int PV> __device__ __forceinline__ void store_codes(uint8_t* dst, unsi
     }
 }
 
+template <int PV> __device__ __forceinline__ void store_packed(uint8_t* dst, unsigned long long vec_index, uint2 w)
+{
+    if (PV == 4) __stcs(reinterpret_cast<uint32_t*>(dst) + vec_index, w.x);
+    else __stcs(reinterpret_cast<uint2*>(dst) + vec_index, w);
+}
+
 // the stochastic words of the PV elements of flat vector u (element i takes word i % 4 of counter i / 4)
 template <int MODE, int PV> __device__ __forceinline__ void sr_words(unsigned long long u, uint32_t k0, uint32_t k1, uint32_t (&rw)[8])
 {
@@ -61,6 +67,29 @@ template <int MODE, int PV> __device__ __forceinline__ void sr_words(unsigned lo
         if (PV == 8) r1 = philox4x32_10((uint32_t)(u * 2 + 1), (uint32_t)((u * 2 + 1) >> 32), k0, k1);
     }
     rw[0] = r0.x; rw[1] = r0.y; rw[2] = r0.z; rw[3] = r0.w; rw[4] = r1.x; rw[5] = r1.y; rw[6] = r1.z; rw[7] = r1.w;
+}
+
+// One vector of a row: round half away through packed words, the other modes element by element.
+template <int SRC, int MODE> __device__ __forceinline__ void encode_row_vector(const ChanParams& p, const SmemTables& sm, const uint4& v, unsigned long long flat,
+                                                                               float scale, uint32_t k0, uint32_t k1)
+{
+    constexpr int PV = SrcTraits<SRC>::kPerVec;
+    if (MODE == HIF8_RND_TA) {
+        const uint32_t s2 = bf16x2_of_pow2(scale);
+        const uint32_t scales2[4] = {s2, s2, s2, s2};
+        const float scales[8] = {scale, scale, scale, scale, scale, scale, scale, scale};
+        store_packed<PV>(p.dst, flat, encode_vector_ta<SRC>(v, scales2, scales, sm.ta));
+        return;
+    }
+    uint32_t rw[8], codes[PV];
+    sr_words<MODE, PV>(flat, k0, k1, rw);
+#pragma unroll
+    for (int k = 0; k < PV; k++) {
+        float x; uint32_t raw;
+        unpack<SRC>(v, k, x, raw);
+        codes[k] = encode_one<MODE, SRC>(x, raw, scale, sm.ta, sm.thr, rw[k]);
+    }
+    store_codes<PV>(p.dst, flat, codes);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -84,7 +113,7 @@ __device__ __forceinline__ uint32_t group_max(uint32_t v, uint32_t* s_part, int 
 }
 
 // Rows that fit in registers (at most NV vectors per thread of a group of gs threads).  A block works through
-// `iters` consecutive sets of kThreads / gs rows; the loads of the next set are issued before the current one is
+// `iters` sets of kThreads / gs rows, one grid apart; the loads of the next set are issued before the current one is
 // reduced and converted, so every row is read exactly once and the memory latency is covered by the arithmetic of the
 // previous row.  Short rows get small groups so that a thread still holds about four vectors.
 template <int SRC, int MODE, int NV>
@@ -93,12 +122,14 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
     __shared__ SmemTables sm;
     __shared__ uint32_t s_part[kThreads / 32];
     constexpr int PV = SrcTraits<SRC>::kPerVec;
+    pdl_launch_dependents();
     setup_tables<true, MODE != HIF8_RND_TA, false, MODE, SRC>(sm, p.flags);
+    pdl_wait_prior_grid();
     const unsigned long long nv = (unsigned long long)p.cols / PV;  // vectors per row (cols is a multiple of PV here)
     const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
     const int groups = kThreads / gs, g = threadIdx.x / gs, t = threadIdx.x % gs;
     const uint4* base = reinterpret_cast<const uint4*>(p.src);
-    const long long first = (long long)blockIdx.x * iters * groups + g;
+    const long long first = (long long)blockIdx.x * groups + g, step = (long long)gridDim.x * groups;
 
     // NV <= kUnroll: two register sets, the next row is in flight while this one is processed; larger rows use one set
     constexpr bool kPrefetch = NV <= kUnroll;
@@ -111,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
         }
     }
     for (int it = 0; it < iters; it++) {
-        const long long row = first + (long long)it * groups, row_next = row + groups;
+        const long long row = first + (long long)it * step, row_next = row + step;
         const bool live = row < p.rows;  // a group past the last row only takes part in the barriers
         if (kPrefetch) {
 #pragma unroll
@@ -133,16 +164,10 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
         int se = 0;
         if (p.d_se_in) se = live ? clamp_exp(p.d_se_in[row]) : 0;
         else {
-            float m = 0.f;
+            uint32_t m = 0u;
 #pragma unroll
-            for (int j = 0; j < NV; j++)
-#pragma unroll
-                for (int k = 0; k < PV; k++) {
-                    float x; uint32_t raw;
-                    unpack<SRC>(cur[j], k, x, raw);
-                    m = amax_step(m, x);
-                }
-            const uint32_t b = group_max(__float_as_uint(m), s_part, gs);
+            for (int j = 0; j < NV; j++) m = amax_vector<SRC>(m, cur[j]);
+            const uint32_t b = group_max(__float_as_uint(amax_value<SRC>(m)), s_part, gs);
             if (t == 0 && live) p.amax_bits[row] = b;
             se = scale_exp_from_amax(b, p.target_exp);
         }
@@ -153,16 +178,7 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
             for (int j = 0; j < NV; j++) {
                 const unsigned long long u = (unsigned long long)j * gs + t;
                 if (u >= nv) continue;
-                const unsigned long long flat = (unsigned long long)row * nv + u;
-                uint32_t rw[8], codes[PV];
-                sr_words<MODE, PV>(flat, k0, k1, rw);
-#pragma unroll
-                for (int k = 0; k < PV; k++) {
-                    float x; uint32_t raw;
-                    unpack<SRC>(cur[j], k, x, raw);
-                    codes[k] = encode_one<MODE, SRC>(x, raw, scale, sm.ta, sm.thr, rw[k]);
-                }
-                store_codes<PV>(p.dst, flat, codes);
+                encode_row_vector<SRC, MODE>(p, sm, cur[j], (unsigned long long)row * nv + u, scale, k0, k1);
             }
         }
     }
@@ -175,7 +191,9 @@ __global__ void __launch_bounds__(kThreads) long_row_channel_kernel(const ChanPa
     __shared__ SmemTables sm;
     __shared__ uint32_t s_part[kThreads / 32];
     constexpr int PV = SrcTraits<SRC>::kPerVec;
+    pdl_launch_dependents();
     setup_tables<true, MODE != HIF8_RND_TA, false, MODE, SRC>(sm, p.flags);
+    pdl_wait_prior_grid();
     const unsigned long long nv = (unsigned long long)p.cols / PV;
     const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
 
@@ -184,7 +202,7 @@ __global__ void __launch_bounds__(kThreads) long_row_channel_kernel(const ChanPa
         int se;
         if (p.d_se_in) se = clamp_exp(p.d_se_in[row]);
         else {
-            float m = 0.f;
+            uint32_t m = 0u;
             for (unsigned long long base = 0; base < nv; base += (unsigned long long)kThreads * kUnroll) {
                 uint4 v[kUnroll];
 #pragma unroll
@@ -193,15 +211,9 @@ __global__ void __launch_bounds__(kThreads) long_row_channel_kernel(const ChanPa
                     v[j] = u < nv ? src[u] : make_uint4(0, 0, 0, 0);  // default caching: the second read wants these lines
                 }
 #pragma unroll
-                for (int j = 0; j < kUnroll; j++)
-#pragma unroll
-                    for (int k = 0; k < PV; k++) {
-                        float x; uint32_t raw;
-                        unpack<SRC>(v[j], k, x, raw);
-                        m = amax_step(m, x);
-                    }
+                for (int j = 0; j < kUnroll; j++) m = amax_vector<SRC>(m, v[j]);
             }
-            const uint32_t b = group_max(__float_as_uint(m), s_part, kThreads);
+            const uint32_t b = group_max(__float_as_uint(amax_value<SRC>(m)), s_part, kThreads);
             if (threadIdx.x == 0) p.amax_bits[row] = b;
             se = scale_exp_from_amax(b, p.target_exp);
         }
@@ -218,16 +230,7 @@ __global__ void __launch_bounds__(kThreads) long_row_channel_kernel(const ChanPa
             for (int j = 0; j < kUnroll; j++) {
                 const unsigned long long u = base + (unsigned long long)j * kThreads + threadIdx.x;
                 if (u >= nv) continue;
-                const unsigned long long flat = (unsigned long long)row * nv + u;
-                uint32_t rw[8], codes[PV];
-                sr_words<MODE, PV>(flat, k0, k1, rw);
-#pragma unroll
-                for (int k = 0; k < PV; k++) {
-                    float x; uint32_t raw;
-                    unpack<SRC>(v[j], k, x, raw);
-                    codes[k] = encode_one<MODE, SRC>(x, raw, scale, sm.ta, sm.thr, rw[k]);
-                }
-                store_codes<PV>(p.dst, flat, codes);
+                encode_row_vector<SRC, MODE>(p, sm, v[j], (unsigned long long)row * nv + u, scale, k0, k1);
             }
         }
     }
@@ -249,9 +252,9 @@ __global__ void __launch_bounds__(kThreads) col_amax_kernel(const ChanParams p, 
     const long long nvc = p.cols / PV;
     const long long cv = ((long long)blockIdx.x * wx + wxi) * 32 + lane;
     const long long r0 = (long long)blockIdx.y * rows_per_block, r1 = min(r0 + rows_per_block, p.rows);
-    float m[PV];
-#pragma unroll
-    for (int k = 0; k < PV; k++) m[k] = 0.f;
+    uint32_t m[4] = {0u, 0u, 0u, 0u};  // running maxima of the vector's words (see amax_word)
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
     if (cv < nvc) {
         const uint4* src = reinterpret_cast<const uint4*>(p.src) + cv;
         for (long long r = r0 + wyi; r < r1; r += wy * kUnroll) {
@@ -259,20 +262,20 @@ __global__ void __launch_bounds__(kThreads) col_amax_kernel(const ChanParams p, 
 #pragma unroll
             for (int j = 0; j < kUnroll; j++) {
                 const long long rr = r + wy * j;
-                v[j] = rr < r1 ? __ldcs(src + rr * nvc) : make_uint4(0, 0, 0, 0);
+                v[j] = rr < r1 ? __ldg(src + rr * nvc) : make_uint4(0, 0, 0, 0);  // default policy: the second pass wants these lines
             }
 #pragma unroll
-            for (int j = 0; j < kUnroll; j++)
-#pragma unroll
-                for (int k = 0; k < PV; k++) {
-                    float x; uint32_t raw;
-                    unpack<SRC>(v[j], k, x, raw);
-                    m[k] = amax_step(m[k], x);
-                }
+            for (int j = 0; j < kUnroll; j++) {
+                m[0] = amax_word<SRC>(m[0], v[j].x); m[1] = amax_word<SRC>(m[1], v[j].y);
+                m[2] = amax_word<SRC>(m[2], v[j].z); m[3] = amax_word<SRC>(m[3], v[j].w);
+            }
         }
     }
 #pragma unroll
-    for (int k = 0; k < PV; k++) s_max[warp][lane * PV + k] = __float_as_uint(m[k]);
+    for (int k = 0; k < PV; k++) {
+        const uint32_t w = m[k * 4 / PV];  // the element's own half of it as a source word of one element
+        s_max[warp][lane * PV + k] = __float_as_uint(amax_value<SRC>(SRC == HIF8_F32 ? w : ((k & 1) ? w >> 16 : w & 0xFFFFu)));
+    }
     __syncthreads();
     for (int idx = threadIdx.x; idx < wx * 32 * PV; idx += kThreads) {  // one atomic per column of the strip
         const int sx = idx / (32 * PV), within = idx % (32 * PV);
@@ -288,7 +291,9 @@ __global__ void __launch_bounds__(kThreads) col_encode_kernel(const ChanParams p
 {
     __shared__ SmemTables sm;
     constexpr int PV = SrcTraits<SRC>::kPerVec;
+    pdl_launch_dependents();
     setup_tables<true, MODE != HIF8_RND_TA, false, MODE, SRC>(sm, p.flags);
+    pdl_wait_prior_grid();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wy = (kThreads / 32) / wx, wxi = warp % wx, wyi = warp / wx;
     const long long nvc = p.cols / PV;
@@ -303,6 +308,11 @@ __global__ void __launch_bounds__(kThreads) col_encode_kernel(const ChanParams p
         scale[k] = pow2f(se);
         if (blockIdx.y == 0 && wyi == 0 && p.d_se_out) p.d_se_out[cv * PV + k] = se;
     }
+    uint32_t scale2[4] = {0u, 0u, 0u, 0u};
+    if (SRC == HIF8_BF16) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) scale2[k] = (__float_as_uint(scale[2 * k % PV]) >> 16) | (__float_as_uint(scale[(2 * k + 1) % PV]) & 0xFFFF0000u);
+    }
     const uint4* src = reinterpret_cast<const uint4*>(p.src) + cv;
     for (long long r = r0 + wyi; r < r1; r += wy * kUnroll) {
         uint4 v[kUnroll];
@@ -316,6 +326,10 @@ __global__ void __launch_bounds__(kThreads) col_encode_kernel(const ChanParams p
             const long long rr = r + wy * j;
             if (rr >= r1) continue;
             const unsigned long long flat = (unsigned long long)rr * nvc + cv;
+            if (MODE == HIF8_RND_TA) {
+                store_packed<PV>(p.dst, flat, encode_vector_ta<SRC>(v[j], scale2, scale, sm.ta));
+                continue;
+            }
             uint32_t rw[8], codes[PV];
             sr_words<MODE, PV>(flat, k0, k1, rw);
 #pragma unroll
@@ -396,22 +410,22 @@ int launch_encode(const ChanParams& p, const Plan& pl, cudaStream_t st)
         const long long nv = p.cols / SrcTraits<SRC>::kPerVec;
         if (nv > (long long)kRowCache * kThreads) {
             const unsigned grid = (unsigned)(p.rows < 0x7FFFFFFFll ? p.rows : 0x7FFFFFFFll);
-            long_row_channel_kernel<SRC, MODE><<<grid, kThreads, 0, st>>>(p);
+            launch_pdl(long_row_channel_kernel<SRC, MODE>, grid, st, p);
         } else {
-            // group size for about four vectors per thread; up to eight sets of rows per block while every SM still
-            // gets eight blocks
+            // group size for about four vectors per thread; with two register sets, as many blocks as are resident (four per SM),
+            // which take the sets of rows in turn: with two consecutive sets a block, 7168 rows of 4096 BF16 values were 3.03
+            // rounds of blocks
             int gs = kThreads;
             while (gs > 32 && nv <= (long long)(gs / 2) * kUnroll) gs >>= 1;
-            const long long sets = (p.rows + kThreads / gs - 1) / (kThreads / gs);
-            int iters = nv <= (long long)kUnroll * gs ? 8 : 1;
-            while (iters > 1 && (sets + iters - 1) / iters < (long long)pl.sms * 8) iters >>= 1;
-            const long long blocks = (sets + iters - 1) / iters;
+            const long long sets = (p.rows + kThreads / gs - 1) / (kThreads / gs), resident = (long long)pl.sms * 4;
+            const long long blocks = nv <= (long long)kUnroll * gs && sets > resident ? resident : sets;
+            const int iters = (int)((sets + blocks - 1) / blocks);
             if (blocks > 0x7FFFFFFFll) return HIF8_ERR_SHAPE;
-            if (nv <= (long long)kUnroll * gs) row_channel_kernel<SRC, MODE, kUnroll><<<(unsigned)blocks, kThreads, 0, st>>>(p, gs, iters);
-            else row_channel_kernel<SRC, MODE, kRowCache><<<(unsigned)blocks, kThreads, 0, st>>>(p, gs, iters);
+            if (nv <= (long long)kUnroll * gs) launch_pdl(row_channel_kernel<SRC, MODE, kUnroll>, (unsigned)blocks, st, p, gs, iters);
+            else launch_pdl(row_channel_kernel<SRC, MODE, kRowCache>, (unsigned)blocks, st, p, gs, iters);
         }
     } else {
-        col_encode_kernel<SRC, MODE><<<pl.grid_encode, kThreads, 0, st>>>(p, pl.rpb_encode, pl.wx);
+        launch_pdl(col_encode_kernel<SRC, MODE>, pl.grid_encode, st, p, pl.rpb_encode, pl.wx);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
@@ -433,7 +447,7 @@ template <int SRC>
 int launch_amax(const ChanParams& p, const Plan& pl, cudaStream_t st)
 {
     if (pl.vec && pl.axis == 0) return HIF8_OK;  // the row kernel reduces its own amax
-    if (pl.vec) col_amax_kernel<SRC><<<pl.grid_amax, kThreads, 0, st>>>(p, pl.rpb_amax, pl.wx);
+    if (pl.vec) launch_pdl(col_amax_kernel<SRC>, pl.grid_amax, st, p, pl.rpb_amax, pl.wx);
     else {
         const long long channels = pl.axis == 0 ? p.rows : p.cols, len = pl.axis == 0 ? p.cols : p.rows;
         // enough (channel, slice) threads to fill the device, slices of at least 64 elements

@@ -286,17 +286,13 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     // (tables under the loads' latency)
     if (kPair16) setup_sum16<MODE, kOneThreads>(sm.ta, sm.thr, p.flags);
     else setup_tables<true, MODE != HIF8_RND_TA, FQ, MODE, SRC, kOneThreads>(sm, p.flags);
-    float amax = amax_step(0.f, x_tail);
+    uint32_t acc = 0u;
 #pragma unroll
     for (int j = 0; j < kOneVecs; j++) {
         if (first + j * step < n_vec) s_src[j * kOneThreads + threadIdx.x] = v[j];
-#pragma unroll
-        for (int k = 0; k < PV; k++) {
-            float x; uint32_t raw;
-            unpack<SRC>(v[j], k, x, raw);
-            amax = amax_step(amax, x);
-        }
+        acc = amax_vector<SRC>(acc, v[j]);
     }
+    const float amax = amax_step(amax_value<SRC>(acc), x_tail);
     uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));  // non-negative floats order as integers
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = m;
     __syncthreads();
@@ -601,6 +597,7 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     const uint4* src = reinterpret_cast<const uint4*>(srcv);
     float amax = 0.f;
+    uint32_t acc = 0u;
     pdl_launch_dependents();
     pdl_wait_prior_grid();
     const unsigned long long stride = (unsigned long long)gridDim.x * kThreads * kUnrollAmax;
@@ -612,15 +609,9 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__
             v[j] = (u < n_vec) ? __ldg(src + u) : make_uint4(0, 0, 0, 0);  // default policy: keep lines for the second pass
         }
 #pragma unroll
-        for (int j = 0; j < kUnrollAmax; j++) {
-#pragma unroll
-            for (int k = 0; k < PV; k++) {
-                float x; uint32_t raw;
-                unpack<SRC>(v[j], k, x, raw);
-                amax = amax_step(amax, x);
-            }
-        }
+        for (int j = 0; j < kUnrollAmax; j++) acc = amax_vector<SRC>(acc, v[j]);
     }
+    amax = amax_value<SRC>(acc);
     const unsigned long long tid = (unsigned long long)blockIdx.x * kThreads + threadIdx.x;
     for (unsigned long long i = n_vec * PV + tid; i < n; i += (unsigned long long)gridDim.x * kThreads) {
         float x; uint32_t raw;

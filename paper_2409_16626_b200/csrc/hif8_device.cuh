@@ -313,6 +313,47 @@ __device__ __forceinline__ void put_signs(const uint4& v, uint32_t& w0, uint32_t
     }
 }
 
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// Two BF16 elements at once: the packed product with a power of two is exact down to 2^-126 (far below half of 2^-22), and its
+// upper twelve magnitude bits are the table's index.  Magnitude codes in bytes 0 and 1; scale2: the scale as two BF16 values.
+__device__ __forceinline__ uint32_t ta_magnitude_codes_bf16x2(uint32_t w, uint32_t scale2, const uint8_t* s_ta)
+{
+    const uint32_t y = mul_bf16x2(w & 0x7FFF7FFFu, scale2);
+    return (uint32_t)s_ta[(y >> 3) & 0xFFFu] | ((uint32_t)s_ta[y >> 19] << 8);
+}
+__device__ __forceinline__ uint32_t bf16x2_of_pow2(float scale) { return (__float_as_uint(scale) >> 16) * 0x00010001u; }
+
+// A source vector under round half away: codes of its elements, packed (w1 only for 16-bit sources).  BF16: one scale per word
+// of two elements; FP32 and FP16: one per element.
+template <int SRC>
+__device__ __forceinline__ uint2 encode_vector_ta(const uint4& v, const uint32_t* scale2, const float* scale, const uint8_t* s_ta)
+{
+    constexpr int PV = SrcTraits<SRC>::kPerVec;
+    uint32_t w0, w1 = 0u;
+    if (SRC == HIF8_BF16) {
+        w0 = ta_magnitude_codes_bf16x2(v.x, scale2[0], s_ta) | (ta_magnitude_codes_bf16x2(v.y, scale2[1], s_ta) << 16);
+        w1 = ta_magnitude_codes_bf16x2(v.z, scale2[2], s_ta) | (ta_magnitude_codes_bf16x2(v.w, scale2[3], s_ta) << 16);
+    } else {
+        uint32_t c[8];
+#pragma unroll
+        for (int k = 0; k < PV; k++) {
+            float x; uint32_t raw;
+            unpack<SRC>(v, k, x, raw);
+            c[k] = ta_magnitude_code(x, scale[k], s_ta);
+        }
+        w0 = c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24);
+        if (PV == 8) w1 = c[4] | (c[5] << 8) | (c[6] << 16) | (c[7] << 24);
+    }
+    put_signs<SRC>(v, w0, w1);
+    return make_uint2(w0, w1);
+}
+
 template <int MODE, int SRC>
 __device__ __forceinline__ uint32_t encode_one(float x, uint32_t raw, float scale, const uint8_t* s_ta,
                                                const uint32_t* s_thr, uint32_t word)
@@ -423,13 +464,6 @@ __device__ __forceinline__ void setup_sum16(uint8_t* code8, uint32_t* inck, unsi
 
 // the negated power-of-two scale as two BF16 values
 __device__ __forceinline__ uint32_t neg_scale_bf16x2(float scale) { return (0x8000u | (__float_as_uint(scale) >> 16)) * 0x00010001u; }
-
-__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b)
-{
-    uint32_t d;
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
 
 __device__ __forceinline__ uint32_t fma_bf16x2(uint32_t a, uint32_t b, uint32_t c)
 {
@@ -586,6 +620,34 @@ __device__ __forceinline__ int resolve_scale_exp(const ConvParams& p)
 // amax contribution of a value: |x| for finite x, ignored (NaN) otherwise; fmaxf drops NaN operands
 __device__ __forceinline__ float amax_step(float acc, float x) { return fmaxf(acc, fmaf(x, 0.0f, fabsf(x))); }
 
+// The same over whole source words.  16-bit sources stay packed, two running maxima in a word: |x| + 0 * |x| is |x| for finite
+// x and NaN otherwise, and the maximum drops NaN operands; 1.5 instructions an element where widening each took 3.5.
+template <int SRC> __device__ __forceinline__ uint32_t amax_word(uint32_t acc, uint32_t w)
+{
+    if (SRC == HIF8_F32) return __float_as_uint(amax_step(__uint_as_float(acc), __uint_as_float(w)));
+    const uint32_t a = w & 0x7FFF7FFFu;
+    uint32_t t, d;
+    if (SRC == HIF8_BF16) {
+        asm("fma.rn.bf16x2 %0, %1, %2, %1;" : "=r"(t) : "r"(a), "r"(0u));
+        asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(acc), "r"(t));
+    } else {
+        asm("fma.rn.f16x2 %0, %1, %2, %1;" : "=r"(t) : "r"(a), "r"(0u));
+        asm("max.f16x2 %0, %1, %2;" : "=r"(d) : "r"(acc), "r"(t));
+    }
+    return d;
+}
+template <int SRC> __device__ __forceinline__ uint32_t amax_vector(uint32_t acc, const uint4& v)
+{
+    return amax_word<SRC>(amax_word<SRC>(amax_word<SRC>(amax_word<SRC>(acc, v.x), v.y), v.z), v.w);
+}
+// ... and their value (finite, non-negative)
+template <int SRC> __device__ __forceinline__ float amax_value(uint32_t acc)
+{
+    if (SRC == HIF8_F32) return __uint_as_float(acc);
+    if (SRC == HIF8_BF16) return fmaxf(__uint_as_float(acc << 16), __uint_as_float(acc & 0xFFFF0000u));
+    return fmaxf(__half2float(__ushort_as_half((unsigned short)(acc & 0xFFFFu))), __half2float(__ushort_as_half((unsigned short)(acc >> 16))));
+}
+
 __device__ __forceinline__ void block_amax_commit(float acc, uint32_t* accum)
 {
     __shared__ uint32_t s_part[kThreads / 32];
@@ -601,10 +663,10 @@ __device__ __forceinline__ void block_amax_commit(float acc, uint32_t* accum)
 
 // launch with programmatic stream serialization (see pdl_* above)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, cudaStream_t st, Args... args)
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
