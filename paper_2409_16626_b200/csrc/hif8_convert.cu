@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const ConvParams p, u
 
 // ------------------------------------------------------------------------------------------------
 // Just-in-time scaling of a small tensor in one launch: a cluster of up to eight blocks holds the source in shared memory,
-// reduces its amax (each block tells the others its own through distributed shared memory, one cluster barrier), and converts
-// from there.  No accumulator in the workspace, so nothing to clear.  Latency and launches bound it: the three launches of the
+// reduces its amax (each block tells the others its own through distributed shared memory, between two cluster barriers, the
+// first of which completes under the loads and the table set-up), and converts from there.  No accumulator in the workspace, so nothing to clear.  Latency and launches bound it: the three launches of the
 // general path (clear, amax, convert) take 3.3 us on the device and 8 us from the host, this 2.3 us and 4 us (512 BF16
 // elements, round half away); 3.9 against 3.1 us at 131072.  The limits are where eight blocks take as long on the device as
 // three launches over all SMs: 256 KiB of source, half of that for dequantized results, which carry more arithmetic
@@ -270,6 +270,7 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     __shared__ uint32_t s_part[kOneThreads / 32], s_block[kOneBlocks];
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     constexpr bool kPair16 = SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ;
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this block has started (waited for before the first remote store)
     pdl_launch_dependents();
     const unsigned first = blockIdx.x * kOneThreads + threadIdx.x, step = gridDim.x * kOneThreads;  // vectors first, first + step, ..
     pdl_wait_prior_grid();
@@ -296,6 +297,7 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));  // non-negative floats order as integers
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = m;
     __syncthreads();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every block of the cluster has started: its shared memory may be written
     if (threadIdx.x < 32) {
         m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kOneThreads / 32 ? s_part[threadIdx.x] : 0u);
         if (threadIdx.x < gridDim.x) {
