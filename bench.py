@@ -12,7 +12,8 @@ figure from profiler counters beside it, and `roofline` describes single kernels
   python bench.py --case NAME [--reps R]        one named workload a few times, for use under a profiler
 
 N > 1 is launched under torch.distributed.run, one rank per GPU; ranks convert independent tensors (no
-data-path collective, weak scaling) and rank 0 prints the single JSON line.
+data-path collective, weak scaling) and rank 0 prints the single JSON line.  Everything measured beside the headline (single
+kernels, other workloads, products) goes to standard error, as one JSON line with the same keys and more.
 `--impl reference` times the CPU oracle (oracle/) on a bounded sample of the same workload.
 """
 import argparse
@@ -134,6 +135,22 @@ def repeats_for(region_ms):
     """How often a timed region is repeated: at least MIN_REPEATS, more for short regions (about half a second of
     device time in all, so that the clock sampler sees the run), never more than 200."""
     return int(min(200, max(MIN_REPEATS, 500.0 / max(region_ms, 1e-3))))
+
+
+HEADLINE_CONFIG = ("workload", "elements", "rounding", "target_exp", "launch", "timed", "ms_per_step_best", "ms_per_step_worst",
+                   "ms_per_step_single_stream", "l2", "bytes_per_step", "elements_per_s")
+HEADLINE_ROOFLINE = ("bound", "kernel", "achieved", "peak", "peak_kind", "unit", "frac", "algorithmic_bytes_per_launch", "avg_launch_ms")
+
+
+def headline(line):
+    """What rank 0 prints on standard output: the measured step and how it was taken, without the tables of other workloads
+    (a few thousand characters at most, so that a reader of the last lines of a log has it whole)."""
+    short = {k: v for k, v in line.items() if k not in ("kernels", "calls", "extra", "sharded")}
+    short["config"] = {k: line["config"][k] for k in HEADLINE_CONFIG}
+    short["roofline"] = {k: line["roofline"][k] for k in HEADLINE_ROOFLINE}
+    if "cpu_baseline" in line:
+        short["cpu_baseline"] = {k: v for k, v in line["cpu_baseline"].items() if not isinstance(v, dict)}
+    return short
 
 
 def load_peaks():
@@ -977,7 +994,8 @@ def main():
             by_config.update(table)
         if world == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_baseline(1 << 23)
-        print(json.dumps(line))
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 

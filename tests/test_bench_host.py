@@ -51,3 +51,23 @@ def test_reference_arm_prints_contract_line_and_other_ranks_stay_silent():
     p = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--steps", "1"],
                        capture_output=True, text=True, env=env1, timeout=600)
     assert p.returncode == 0 and p.stdout.strip() == ""
+
+
+def test_headline_is_short_and_whole():
+    """Standard output carries the contract's keys in a line that a bounded tail of a log holds; tables of any size stay out."""
+    import bench
+    table = {f"workload_{i}": {"ms": 1.0 / 3.0, "note": "x" * 200} for i in range(100)}
+    text = "x" * 130
+    line = {"metric": bench.METRIC, "value": 7000.0 / 3, "unit": "GB/s", "n_gpus": 1, "steps": 20, "warmup": 5, "ms_per_step": 0.1 / 3,
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u8", "data": "synthetic",
+            "config": dict({k: text for k in bench.HEADLINE_CONFIG}, step_dram=table),
+            "clocks": {"sm_mhz": 1965.0, "sm_max_mhz": 1965, "reasons": ["sw_power_cap"], "samples": 100},
+            "e2e": {"value": 100.0 / 3, "unit": "GB/s", "ms_per_step": 1.7 / 3, "h2d_bytes_per_step": 1 << 26, "d2h_bytes_per_step": 5 << 24},
+            "gpu_launches": 80, "roofline": dict({k: 1.0 / 3 for k in bench.HEADLINE_ROOFLINE}, by_config=table),
+            "cpu_baseline": {"value": 0.07, "unit": "GB/s", "cores": 16, "kind": "oracle", "sample": text, "elements_per_s": 1e7 / 3, "legs": table},
+            "kernels": table, "calls": table, "extra": table, "sharded": table}
+    short = bench.headline(line)
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype",
+                "data", "clocks", "e2e", "gpu_launches"):
+        assert short[key] == line[key]
+    assert short["cpu_baseline"]["value"] == 0.07 and short["config"]["workload"] == text and len(json.dumps(short)) < 3800
