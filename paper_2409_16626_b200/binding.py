@@ -12,6 +12,8 @@ import os
 
 import torch
 
+from .build import CALL as CALL_PATH
+
 F32, BF16, F16 = 0, 1, 2
 RND_TA, RND_HR, RND_SSR, RND_TE, RND_SR = 0, 1, 2, 3, 4
 FLAG_SATURATE, FLAG_NAN_TO_ZERO = 1, 2
@@ -27,12 +29,15 @@ EXPORTS = ["hif8_encode", "hif8_decode", "hif8_amax", "hif8_amax_scale_encode", 
            "hif8_scale_state_init", "hif8_delayed_scale_encode", "hif8_gemm_ex", "hif8_encode_transpose", "hif8_als_state_init", "hif8_als_update", "hif8_check_finite", "hif8_encode_from_amax",
            "hif8_amax_scale_encode_static", "hif8_encode_f32_patterns", "hif8_last_device_status", "hif8_selftest_host_caches", "hif8_gemm_path_policy", "hif8_workspace_bytes", "hif8_status_string", "hif8_launch_count"]
 
-if not os.path.exists(LIB_PATH):
-    raise ImportError(f"{LIB_PATH} is missing: run `python -m paper_2409_16626_b200.build` (needs nvcc)")
+for _path in (LIB_PATH, CALL_PATH):
+    if not os.path.exists(_path):
+        raise ImportError(f"{_path} is missing: run `python -m paper_2409_16626_b200.build` (needs nvcc and g++)")
 lib = C.CDLL(LIB_PATH)
 from . import _hif8_call as _c  # noqa: E402  (linked against the library above)
 
-_c.set_up(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+if hasattr(torch._C, "_cuda_getDevice") and hasattr(torch._C, "_cuda_getCurrentRawStream"):
+    # (a torch without CUDA has neither; then the flag below stays off and streams are always asked for through torch)
+    _c.set_up(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
 os.register_at_fork(after_in_child=lambda: _c.set_cuda_ready(False))
 
 _vp, _sz, _i, _u, _u64, _i64 = C.c_void_p, C.c_size_t, C.c_int, C.c_uint, C.c_uint64, C.c_int64
@@ -306,4 +311,4 @@ def hif8_encode_from_amax(src, src_dtype, dst, n, target_exp, rnd, flags, seed, 
 
 
 # the names that the package itself offers (see the package's __getattr__)
-PUBLIC = frozenset(n for n in globals() if not n.startswith("_") and n not in ("C", "lib", "os", "torch"))
+PUBLIC = frozenset(n for n in globals() if not n.startswith("_") and n not in ("C", "CALL_PATH", "lib", "os", "torch"))

@@ -9,7 +9,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhif8.so")
-CALL_SRC, CALL = os.path.join(CSRC, "hif8_call.cpp"), os.path.join(HERE, "_hif8_call.so")
+# (named for the interpreter it is built against, so that another one does not load it)
+CALL_SRC, CALL = os.path.join(CSRC, "hif8_call.cpp"), os.path.join(HERE, "_hif8_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 CXX = os.environ.get("CXX", "g++")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -45,6 +46,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB] + objs + ["-lcudart"])
     subprocess.check_call([CXX, "-O2", "-std=c++17", "-Wall", "-fPIC", "-shared", "-I" + os.path.join(ROOT, "include"),
                            "-I" + sysconfig.get_paths()["include"], CALL_SRC, "-o", CALL, "-L" + HERE, "-l:libhif8.so", "-Wl,-rpath,$ORIGIN"])
+    untagged = os.path.join(HERE, "_hif8_call.so")
+    if untagged != CALL and os.path.exists(untagged):  # any interpreter would load that one
+        os.remove(untagged)
     return LIB
 
 

@@ -1,6 +1,11 @@
 """The CPython entry (csrc/hif8_call.cpp) against the same calls through ctypes, on the CPU: argument errors are found
 before anything touches a device, so status codes and exceptions can be compared without one."""
 import ctypes
+import os
+import shutil
+import subprocess
+import sys
+import sysconfig
 
 import pytest
 
@@ -70,6 +75,36 @@ def test_other_arguments_are_reported_by_ctypes(bad):
 def test_current_stream_is_left_to_torch_before_initialisation():
     call.set_cuda_ready(False)
     assert call.hif8_encode(A, 0, B, 0, 0, 0, 0, 0, None) is None
+
+
+PACKAGE = os.path.dirname(os.path.abspath(binding.__file__))
+
+
+def import_elsewhere(tmp_path, files, before=""):
+    """`import paper_2409_16626_b200.binding` of a copy that has only these built files, in a process of its own."""
+    copy = tmp_path / "paper_2409_16626_b200"
+    copy.mkdir()
+    for f in ["__init__.py", "binding.py", "build.py"] + files:
+        shutil.copy(os.path.join(PACKAGE, f), copy)
+    code = before + "import paper_2409_16626_b200 as H, ctypes; print(H.hif8_workspace_bytes(H.WS_GEMM, 0), H.hif8_encode(65536, 7, 131072, 16, stream=0, check=False))"
+    return subprocess.run([sys.executable, "-c", code], cwd=tmp_path, capture_output=True, text=True, timeout=300)
+
+
+def test_entry_is_named_for_its_interpreter():
+    tag = sysconfig.get_config_var("EXT_SUFFIX")
+    assert os.path.basename(call.__file__) == "_hif8_call" + tag and tag != ".so" and not os.path.exists(os.path.join(PACKAGE, "_hif8_call.so"))
+
+
+def test_missing_entry_says_how_to_build_it(tmp_path):
+    p = import_elsewhere(tmp_path, ["libhif8.so"])
+    assert p.returncode != 0 and "ImportError" in p.stderr and "paper_2409_16626_b200.build" in p.stderr
+
+
+def test_import_with_a_torch_without_cuda(tmp_path):
+    p = import_elsewhere(tmp_path, ["libhif8.so", os.path.basename(call.__file__)],
+                         "import torch; del torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream\n")
+    assert p.returncode == 0, p.stderr
+    assert p.stdout.split() == ["256", "2"]
 
 
 def test_errors_and_check():
