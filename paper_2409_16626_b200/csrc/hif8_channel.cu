@@ -113,7 +113,7 @@ __device__ __forceinline__ uint32_t group_max(uint32_t v, uint32_t* s_part, int 
 }
 
 // Rows that fit in registers (at most NV vectors per thread of a group of gs threads).  A block works through
-// `iters` sets of kThreads / gs rows, one grid apart; the loads of the next set are issued before the current one is
+// `iters` consecutive sets of kThreads / gs rows; the loads of the next set are issued before the current one is
 // reduced and converted, so every row is read exactly once and the memory latency is covered by the arithmetic of the
 // previous row.  Short rows get small groups so that a thread still holds about four vectors.
 template <int SRC, int MODE, int NV>
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
     const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
     const int groups = kThreads / gs, g = threadIdx.x / gs, t = threadIdx.x % gs;
     const uint4* base = reinterpret_cast<const uint4*>(p.src);
-    const long long first = (long long)blockIdx.x * groups + g, step = (long long)gridDim.x * groups;
+    const long long first = (long long)blockIdx.x * iters * groups + g;
 
     // NV <= kUnroll: two register sets, the next row is in flight while this one is processed; larger rows use one set
     constexpr bool kPrefetch = NV <= kUnroll;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
         }
     }
     for (int it = 0; it < iters; it++) {
-        const long long row = first + (long long)it * step, row_next = row + step;
+        const long long row = first + (long long)it * groups, row_next = row + groups;
         const bool live = row < p.rows;  // a group past the last row only takes part in the barriers
         if (kPrefetch) {
 #pragma unroll
@@ -412,14 +412,14 @@ int launch_encode(const ChanParams& p, const Plan& pl, cudaStream_t st)
             const unsigned grid = (unsigned)(p.rows < 0x7FFFFFFFll ? p.rows : 0x7FFFFFFFll);
             launch_pdl(long_row_channel_kernel<SRC, MODE>, grid, st, p);
         } else {
-            // group size for about four vectors per thread; with two register sets, as many blocks as are resident (four per SM),
-            // which take the sets of rows in turn: with two consecutive sets a block, 7168 rows of 4096 BF16 values were 3.03
-            // rounds of blocks
+            // group size for about four vectors per thread; up to eight sets of rows per block while every SM still
+            // gets eight blocks
             int gs = kThreads;
             while (gs > 32 && nv <= (long long)(gs / 2) * kUnroll) gs >>= 1;
-            const long long sets = (p.rows + kThreads / gs - 1) / (kThreads / gs), resident = (long long)pl.sms * 4;
-            const long long blocks = nv <= (long long)kUnroll * gs && sets > resident ? resident : sets;
-            const int iters = (int)((sets + blocks - 1) / blocks);
+            const long long sets = (p.rows + kThreads / gs - 1) / (kThreads / gs);
+            int iters = nv <= (long long)kUnroll * gs ? 8 : 1;
+            while (iters > 1 && (sets + iters - 1) / iters < (long long)pl.sms * 8) iters >>= 1;
+            const long long blocks = (sets + iters - 1) / iters;
             if (blocks > 0x7FFFFFFFll) return HIF8_ERR_SHAPE;
             if (nv <= (long long)kUnroll * gs) launch_pdl(row_channel_kernel<SRC, MODE, kUnroll>, (unsigned)blocks, st, p, gs, iters);
             else launch_pdl(row_channel_kernel<SRC, MODE, kRowCache>, (unsigned)blocks, st, p, gs, iters);

@@ -102,6 +102,55 @@ def test_channel_encode_given_exponents_and_odd_layouts(dtype, axis):
         assert np.array_equal(q2, O.channel_encode(x, dtype, axis, se_o, quick=True))
 
 
+@pytest.mark.parametrize("flags", [0, H.FLAG_SATURATE | H.FLAG_NAN_TO_ZERO])
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("dtype", [H.BF16, H.F16])
+def test_channel_encode_every_16_bit_pattern_at_extreme_exponents(dtype, axis, flags):
+    # the exponents go round the channels, one further on with each shift: each pattern meets each exponent
+    x = np.arange(65536, dtype=np.uint16).reshape(256, 256)
+    exps = np.array([0, -126, 126, 14, -22, 126, 1, -126, 63, -64, 7], dtype=np.int32)
+    for shift in range(len(exps)):
+        given = exps[(np.arange(256) + shift) % len(exps)]
+        q, _, se = run_channel(x, dtype, axis, given=given, flags=flags)
+        assert np.array_equal(se, given)
+        assert np.array_equal(q, O.channel_encode(x, dtype, axis, given, flags=flags, quick=True)), shift
+
+
+def test_channel_calls_replay_from_a_cuda_graph():
+    # rows (one launch), columns (a memset node in front of two launches with programmatic serialization) and the element-wise
+    # path, captured into one graph and replayed on new contents
+    shapes = [((300, 520), 0), ((300, 520), 1), ((70, 131), 1)]
+    src = [torch.empty(r * c, dtype=torch.int16, device="cuda") for (r, c), _ in shapes]
+    dst = [torch.empty(r * c, dtype=torch.uint8, device="cuda") for (r, c), _ in shapes]
+    amax = [torch.full((s[ax],), -1.0, device="cuda") for s, ax in shapes]
+    exps = [torch.full((s[ax],), 77, dtype=torch.int32, device="cuda") for s, ax in shapes]
+
+    def calls():
+        for i, ((r, c), ax) in enumerate(shapes):
+            H.hif8_channel_amax_scale_encode(src[i], H.BF16, dst[i], r, c, ax, 14, H.RND_TA, 0, 0, None, amax[i], exps[i])
+
+    def load(seed):
+        xs = [weight(r, c, seed=seed + i, dtype=H.BF16) for i, ((r, c), _) in enumerate(shapes)]
+        for t, x in zip(src, xs):
+            t.copy_(torch.from_numpy(x.reshape(-1).view(np.int16)))
+        return xs
+
+    load(1)
+    calls()                                                   # eager first: one-time set-up happens outside the capture
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        calls()
+    for seed in (20, 40):
+        xs = load(seed)
+        g.replay()
+        torch.cuda.synchronize()
+        for i, ((r, c), ax) in enumerate(shapes):
+            amax_o, se_o = O.channel_amax_scale(xs[i], H.BF16, ax, 14)
+            assert np.array_equal(amax[i].cpu().numpy(), amax_o) and np.array_equal(exps[i].cpu().numpy(), se_o)
+            assert np.array_equal(dst[i].cpu().numpy().reshape(r, c), O.channel_encode(xs[i], H.BF16, ax, se_o, quick=True))
+
+
 def test_channel_encode_degenerate_shapes():
     d_amax = torch.full((5,), -1.0, device="cuda")
     d_se = torch.full((5,), 9, dtype=torch.int32, device="cuda")
