@@ -69,12 +69,13 @@ template <int MODE, int PV> __device__ __forceinline__ void sr_words(unsigned lo
     rw[0] = r0.x; rw[1] = r0.y; rw[2] = r0.z; rw[3] = r0.w; rw[4] = r1.x; rw[5] = r1.y; rw[6] = r1.z; rw[7] = r1.w;
 }
 
-// One vector of a row: round half away through packed words, the other modes element by element.
+// One vector of a row: BF16 under round half away through packed words, the rest element by element (FP16, 28672 x 8192: 125 us a call
+// through packed words, 118 us so).
 template <int SRC, int MODE> __device__ __forceinline__ void encode_row_vector(const ChanParams& p, const SmemTables& sm, const uint4& v, unsigned long long flat,
                                                                                float scale, uint32_t k0, uint32_t k1)
 {
     constexpr int PV = SrcTraits<SRC>::kPerVec;
-    if (MODE == HIF8_RND_TA) {
+    if (MODE == HIF8_RND_TA && SRC == HIF8_BF16) {
         const uint32_t s2 = bf16x2_of_pow2(scale);
         const uint32_t scales2[4] = {s2, s2, s2, s2};
         const float scales[8] = {scale, scale, scale, scale, scale, scale, scale, scale};
