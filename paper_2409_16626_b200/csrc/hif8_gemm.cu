@@ -24,6 +24,7 @@
 #include <cstdint>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "hif8.h"
 #include "hif8_host_cache.h"
@@ -1167,10 +1168,13 @@ struct TilePlan {
 };
 
 // Eight finished sums of this thread's weight column, activation rows m .. m + 7 of which `rows` exist, to C: `out` is the
-// place of the first, `pitch` the bytes from row to row (below 2^32: more than 64 rows fit in memory).  For one row a warp
-// writes 32 consecutive columns.  Issue slots bound this: with two scale factors, 64-bit row addresses and a test per row
-// the epilogue of a 256 x 256 tile took 5300 cycles, 19 instructions a store.
-__device__ __forceinline__ void store_columns(unsigned char* out, uint32_t pitch, int is_f32, int accumulate, int rows, float (&v)[8])
+// place of the first, `pitch` the bytes from row to row.  For one row a warp writes 32 consecutive columns.  Issue slots bound
+// this: with two scale factors, 64-bit row addresses and a test per row the epilogue of a 256 x 256 tile took 5300 cycles, 19
+// instructions a store.  So the pitch has 32 bits, one multiply-add per row, unless rows lie 4 GiB apart or more (a few rows of
+// a large buffer): that is an instantiation of its own, since 64-bit products for all cost 1 % (4096 x 28672 x 8192 with
+// expanded activations: 1320 -> 1352 us).
+template <typename Pitch>
+__device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, int is_f32, int accumulate, int rows, float (&v)[8])
 {
     auto at = [&](int i) { return out + (unsigned long long)pitch * (uint32_t)i; };
     if (accumulate) {
@@ -1206,7 +1210,8 @@ __device__ __forceinline__ void store_columns(unsigned char* out, uint32_t pitch
     }
 }
 
-template <bool W_IS_NK, int ACT>
+// FAR: the rows of C lie 4 GiB apart or more
+template <bool W_IS_NK, int ACT, bool FAR>
 __global__ void __launch_bounds__(kThreadsWd, 1)
 hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_act, const GemmParams p, const TilePlan tp)
 {
@@ -1529,7 +1534,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
 #pragma unroll
                     for (int i = 0; i < 8; i++) v[i] *= f2;
                 }
-                if (n < p.N) store_columns(out + j * 8 * pitch, (uint32_t)pitch, p.c_is_f32, p.accumulate, cols - j * 8, v);
+                if (n < p.N) store_columns(out + j * 8 * pitch, (std::conditional_t<FAR, unsigned long long, uint32_t>)pitch, p.c_is_f32, p.accumulate, cols - j * 8, v);
             }
             tc_fence_before();
             __syncwarp();
@@ -1994,12 +1999,15 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
         std::memset(out->wd_clusters, 0, sizeof out->wd_clusters);
         std::memset(out->nw_clusters, 0, sizeof out->nw_clusters);
         const void* pair[2] = {(const void*)bf16_gemm_pair_kernel<false>, (const void*)bf16_gemm_pair_kernel<true>};
-        const void* wd[6] = {(const void*)hif8_gemm_weights_kernel<false, kActExpanded>, (const void*)hif8_gemm_weights_kernel<true, kActExpanded>,
-                             (const void*)hif8_gemm_weights_kernel<false, kActRows>, (const void*)hif8_gemm_weights_kernel<true, kActRows>,
-                             (const void*)hif8_gemm_weights_kernel<false, kActColumns>, (const void*)hif8_gemm_weights_kernel<true, kActColumns>};
+        const void* wd[12] = {(const void*)hif8_gemm_weights_kernel<false, kActExpanded, false>, (const void*)hif8_gemm_weights_kernel<true, kActExpanded, false>,
+                              (const void*)hif8_gemm_weights_kernel<false, kActRows, false>, (const void*)hif8_gemm_weights_kernel<true, kActRows, false>,
+                              (const void*)hif8_gemm_weights_kernel<false, kActColumns, false>, (const void*)hif8_gemm_weights_kernel<true, kActColumns, false>,
+                              (const void*)hif8_gemm_weights_kernel<false, kActExpanded, true>, (const void*)hif8_gemm_weights_kernel<true, kActExpanded, true>,
+                              (const void*)hif8_gemm_weights_kernel<false, kActRows, true>, (const void*)hif8_gemm_weights_kernel<true, kActRows, true>,
+                              (const void*)hif8_gemm_weights_kernel<false, kActColumns, true>, (const void*)hif8_gemm_weights_kernel<true, kActColumns, true>};
         for (int i = 0; i < 2 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(pair[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2);
-        for (int i = 0; i < 6 && out->rc == cudaSuccess; i++)
+        for (int i = 0; i < 12 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(wd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
         for (int s = 1; s <= kWdMaxSplit && out->rc == cudaSuccess; s *= 2) {
             cudaLaunchConfig_t cfg{};
@@ -2162,8 +2170,11 @@ template <int ACT>
 static cudaError_t launch_weights_kernel(const cudaLaunchConfig_t& cfg, int w_is_nk, const CUtensorMap& map_w, const CUtensorMap& map_act, const GemmParams& p,
                                          const TilePlan& tp)
 {
-    return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true, ACT>, map_w, map_act, p, tp)
-                   : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false, ACT>, map_w, map_act, p, tp);
+    if ((p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32)
+        return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true, ACT, true>, map_w, map_act, p, tp)
+                       : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false, ACT, true>, map_w, map_act, p, tp);
+    return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true, ACT, false>, map_w, map_act, p, tp)
+                   : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false, ACT, false>, map_w, map_act, p, tp);
 }
 
 // C = A W with the weights decoded inside the kernel.  act = kActExpanded: `a` is BF16 [M,K], written by the launch in front of

@@ -231,3 +231,33 @@ def test_gemm_ex_argument_checks():
     assert H.hif8_gemm_ex(A, 64, 1, A, 64, 0, C, 64, 5, 64, 64, 64, **ok) == 2
     assert H.hif8_gemm_ex(A, 64, 1, A, 64, 0, C, 64, H.F32, 64, 64, 64, workspace=None, workspace_bytes=0, check=False) == 8
     assert H.hif8_gemm_ex(A, 64, 1, A, 64, 0, C, 64, H.F32, 0, 64, 64, **ok) == 0     # empty output
+
+
+@pytest.mark.parametrize("c_dtype,accumulate", [(H.F32, 0), (H.F32, 1), (H.BF16, 0), (H.BF16, 1)])
+def test_gemm_ex_rows_of_c_more_than_4_gib_apart(c_dtype, accumulate):
+    # few activation rows given as [K,M]: C may be a strided view of a large buffer, a row pitch needs 64 bits
+    M, N, K, lda = 9, 24, 32, 16
+    ldc = (2 ** 32 + 64) // (4 if c_dtype == H.F32 else 2)
+    if torch.cuda.mem_get_info()[0] < 48 << 30:
+        pytest.skip("needs 35 GiB of device memory")
+    Amk, Wkn = codes((M, K), 11), codes((K, N), 12)
+    A = np.zeros((K, lda), dtype=np.uint8)
+    A[:, :M] = Amk.T
+    Wq = np.pad(Wkn, ((0, 0), (0, 8)))
+    buf = torch.empty((M - 1) * ldc + N, dtype=torch.float32 if c_dtype == H.F32 else torch.bfloat16, device="cuda")
+    C = torch.as_strided(buf, (M, N), (ldc, 1))
+    C.copy_(torch.from_numpy((np.random.default_rng(1).standard_normal((M, N)) * 50).astype(np.float32)))
+    c0 = C.float().cpu().numpy().astype(np.float64)
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    H.hif8_gemm_ex(to_dev(A), lda, 1, to_dev(Wq), N + 8, 0, buf, ldc, c_dtype, M, N, K, None, None, None, accumulate, ws, 256)
+    assert H.hif8_gemm_status(ws) == 0
+    out = C.float().cpu().numpy().astype(np.float64)
+    del buf, C
+    torch.cuda.empty_cache()
+    rows, cols = np.divmod(np.arange(M * N), N)
+    P, S = O.gemm_entries_ex(A, 1, Wkn, 0, 0, 0, rows, cols)
+    want = P.reshape(M, N) + (c0 if accumulate else 0.0)
+    tol = 1e-5 * S.reshape(M, N) + 2.0 ** -24 * np.abs(want)
+    if c_dtype == H.BF16:
+        tol = tol + bf16_half_ulp(np.abs(want) + tol)
+    assert np.all(np.abs(out - want) <= tol)
