@@ -384,7 +384,7 @@ __device__ __forceinline__ uint4 decode8(uint2 v, uint32_t lut_lane)
 
 __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int& tile_m, int& tile_n)
 {
-    constexpr int kGroupM = 8;  // groups of 8 tile-rows sweep N together: their W tiles stay in L2
+    constexpr int kGroupM = 8;  // groups of 8 tile-rows sweep N together: their W tiles stay in L2 (kGroupPieces is the same number)
     const int per_group = kGroupM * tiles_n;
     const int g = t / per_group, first_m = g * kGroupM;
     const int rows_in_group = min(kGroupM, tiles_m - first_m);
@@ -1162,7 +1162,11 @@ static_assert((kWdMaxSplit - 1) * (BN / kWdMaxSplit) * BM * 4 <= 2 * kWdStages *
 
 struct TilePlan {
     int first, count;  // tiles [first, first + count) of the product
-    int chunks, bn;    // activation rows in `chunks` pieces of bn (a multiple of 32); tile t = weight slab t / chunks, piece t % chunks
+    int chunks, bn;    // activation rows in `chunks` pieces of bn (a multiple of 32)
+    // Tiles in groups of eight pieces that sweep the `slabs` of 256 weight columns together (tile_coords).  Slab by slab, with 32
+    // pieces one round of 74 tiles read all of the activations: 8192 x 28672 x 8192 with expanded activations (134 MB, more than
+    // L2 holds) 2905 us, in groups 2614 to 2636.
+    int slabs;
     int split;
     int clear_status;  // nonzero: no launch in front of this one clears the status word
 };
@@ -1210,8 +1214,11 @@ __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, i
     }
 }
 
-// FAR: the rows of C lie 4 GiB apart or more
-template <bool W_IS_NK, int ACT, bool FAR>
+// Instantiations by tile order and row pitch.  (With the choice of the order made in the kernel, its divisions in everybody's way,
+// 128 x 512 x 512 took 10.0 us instead of 9.8.)
+enum WeightsForm { kOneGroup, kGroups, kFarRows };  // up to eight pieces; more; the rows of C 4 GiB apart or more (any number of pieces)
+constexpr int kGroupPieces = 8;
+template <bool W_IS_NK, int ACT, int FORM>
 __global__ void __launch_bounds__(kThreadsWd, 1)
 hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_act, const GemmParams p, const TilePlan tp)
 {
@@ -1252,14 +1259,24 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     // ---- set-up.  A call of a small product is mostly latency: the first weight copies go out under the table set-up, and only
     // what touches the other CTAs waits for the cluster (its barrier takes 1400 to 1900 cycles from the start of the kernel,
     // in which a first k-block is copied and decoded).
+    auto place = [&](int t, int& slab, int& m0) {  // tile t: its weight slab and its first activation row
+        int piece;
+        if (FORM == kOneGroup) {
+            slab = t / tp.chunks;
+            piece = t - slab * tp.chunks;
+        } else tile_coords(t, tp.chunks, tp.slabs, piece, slab);
+        m0 = piece * tp.bn;
+    };
     auto copy_bytes = [&](int it, int t, int kb) {  // tile t's bytes of k-block kb into stage it % kWdStages, which is free
-        const int s = it % kWdStages, slab = t / tp.chunks, n0 = slab * 2 * BM + (int)half * BM;
+        int slab, m0;
+        place(t, slab, m0);
+        const int s = it % kWdStages, n0 = slab * 2 * BM + (int)half * BM;
         const uint32_t dst = lay.u8(s), bar = bar_u8_full(s);
         mbar_arrive_expect_tx(bar, Smem::kW8 + (ACT == kActExpanded ? 0u : (uint32_t)(tp.bn / 2) * KB));
         if (W_IS_NK) tma_load_2d(dst, &map_w, kb * KB, n0, bar);
         else tma_load_2d(dst, &map_w, n0, kb * KB, bar);
         if (ACT != kActExpanded) {
-            const int m0 = (t - slab * tp.chunks) * tp.bn + (int)half * (tp.bn / 2);
+            m0 += (int)half * (tp.bn / 2);
             if (ACT == kActRows) tma_load_2d(dst + Smem::kW8, &map_act, kb * KB, m0, bar);
             else tma_load_2d(dst + Smem::kW8, &map_act, m0, kb * KB, bar);
         }
@@ -1329,7 +1346,10 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             int it = 0;
             bool ok = ACT == kActExpanded;
             for (int t = t0; t < t_end && ok; t += t_step) {
-                const int m0 = t % tp.chunks * tp.bn + (int)half * (tp.bn / 2);
+                int slab, m0;
+                if (FORM == kOneGroup) m0 = t % tp.chunks * tp.bn;
+                else place(t, slab, m0);
+                m0 += (int)half * (tp.bn / 2);
                 for (int kb = kb0; kb < kb1; kb++, it++) {
                     const int s = it % kWdStages;
                     if (it >= kWdStages) ok = mbar_wait(bar_bf_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 46);
@@ -1476,7 +1496,9 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                 continue;
             }
             if (!joined) { __syncwarp(); cluster_wait(); joined = true; }
-            const int slab = t / tp.chunks, m0 = (t - slab * tp.chunks) * tp.bn, n = slab * 2 * BM + (int)half * BM + row;
+            int slab, m0;
+            place(t, slab, m0);
+            const int n = slab * 2 * BM + (int)half * BM + row;
             // 2^sc as one factor, and a second one for the few scales that need it
             const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = max(-126, min(126, sc));
             const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(sc - s1 + 127) << 23);
@@ -1534,7 +1556,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
 #pragma unroll
                     for (int i = 0; i < 8; i++) v[i] *= f2;
                 }
-                if (n < p.N) store_columns(out + j * 8 * pitch, (std::conditional_t<FAR, unsigned long long, uint32_t>)pitch, p.c_is_f32, p.accumulate, cols - j * 8, v);
+                if (n < p.N) store_columns(out + j * 8 * pitch, (std::conditional_t<FORM == kFarRows, unsigned long long, uint32_t>)pitch, p.c_is_f32, p.accumulate, cols - j * 8, v);
             }
             tc_fence_before();
             __syncwarp();
@@ -1991,6 +2013,14 @@ struct GemmDeviceSetup {
 };
 PerDevice<GemmDeviceSetup> g_gemm_setup;
 
+template <int FORM>
+void weights_kernels(const void** k)
+{
+    k[0] = (const void*)hif8_gemm_weights_kernel<false, kActExpanded, FORM>; k[1] = (const void*)hif8_gemm_weights_kernel<true, kActExpanded, FORM>;
+    k[2] = (const void*)hif8_gemm_weights_kernel<false, kActRows, FORM>; k[3] = (const void*)hif8_gemm_weights_kernel<true, kActRows, FORM>;
+    k[4] = (const void*)hif8_gemm_weights_kernel<false, kActColumns, FORM>; k[5] = (const void*)hif8_gemm_weights_kernel<true, kActColumns, FORM>;
+}
+
 bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nullptr, const int** nw_clusters = nullptr)
 {
     const GemmDeviceSetup* s = g_gemm_setup.get(dev, [](int d, GemmDeviceSetup* out) {
@@ -1999,15 +2029,11 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
         std::memset(out->wd_clusters, 0, sizeof out->wd_clusters);
         std::memset(out->nw_clusters, 0, sizeof out->nw_clusters);
         const void* pair[2] = {(const void*)bf16_gemm_pair_kernel<false>, (const void*)bf16_gemm_pair_kernel<true>};
-        const void* wd[12] = {(const void*)hif8_gemm_weights_kernel<false, kActExpanded, false>, (const void*)hif8_gemm_weights_kernel<true, kActExpanded, false>,
-                              (const void*)hif8_gemm_weights_kernel<false, kActRows, false>, (const void*)hif8_gemm_weights_kernel<true, kActRows, false>,
-                              (const void*)hif8_gemm_weights_kernel<false, kActColumns, false>, (const void*)hif8_gemm_weights_kernel<true, kActColumns, false>,
-                              (const void*)hif8_gemm_weights_kernel<false, kActExpanded, true>, (const void*)hif8_gemm_weights_kernel<true, kActExpanded, true>,
-                              (const void*)hif8_gemm_weights_kernel<false, kActRows, true>, (const void*)hif8_gemm_weights_kernel<true, kActRows, true>,
-                              (const void*)hif8_gemm_weights_kernel<false, kActColumns, true>, (const void*)hif8_gemm_weights_kernel<true, kActColumns, true>};
+        const void* wd[18];
+        weights_kernels<kOneGroup>(wd); weights_kernels<kGroups>(wd + 6); weights_kernels<kFarRows>(wd + 12);
         for (int i = 0; i < 2 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(pair[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2);
-        for (int i = 0; i < 12 && out->rc == cudaSuccess; i++)
+        for (int i = 0; i < 18 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(wd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
         for (int s = 1; s <= kWdMaxSplit && out->rc == cudaSuccess; s *= 2) {
             cudaLaunchConfig_t cfg{};
@@ -2166,15 +2192,21 @@ struct WeightsTiling {
     }
 };
 
+template <int ACT, int FORM>
+static cudaError_t launch_weights_form(const cudaLaunchConfig_t& cfg, int w_is_nk, const CUtensorMap& map_w, const CUtensorMap& map_act, const GemmParams& p,
+                                       const TilePlan& tp)
+{
+    return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true, ACT, FORM>, map_w, map_act, p, tp)
+                   : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false, ACT, FORM>, map_w, map_act, p, tp);
+}
+
 template <int ACT>
 static cudaError_t launch_weights_kernel(const cudaLaunchConfig_t& cfg, int w_is_nk, const CUtensorMap& map_w, const CUtensorMap& map_act, const GemmParams& p,
                                          const TilePlan& tp)
 {
-    if ((p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32)
-        return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true, ACT, true>, map_w, map_act, p, tp)
-                       : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false, ACT, true>, map_w, map_act, p, tp);
-    return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<true, ACT, false>, map_w, map_act, p, tp)
-                   : cudaLaunchKernelEx(&cfg, hif8_gemm_weights_kernel<false, ACT, false>, map_w, map_act, p, tp);
+    if ((p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) return launch_weights_form<ACT, kFarRows>(cfg, w_is_nk, map_w, map_act, p, tp);
+    return tp.chunks > kGroupPieces ? launch_weights_form<ACT, kGroups>(cfg, w_is_nk, map_w, map_act, p, tp)
+                                    : launch_weights_form<ACT, kOneGroup>(cfg, w_is_nk, map_w, map_act, p, tp);
 }
 
 // C = A W with the weights decoded inside the kernel.  act = kActExpanded: `a` is BF16 [M,K], written by the launch in front of
@@ -2195,8 +2227,8 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, int 
     if (!okw || !oka) return HIF8_ERR_CUDA;
     const int rem = (int)tl.cost.remainder(tiles), clear = act != kActExpanded;
     TilePlan launch[2];
-    launch[0] = TilePlan{0, tiles - rem, tl.chunks, tl.bn, tiles <= pairs ? tl.cost.best_split(tiles) : 1, clear};
-    launch[1] = TilePlan{tiles - rem, rem, tl.chunks, tl.bn, rem ? tl.cost.best_split(rem) : 1, 0};
+    launch[0] = TilePlan{0, tiles - rem, tl.chunks, tl.bn, tiles / tl.chunks, tiles <= pairs ? tl.cost.best_split(tiles) : 1, clear};
+    launch[1] = TilePlan{tiles - rem, rem, tl.chunks, tl.bn, tiles / tl.chunks, rem ? tl.cost.best_split(rem) : 1, 0};
     for (int i = 0; i < (rem ? 2 : 1); i++) {
         const TilePlan& tp = launch[i];
         cudaLaunchConfig_t cfg{};
