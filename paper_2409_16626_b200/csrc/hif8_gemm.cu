@@ -15,8 +15,9 @@
 // (128 bytes), eight rows form a 1024-byte swizzle atom, 16-byte chunk j of row r is stored at chunk j ^ (r % 8).
 // MN-major operands have atoms of 8 k-rows x 64 columns.
 //
-// Every wait on an mbarrier is bounded; a wait that runs out records a status word, makes all roles leave their
-// loops, lets outstanding TMA copies land, frees TMEM and returns.
+// Every wait on an mbarrier is bounded; a wait that runs out records a status word and makes all roles leave their
+// loops.  Whoever issued copies or MMAs waits for them (again with a limit) before the block leaves and its shared memory may
+// become another's; then TMEM is freed.  Copies whose barrier counts other parties too are made waitable by those parties.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -102,6 +103,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
             }
         }
     }
+}
+
+// Lets the use-th use of a ring of `stages` barriers complete, `bar` its own, within the limit of a wait.
+__device__ __forceinline__ void wait_landed(uint32_t bar, int use, int stages)
+{
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try_wait(bar, (uint32_t)(use / stages) & 1u) && global_ns() - t0 < kWaitLimitNs) {}
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar)
@@ -207,6 +215,11 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr)
 __device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+__device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -330,6 +343,12 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
 {
     uint32_t v;
     asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_volatile_u32(uint32_t addr)
+{
+    uint32_t v;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ uint2 lds_v2(uint32_t addr)
@@ -754,12 +773,8 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                 issued = it + 1;
                 if (++s == S8) { s = 0; ph ^= 1u; }
             }
-            if (*abort_flag) {  // let the copies already issued land before this CTA's shared memory goes away
-                for (int it = max(0, issued - S8); it < issued; it++) {
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(bar_u8_full(it % S8), (it / S8) & 1) && global_ns() - t0 < kWaitLimitNs) {}
-                }
-            }
+            if (*abort_flag)
+                for (int it = max(0, issued - S8); it < issued; it++) wait_landed(bar_u8_full(it % S8), it, S8);
         }
     } else if (warp == kNwActWarp) {
         // Activations expanded to BF16 beforehand (map_act is then the map of that copy): the tile of every k-block goes
@@ -776,12 +791,8 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                 issued = it + 1;
                 if (++kb == num_kb) kb = 0;
             }
-            if (*abort_flag) {
-                for (int it = max(0, issued - S); it < issued; it++) {
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(bar_bf_full(it % S), (it / S) & 1) && global_ns() - t0 < kWaitLimitNs) {}
-                }
-            }
+            if (*abort_flag)
+                for (int it = max(0, issued - S); it < issued; it++) wait_landed(bar_bf_full(it % S), it, S);
         }
     } else if (warp == kMmaWarp || warp >= kFirstDecodeWarp + kDecodeWarps) {
         const int q = warp == kMmaWarp ? 0 : warp - (kFirstDecodeWarp + kDecodeWarps) + 1;  // issuer number
@@ -792,8 +803,8 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             // descriptor of stage 0; a stage or a 16-k step further on adds to the address field only
             const uint64_t da0 = make_smem_desc(lay.bf(0), 16, 1024);
             bool ok = true, first = true;
-            int kb = 2 * pb0, seg = 0;
-            for (int it = 0; it < n_it && ok; it++) {
+            int kb = 2 * pb0, seg = 0, it = 0;
+            for (; it < n_it && ok; it++) {
                 const int buf = bufs == 2 ? seg & 1 : 0, use = bufs == 2 ? seg >> 1 : seg;  // use: how often the buffer was filled before
                 if ((it & (issuers - 1)) == q) {
                     const int s = it % S, round = it / S;
@@ -822,6 +833,10 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                     kb = 0; seg++; first = true;
                 }
             }
+            if (!ok && it > q) {  // its last MMAs: of the last k-block before this one that it took
+                const int last = it - 1 - ((it - 1 - q) & (issuers - 1));
+                wait_landed(bar_bf_empty(last % S), last, S);
+            }
         }
     } else if (warp >= kFirstDecodeWarp) {
         const int group = (warp - kFirstDecodeWarp) / kGroupWarps;
@@ -835,7 +850,13 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             const int s = it % S, r = it / S;
             ok = mbar_wait(bar_u8_full(s8), ph8, abort_flag, p.status, 33);
             if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 34);
-            if (!ok) break;
+            if (!ok) {
+                // The barrier of an expanded activation tile counts this group too: its arrivals for the tiles that may have been
+                // issued, one per stage, so that they can be waited for.
+                if (ACT_BF16 && lane == 0)
+                    for (int i = it; i < min(it + S, n_it); i += kDecodeGroups) mbar_arrive(bar_bf_full(i % S));
+                break;
+            }
             const uint32_t w8 = lay.u8(s8), a8 = w8 + kU8Act + (uint32_t)h * BK;
             const uint32_t abf = lay.bf(s);
             uint2 va[kNarrowMaxM * (BK / 8) / kGroupThreads];
@@ -1148,13 +1169,14 @@ struct WdSmem {
             front = min((int)((lut - base) / kSlotBytes), 2 * kWdStages);
             bars = lut + kLutBytesWide + (uint32_t)(2 * kWdStages - front) * kSlotBytes;
         }
-        end = bars + n_bars * 8 + 8;
+        end = bars + n_bars * 8 + 12;
     }
     __device__ uint32_t slot(int i) const { return i < front ? base + (uint32_t)i * kSlotBytes : lut + kLutBytesWide + (uint32_t)(i - front) * kSlotBytes; }
     __device__ uint32_t act(int s) const { return ACT == kActExpanded ? base + (uint32_t)s * kActStage : slot(s); }
     __device__ uint32_t u8(int s) const { return ACT == kActExpanded ? base + kWdStages * kActStage + (uint32_t)s * kW8 : slot(kWdStages + s); }
     __device__ uint32_t tmem_slot() const { return bars + n_bars * 8; }
     __device__ uint32_t abort_flag() const { return tmem_slot() + 4; }
+    __device__ uint32_t other_issued() const { return tmem_slot() + 8; }  // 1 + the activation tiles that the pair's other CTA issued in all (0: not through yet)
 };
 static_assert(WdSmem<kActRows>::kActStage == kSlotBytes && 2 * WdSmem<kActRows>::kW8 == kSlotBytes, "one stage per slot");
 static_assert((kWdMaxSplit - 1) * (BN / kWdMaxSplit) * BM * 4 <= 2 * kWdStages * kSlotBytes && (2 - 1) * (BN / 2) * BM * 4 <= 2 * kWdStages * kSlotBytes,
@@ -1214,10 +1236,11 @@ __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, i
     }
 }
 
-// Instantiations by tile order and row pitch.  (With the choice of the order made in the kernel, its divisions in everybody's way,
-// 128 x 512 x 512 took 10.0 us instead of 9.8.)
+// Instantiations by tile order and row pitch.  (With the choice of the order made in the kernel, the divisions of the other one in
+// the way of the first copies, 128 x 512 x 512 took 10.0 us instead of 9.8.)
 enum WeightsForm { kOneGroup, kGroups, kFarRows };  // up to eight pieces; more; the rows of C 4 GiB apart or more (any number of pieces)
 constexpr int kGroupPieces = 8;
+
 template <bool W_IS_NK, int ACT, int FORM>
 __global__ void __launch_bounds__(kThreadsWd, 1)
 hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_act, const GemmParams p, const TilePlan tp)
@@ -1289,6 +1312,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         }
         mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps));
         *abort_flag = 0;
+        if (ACT == kActExpanded) *reinterpret_cast<volatile uint32_t*>(sm + lay.other_issued()) = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         if (ACT == kActExpanded) copy_bytes(0, t0, kb0);
@@ -1329,12 +1353,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                     copy_bytes(it, t, kb);
                 }
             }
-            if (*abort_flag) {
-                for (int i = max(0, it - kWdStages); i < it; i++) {  // let the copies already issued land
-                    const unsigned long long c0 = global_ns();
-                    while (!mbar_try_wait(bar_u8_full(i % kWdStages), (i / kWdStages) & 1) && global_ns() - c0 < kWaitLimitNs) {}
-                }
-            }
+            if (*abort_flag)
+                for (int i = max(0, it - kWdStages); i < it; i++) wait_landed(bar_u8_full(i % kWdStages), i, kWdStages);
         }
     } else if (warp == kWdActWarp) {
         // ------------------------------------------------------------------ expanded activations: this CTA's bn / 2 rows, two boxes of
@@ -1343,8 +1363,13 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         if (lane == 0) {
             asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            int it = 0;
+            // A tile's barrier (in the pair's leader) counts the bytes of both CTAs' halves.  A thread that gives up tells the other CTA's
+            // how many tiles it has issued, and the one that is behind issues its halves of the tiles that the other one
+            // issued: their stages were free for both, and hold nothing that anybody still wants.
+            constexpr int kNoLimit = 0x7FFFFFFF;
+            int it = 0, limit = kNoLimit;
             bool ok = ACT == kActExpanded;
+            auto tell = [&]() { st_cluster_u32(map_to_cta(lay.other_issued(), rank ^ 1u), (uint32_t)it + 1u); };
             for (int t = t0; t < t_end && ok; t += t_step) {
                 int slab, m0;
                 if (FORM == kOneGroup) m0 = t % tp.chunks * tp.bn;
@@ -1352,17 +1377,24 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                 m0 += (int)half * (tp.bn / 2);
                 for (int kb = kb0; kb < kb1; kb++, it++) {
                     const int s = it % kWdStages;
-                    if (it >= kWdStages) ok = mbar_wait(bar_bf_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 46);
-                    if (!ok || *abort_flag) { ok = false; break; }
+                    if (limit == kNoLimit && ((it >= kWdStages && !mbar_wait(bar_bf_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 46)) || *abort_flag)) {
+                        tell();
+                        const unsigned long long c0 = global_ns();
+                        do limit = (int)lds_volatile_u32(lay.other_issued()) - 1;  // (the other CTA's waits are bounded as well)
+                        while (limit < 0 && global_ns() - c0 < 2 * kWaitLimitNs);
+                    }
+                    if (it >= limit) { ok = false; break; }
                     if (leader) mbar_arrive_expect_tx(bar_bf_full(s), (uint32_t)tp.bn * KB * 2u);
                     const uint32_t full = map_to_cta(bar_bf_full(s), lead);
                     tma_load_3d_pair(lay.act(s), &map_act, kb * KB, m0, 0, full);
                     tma_load_3d_pair(lay.act(s) + Smem::kActStage / 2, &map_act, kb * KB + BK, m0, 0, full);
                 }
             }
-            if (ACT == kActExpanded && *abort_flag) {  // (their barrier also counts the decode groups, which have given up: a fixed 50 us instead)
-                const unsigned long long c0 = global_ns();
-                while (global_ns() - c0 < 50000ull) {}
+            if (ACT == kActExpanded) {
+                if (limit == kNoLimit) tell();
+                if (leader && *abort_flag) {
+                    for (int i = max(0, it - kWdStages); i < it; i++) wait_landed(bar_bf_full(i % kWdStages), i, kWdStages);
+                }
             }
         }
     } else if (warp == kMmaWarp) {
@@ -1393,6 +1425,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                 }
                 if (ok) tc_commit_pair(bar_acc_full, lead);
             }
+            if (!ok && it > 0) wait_landed(bar_bf_empty((it - 1) % kWdStages), it - 1, kWdStages);
         }
     } else if (warp < kFirstDecodeWarp) cluster_wait();  // warps 0-3
 
@@ -1412,7 +1445,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         const long long pitch = p.ldc * c_size;
         const uint32_t tl = tmem_base + ((uint32_t)(quarter * 32) << 16), mine = base + (uint32_t)row * 16u, tlane = tl + kTmemColsAcc;
         const int n_kb = kb1 - kb0;
-        int it = decodes ? group : 0x7FFFFFFF, tile_it = 0, local = 0;  // next k-block of the group; first k-block of the tile to finish next
+        constexpr int kGaveUp = 1 << 30;
+        int it = decodes ? group : kGaveUp, tile_it = 0, local = 0;  // next k-block of the group; first k-block of the tile to finish next
         bool joined = !decodes;
         for (int t = t0; t < t_end;) {
             // the group's k-blocks of this tile, and one of the next
@@ -1421,7 +1455,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                 const int s = it % kWdStages, r = it / kWdStages;
                 bool ok = mbar_wait(bar_u8_full(s), r & 1, abort_flag, p.status, 43);
                 if (ok && r > 0) ok = mbar_wait(bar_bf_empty(s), (r - 1) & 1, abort_flag, p.status, 44);
-                if (!ok) { it = 0x7FFFFFFF; continue; }  // (gives up at the next wait)
+                if (!ok) { it += kGaveUp; continue; }  // (no further k-block: gives up at the next wait)
                 const uint32_t w8 = lay.u8(s), dst = tlane + (uint32_t)(s * (KB / 2));
                 // activations as bytes: eight 8-byte chunks of the tile per thread at most (it lies in a row, [M,K] or [K,M])
                 const int dt = threadIdx.x - (kFirstDecodeWarp + group * kGroupWarps) * 32, n_chunks = tp.bn / 2 * (BK / 8);
@@ -1564,6 +1598,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             t += t_step; tile_it += n_kb; local++;
         }
         if (!joined) { __syncwarp(); cluster_wait(); }
+        // (gave up: the barrier of an expanded activation tile counts this group too; its arrival, so that the tile can be waited for)
+        if (ACT == kActExpanded && decodes && it >= kGaveUp && lane == 0) mbar_arrive_remote(map_to_cta(bar_bf_full((it - kGaveUp) % kWdStages), lead));
     }
 
     // ---- teardown: all waits are bounded, so everybody arrives; nobody leaves while the peer may still read this
@@ -1607,7 +1643,9 @@ struct SmemLayout2 {
     static constexpr uint32_t n_bars = 2 * kStages2 + 4 + 2 * kEpiWarps;
     static constexpr uint32_t tmem_slot = bars + n_bars * 8;
     static constexpr uint32_t abort_flag = tmem_slot + 4;
-    static constexpr uint32_t total = abort_flag + 4;
+    static constexpr uint32_t gave_up = abort_flag + 4;    // a CTA of the pair gave up
+    static constexpr uint32_t issued = gave_up + 4;        // k-blocks issued by the pair's four copying threads
+    static constexpr uint32_t total = issued + 4 * 4;
 };
 constexpr uint32_t kSmemBytes2 = SmemLayout2::total + 1024;
 static_assert(kSmemBytes2 <= 227 * 1024, "shared memory of one CTA");
@@ -1643,6 +1681,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         for (int a = 0; a < 2; a++) { mbar_init(bar_acc_full(a), 1); mbar_init(bar_acc_empty(a), 2 * kEpiWarps); }
         for (int i = 0; i < 2 * kEpiWarps; i++) mbar_init(bar_old(i), 1);
         *abort_flag = 0;
+        *reinterpret_cast<volatile int*>(sm + SmemLayout2::gave_up) = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kMmaWarp) {
@@ -1657,10 +1696,23 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     const uint32_t tmem_base = *tmem_slot;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // (set-up above runs under the launch in front, which expands the weights)
 
+    int progress = 0;  // of this thread's role: k-blocks issued or committed
+    const bool loads_a = warp == kTmaWarp;
+    auto copy_block = [&](int m0, int n0, int ia, int iw, int kb, int s) {  // this thread's operand of k-block kb into stage s, which is free
+        const uint32_t dst_a = base + s * kStageBytes2, dst_b = dst_a + kABfBytes;
+        const uint32_t full = map_to_cta(bar_full(s), 0);
+        if (loads_a) {
+            if (leader) mbar_arrive_expect_tx(bar_full(s), 2 * kStageBytes2);  // bytes of both CTAs, both operands
+            tma_load_3d_pair(dst_a, &map_a, kb * BK, m0, ia, full);
+        } else if (W_IS_NK) tma_load_3d_pair(dst_b, &map_w, kb * BK, n0, iw, full);
+        else {
+#pragma unroll
+            for (int c = 0; c < BN / 2 / 64; c++)
+                tma_load_3d_pair(dst_b + c * 8192, &map_w, n0 + c * 64, kb * BK, iw, full);
+        }
+    };
     if (warp == kTmaWarp || warp == kTmaWarpW) {
         if (lane == 0) {
-            const bool loads_a = warp == kTmaWarp;
-            long long issued = 0;
             int s = 0;            // stage of the next k-block
             uint32_t ph = 0;      // parity of the round the ring is in
             bool ok = true, wrapped = false;
@@ -1672,28 +1724,12 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                 for (int kb = 0; kb < num_kb; kb++) {
                     if (wrapped) ok = mbar_wait(bar_empty(s), ph ^ 1u, abort_flag, p.status, 21);  // the previous round's use of the stage
                     if (!ok || *abort_flag) { ok = false; break; }
-                    const uint32_t dst_a = base + s * kStageBytes2, dst_b = dst_a + kABfBytes;
-                    const uint32_t full = map_to_cta(bar_full(s), 0);
-                    if (loads_a) {
-                        if (leader) mbar_arrive_expect_tx(bar_full(s), 2 * kStageBytes2);  // bytes of both CTAs, both operands
-                        tma_load_3d_pair(dst_a, &map_a, kb * BK, m0, ia, full);
-                    } else if (W_IS_NK) tma_load_3d_pair(dst_b, &map_w, kb * BK, n0, iw, full);
-                    else {
-#pragma unroll
-                        for (int c = 0; c < BN / 2 / 64; c++)
-                            tma_load_3d_pair(dst_b + c * 8192, &map_w, n0 + c * 64, kb * BK, iw, full);
-                    }
-                    issued++;
+                    copy_block(m0, n0, ia, iw, kb, s);
+                    progress++;
                     if (++s == kStages2) { s = 0; ph ^= 1u; wrapped = true; }
                 }
             }
-            if (*abort_flag && leader && loads_a) {  // let copies in flight land (their completions are counted on the leader)
-                for (long long j = issued > kStages2 ? issued - kStages2 : 0; j < issued; j++) {
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(bar_full((int)(j % kStages2)), (uint32_t)((j / kStages2) & 1)) &&
-                           global_ns() - t0 < kWaitLimitNs) {}
-                }
-            }
+            for (uint32_t r = 0; r < 2; r++) st_cluster_u32(map_to_cta(base + SmemLayout2::issued + 4u * (2u * rank + (loads_a ? 0u : 1u)), r), (uint32_t)progress);
         }
     } else if (warp == kMmaWarp) {
         if (lane == 0 && leader) {
@@ -1722,6 +1758,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                         tc_mma_bf16_pair(d_tmem, da, db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                     }
                     tc_commit_pair(bar_empty(s));
+                    progress++;
                     if (++s == kStages2) { s = 0; ph ^= 1u; }
                 }
                 if (ok) tc_commit_pair(bar_acc_full(acc));
@@ -1738,7 +1775,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         };
         const int piece_cols = p.c_is_f32 ? 32 : 64;
         const uint32_t staging = base + SmemLayout2::out + (uint32_t)warp * 2 * kOutBytes;  // this warp's two pieces
-        uint32_t n_old = 0;  // old pieces waited for, over all tiles
+        uint32_t n_old = 0, n_fetched = 0;  // old pieces waited for and (lane 0) asked for, over all tiles: parities of the two buffers
         for (int t = pair_id; t < tiles; t += pairs, local++) {
             const int acc = local & 1, use = local >> 1;
             int tile_m, tile_n;
@@ -1750,6 +1787,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                 const uint32_t bar = bar_old(2 * warp + (i & 1));
                 mbar_arrive_expect_tx(bar, kOutBytes);
                 tma_load_2d(staging + (uint32_t)(i & 1) * kOutBytes, &map_c, n0 + i * piece_cols, row0, bar);
+                n_fetched ^= 1u << (i & 1);
             };
             if (p.c_by_tma && p.accumulate && lane == 0) {
                 asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -1854,10 +1892,9 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         }
         if (p.err_sum) flush_error();
         if (p.c_by_tma && lane == 0) {
-            if (p.accumulate && *abort_flag) {  // old pieces still on their way land before this CTA's shared memory goes away
-                const unsigned long long c0 = global_ns();
-                while (global_ns() - c0 < 50000ull) {}
-            }
+            // old pieces still on their way (a wait gave up) land before this CTA's shared memory goes away
+            for (uint32_t i = 0; i < 2; i++)
+                if (((n_fetched ^ n_old) >> i) & 1u) wait_landed(bar_old(2 * warp + i), (int)(n_old >> i), 1);
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         }
     }
@@ -1865,7 +1902,32 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     // nobody leaves while the other CTA may still read this CTA's shared memory or signal its barriers
     tc_fence_before();
     __syncthreads();
+    if (*abort_flag && threadIdx.x == 0)
+        for (uint32_t r = 0; r < 2; r++) st_cluster_u32(map_to_cta(base + SmemLayout2::gave_up, r), 1u);
+    __syncwarp();
     cluster_sync_all();
+    if (*reinterpret_cast<volatile int*>(sm + SmemLayout2::gave_up)) {
+        // A wait gave up in one of the CTAs (the same answer in both).  A stage's barrier counts the copies of four threads: those
+        // that are behind issue theirs of the k-blocks that another one issued (whose stages were free for all), and the leader
+        // waits for them all, and for its last MMAs.
+        if (lane == 0) {
+            if (warp == kTmaWarp || warp == kTmaWarpW) {
+                const volatile int* issued = reinterpret_cast<const volatile int*>(sm + SmemLayout2::issued);
+                const int top = max(max(issued[0], issued[1]), max(issued[2], issued[3]));
+#pragma unroll 1
+                for (int i = progress; i < top; i++) {
+                    int tile_m, tile_n;
+                    const int t = pair_id + i / num_kb * pairs, b = t / tiles_one, ia = b / nb;
+                    tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n);
+                    copy_block(tile_m * 2 * BM + (int)rank * BM, tile_n * BN + (int)rank * (BN / 2), ia, b - ia * nb, i % num_kb, i % kStages2);
+                }
+                if (leader && loads_a)
+                    for (int i = max(0, top - kStages2); i < top; i++) wait_landed(bar_full(i % kStages2), i, kStages2);
+            } else if (warp == kMmaWarp && leader && progress > 0) wait_landed(bar_empty((progress - 1) % kStages2), progress - 1, kStages2);
+        }
+        __syncwarp();
+        cluster_sync_all();
+    }
     if (warp == kMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");

@@ -8,7 +8,7 @@ import re
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2409_16626_b200", "csrc")
-REMOTE = ("st.shared::cluster", "st_cluster_v4(", "mbar_arrive_remote(", "atom.shared::cluster", "red.shared::cluster", "ld.shared::cluster")
+REMOTE = ("st.shared::cluster", "st_cluster_v4(", "st_cluster_u32(", "mbar_arrive_remote(", "atom.shared::cluster", "red.shared::cluster", "ld.shared::cluster")
 WAIT = ("barrier.cluster.wait", "cluster_wait()", "cluster_sync_all()")
 
 

@@ -1,0 +1,36 @@
+"""What a GEMM kernel has in flight when one of its bounded waits gives up must land before the block leaves and its shared
+memory becomes another's.  Running into that would take a kernel broken on purpose, so the sources are checked, on the CPU:
+for every barrier that copies complete on, the kernel waits at its end, and no fixed delay stands in for a wait."""
+import os
+import re
+
+import pytest
+
+SOURCE = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2409_16626_b200", "csrc", "hif8_gemm.cu")
+TEXT = re.sub(r"//[^\n]*", "", open(SOURCE).read())
+
+
+def body(name):
+    start = re.search(r"\n%s\(const __grid_constant__" % name, TEXT).end()
+    return TEXT[start:TEXT.find("\n}\n", start)]
+
+
+@pytest.mark.parametrize("kernel,barriers", [("hif8_gemm_narrow_kernel", ["bar_u8_full", "bar_bf_full"]),
+                                             ("hif8_gemm_weights_kernel", ["bar_u8_full", "bar_bf_full"]),
+                                             ("bf16_gemm_pair_kernel", ["bar_full", "bar_old"])])
+def test_copies_are_waited_for(kernel, barriers):
+    text = body(kernel)
+    assert "tma_load" in text
+    for b in barriers:
+        assert f"wait_landed({b}(" in text, b
+
+
+@pytest.mark.parametrize("kernel,barrier", [("hif8_gemm_narrow_kernel", "bar_bf_empty"), ("hif8_gemm_weights_kernel", "bar_bf_empty"),
+                                            ("bf16_gemm_pair_kernel", "bar_empty")])
+def test_mmas_are_waited_for(kernel, barrier):
+    assert f"wait_landed({barrier}(" in body(kernel)
+
+
+def test_every_wait_has_the_limit_and_there_is_no_fixed_delay():
+    loops = re.findall(r"while \([^;{]*global_ns\(\)[^;{]*[;{]", TEXT)
+    assert loops and all("kWaitLimitNs" in w for w in loops), loops
