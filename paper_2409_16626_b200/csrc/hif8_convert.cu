@@ -253,11 +253,12 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const ConvParams p, u
 // ------------------------------------------------------------------------------------------------
 // Just-in-time scaling of a small tensor in one launch: a cluster of up to eight blocks holds the source in shared memory,
 // reduces its amax (each block tells the others its own through distributed shared memory, between two cluster barriers, the
-// first of which completes under the loads and the table set-up), and converts from there.  No accumulator in the workspace, so nothing to clear.  Latency and launches bound it: the three launches of the
-// general path (clear, amax, convert) take 3.3 us on the device and 8 us from the host, this 2.3 us and 4 us (512 BF16
-// elements, round half away); 3.9 against 3.1 us at 131072.  The limits are where eight blocks take as long on the device as
-// three launches over all SMs: 256 KiB of source, half of that for dequantized results, which carry more arithmetic
-// (131072 BF16 elements under hybrid rounding: 4.5 us by three launches, 5.0 us by one).
+// first of which completes under the loads and the table set-up), and converts from there.  No accumulator in the workspace,
+// so nothing to clear.  Latency and launches bound it: the three launches of the general path (clear, amax, convert) take 3.3 us
+// on the device and 8 us from the host, this 2.3 us and 4 us (512 BF16 elements, round half away); 3.9 against 3.1 us on the device
+// at 131072.  To bytes it takes what eight blocks hold without an opt-in to more than 48 KiB of shared memory each: 256 KiB of
+// source, where it is still the faster one.  Dequantized results carry more arithmetic, and at that size eight blocks are the
+// slower form (131072 BF16 elements under hybrid rounding: 4.5 us by three launches, 5.0 us by one): half of it.
 // ------------------------------------------------------------------------------------------------
 constexpr int kOneThreads = 512, kOneVecs = 4, kOneBlocks = 8;  // 32 KiB of source per block
 constexpr unsigned long long kOneMaxVecs = (unsigned long long)kOneThreads * kOneVecs * kOneBlocks, kOneMaxVecsFq = kOneMaxVecs / 2;

@@ -412,68 +412,45 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
 }
 
 
-// Epilogue of one 32-column chunk of one accumulator row: descale by f1 * f2 (two exact powers of two) and store as
-// FP32 or BF16 (round to nearest even); rows / columns outside the matrix are skipped.
-__device__ __forceinline__ void store_chunk(const GemmParams& p, int row, int col, const uint32_t (&r)[32], float f1, float f2)
+// One 32-column chunk of one accumulator row, descaled by f1 * f2 (two exact powers of two), added to BF16 results that are
+// there already and rounded to nearest even; rows / columns outside the matrix are skipped.
+__device__ __forceinline__ void add_chunk_bf16(const GemmParams& p, int row, int col, const uint32_t (&r)[32], float f1, float f2)
 {
     if (row >= p.M || col >= p.N) return;
     const bool full = col + 32 <= p.N;
-    if (p.c_is_f32) {
-        float* out = reinterpret_cast<float*>(p.C) + (long long)row * p.ldc + col;
-        if (full) {
-            // C is touched once: streaming loads and stores, so that it does not push operand tiles out of L2; all the
-            // loads of the chunk are issued before the first store (they cannot be moved across it by the compiler)
-            float4 c[8];
+    unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + (long long)row * p.ldc + col;
+    uint32_t h[32];  // previous contents of C, widened exactly
+    if (full) {
 #pragma unroll
-            for (int i = 0; i < 8; i++) c[i] = p.accumulate ? __ldcs(reinterpret_cast<const float4*>(out) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int i = 0; i < 8; i++)
-                __stcs(reinterpret_cast<float4*>(out) + i,
-                       make_float4(__uint_as_float(r[4 * i]) * f1 * f2 + c[i].x, __uint_as_float(r[4 * i + 1]) * f1 * f2 + c[i].y,
-                                   __uint_as_float(r[4 * i + 2]) * f1 * f2 + c[i].z, __uint_as_float(r[4 * i + 3]) * f1 * f2 + c[i].w));
-        } else {
-            // (every index a compile-time constant: a loop that stops at the ragged edge would index the chunk by a
-            // variable and put it, for all paths, into local memory -- which has next to no L1 behind it in these kernels)
-#pragma unroll
-            for (int i = 0; i < 32; i++)
-                if (col + i < p.N) out[i] = __uint_as_float(r[i]) * f1 * f2 + (p.accumulate ? out[i] : 0.f);
+        for (int i = 0; i < 32; i += 8) {
+            const uint4 c = __ldcs(reinterpret_cast<const uint4*>(out + i));
+            h[i] = c.x << 16; h[i + 1] = c.x & 0xFFFF0000u; h[i + 2] = c.y << 16; h[i + 3] = c.y & 0xFFFF0000u;
+            h[i + 4] = c.z << 16; h[i + 5] = c.z & 0xFFFF0000u; h[i + 6] = c.w << 16; h[i + 7] = c.w & 0xFFFF0000u;
         }
     } else {
-        unsigned short* out = reinterpret_cast<unsigned short*>(p.C) + (long long)row * p.ldc + col;
-        uint32_t h[32];
-        if (p.accumulate) {  // previous contents of C, widened exactly
-            if (full) {
+        // (every index a compile-time constant: a loop that stops at the ragged edge would index the chunk by a
+        // variable and put it, for all paths, into local memory -- which has next to no L1 behind it in these kernels)
 #pragma unroll
-                for (int i = 0; i < 32; i += 8) {
-                    const uint4 c = __ldcs(reinterpret_cast<const uint4*>(out + i));
-                    h[i] = c.x << 16; h[i + 1] = c.x & 0xFFFF0000u; h[i + 2] = c.y << 16; h[i + 3] = c.y & 0xFFFF0000u;
-                    h[i + 4] = c.z << 16; h[i + 5] = c.z & 0xFFFF0000u; h[i + 6] = c.w << 16; h[i + 7] = c.w & 0xFFFF0000u;
-                }
-            } else {
+        for (int i = 0; i < 32; i++) h[i] = (col + i < p.N) ? (uint32_t)out[i] << 16 : 0u;
+    }
+    uint32_t pk[16];  // two BF16 per word, rounded to nearest even by the conversion instruction (a NaN stays a NaN)
 #pragma unroll
-                for (int i = 0; i < 32; i++) h[i] = (col + i < p.N) ? (uint32_t)out[i] << 16 : 0u;
-            }
-        }
-        uint32_t pk[16];  // two BF16 per word, rounded to nearest even by the conversion instruction (a NaN stays a NaN)
+    for (int i = 0; i < 32; i += 2) {
+        const float v0 = __uint_as_float(r[i]) * f1 * f2 + __uint_as_float(h[i]), v1 = __uint_as_float(r[i + 1]) * f1 * f2 + __uint_as_float(h[i + 1]);
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[i >> 1]) : "f"(v1), "f"(v0));  // first source -> upper half
+    }
+    if (full) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 2) {
-            float v0 = __uint_as_float(r[i]) * f1 * f2, v1 = __uint_as_float(r[i + 1]) * f1 * f2;
-            if (p.accumulate) { v0 += __uint_as_float(h[i]); v1 += __uint_as_float(h[i + 1]); }
-            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[i >> 1]) : "f"(v1), "f"(v0));  // first source -> upper half
-        }
-        if (full) {
+        for (int i = 0; i < 16; i += 4)
+            __stcs(reinterpret_cast<uint4*>(out + 2 * i), make_uint4(pk[i], pk[i + 1], pk[i + 2], pk[i + 3]));
+    } else {
 #pragma unroll
-            for (int i = 0; i < 16; i += 4)
-                __stcs(reinterpret_cast<uint4*>(out + 2 * i), make_uint4(pk[i], pk[i + 1], pk[i + 2], pk[i + 3]));
-        } else {
-#pragma unroll
-            for (int i = 0; i < 32; i++)
-                if (col + i < p.N) out[i] = (unsigned short)(pk[i >> 1] >> (16 * (i & 1)));
-        }
+        for (int i = 0; i < 32; i++)
+            if (col + i < p.N) out[i] = (unsigned short)(pk[i >> 1] >> (16 * (i & 1)));
     }
 }
 
-// The same chunk, descaled and rounded to BF16, into a staging tile in shared memory from which a tile store writes C:
+// A chunk, descaled and rounded to BF16, into a staging tile in shared memory from which a tile store writes C:
 // boxes of 64 columns x 128 rows in the 128-byte-swizzled layout of the tensor map (16-byte piece j of row r sits at
 // piece j ^ (r % 8) of its 128-byte line; lines of eight rows form 1024-byte atoms).  `piece0` = first 16-byte piece of
 // the chunk within its row of the box (0 or 4).  A thread's four stores hit four different pieces; the eight rows of an
@@ -542,7 +519,7 @@ constexpr int kNwMaxByteStages = 6, kNwMinByteStages = 4;
 // that a group starts its next k-block without waiting for the MMAs of its previous one
 constexpr int kNwTmemStages = 2 * kDecodeGroups;
 constexpr uint32_t kNwBars = 2 * kNwMaxByteStages + 2 * kNwTmemStages + 4;
-// Where the narrow kernel keeps what (mp activation rows).  WIDE ([N,K] weights with the activations expanded beforehand):
+// Where the narrow kernel keeps what (mp activation rows).  WIDE (activations expanded beforehand):
 // the decode table has rows of 256 bytes and starts on a 64 KiB boundary of the shared window, so that one byte permute makes
 // a lookup's address (see decode8); operand stages and then byte stages as they fit in front of it, the rest behind it.
 // Otherwise: operand stages, byte stages and the 32 KiB table in a row.
@@ -1874,7 +1851,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                             }
                         } else {
 #pragma unroll
-                            for (int i = 0; i < 32; i++) {  // (constant indices: see store_chunk)
+                            for (int i = 0; i < 32; i++) {  // (constant indices: see add_chunk_bf16)
                                 if (col + i < p.N) {
                                     const double d = (double)(__uint_as_float(r[i]) * f1 * f2) - (double)__ldg(ref + i);
                                     err_acc += d * d;
@@ -1882,7 +1859,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                             }
                         }
                     }
-                } else store_chunk(p, row, col, r, f1, f2);
+                } else add_chunk_bf16(p, row, col, r, f1, f2);
             }
             tc_fence_before();
             __syncwarp();

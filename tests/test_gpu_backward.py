@@ -261,3 +261,36 @@ def test_gemm_ex_rows_of_c_more_than_4_gib_apart(c_dtype, accumulate):
     if c_dtype == H.BF16:
         tol = tol + bf16_half_ulp(np.abs(want) + tol)
     assert np.all(np.abs(out - want) <= tol)
+
+
+@pytest.fixture(scope="module")
+def many_tiles():
+    # 11 x 16 tiles of 256 x 256 on 74 CTA pairs: two and three tiles per pair; ragged rows, and a last column tile of three
+    # pieces of 32 columns (FP32 results) or of one and a half of 64 (BF16)
+    M, N, K = 2570, 3936, 80
+    Aq, Wq = codes((M, K), 21), codes((K, N), 22)
+    return Aq, Wq, O.gemm_full(Aq, Wq, False, 3, -4)
+
+
+@pytest.mark.parametrize("accumulate", [0, 1])
+@pytest.mark.parametrize("c_dtype", [H.F32, H.BF16])
+def test_gemm_both_operands_expanded_many_tiles_per_pair(many_tiles, c_dtype, accumulate):
+    Aq, Wq, (Cs, S) = many_tiles
+    (M, K), N = Aq.shape, Wq.shape[1]
+    ldc = N + 8
+    c0 = (np.random.default_rng(4).standard_normal((M, ldc)) * 50).astype(np.float32)
+    C = torch.from_numpy(c0).cuda().to(torch.float32 if c_dtype == H.F32 else torch.bfloat16)
+    c0 = C.float().cpu().numpy().astype(np.float64)
+    wsb = H.hif8_workspace_bytes(H.WS_GEMM, M * K + K * N)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    with both_operands_expanded(True):
+        H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wq), N, 0, C, ldc, c_dtype, M, N, K, torch.tensor([3], dtype=torch.int32, device="cuda"),
+                       torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    assert H.hif8_gemm_status(ws) == 0
+    out = C.float().cpu().numpy().astype(np.float64)
+    assert np.array_equal(out[:, N:], c0[:, N:])
+    want = Cs + (c0[:, :N] if accumulate else 0.0)
+    tol = 1e-5 * S + (2.0 ** -24 * np.abs(want) if accumulate else 0.0)
+    if c_dtype == H.BF16:
+        tol = tol + bf16_half_ulp(np.abs(want) + tol)
+    assert np.all(np.abs(out[:, :N] - want) <= tol)

@@ -261,8 +261,8 @@ def test_gemm_narrow_channel_scales_and_accumulate(K):
 
 
 def test_gemm_calls_replay_from_a_cuda_graph():
-    # the narrow call is two launches chained by programmatic stream serialization, the general one a memset node and a
-    # cluster launch: both are captured into one graph and replayed on new operand contents
+    # the narrow call is two launches chained by programmatic stream serialization, the general one (nothing but the status word)
+    # a cluster launch that clears it: both are captured into one graph and replayed on new operand contents
     M, N, K = 16, 1168, 2432
     M2 = 256
     dA, dW = torch.empty(M2 * K, dtype=torch.uint8, device="cuda"), torch.empty(K * N, dtype=torch.uint8, device="cuda")
