@@ -119,10 +119,10 @@ __device__ __forceinline__ uint32_t group_max(uint32_t v, uint32_t* s_part, int 
 // do not fit in registers) dependents are let go at the end (20.3 and 4.9 us), elsewhere at once (a call is 2 us shorter).
 
 // Rows that fit in registers (at most NV vectors per thread of a group of gs threads).  A block works through
-// `iters` consecutive sets of kThreads / gs rows; the loads of the next set are issued before the current one is
+// `iters` sets of kThreads / gs rows, consecutive ones or (APART) one grid apart; the loads of the next set are issued before the current one is
 // reduced and converted, so every row is read exactly once and the memory latency is covered by the arithmetic of the
 // previous row.  Short rows get small groups so that a thread still holds about four vectors.
-template <int SRC, int MODE, int NV>
+template <int SRC, int MODE, int NV, bool APART = false>
 __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanParams p, int gs, int iters)
 {
     __shared__ SmemTables sm;
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
     const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
     const int groups = kThreads / gs, g = threadIdx.x / gs, t = threadIdx.x % gs;
     const uint4* base = reinterpret_cast<const uint4*>(p.src);
-    const long long first = (long long)blockIdx.x * iters * groups + g;
+    const long long step = APART ? (long long)gridDim.x * groups : groups, first = (long long)blockIdx.x * (APART ? 1 : iters) * groups + g;
 
     // NV <= kUnroll: two register sets, the next row is in flight while this one is processed; larger rows use one set
     constexpr bool kPrefetch = NV <= kUnroll;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
         }
     }
     for (int it = 0; it < iters; it++) {
-        const long long row = first + (long long)it * groups, row_next = row + groups;
+        const long long row = first + (long long)it * step, row_next = row + step;
         const bool live = row < p.rows;  // a group past the last row only takes part in the barriers
         if (kPrefetch) {
 #pragma unroll
@@ -429,9 +429,18 @@ int launch_encode(const ChanParams& p, const Plan& pl, cudaStream_t st)
             const long long sets = (p.rows + kThreads / gs - 1) / (kThreads / gs);
             int iters = nv <= (long long)kUnroll * gs ? 8 : 1;
             while (iters > 1 && (sets + iters - 1) / iters < (long long)pl.sms * 8) iters >>= 1;
-            const long long blocks = (sets + iters - 1) / iters;
+            // Few sets, with two register sets: as many blocks as are resident (four per SM) and their sets one grid apart, since blocks
+            // of consecutive sets then end in a round that is nearly empty (7168 x 4096 BF16, 6 sets a block: 19.55 us, apart 18.7;
+            // 8192 x 64 4.5 and 4.1).  With more than eight a block consecutive sets are faster (12288 x 4096 BF16, 10 a block: 27.7,
+            // apart 28.7; 28672 x 8192, 48 a block, under hybrid rounding with given exponents 158 and 168).  (An instantiation: a stride that is
+            // an argument cost the other calls 2 to 10 %.)
+            const long long resident = (long long)pl.sms * 4;
+            const bool apart = nv <= (long long)kUnroll * gs && sets > resident && sets <= 8 * resident;
+            if (apart) iters = (int)((sets + resident - 1) / resident);
+            const long long blocks = apart ? resident : (sets + iters - 1) / iters;
             if (blocks > 0x7FFFFFFFll) return HIF8_ERR_SHAPE;
-            if (nv <= (long long)kUnroll * gs) launch_pdl(row_channel_kernel<SRC, MODE, kUnroll>, (unsigned)blocks, st, p, gs, iters);
+            if (apart) launch_pdl(row_channel_kernel<SRC, MODE, kUnroll, true>, (unsigned)blocks, st, p, gs, iters);
+            else if (nv <= (long long)kUnroll * gs) launch_pdl(row_channel_kernel<SRC, MODE, kUnroll>, (unsigned)blocks, st, p, gs, iters);
             else launch_pdl(row_channel_kernel<SRC, MODE, kRowCache>, (unsigned)blocks, st, p, gs, iters);
         }
     } else {

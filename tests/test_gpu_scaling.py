@@ -73,6 +73,18 @@ def test_channel_encode_large(axis, dtype, shape):
     assert np.array_equal(q, O.channel_encode(x, dtype, axis, se_o, rnd=H.RND_HR, quick=True))
 
 
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16])
+@pytest.mark.parametrize("sets", [592, 593, 1184, 1185, 8 * 592, 8 * 592 + 1])
+def test_channel_encode_rows_by_sets_per_block(sets, dtype):
+    # around the sizes where a block takes one set of eight short rows, several that lie one grid apart, or consecutive ones
+    # (592 blocks are resident on 148 SMs); the last set is not full
+    x = weight(8 * sets - 3, 64, seed=sets, dtype=dtype)
+    q, amax, se = run_channel(x, dtype, 0)
+    amax_o, se_o = O.channel_amax_scale(x, dtype, 0, 14)
+    assert np.array_equal(amax, amax_o) and np.array_equal(se, se_o)
+    assert np.array_equal(q, O.channel_encode(x, dtype, 0, se_o, quick=True))
+
+
 @pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("axis", [0, 1])
 @pytest.mark.parametrize("dtype", [H.F32, H.BF16])
