@@ -315,20 +315,20 @@ __device__ const Bf16OfCode g_bf16_of_code = make_bf16_of_code();
 
 // Fills the decode table: entry (code c, lane l) at word c * ROW_WORDS + l holds the BF16 bits of code c (one copy per
 // lane, so that a warp's lookups never meet in a bank).  A warp writes four rows per step, eight lanes with 16 bytes each to
-// a row; at most three steps for the 22 warps or more of a block, their values loaded together.  (What runs once at the head
+// a row; STEPS steps, their values loaded together (three for the 22 warps or more of most blocks).  (What runs once at the head
 // of a kernel costs its instruction fetches above all, so the values come from a table in global memory and not from the
 // field definitions: 1050 -> 600 cycles; eight warps with 32 codes each, handed round by shuffles, took 1300.)
-template <int ROW_WORDS>
+template <int ROW_WORDS, int STEPS = 3>
 __device__ __forceinline__ void fill_decode_table(uint32_t* table, int warp, int lane, int n_warps)
 {
-    uint32_t v[3];
+    uint32_t v[STEPS];
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
+    for (int k = 0; k < STEPS; k++) {
         const int i = warp + k * n_warps;
         v[k] = i < 64 ? __ldg(g_bf16_of_code.v + 4 * i + (lane >> 3)) : 0u;
     }
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
+    for (int k = 0; k < STEPS; k++) {
         const int i = warp + k * n_warps;
         if (i < 64) *reinterpret_cast<uint4*>(table + (4 * i + (lane >> 3)) * ROW_WORDS + (lane & 7) * 4) = make_uint4(v[k], v[k], v[k], v[k]);
     }
@@ -489,6 +489,8 @@ __device__ __forceinline__ void apply_channel_scale(const GemmParams& p, int col
                                __uint_as_float((uint32_t)(s2 + 127) << 23));
     }
 }
+
+#include "hif8_gemm_warp.cuh"
 
 // ---------------------------------------------------------------------------------------------------------
 // Narrow products (M <= 64 rows of activations: the decode phase of inference).  The product is bound by reading the
@@ -2048,6 +2050,7 @@ struct GemmDeviceSetup {
     cudaError_t rc;
     int sm_count;
     int nw_clusters[kNwMaxSplit + 1];  // clusters of s CTAs of the narrow kernel, s = 1, 2, 4, 8
+    int wp_clusters[kWarpMaxCluster + 1];  // clusters of s blocks of hif8_gemm_warp_kernel, s = 1 .. 8
     int wd_clusters[kWdMaxSplit + 1];  // clusters of s pairs of hif8_gemm_weights_kernel that fit on the device at once, s = 1, 2, 4
 };
 PerDevice<GemmDeviceSetup> g_gemm_setup;
@@ -2060,7 +2063,13 @@ void weights_kernels(const void** k)
     k[4] = (const void*)hif8_gemm_weights_kernel<false, kActColumns, FORM>; k[5] = (const void*)hif8_gemm_weights_kernel<true, kActColumns, FORM>;
 }
 
-bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nullptr, const int** nw_clusters = nullptr)
+template <int MT>
+void warp_kernels(const void** k)
+{
+    k[0] = (const void*)hif8_gemm_warp_kernel<false, false, MT>; k[1] = (const void*)hif8_gemm_warp_kernel<true, false, MT>;
+}
+
+bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nullptr, const int** nw_clusters = nullptr, const int** wp_clusters = nullptr)
 {
     const GemmDeviceSetup* s = g_gemm_setup.get(dev, [](int d, GemmDeviceSetup* out) {
         out->rc = cudaSuccess;
@@ -2098,12 +2107,28 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
             cfg.attrs = attr; cfg.numAttrs = 1;
             out->rc = cudaOccupancyMaxActiveClusters(&out->nw_clusters[s], narrow[7], &cfg);
         }
+        std::memset(out->wp_clusters, 0, sizeof out->wp_clusters);
+        const void* wp[8];
+        warp_kernels<1>(wp); warp_kernels<2>(wp + 2); warp_kernels<4>(wp + 4);
+        wp[6] = (const void*)hif8_gemm_warp_kernel<false, true, 4>; wp[7] = (const void*)hif8_gemm_warp_kernel<true, true, 4>;
+        for (int i = 0; i < 8 && out->rc == cudaSuccess; i++)
+            out->rc = cudaFuncSetAttribute(wp[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
+        for (int s = 1; s <= kWarpMaxCluster && out->rc == cudaSuccess; s++) {
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = s; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            cfg.gridDim = dim3(s); cfg.blockDim = dim3(kWarpThreads); cfg.dynamicSmemBytes = kSmemBytesMax;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            out->rc = cudaOccupancyMaxActiveClusters(&out->wp_clusters[s], wp[7], &cfg);
+        }
         if (out->rc == cudaSuccess) out->rc = cudaDeviceGetAttribute(&out->sm_count, cudaDevAttrMultiProcessorCount, d);
     });
     if (!s) return false;
     *sm_count_out = s->sm_count;
     if (wd_clusters) *wd_clusters = s->wd_clusters;
     if (nw_clusters) *nw_clusters = s->nw_clusters;
+    if (wp_clusters) *wp_clusters = s->wp_clusters;
     return s->rc == cudaSuccess && s->sm_count > 0 && s->wd_clusters[1] > 0;
 }
 
@@ -2180,18 +2205,19 @@ int launch_bf16_pair_gemm(const void* a_bf, const void* w_bf, int w_is_nk, GemmP
 
 using namespace hif8;
 
-// Time of the weights kernel in cycles, from measurements: a k-block (64 k with activations as bytes, 128 k otherwise) and a
-// tile's drain; what the exchange of a split tile costs beyond that (two cluster barriers, the sums at 20 bytes a cycle, less
-// what the shared epilogue saves) at bn = 256, about half of it at 128; a launch of its own for the last round (set-up, first
-// copies).
+// Time of the weights kernel in cycles, from measurements: a k-block (128 k with expanded activations; 64 k with bytes, where the
+// activations' lookups count too) and a tile's drain; what the exchange of a split tile costs beyond that (two cluster barriers,
+// the sums at 20 bytes a cycle, less what the shared epilogue saves) at bn = 256, about half of it at 128; a launch of its own for
+// the last round (set-up, first copies).
 struct WeightsCost {
     int num_kb, bn;
+    bool expanded;
     const int* clusters;  // clusters of s pairs that the device holds
-    static constexpr double kblock = 1150.0;
     double tiles(long long n, int split) const
     {
         if (split > num_kb || clusters[split] <= 0) return 1e30;
         const double f = bn / 256.0, exchange = split == 1 ? 0.0 : (split == 2 ? 1300.0 + 2000.0 * f : 2100.0 + 5300.0 * f);
+        const double kblock = expanded ? 1150.0 : 730.0 + 270.0 * f;
         return (double)((n + clusters[split] - 1) / clusters[split]) * ((num_kb + split - 1) / split * kblock + 5000.0 * f + exchange);
     }
     int best_split(long long n) const
@@ -2216,18 +2242,28 @@ struct WeightsCost {
     }
 };
 
+// How the weights kernel divides a product for one form of the activations.  Pieces of up to 256 activation rows, a multiple of 32
+// (of 128 as bytes [K,M]: whole 64-column atoms per CTA): as few as possible, or, where that leaves the device idle, more and
+// smaller ones, which need no exchange between pairs (256 x 768 x 1536 with bytes, one piece split in four 12.8 us, four pieces
+// split in four 9.9; 128 x 512 x 512 9.1 in one piece, 6.9 in four).
 struct WeightsTiling {
-    int chunks, bn;
-    long long tiles;
-    WeightsCost cost;
-    WeightsTiling(int M, int N, int K, int act, const int* clusters)
+    int act = kActExpanded, chunks = 0, bn = 0;
+    long long tiles = 0;
+    WeightsCost cost{};
+    double cycles = 1e30;  // of the kernel and of the launch that expands the activations, from call to results
+    WeightsTiling() = default;
+    WeightsTiling(int M, int N, int K, int act_, bool a_is_km, const int* clusters) : act(act_)
     {
-        // activation rows in pieces of at most 256, a multiple of 32 (of 128 as bytes [K,M]: whole 64-column atoms per CTA)
-        const int unit = act == kActColumns ? 128 : 32, kb = act == kActExpanded ? 2 * BK : BK;
-        chunks = (M + BN - 1) / BN;
-        bn = ((M + chunks - 1) / chunks + unit - 1) / unit * unit;
-        tiles = (long long)((N + 2 * BM - 1) / (2 * BM)) * chunks;
-        cost = WeightsCost{(K + kb - 1) / kb, bn, clusters};
+        const int unit = act == kActColumns ? 128 : 32, kb = act == kActExpanded ? 2 * BK : BK, least = (M + BN - 1) / BN;
+        const long long slabs = (N + 2 * BM - 1) / (2 * BM);
+        // (the launch that expands, its passing over to the kernel, and 1 / 430 or, transposed, 1 / 260 of a cycle per element)
+        const double before = act == kActExpanded ? 11000.0 + (double)M * K * (a_is_km ? 0.0039 : 0.0023) : 7500.0;
+        for (int pieces = least; pieces == least || (slabs * pieces <= clusters[1] && (pieces - 1) * unit < M); pieces++) {
+            const int rows = ((M + pieces - 1) / pieces + unit - 1) / unit * unit, n = (M + rows - 1) / rows;
+            const WeightsCost c{(K + kb - 1) / kb, rows, act == kActExpanded, clusters};
+            const double t = before + c.all(slabs * n);
+            if (t < cycles) { cycles = t; chunks = n; bn = rows; tiles = slabs * n; cost = c; }
+        }
     }
 };
 
@@ -2250,11 +2286,10 @@ static cudaError_t launch_weights_kernel(const cudaLaunchConfig_t& cfg, int w_is
 
 // C = A W with the weights decoded inside the kernel.  act = kActExpanded: `a` is BF16 [M,K], written by the launch in front of
 // this one, which also clears the status word; otherwise the caller's bytes.
-static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, int act, const void* a, int64_t lda, const GemmParams& p, const int* clusters,
-                               cudaStream_t st)
+static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, const WeightsTiling& tl, const void* a, int64_t lda, const GemmParams& p,
+                               const int* clusters, cudaStream_t st)
 {
-    const int M = p.M, N = p.N, K = p.K, kb = act == kActExpanded ? 2 * BK : BK;
-    const WeightsTiling tl(M, N, K, act, clusters);
+    const int M = p.M, N = p.N, K = p.K, act = tl.act, kb = act == kActExpanded ? 2 * BK : BK;
     if (tl.tiles > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
     const int tiles = (int)tl.tiles, pairs = clusters[1];
     CUtensorMap map_w, map_act;
@@ -2298,12 +2333,158 @@ static cudaError_t launch_narrow_kernel(const cudaLaunchConfig_t& cfg, bool clus
                    : cudaLaunchKernelEx(&cfg, hif8_gemm_narrow_kernel<W_IS_NK, ACT_BF16, false>, map_act, map_w, p, mp, plan);
 }
 
+// How the warp kernel divides a product, and what that takes in cycles from call to results.  The terms are fitted to 670 measured
+// calls (1 to 256 rows, N and K 512 to 8192, all divisions; within 15 % of most): the activations that a block decodes, the weights
+// that go through its shared memory, deposits, and what a unit costs a warp one after the other.
+struct WarpTiling {
+    WarpPlan plan{};
+    int mt = 0, row_blocks = 0;
+    double cycles = 1e30;
+    WarpTiling() = default;
+    WarpTiling(int M, int N, int K, bool w_is_nk, bool a_is_km, const int* clusters)
+    {
+        if ((double)M * N * K > 4e9 || K > 4096 * kWarpMaxCluster || (!w_is_nk && (N & 3))) return;  // (far beyond what it is good for; a thread loads four columns of [K,N] in one piece)
+        for (int m = a_is_km ? 4 : 1; m <= 4; m *= 2)
+            if (m == 1 ? M <= 8 : (a_is_km || 4 * m < M)) divide(M, N, K, w_is_nk, m, clusters);
+    }
+    void divide(int M, int N, int K, bool w_is_nk, int m, const int* clusters)
+    {
+        const int blocks = (M + 8 * m - 1) / (8 * m), ut = w_is_nk ? 1 : 2, max_chunks = (w_is_nk ? 4 : 2) / (m == 4 ? 2 : 1), cols = 16 * ut;
+        const int units = (N + cols - 1) / cols, kb = (K + 63) / 64;
+        const uint32_t deposit = (uint32_t)(cols * 8 * m * 4);
+        for (int c = 1; c <= kWarpMaxCluster; c++) {
+            if (clusters[c] <= 0) continue;
+            const int fit = clusters[c] / blocks, n = fit < 1 ? 1 : (fit < units ? fit : units), nu = (units + n - 1) / n;
+            const int rounds = fit < 1 ? (blocks + clusters[c] - 1) / clusters[c] : 1;
+            if ((uint32_t)(units / n + 1) * deposit > kWarpSumBytes) continue;
+            for (int s = 1; s <= kWarpWarps; s++) {
+                const int chunks = (kb + c * s - 1) / (c * s), lanes = kWarpWarps / s;
+                if (chunks > max_chunks || (kb + chunks - 1) / chunks <= (c - 1) * s) continue;  // (the latter: a block of the cluster without work)
+                const int turns = (nu + lanes - 1) / lanes, active = s * (lanes < nu ? lanes : nu);
+                const double t = rounds * (w_is_nk ? 3500.0 + 40.0 * active * chunks * m + 46.0 * nu * s * m + 450.0 * turns + 890.0 * turns * chunks + (c > 1 ? 4100.0 : 0.0)
+                                                   : 3300.0 + 24.0 * active * chunks * m + 122.0 * nu * s * chunks + 34.0 * nu * s * m + 970.0 * turns +
+                                                         1240.0 * turns * chunks + (c > 1 ? 4400.0 : 0.0));
+                if (t < cycles) {
+                    cycles = t; mt = m; row_blocks = blocks;
+                    plan.chunks = chunks; plan.slices = s; plan.lanes = lanes; plan.cluster = c; plan.units = units;
+                    plan.q = units / n; plan.rem = units % n;
+                }
+            }
+        }
+    }
+    int clusters_used() const { return plan.q > 0 ? (plan.units - plan.rem) / plan.q : plan.rem; }
+};
+
+template <int MT>
+static cudaError_t launch_warp_kernel(const cudaLaunchConfig_t& cfg, bool w_is_nk, const uint8_t* A, long long lda, const uint8_t* W, long long ldw,
+                                      const GemmParams& p, const WarpPlan& plan)
+{
+    return w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_warp_kernel<true, false, MT>, A, lda, W, ldw, p, plan)
+                   : cudaLaunchKernelEx(&cfg, hif8_gemm_warp_kernel<false, false, MT>, A, lda, W, ldw, p, plan);
+}
+
+static int launch_warp_gemm(const uint8_t* A, int64_t lda, int a_is_km, const uint8_t* W, int64_t ldw, int w_is_nk, const GemmParams& p, const WarpTiling& tl,
+                            cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(tl.clusters_used() * tl.plan.cluster), (unsigned)tl.row_blocks);
+    cfg.blockDim = dim3(kWarpThreads);
+    cfg.dynamicSmemBytes = kSmemBytesMax;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)tl.plan.cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = tl.plan.cluster > 1 ? 2 : 1;
+    cudaError_t rc;
+    if (a_is_km)
+        rc = w_is_nk ? cudaLaunchKernelEx(&cfg, hif8_gemm_warp_kernel<true, true, 4>, A, (long long)lda, W, (long long)ldw, p, tl.plan)
+                     : cudaLaunchKernelEx(&cfg, hif8_gemm_warp_kernel<false, true, 4>, A, (long long)lda, W, (long long)ldw, p, tl.plan);
+    else if (tl.mt == 1) rc = launch_warp_kernel<1>(cfg, w_is_nk, A, lda, W, ldw, p, tl.plan);
+    else if (tl.mt == 2) rc = launch_warp_kernel<2>(cfg, w_is_nk, A, lda, W, ldw, p, tl.plan);
+    else rc = launch_warp_kernel<4>(cfg, w_is_nk, A, lda, W, ldw, p, tl.plan);
+    if (rc != cudaSuccess) return HIF8_ERR_CUDA;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+}
+
 static std::atomic<int> g_path_policy{HIF8_GEMM_PATH_AUTO};
 
 extern "C" int hif8_gemm_path_policy(int policy)
 {
     if (policy != HIF8_GEMM_PATH_AUTO && policy != HIF8_GEMM_PATH_EXPAND_BOTH) return HIF8_ERR_FLAGS;
     return g_path_policy.exchange(policy, std::memory_order_relaxed);
+}
+
+// How the narrow kernel divides a product.  Cycles: a k-block takes about 500 (mp = 16) to 590 (64); a cluster's exchange 4000, and
+// clusters of eight start later; ranges of slabs end in a reduction of 2500 + 290 mp.  A cluster per slab (or one CTA: split 1), or,
+// when the workspace holds the partial sums of the slabs that a range boundary cuts, one CTA per SM with equal ranges: for many
+// slabs that do not divide among the SMs, and few rows.
+struct NarrowTiling {
+    int split = 0;         // of the best clusters
+    bool ranges = false;   // ranges are better
+    long long grid = 0, pmax = 0;
+    double cycles = 1e30;
+    NarrowTiling(int M, int N, int K, int sm_count, const int* clusters, bool with_ranges)
+    {
+        const int mp = (M + 15) & ~15;
+        const long long slabs = (N + BM - 1) / BM, num_pb = (K + BK2 - 1) / BK2, total = slabs * num_pb;  // pair blocks: two k-blocks
+        const double c_pb = 2.0 * (470.0 + 1.9 * mp);
+        for (int s = 1; s <= kNwMaxSplit && s <= num_pb; s *= 2) {
+            if (clusters[s] <= 0) continue;
+            const long long rounds = (slabs + clusters[s] - 1) / clusters[s];
+            const double c = (double)rounds * ((double)((num_pb + s - 1) / s) * c_pb + 4500.0 + (s == 1 ? 0.0 : (s < 8 ? 4000.0 : 6000.0)));
+            if (c < cycles) { cycles = c; split = s; }
+        }
+        // four or more pair blocks per CTA, but never fewer CTAs than slabs
+        grid = total / 4 < sm_count ? total / 4 : sm_count;
+        const long long floor_g = slabs < sm_count ? slabs : sm_count;
+        if (grid < floor_g) grid = floor_g;
+        const long long per = total / grid;
+        pmax = (num_pb + per - 1) / per + 1;
+        const double c = (double)(per + 1) * c_pb + 4500.0 + 2500.0 + 290.0 * mp;
+        if (with_ranges && c < cycles) { cycles = c; ranges = true; }
+    }
+};
+
+// Which kernel takes a product, and how it divides it: a function of the sizes, the layouts and what the workspace has room for, so
+// it is worked out once for each (the search over divisions takes a few microseconds).
+enum GemmForm { kFormWarp, kFormNarrow, kFormWeights, kFormPair };
+struct GemmKey {
+    int M, N, K, dev, w_is_nk, a_is_km, room, policy;
+};
+struct GemmChoice {
+    GemmForm form;
+    WarpTiling warp;
+    WeightsTiling weights;
+};
+static LruCache<GemmKey, GemmChoice, 64> g_choices;
+
+static bool choose(const GemmKey& k, int sm_count, const int* wd_clusters, const int* nw_clusters, const int* wp_clusters, GemmChoice* out)
+{
+    const bool narrow = !k.a_is_km && k.M <= kNarrowMaxM;
+    out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters);
+    const WeightsTiling bytes(k.M, k.N, k.K, k.a_is_km ? kActColumns : kActRows, k.a_is_km, wd_clusters);
+    const WeightsTiling expanded(k.M, k.N, k.K, kActExpanded, k.a_is_km, wd_clusters);
+    out->weights = k.room && expanded.cycles < bytes.cycles ? expanded : bytes;
+    out->form = narrow ? kFormNarrow : kFormWeights;
+    // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element moved, at
+    // 3300 bytes a cycle, and a launch) by the cheaper k-blocks and tiles of the pair kernel: 545 cycles per
+    // 64 k and nothing between tiles, against the weights kernel's cost above.  Measured (us, both expanded / weights decoded in
+    // the kernel): 2048 x 7168 x 4096 105 / 98, 3072 rows 130 / 133, 4096 rows 172 / 176; 1536 x 8192 x 1024 28.5 / 33;
+    // 2048 x 16384 x 8192 381 / 357, 4096 rows 702 / 732.
+    const long long pair_rounds = ((long long)((k.M + 2 * BM - 1) / (2 * BM)) * ((k.N + BN - 1) / BN) + sm_count / 2 - 1) / (sm_count / 2);
+    const double expand_w = 6000.0 + 3.0 * (double)k.K * k.N / 3300.0, pair_cycles = (double)pair_rounds * ((k.K + BK - 1) / BK * 545.0 + 500.0);
+    if (!narrow && k.room == 2 && (k.policy == HIF8_GEMM_PATH_EXPAND_BOTH ||
+                                   expand_w + pair_cycles < 1.03 * expanded.cost.all(expanded.tiles))) {  // (equal at 1.03: the lookups also cost clock under the power limit)
+        out->form = kFormPair;
+        return true;
+    }
+    // (1.08: the search takes the division whose time is underestimated most; 6000: the launch in front of the narrow kernel, its start and end)
+    const double other = narrow ? NarrowTiling(k.M, k.N, k.K, sm_count, nw_clusters, k.room > 0).cycles + 6000.0 : out->weights.cycles;
+    if (1.08 * out->warp.cycles < other) out->form = kFormWarp;
+    return true;
 }
 
 static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t* Wq, int64_t ldw, int w_is_nk, void* C,
@@ -2337,13 +2518,29 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     note_status_word(st, reinterpret_cast<const int*>(workspace));
 
     int sm_count = 0;
-    const int *wd_clusters = nullptr, *nw_clusters = nullptr;
-    if (!gemm_kernels_ready(dev, &sm_count, &wd_clusters, &nw_clusters)) return HIF8_ERR_CUDA;
+    const int *wd_clusters = nullptr, *nw_clusters = nullptr, *wp_clusters = nullptr;
+    if (!gemm_kernels_ready(dev, &sm_count, &wd_clusters, &nw_clusters, &wp_clusters)) return HIF8_ERR_CUDA;
+
+
+    // Operands as BF16 in the workspace: none, the activations, both.
+    const size_t bytes_a = (((size_t)M * K * 2) + 255) & ~(size_t)255, bytes_w = (((size_t)K * N * 2) + 255) & ~(size_t)255;
+    const bool a_contiguous = lda == (a_is_km ? M : K), w_contiguous = ldw == (w_is_nk ? K : N), ws_aligned = !(reinterpret_cast<uintptr_t>(workspace) & 255);
+    const bool room_a = a_contiguous && ws_aligned && workspace_bytes >= kGemmWorkspaceBytes + bytes_a;
+    const bool room_w = room_a && w_contiguous && workspace_bytes >= kGemmWorkspaceBytes + bytes_a + bytes_w;
+    GemmKey key;
+    std::memset(&key, 0, sizeof key);
+    key.M = M; key.N = N; key.K = K; key.dev = dev;
+    key.w_is_nk = w_is_nk != 0; key.a_is_km = a_is_km != 0; key.room = room_w ? 2 : (room_a ? 1 : 0);
+    key.policy = g_path_policy.load(std::memory_order_relaxed);
+    GemmChoice choice;
+    if (!g_choices.lookup_or_make(key, &choice, [&](const GemmKey& k, GemmChoice* out) { return choose(k, sm_count, wd_clusters, nw_clusters, wp_clusters, out); }))
+        return HIF8_ERR_SHAPE;
+    if (choice.form == kFormWarp) return launch_warp_gemm(Aq, lda, a_is_km, Wq, ldw, w_is_nk, p, choice.warp, st);
     // the status word is cleared on the stream before the kernels; the narrow path clears its tickets in the same operation
     size_t clear_bytes = 4;
 
     // Narrow products: the weight-streaming kernel, whatever the workspace
-    if (!a_is_km && M <= kNarrowMaxM) {
+    if (choice.form == kFormNarrow) {
         const int mp = (M + 15) & ~15;
         CUtensorMap map_act, map_ws;
         if (!make_map(&map_act, Aq, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK2, (uint32_t)mp)) return HIF8_ERR_CUDA;
@@ -2355,36 +2552,19 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         NarrowPlan plan{};
         const long long total = slabs * num_pb;
         if (total > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
-        // Cycles: a k-block takes about 500 (mp = 16) to 590 (64); a cluster's exchange 4000, and clusters of eight start later;
-        // ranges of slabs end in a reduction of 2500 + 290 mp.  A cluster per slab (or one CTA: split 1), or, when the workspace
-        // holds the partial sums of the slabs that a range boundary cuts, one CTA per SM with equal ranges: for many slabs that do
-        // not divide among the SMs, and few rows.
-        const double c_pb = 2.0 * (470.0 + 1.9 * mp);
-        double best = 1e30;
-        for (int s = 1; s <= kNwMaxSplit && s <= num_pb; s *= 2) {
-            if (nw_clusters[s] <= 0) continue;
-            const long long rounds = (slabs + nw_clusters[s] - 1) / nw_clusters[s];
-            const double c = (double)rounds * ((double)((num_pb + s - 1) / s) * c_pb + 4500.0 + (s == 1 ? 0.0 : (s < 8 ? 4000.0 : 6000.0)));
-            if (c < best) { best = c; plan.split = s; }
-        }
+        const NarrowTiling nt(M, N, K, sm_count, nw_clusters, true);
+        plan.split = nt.split;
         long long grid = slabs * plan.split;
-        {
-            // four or more pair blocks per CTA, but never fewer CTAs than slabs
-            long long g = total / 4 < sm_count ? total / 4 : sm_count;
-            const long long floor_g = slabs < sm_count ? slabs : sm_count;
-            if (g < floor_g) g = floor_g;
-            const long long per = total / g;
-            const long long pmax = (num_pb + per - 1) / per + 1;
+        if (nt.ranges) {
             const size_t ticket_bytes = (((size_t)slabs * kEpiWarps * 4) + 255) & ~(size_t)255;
-            const size_t part_bytes = (size_t)slabs * pmax * mp * BM * 4;
-            const double c = (double)(per + 1) * c_pb + 4500.0 + 2500.0 + 290.0 * mp;
-            if (c < best && workspace_bytes >= kGemmWorkspaceBytes + ticket_bytes + part_bytes && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
+            const size_t part_bytes = (size_t)slabs * nt.pmax * mp * BM * 4;
+            if (workspace_bytes >= kGemmWorkspaceBytes + ticket_bytes + part_bytes && ws_aligned) {
                 unsigned char* wsb = reinterpret_cast<unsigned char*>(workspace) + kGemmWorkspaceBytes;
                 plan.tickets = reinterpret_cast<unsigned*>(wsb);
                 plan.part = reinterpret_cast<float*>(wsb + ticket_bytes);
-                plan.pmax = (int)pmax;
+                plan.pmax = (int)nt.pmax;
                 plan.split = 0;
-                grid = g;
+                grid = nt.grid;
                 clear_bytes = kGemmWorkspaceBytes + ticket_bytes;  // the tickets follow the status block
             }
         }
@@ -2435,37 +2615,18 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
     }
 
-    // Decode-once path: with room for both operands as BF16 in the workspace (and contiguous operands), each HiF8
-    // byte is decoded exactly once by the conversion kernel and the tensor-core kernel reads BF16 tiles through TMA.
-    // Otherwise the weights are decoded inside the tensor-core kernel, and the activations too when there is no room for them.
-    const size_t bytes_a = (((size_t)M * K * 2) + 255) & ~(size_t)255, bytes_w = (((size_t)K * N * 2) + 255) & ~(size_t)255;
-    const bool a_contiguous = lda == (a_is_km ? M : K), w_contiguous = ldw == (w_is_nk ? K : N);
-    // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element moved, at
-    // 3300 bytes a cycle, and a launch) by the cheaper k-blocks and tiles of the pair kernel: 545 cycles per
-    // 64 k and nothing between tiles, against the weights kernel's cost above.  Measured (us, both expanded / weights decoded in
-    // the kernel): 2048 x 7168 x 4096 105 / 98, 3072 rows 130 / 133, 4096 rows 172 / 176; 1536 x 8192 x 1024 28.5 / 33;
-    // 2048 x 16384 x 8192 381 / 357, 4096 rows 702 / 732.
-    const WeightsTiling tl(M, N, K, kActExpanded, wd_clusters);
-    const long long pair_rounds = ((long long)((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN) + sm_count / 2 - 1) / (sm_count / 2);
-    const double expand_w = 6000.0 + 3.0 * (double)K * N / 3300.0, pair_cycles = (double)pair_rounds * ((K + BK - 1) / BK * 545.0 + 500.0);
-    const bool w_expansion_pays = g_path_policy.load(std::memory_order_relaxed) == HIF8_GEMM_PATH_EXPAND_BOTH ||
-                                  expand_w + pair_cycles < 1.03 * tl.cost.all(tl.tiles);  // (equal at 1.03: the lookups also cost clock under the power limit)
-    if (a_contiguous && workspace_bytes >= kGemmWorkspaceBytes + bytes_a && !(reinterpret_cast<uintptr_t>(workspace) & 255)) {
-        unsigned char* a_bf = reinterpret_cast<unsigned char*>(workspace) + kGemmWorkspaceBytes;
-        // (an A given as [K,M] is written as [M,K] while it is expanded; either launch clears the status word)
-        int rc = HIF8_OK;
-        if (a_is_km) rc = decode_transpose_bf16(Aq, a_bf, K, M, reinterpret_cast<uint32_t*>(workspace), st);
-        else if (launch_expand_activations(Aq, a_bf, (unsigned long long)M * K, workspace, 4, sm_count, st) != cudaSuccess) rc = HIF8_ERR_CUDA;
-        if (rc != HIF8_OK) return rc;
-        if (w_contiguous && w_expansion_pays && workspace_bytes >= kGemmWorkspaceBytes + bytes_a + bytes_w) {
-            unsigned char* w_bf = a_bf + bytes_a;
-            rc = hif8_decode(Wq, w_bf, HIF8_BF16, (size_t)K * N, 0, stream);
-            return rc != HIF8_OK ? rc : launch_bf16_pair_gemm(a_bf, w_bf, w_is_nk, p, st);
-        }
-        return launch_weights_gemm(Wq, ldw, w_is_nk, kActExpanded, a_bf, K, p, wd_clusters, st);
-    }
-    // No room for the activations: both operands are decoded in the kernel.
-    return launch_weights_gemm(Wq, ldw, w_is_nk, a_is_km ? kActColumns : kActRows, Aq, lda, p, wd_clusters, st);
+    if (choice.form == kFormWeights && choice.weights.act != kActExpanded) return launch_weights_gemm(Wq, ldw, w_is_nk, choice.weights, Aq, lda, p, wd_clusters, st);
+    // The activations are expanded once (an A given as [K,M] is written as [M,K] meanwhile); either launch clears the status word.
+    // For the pair kernel the weights too: each HiF8 byte is then decoded exactly once.
+    unsigned char* a_bf = reinterpret_cast<unsigned char*>(workspace) + kGemmWorkspaceBytes;
+    int rc = HIF8_OK;
+    if (a_is_km) rc = decode_transpose_bf16(Aq, a_bf, K, M, reinterpret_cast<uint32_t*>(workspace), st);
+    else if (launch_expand_activations(Aq, a_bf, (unsigned long long)M * K, workspace, 4, sm_count, st) != cudaSuccess) rc = HIF8_ERR_CUDA;
+    if (rc != HIF8_OK) return rc;
+    if (choice.form == kFormWeights) return launch_weights_gemm(Wq, ldw, w_is_nk, choice.weights, a_bf, K, p, wd_clusters, st);
+    unsigned char* w_bf = a_bf + bytes_a;
+    rc = hif8_decode(Wq, w_bf, HIF8_BF16, (size_t)K * N, 0, stream);
+    return rc != HIF8_OK ? rc : launch_bf16_pair_gemm(a_bf, w_bf, w_is_nk, p, st);
 }
 
 extern "C" int hif8_gemm(const uint8_t* Aq, int64_t lda, const uint8_t* Wq, int64_t ldw, int w_is_nk, void* C, int64_t ldc,
