@@ -1170,6 +1170,11 @@ struct TilePlan {
     int slabs;
     int split;
     int clear_status;  // nonzero: no launch in front of this one clears the status word
+    // nonzero: the launch in front of this one is the same product's other tiles.  It lets this one start once everything before itself
+    // is complete, so nothing is waited for at the start, and its end at this one's end, for whoever comes after.
+    int follows;
+    // kParts: `first` and `count` are in parts of tiles, `parts` to a tile, whose activation rows are `tile_rows`; bn is a part's
+    int parts, tile_rows;
 };
 
 // Eight finished sums of this thread's weight column, activation rows m .. m + 7 of which `rows` exist, to C: `out` is the
@@ -1217,7 +1222,10 @@ __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, i
 
 // Instantiations by tile order and row pitch.  (With the choice of the order made in the kernel, the divisions of the other one in
 // the way of the first copies, 128 x 512 x 512 took 10.0 us instead of 9.8.)
-enum WeightsForm { kOneGroup, kGroups, kFarRows };  // up to eight pieces; more; the rows of C 4 GiB apart or more (any number of pieces)
+// kParts is the last, incomplete round of a large product in tiles of fewer activation rows: divided along K alone, two tiles of
+// 2048 x 7168 x 4096 kept 8 pairs of 74 busy (with it 104 -> 101.5 us, with activations as bytes 144 -> 140; that launch waits for
+// nothing of the one in front of it, see TilePlan::follows, which is 1 us of it).
+enum WeightsForm { kOneGroup, kGroups, kFarRows, kParts };  // up to eight pieces; more; the rows of C 4 GiB apart or more (any number of pieces); parts of tiles
 constexpr int kGroupPieces = 8;
 
 template <bool W_IS_NK, int ACT, int FORM>
@@ -1266,8 +1274,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         if (FORM == kOneGroup) {
             slab = t / tp.chunks;
             piece = t - slab * tp.chunks;
-        } else tile_coords(t, tp.chunks, tp.slabs, piece, slab);
-        m0 = piece * tp.bn;
+        } else tile_coords(FORM == kParts ? t / tp.parts : t, tp.chunks, tp.slabs, piece, slab);
+        m0 = FORM == kParts ? piece * tp.tile_rows + t % tp.parts * tp.bn : piece * tp.bn;
     };
     auto copy_bytes = [&](int it, int t, int kb) {  // tile t's bytes of k-block kb into stage it % kWdStages, which is free
         int slab, m0;
@@ -1309,7 +1317,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     const uint32_t tmem_base = *tmem_slot;
     if (ACT != kActExpanded) {
         // Nothing was launched in front of this kernel to order it behind what produces its operands.
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (!tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
         if (tp.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile int*>(p.status) = 0;  // (a wait gives up seconds later)
     }
 
@@ -1340,7 +1348,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         // 64 k (the swizzle span); both CTAs' copies complete on the leader's "operands ready" barrier
         cluster_wait();
         if (lane == 0) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
+            if (!tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             // A tile's barrier (in the pair's leader) counts the bytes of both CTAs' halves.  A thread that gives up tells the other CTA's
             // how many tiles it has issued, and the one that is behind issues its halves of the tiles that the other one
@@ -1515,7 +1523,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             // 2^sc as one factor, and a second one for the few scales that need it
             const int sc = -(sa + (p.d_sw_channel ? (n < p.N ? __ldg(p.d_sw_channel + n) : 0) : sw_all)), s1 = max(-126, min(126, sc));
             const float f1 = __uint_as_float((uint32_t)(s1 + 127) << 23), f2 = __uint_as_float((uint32_t)(sc - s1 + 127) << 23);
-            const int cols = min(tp.bn, p.M - m0), pieces = (cols + 7) / 8, per = split == 1 ? pieces : (pieces + split - 1) / split;
+            const int past = FORM == kParts ? min(p.M, (m0 / tp.tile_rows + 1) * tp.tile_rows) : p.M;  // (the last part of a tile may be a shorter one)
+            const int cols = max(0, min(tp.bn, past - m0)), pieces = (cols + 7) / 8, per = split == 1 ? pieces : (pieces + split - 1) / split;
             unsigned char* out = reinterpret_cast<unsigned char*>(p.C) + (long long)m0 * pitch + (long long)n * c_size;
             const bool ok = mbar_wait(bar_acc_full, local & 1, abort_flag, p.status, 47);
             if (!ok && split == 1) break;
@@ -1583,6 +1592,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
 
     // ---- teardown: all waits are bounded, so everybody arrives; nobody leaves while the peer may still read this
     // CTA's operands or signal its barriers; then the allocating warps free TMEM
+    if (tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();
@@ -2077,11 +2087,11 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
         std::memset(out->wd_clusters, 0, sizeof out->wd_clusters);
         std::memset(out->nw_clusters, 0, sizeof out->nw_clusters);
         const void* pair[2] = {(const void*)bf16_gemm_pair_kernel<false>, (const void*)bf16_gemm_pair_kernel<true>};
-        const void* wd[18];
-        weights_kernels<kOneGroup>(wd); weights_kernels<kGroups>(wd + 6); weights_kernels<kFarRows>(wd + 12);
+        const void* wd[24];
+        weights_kernels<kOneGroup>(wd); weights_kernels<kGroups>(wd + 6); weights_kernels<kFarRows>(wd + 12); weights_kernels<kParts>(wd + 18);
         for (int i = 0; i < 2 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(pair[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2);
-        for (int i = 0; i < 18 && out->rc == cudaSuccess; i++)
+        for (int i = 0; i < 24 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(wd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
         for (int s = 1; s <= kWdMaxSplit && out->rc == cudaSuccess; s *= 2) {
             cudaLaunchConfig_t cfg{};
@@ -2210,7 +2220,7 @@ using namespace hif8;
 // the sums at 20 bytes a cycle, less what the shared epilogue saves) at bn = 256, about half of it at 128; a launch of its own for
 // the last round (set-up, first copies).
 struct WeightsCost {
-    int num_kb, bn;
+    int num_kb, bn, unit;  // unit: the activation rows of a tile are a multiple of this
     bool expanded;
     const int* clusters;  // clusters of s pairs that the device holds
     double tiles(long long n, int split) const
@@ -2227,18 +2237,33 @@ struct WeightsCost {
             if (tiles(n, s) < tiles(n, best)) best = s;
         return best;
     }
-    // tiles of the last round that a launch of their own, split, finishes earlier (0: none)
-    long long remainder(long long n) const
+    // The tiles of the last, incomplete round, in a launch of their own when that finishes earlier: in parts of fewer activation
+    // rows, each split along K.
+    struct Rest {
+        long long tiles = 0;  // 0: no such launch
+        int parts = 1, rows = 0, split = 1;
+        double cycles = 0.0;
+    };
+    Rest rest(long long n) const
     {
+        Rest r;
         const long long rem = n > clusters[1] ? n % clusters[1] : 0;
-        if (!rem) return 0;
-        const int s = best_split(rem);
-        return s > 1 && tiles(rem, s) + 4200.0 < tiles(rem, 1) ? rem : 0;
+        if (!rem) return r;
+        r.cycles = tiles(rem, 1);
+        for (int want = 1; want <= 8; want *= 2) {
+            WeightsCost c = *this;
+            c.bn = (bn + want * unit - 1) / (want * unit) * unit;
+            const int parts = (bn + c.bn - 1) / c.bn, split = c.best_split(rem * parts);
+            const double t = c.tiles(rem * parts, split) + 4200.0;
+            if ((split > 1 || parts > 1) && rem * parts <= clusters[split] && t < r.cycles) r = Rest{rem, parts, c.bn, split, t};
+        }
+        return r;
     }
     double all(long long n) const
     {
-        const long long rem = remainder(n);
-        return n <= clusters[1] ? tiles(n, best_split(n)) : (rem ? tiles(n - rem, 1) + tiles(rem, best_split(rem)) + 4200.0 : tiles(n, 1));
+        if (n <= clusters[1]) return tiles(n, best_split(n));
+        const long long rem = n % clusters[1];
+        return tiles(n - rem, 1) + rest(n).cycles;
     }
 };
 
@@ -2260,7 +2285,7 @@ struct WeightsTiling {
         const double before = act == kActExpanded ? 11000.0 + (double)M * K * (a_is_km ? 0.0039 : 0.0023) : 7500.0;
         for (int pieces = least; pieces == least || (slabs * pieces <= clusters[1] && (pieces - 1) * unit < M); pieces++) {
             const int rows = ((M + pieces - 1) / pieces + unit - 1) / unit * unit, n = (M + rows - 1) / rows;
-            const WeightsCost c{(K + kb - 1) / kb, rows, act == kActExpanded, clusters};
+            const WeightsCost c{(K + kb - 1) / kb, rows, unit, act == kActExpanded, clusters};
             const double t = before + c.all(slabs * n);
             if (t < cycles) { cycles = t; chunks = n; bn = rows; tiles = slabs * n; cost = c; }
         }
@@ -2280,6 +2305,7 @@ static cudaError_t launch_weights_kernel(const cudaLaunchConfig_t& cfg, int w_is
                                          const TilePlan& tp)
 {
     if ((p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) return launch_weights_form<ACT, kFarRows>(cfg, w_is_nk, map_w, map_act, p, tp);
+    if (tp.parts > 1) return launch_weights_form<ACT, kParts>(cfg, w_is_nk, map_w, map_act, p, tp);
     return tp.chunks > kGroupPieces ? launch_weights_form<ACT, kGroups>(cfg, w_is_nk, map_w, map_act, p, tp)
                                     : launch_weights_form<ACT, kOneGroup>(cfg, w_is_nk, map_w, map_act, p, tp);
 }
@@ -2292,19 +2318,23 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
     const int M = p.M, N = p.N, K = p.K, act = tl.act, kb = act == kActExpanded ? 2 * BK : BK;
     if (tl.tiles > 0x3FFFFFFF) return HIF8_ERR_SHAPE;
     const int tiles = (int)tl.tiles, pairs = clusters[1];
-    CUtensorMap map_w, map_act;
+    CUtensorMap map_w;
     const bool okw = w_is_nk ? make_map(&map_w, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, (uint32_t)kb, BM, false, (uint32_t)kb)
                              : make_map(&map_w, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, (uint32_t)kb, false, 128);
-    const bool oka = act == kActExpanded ? make_map3(&map_act, a, (uint64_t)K, (uint64_t)M, 1, 0, BK, (uint32_t)tl.bn / 2)
-                     : act == kActRows   ? make_map(&map_act, a, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, (uint32_t)tl.bn / 2)
-                                         : make_map(&map_act, a, (uint64_t)M, (uint64_t)K, (uint64_t)lda, (uint32_t)tl.bn / 2, BK);
-    if (!okw || !oka) return HIF8_ERR_CUDA;
-    const int rem = (int)tl.cost.remainder(tiles), clear = act != kActExpanded;
+    if (!okw) return HIF8_ERR_CUDA;
+    WeightsCost::Rest rest = tl.cost.rest(tiles);
+    if (rest.parts > 1 && (p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) rest = WeightsCost::Rest{};  // (rows of C 4 GiB apart have an instantiation for whole tiles)
+    const int rem = (int)rest.tiles, clear = act != kActExpanded, slabs = tiles / tl.chunks;
     TilePlan launch[2];
-    launch[0] = TilePlan{0, tiles - rem, tl.chunks, tl.bn, tiles / tl.chunks, tiles <= pairs ? tl.cost.best_split(tiles) : 1, clear};
-    launch[1] = TilePlan{tiles - rem, rem, tl.chunks, tl.bn, tiles / tl.chunks, rem ? tl.cost.best_split(rem) : 1, 0};
+    launch[0] = TilePlan{0, tiles - rem, tl.chunks, tl.bn, slabs, tiles <= pairs ? tl.cost.best_split(tiles) : 1, clear, 0, 1, tl.bn};
+    launch[1] = TilePlan{(tiles - rem) * rest.parts, rem * rest.parts, tl.chunks, rest.rows, slabs, rest.split, 0, 1, rest.parts, tl.bn};
     for (int i = 0; i < (rem ? 2 : 1); i++) {
         const TilePlan& tp = launch[i];
+        CUtensorMap map_act;
+        const bool oka = act == kActExpanded ? make_map3(&map_act, a, (uint64_t)K, (uint64_t)M, 1, 0, BK, (uint32_t)tp.bn / 2)
+                         : act == kActRows   ? make_map(&map_act, a, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, (uint32_t)tp.bn / 2)
+                                             : make_map(&map_act, a, (uint64_t)M, (uint64_t)K, (uint64_t)lda, (uint32_t)tp.bn / 2, BK);
+        if (!oka) return HIF8_ERR_CUDA;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(2u * (unsigned)(tp.split > 1 ? tp.count * tp.split : (tp.count < pairs ? tp.count : pairs)));
         cfg.blockDim = dim3(kThreadsWd);

@@ -106,3 +106,28 @@ def test_gemm_pieces_of_activation_rows(shape, form):
     rows, cols = np.concatenate([rng.integers(0, M, 30000), np.repeat(np.arange(M), 16)]), np.concatenate([rng.integers(0, N, 30000), np.tile(np.arange(N - 16, N), M)])
     P, S = O.gemm_entries(Amk, Wkn, False, 0, 0, rows, cols)
     assert np.all(np.abs(C.cpu().numpy().astype(np.float64)[rows, cols] - P) <= 1e-5 * S)
+
+
+@pytest.mark.parametrize("accumulate", [0, 1])
+@pytest.mark.parametrize("form", ["rows", "columns", "expanded"])
+@pytest.mark.parametrize("shape", [(1216, 3904, 144), (1200, 3904, 1040), (512, 10000, 528), (2400, 4096, 272)])
+def test_gemm_last_round_in_parts(shape, form, accumulate):
+    # 80 and a few more tiles of up to 256 activation rows on 74 pairs: the last ones in parts of fewer rows, split along K, in a
+    # launch of their own; the last part of a tile and the last piece of the matrix shorter than the others; more pieces than one
+    # group of eight.  Each output is written (or added to) once.
+    M, N, K = shape
+    Amk, Wkn = codes((M, K), M), codes((K, N), N)
+    A = np.ascontiguousarray(Amk.T) if form == "columns" else Amk
+    rng = np.random.default_rng(M)
+    c0 = (rng.standard_normal((M, N)) * 50).astype(np.float32)
+    C = torch.from_numpy(c0.copy()).cuda()
+    wsb = 256 + (2 * M * K + 255) // 256 * 256 if form == "expanded" else 256
+    ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")
+    H.hif8_gemm_ex(to_dev(A), A.shape[1], form == "columns", to_dev(Wkn), N, 0, C, N, H.F32, M, N, K, torch.tensor([3], dtype=torch.int32, device="cuda"),
+                   torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    assert H.hif8_gemm_status(ws) == 0
+    rows = np.concatenate([rng.integers(0, M, 40000), np.repeat(np.arange(M), 24)])
+    cols = np.concatenate([rng.integers(0, N, 40000), np.tile(np.arange(N - 24, N), M)])
+    P, S = O.gemm_entries(Amk, Wkn, False, 3, -4, rows, cols)
+    want = P + c0[rows, cols] if accumulate else P
+    assert np.all(np.abs(C.cpu().numpy().astype(np.float64)[rows, cols] - want) <= 1e-5 * S + 2.0 ** -24 * np.abs(want))
