@@ -216,6 +216,12 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a,
 {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+// the same, its 16 bytes counted by a barrier of the CTA that gets them
+__device__ __forceinline__ void st_async_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t cluster_bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(cluster_bar) : "memory");
+}
 
 __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v)
 {
@@ -223,6 +229,10 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v
 }
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// Arrival that publishes nothing: "this CTA is through with what others may now overwrite".  One with release waits for every store
+// the SM has in flight, results included (256 x 1536 x 768 split in two: the two such barriers of a call took 1700 and 1260 cycles,
+// now 1500 and 410).
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all()
 {
@@ -1036,7 +1046,8 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
         const bool ok = mbar_wait(bar_acc_full(0), 0, abort_flag, p.status, 38);
         tc_fence_after();
         __syncwarp();
-        cluster_sync_all();  // all CTAs are done with their stages
+        cluster_arrive_relaxed();
+        cluster_wait();  // all CTAs are done with their stages
         if (ok) {
 #pragma unroll 1
             for (int j = warp >> 2; j < pieces; j += shares) {
@@ -1135,7 +1146,7 @@ template <int ACT>
 struct WdSmem {
     static constexpr int KB = ACT == kActExpanded ? 2 * BK : BK;  // k per k-block
     static constexpr uint32_t kActStage = (BN / 2) * KB * 2, kW8 = BM * KB;
-    static constexpr uint32_t n_bars = 4 * kWdStages + 2;
+    static constexpr uint32_t n_bars = 4 * kWdStages + 3;
     uint32_t base, lut, bars, end;
     int front;
     __device__ explicit WdSmem(uint32_t raw)
@@ -1257,6 +1268,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     auto bar_bf_empty = [&](int s) { return bars + 8u * (3 * kWdStages + s); };    // per CTA, leader's commits
     const uint32_t bar_acc_full = bars + 8u * (4 * kWdStages);                     // per CTA, leader's commit
     const uint32_t bar_acc_empty = bars + 8u * (4 * kWdStages + 1);                // leader: both CTAs' epilogue warps
+    const uint32_t bar_sums = bars + 8u * (4 * kWdStages + 2);                     // per CTA: the sums of the other pairs have arrived
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + lay.abort_flag());
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + lay.tmem_slot());
     const uint32_t lut = lay.lut + 4u * lane;
@@ -1297,7 +1309,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             // operands ready: both CTAs' groups, plus (expanded activations) the leader's announcement of the tile bytes
             mbar_init(bar_bf_full(s), 2 * kGroupWarps + (ACT == kActExpanded ? 1 : 0)); mbar_init(bar_bf_empty(s), 1);
         }
-        mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps));
+        mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps)); mbar_init(bar_sums, 1);
         *abort_flag = 0;
         if (ACT == kActExpanded) *reinterpret_cast<volatile uint32_t*>(sm + lay.other_issued()) = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1312,7 +1324,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     }
     tc_fence_before();
     __syncthreads();
-    cluster_arrive();  // barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once
+    cluster_arrive_relaxed();  // (the barriers' initialisation has been released) barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     if (ACT != kActExpanded) {
@@ -1529,9 +1541,12 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             const bool ok = mbar_wait(bar_acc_full, local & 1, abort_flag, p.status, 47);
             if (!ok && split == 1) break;
             tc_fence_after();
+            const int j0 = part * per, j1 = min(pieces, j0 + per);
             if (split > 1) {
+                if (threadIdx.x == 0) mbar_arrive_expect_tx(bar_sums, (uint32_t)((split - 1) * max(0, j1 - j0)) * 8u * BM * 4u);
                 __syncwarp();
-                cluster_sync_all();  // every pair's MMAs and copies are done: the stages of all CTAs are free
+                cluster_arrive_relaxed();
+                cluster_wait();  // every pair's MMAs and copies are done: the stages of all CTAs are free
                 if (ok) {
 #pragma unroll 1
                     for (int j = share; j < pieces; j += shares) {
@@ -1542,15 +1557,14 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                         tmem_ld_wait();
                         const int slot = part < owner ? part : part - 1;
                         const uint32_t to = map_to_cta(mine + (uint32_t)((slot * per + (j - owner * per)) * 8 * BM) * 4u, 2u * owner + half);
-                        st_cluster_v4(to, r[0], r[1], r[2], r[3]);
-                        st_cluster_v4(to + BM * 16, r[4], r[5], r[6], r[7]);
+                        const uint32_t bar = map_to_cta(bar_sums, 2u * owner + half);
+                        st_async_v4(to, r[0], r[1], r[2], r[3], bar);
+                        st_async_v4(to + BM * 16, r[4], r[5], r[6], r[7], bar);
                     }
                 }
-                __syncwarp();
-                cluster_sync_all();
-                if (!ok) break;
+                // (counted by a barrier here: a cluster barrier with release and acquire took 1800 cycles, this 800; in the narrow kernel, whose exchange is smaller, nothing is gained)
+                if (!ok || !mbar_wait(bar_sums, 0, abort_flag, p.status, 48)) break;
             }
-            const int j0 = part * per, j1 = min(pieces, j0 + per);
 #pragma unroll 1
             for (int j = j0 + share; j < j1; j += shares) {
                 uint32_t r[8];
@@ -1595,7 +1609,9 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     if (tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();
+    if (*abort_flag) cluster_arrive();  // (signals to other CTAs that nobody waited for land first)
+    else cluster_arrive_relaxed();
+    cluster_wait();
     if (warp == kMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
@@ -2511,9 +2527,9 @@ static bool choose(const GemmKey& k, int sm_count, const int* wd_clusters, const
         out->form = kFormPair;
         return true;
     }
-    // (1.08: the search takes the division whose time is underestimated most; 6000: the launch in front of the narrow kernel, its start and end)
+    // (1.2: the search takes the division whose time is underestimated most; 6000: the launch in front of the narrow kernel, its start and end)
     const double other = narrow ? NarrowTiling(k.M, k.N, k.K, sm_count, nw_clusters, k.room > 0).cycles + 6000.0 : out->weights.cycles;
-    if (1.08 * out->warp.cycles < other) out->form = kFormWarp;
+    if (1.2 * out->warp.cycles < other) out->form = kFormWarp;
     return true;
 }
 

@@ -376,5 +376,8 @@ hif8_gemm_warp_kernel(const uint8_t* __restrict__ A, long long lda, const uint8_
             }
         }
     }
-    if (c > 1) cluster_sync_all();  // nobody leaves while another block reads its sums
+    if (c > 1) {  // nobody leaves while another block reads its sums
+        cluster_arrive_relaxed();
+        cluster_wait();
+    }
 }
