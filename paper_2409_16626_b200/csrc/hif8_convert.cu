@@ -688,6 +688,57 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const uint8_t* __restr
     }
 }
 
+// The same for 16-bit results of large tensors, with a table that has a copy per lane: the conflicts of one table for all lanes, 3.5
+// wavefronts per 32 lookups, took longer than the transfer (BF16, us, one table / a copy per lane: 3001 x 4099 codes 7.8 / 7.2, 8 M
+// 5.8 / 5.2, 100 M 49.1 / 46.0).  Filling it takes a block as long as half of its lookups, so a block of 512 threads has 16384 codes
+// (8192: 7.9, 32768: 7.6 us); below two million codes that leaves too few blocks (1 M: 2.1 / 2.2).  FP32 results store twice the
+// bytes a code and gain nothing (100 M: 75.3 / 76.4).
+constexpr int kDecodeThreads = 512, kDecodeCodes = 32;  // codes per thread
+constexpr size_t kDecodeStreamFrom = (size_t)1 << 21;
+template <int DT>
+__global__ void __launch_bounds__(kDecodeThreads) decode_stream_kernel(const uint8_t* __restrict__ src, void* __restrict__ dst,
+                                                                unsigned long long n, unsigned long long n_vec, int se)
+{
+    static_assert(DT != HIF8_F32, "16-bit results");
+    __shared__ __align__(16) uint32_t s_out[kLaneTableWords];
+    pdl_launch_dependents();
+    {
+        const int da = (-se) / 2, db = -se - da;
+        fill_lane_table(s_out, to_bits<DT>(__uint_as_float(decode_bits_f32(threadIdx.x & 255u)) * pow2f(da) * pow2f(db)));
+    }
+    __syncthreads();
+    pdl_wait_prior_grid();
+    constexpr int PV = SrcTraits<DT>::kPerVec, U = kDecodeCodes / PV;  // codes per 16-byte store, vectors per thread
+    const uint32_t lane4 = (threadIdx.x & 31u) * 4u;
+    // one group of U vectors per thread; a group wholly inside the tensor runs without bounds checks
+    auto group = [&](unsigned long long base, auto full_tag) {
+        constexpr bool FULL = decltype(full_tag)::value;
+        uint2 v[U];
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            unsigned long long u = base + (unsigned long long)j * kDecodeThreads + threadIdx.x;
+            v[j] = make_uint2(0, 0);
+            if (FULL || u < n_vec) v[j] = __ldcs(reinterpret_cast<const uint2*>(src) + u);
+        }
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            unsigned long long u = base + (unsigned long long)j * kDecodeThreads + threadIdx.x;
+            if (!FULL && u >= n_vec) continue;
+            const uint2 lo = lane_lookup4(s_out, v[j].x, lane4), hi = lane_lookup4(s_out, v[j].y, lane4);
+            __stcs(reinterpret_cast<uint4*>(dst) + u, make_uint4(lo.x, lo.y, hi.x, hi.y));
+        }
+    };
+    const unsigned long long stride = (unsigned long long)gridDim.x * kDecodeThreads * U;
+    for (unsigned long long base = (unsigned long long)blockIdx.x * kDecodeThreads * U; base < n_vec; base += stride) {
+        if (base + (unsigned long long)kDecodeThreads * U <= n_vec) group(base, std::true_type{});
+        else group(base, std::false_type{});
+    }
+    const unsigned long long tid = (unsigned long long)blockIdx.x * kDecodeThreads + threadIdx.x;
+    for (unsigned long long i = n_vec * PV + tid; i < n; i += (unsigned long long)gridDim.x * kDecodeThreads) {
+        reinterpret_cast<unsigned short*>(dst)[i] = (unsigned short)lane_lookup<0>(s_out, src[i], lane4);
+    }
+}
+
 // ------------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------------
@@ -929,8 +980,16 @@ int hif8_decode(const uint8_t* src, void* dst, int dst_dtype, size_t n, int scal
     unsigned long long pv = dst_dtype == HIF8_F32 ? 4 : 8;
     bool vec_ok = aligned16(dst) && (reinterpret_cast<uintptr_t>(src) % pv) == 0;
     unsigned long long n_vec = vec_ok ? n / pv : 0;
-    unsigned grid = grid_for(n_vec, n, sms);
     cudaStream_t st = (cudaStream_t)stream;
+    if (dst_dtype != HIF8_F32 && vec_ok && n >= kDecodeStreamFrom) {
+        const size_t blocks = (n + kDecodeThreads * kDecodeCodes - 1) / (kDecodeThreads * kDecodeCodes);
+        const dim3 grid((unsigned)(blocks < 0x7FFFFFFF ? blocks : 0x7FFFFFFF));
+        if (dst_dtype == HIF8_BF16) launch_pdl_threads(kDecodeThreads, decode_stream_kernel<HIF8_BF16>, grid, st, src, dst, n, n_vec, scale_exp);
+        else launch_pdl_threads(kDecodeThreads, decode_stream_kernel<HIF8_F16>, grid, st, src, dst, n, n_vec, scale_exp);
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+    }
+    unsigned grid = grid_for(n_vec, n, sms);
     switch (dst_dtype) {
         case HIF8_F32: launch_pdl(decode_kernel<HIF8_F32>, grid, st, src, dst, n, n_vec, scale_exp); break;
         case HIF8_BF16: launch_pdl(decode_kernel<HIF8_BF16>, grid, st, src, dst, n, n_vec, scale_exp); break;

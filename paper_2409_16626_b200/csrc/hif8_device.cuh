@@ -664,11 +664,11 @@ __device__ __forceinline__ void block_amax_commit(float acc, uint32_t* accum)
 
 // launch with programmatic stream serialization (see pdl_* above)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, cudaStream_t st, Args... args)
+cudaError_t launch_pdl_threads(int threads, void (*kernel)(KArgs...), dim3 grid, cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -677,6 +677,11 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, cudaStream_t st, Arg
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, cudaStream_t st, Args... args)
+{
+    return launch_pdl_threads(kThreads, kernel, grid, st, args...);
 }
 
 }  // namespace

@@ -41,6 +41,32 @@ int decode_transpose_bf16(const uint8_t* src, void* dst, long long rows, long lo
 // latest GEMM-class call on stream `st` of the current device; hif8_last_device_status reads it back.
 void note_status_word(cudaStream_t st, const int* word);
 
+// Table of 256 words, one copy per lane: word 32 c + l belongs to code c and lane l, so that a warp's lookups never meet in a bank.
+// (One copy for all takes 3.5 wavefronts per 32 lookups of codes as they are distributed: more time than the bytes take from DRAM.)
+// 32 KiB; filled by 256 threads or more, thread c < 256 with the word of code c.
+constexpr int kLaneTableWords = 256 * 32;
+__device__ __forceinline__ void fill_lane_table(uint32_t* table, uint32_t word)
+{
+    if (threadIdx.x < 256) {
+#pragma unroll
+        for (uint32_t j = 0; j < 8; j++)  // (eight rows meet in a bank unless each starts with another 16 bytes)
+            *reinterpret_cast<uint4*>(table + threadIdx.x * 32 + ((j + threadIdx.x) & 7u) * 4) = make_uint4(word, word, word, word);
+    }
+}
+// the word of byte K of w; `lane4` is four times the lane
+template <int K>
+__device__ __forceinline__ uint32_t lane_lookup(const uint32_t* table, uint32_t w, uint32_t lane4)
+{
+    const uint32_t at = ((K == 0 ? w << 7 : w >> (8 * K - (K == 0 ? 0 : 7))) & 0x7F80u) | lane4;
+    return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned char*>(table) + at);
+}
+// four codes -> two words of two 16-bit values (the low halves of the table's words)
+__device__ __forceinline__ uint2 lane_lookup4(const uint32_t* table, uint32_t w, uint32_t lane4)
+{
+    return make_uint2(__byte_perm(lane_lookup<0>(table, w, lane4), lane_lookup<1>(table, w, lane4), 0x5410),
+                      __byte_perm(lane_lookup<2>(table, w, lane4), lane_lookup<3>(table, w, lane4), 0x5410));
+}
+
 // True when the byte ranges [a, a + a_bytes) and [b, b + b_bytes) share at least one byte (empty ranges share none).
 inline bool ranges_overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes)
 {
