@@ -268,6 +268,8 @@ int hif8_fake_quant(const void* src, void* dst, int dtype, size_t n, int use_ama
  * the product is too small to win the pass over W back (see hif8_gemm_path_policy).
  * Products with at most 64 rows of A (and A given as [M,K]) take a weight-streaming kernel whatever the workspace;
  * with the workspace size above it first expands the few rows of A to BF16 there (one small launch more, A contiguous).
+ * Products of few rows and a small weight, and those of few tiles, take A as bytes in one launch even when the workspace
+ * has room for it, where that is faster.
  * Where several SMs share the sum of an output (K split among them), the parts are added in a fixed order: results are
  * reproducible run to run; how K is split depends on the sizes, the device and the workspace.
  */

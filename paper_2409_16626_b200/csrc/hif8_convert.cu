@@ -923,6 +923,31 @@ constexpr size_t kConvWorkspaceBytes = 256;
 
 int checked_device(int* sms) { return device_info(sms); }
 
+int decode_codes(const uint8_t* src, void* dst, int dst_dtype, size_t n, int scale_exp, size_t stream_from, cudaStream_t st)
+{
+    int sms; int rc = device_info(&sms);
+    if (rc) return rc;
+    unsigned long long pv = dst_dtype == HIF8_F32 ? 4 : 8;
+    bool vec_ok = aligned16(dst) && (reinterpret_cast<uintptr_t>(src) % pv) == 0;
+    unsigned long long n_vec = vec_ok ? n / pv : 0;
+    if (dst_dtype != HIF8_F32 && vec_ok && n >= stream_from) {
+        const size_t blocks = (n + kDecodeThreads * kDecodeCodes - 1) / (kDecodeThreads * kDecodeCodes);
+        const dim3 grid((unsigned)(blocks < 0x7FFFFFFF ? blocks : 0x7FFFFFFF));
+        if (dst_dtype == HIF8_BF16) launch_pdl_threads(kDecodeThreads, decode_stream_kernel<HIF8_BF16>, grid, st, src, dst, n, n_vec, scale_exp);
+        else launch_pdl_threads(kDecodeThreads, decode_stream_kernel<HIF8_F16>, grid, st, src, dst, n, n_vec, scale_exp);
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+    }
+    unsigned grid = grid_for(n_vec, n, sms);
+    switch (dst_dtype) {
+        case HIF8_F32: launch_pdl(decode_kernel<HIF8_F32>, grid, st, src, dst, n, n_vec, scale_exp); break;
+        case HIF8_BF16: launch_pdl(decode_kernel<HIF8_BF16>, grid, st, src, dst, n, n_vec, scale_exp); break;
+        default: launch_pdl(decode_kernel<HIF8_F16>, grid, st, src, dst, n, n_vec, scale_exp); break;
+    }
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+}
+
 }  // namespace hif8
 
 using namespace hif8;
@@ -981,28 +1006,7 @@ int hif8_decode(const uint8_t* src, void* dst, int dst_dtype, size_t n, int scal
     if (n == 0) return HIF8_OK;
     if (!src || !dst) return HIF8_ERR_NULL;
     if (ranges_overlap(src, n, dst, n * dtype_bytes(dst_dtype))) return HIF8_ERR_OVERLAP;
-    int sms; int rc = device_info(&sms);
-    if (rc) return rc;
-    unsigned long long pv = dst_dtype == HIF8_F32 ? 4 : 8;
-    bool vec_ok = aligned16(dst) && (reinterpret_cast<uintptr_t>(src) % pv) == 0;
-    unsigned long long n_vec = vec_ok ? n / pv : 0;
-    cudaStream_t st = (cudaStream_t)stream;
-    if (dst_dtype != HIF8_F32 && vec_ok && n >= kDecodeStreamFrom) {
-        const size_t blocks = (n + kDecodeThreads * kDecodeCodes - 1) / (kDecodeThreads * kDecodeCodes);
-        const dim3 grid((unsigned)(blocks < 0x7FFFFFFF ? blocks : 0x7FFFFFFF));
-        if (dst_dtype == HIF8_BF16) launch_pdl_threads(kDecodeThreads, decode_stream_kernel<HIF8_BF16>, grid, st, src, dst, n, n_vec, scale_exp);
-        else launch_pdl_threads(kDecodeThreads, decode_stream_kernel<HIF8_F16>, grid, st, src, dst, n, n_vec, scale_exp);
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
-    }
-    unsigned grid = grid_for(n_vec, n, sms);
-    switch (dst_dtype) {
-        case HIF8_F32: launch_pdl(decode_kernel<HIF8_F32>, grid, st, src, dst, n, n_vec, scale_exp); break;
-        case HIF8_BF16: launch_pdl(decode_kernel<HIF8_BF16>, grid, st, src, dst, n, n_vec, scale_exp); break;
-        default: launch_pdl(decode_kernel<HIF8_F16>, grid, st, src, dst, n, n_vec, scale_exp); break;
-    }
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+    return decode_codes(src, dst, dst_dtype, n, scale_exp, kDecodeStreamFrom, (cudaStream_t)stream);
 }
 
 // shared by hif8_amax_scale_encode and hif8_fake_quant

@@ -2,10 +2,11 @@
 //
 //   C[m,n] = 2^-(sa+sw) * sum_k value(Aq[m,k]) * value(Wq[k,n])       (Algorithm 1, "MatMul & Restore")
 //
-// Three kernels behind one entry point, chosen by the sizes and by what fits in the caller's workspace:
+// Four kernels behind one entry point, chosen by the sizes and by what fits in the caller's workspace (see choose()):
+//   warp     few activation rows and a small weight: every warp alone on a slice of K (hif8_gemm_warp.cuh)
 //   narrow   up to 64 activation rows: bound by reading the weight bytes once
 //   weights  weights decoded into tensor memory by the tensor-core kernel; the activations come expanded to BF16 from the
-//            workspace, or, with no room there, as bytes that are decoded in the kernel too
+//            workspace, or, with no room there or too few of them, as bytes that are decoded in the kernel too
 //   pair     both operands expanded to BF16 in the workspace (large products)
 //
 // Every HiF8 value has at most 4 significant bits and an exponent in [-22, 15], so it is exact in BF16 and every
@@ -2703,7 +2704,9 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     if (rc != HIF8_OK) return rc;
     if (choice.form == kFormWeights) return launch_weights_gemm(Wq, ldw, w_is_nk, choice.weights, a_bf, K, p, wd_clusters, st);
     unsigned char* w_bf = a_bf + bytes_a;
-    rc = hif8_decode(Wq, w_bf, HIF8_BF16, (size_t)K * N, 0, stream);
+    // (a block of the pair kernel, which starts under this launch, has no room beside blocks that hold a 32 KiB table: below eight
+    // million codes that costs more than such a table saves, 2758 x 2816 x 848 21.1 -> 22.3 us)
+    rc = decode_codes(Wq, w_bf, HIF8_BF16, (size_t)K * N, 0, (size_t)1 << 23, st);
     return rc != HIF8_OK ? rc : launch_bf16_pair_gemm(a_bf, w_bf, w_is_nk, p, st);
 }
 

@@ -37,6 +37,10 @@ int launch_bf16_pair_gemm(const void* a_bf, const void* w_bf, int w_is_nk, GemmP
 // pointers 16-byte aligned.  The launch also clears the device word `clear_word` (may be null).
 int decode_transpose_bf16(const uint8_t* src, void* dst, long long rows, long long cols, uint32_t* clear_word, cudaStream_t st);
 
+// hif8_decode without its checks of the arguments.  From `stream_from` codes on, 16-bit results take the kernel whose blocks hold a
+// 32 KiB table.
+int decode_codes(const uint8_t* src, void* dst, int dst_dtype, size_t n, int scale_exp, size_t stream_from, cudaStream_t st);
+
 // Remembers `word` (a device int that a kernel sets when one of its bounded waits gives up) as the status word of the
 // latest GEMM-class call on stream `st` of the current device; hif8_last_device_status reads it back.
 void note_status_word(cudaStream_t st, const int* word);
