@@ -1624,7 +1624,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             }
             tc_fence_before();
             __syncwarp();
-            if (!one_tile && lane == 0) mbar_arrive_remote(map_to_cta(bar_acc_empty, lead));
+            // (not after the last tile: nobody waits for that one, so it could reach the leader after the leader has left)
+            if (t + t_step < t_end && lane == 0) mbar_arrive_remote(map_to_cta(bar_acc_empty, lead));
             t += t_step; tile_it += n_kb; local++;
         }
         if (!joined) { __syncwarp(); cluster_wait(); }

@@ -34,3 +34,12 @@ def test_mmas_are_waited_for(kernel, barrier):
 def test_every_wait_has_the_limit_and_there_is_no_fixed_delay():
     loops = re.findall(r"while \([^;{]*global_ns\(\)[^;{]*[;{]", TEXT)
     assert loops and all("kWaitLimitNs" in w for w in loops), loops
+
+
+def test_last_tile_sends_no_signal_that_nobody_waits_for():
+    # the MMA thread waits for the epilogue of a tile before it starts another; the arrivals of the last one would be on their way to
+    # the leader, unordered by the relaxed barrier at the end, while it leaves
+    text = body("hif8_gemm_weights_kernel")
+    arrivals = re.findall(r"[^\n]*mbar_arrive_remote\(map_to_cta\(bar_acc_empty[^\n]*", text)
+    assert len(arrivals) == 1 and "if (t + t_step < t_end && lane == 0)" in arrivals[0], arrivals
+    assert "if (local > 0) ok = mbar_wait(bar_acc_empty, (local - 1) & 1" in text
