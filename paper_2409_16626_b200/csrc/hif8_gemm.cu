@@ -234,6 +234,8 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 // the SM has in flight, results included (256 x 1536 x 768 split in two: the two such barriers of a call took 1700 and 1260 cycles,
 // now 1500 and 410).
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+// What this thread stored before it is there for everybody by the cluster's next barrier, also where the thread arrives on that relaxed.
+__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all()
 {
@@ -1352,7 +1354,10 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     }
     tc_fence_before();
     __syncthreads();
-    cluster_arrive_relaxed();  // (the barriers' initialisation has been released) barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once
+    // Barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once.  (The barriers' initialisation has been
+    // released; the words beside them that other CTAs write were zeroed by the copying warp.)
+    if (warp == kTmaWarp) cluster_arrive();
+    else cluster_arrive_relaxed();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     if (ACT != kActExpanded) {
@@ -1419,6 +1424,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             }
             if (ACT == kActExpanded) {
                 if (limit == kNoLimit) tell();
+                fence_cluster();  // (the barrier at the end is relaxed, and nobody waits for this word in a run that succeeds)
                 if (leader && *abort_flag) {
                     for (int i = max(0, it - kWdStages); i < it; i++) wait_landed(bar_bf_full(i % kWdStages), i, kWdStages);
                 }

@@ -43,3 +43,16 @@ def test_last_tile_sends_no_signal_that_nobody_waits_for():
     arrivals = re.findall(r"[^\n]*mbar_arrive_remote\(map_to_cta\(bar_acc_empty[^\n]*", text)
     assert len(arrivals) == 1 and "if (t + t_step < t_end && lane == 0)" in arrivals[0], arrivals
     assert "if (local > 0) ok = mbar_wait(bar_acc_empty, (local - 1) & 1" in text
+
+
+def test_stores_to_another_block_land_before_the_relaxed_barrier():
+    # plain stores to the pair's other CTA: the thread that made them fences at cluster scope before the barrier at the end, and the
+    # thread that zeroes such words releases that at the barrier in front of the first of them
+    text = body("hif8_gemm_weights_kernel")
+    stores = [m.start() for m in re.finditer(r"tell\(\);", text)]
+    fences = [m.start() for m in re.finditer(r"fence_cluster\(\);", text)]
+    end = text.rfind("cluster_arrive_relaxed()")
+    assert stores and all(any(s < f < end for f in fences) for s in stores)
+    setup = text[:text.find("cluster_wait()")]
+    zeroed = setup.rfind("lay.other_issued()) = 0u")
+    assert "threadIdx.x == kTmaWarp * 32" in setup[:zeroed] and re.search(r"if \(warp == kTmaWarp\) cluster_arrive\(\);\s*else cluster_arrive_relaxed\(\);", setup[zeroed:])
