@@ -1189,13 +1189,14 @@ struct WdSmem {
             front = min((int)((lut - base) / kSlotBytes), 2 * kWdStages);
             bars = lut + kLutBytesWide + (uint32_t)(2 * kWdStages - front) * kSlotBytes;
         }
-        end = bars + n_bars * 8 + 12;
+        end = bars + n_bars * 8 + 16;
     }
     __device__ uint32_t slot(int i) const { return i < front ? base + (uint32_t)i * kSlotBytes : lut + kLutBytesWide + (uint32_t)(i - front) * kSlotBytes; }
     __device__ uint32_t act(int s) const { return ACT == kActExpanded ? base + (uint32_t)s * kActStage : slot(s); }
     __device__ uint32_t u8(int s) const { return ACT == kActExpanded ? base + kWdStages * kActStage + (uint32_t)s * kW8 : slot(kWdStages + s); }
     __device__ uint32_t tmem_slot() const { return bars + n_bars * 8; }
     __device__ uint32_t abort_flag() const { return tmem_slot() + 4; }
+    __device__ uint32_t gave_up() const { return tmem_slot() + 12; }  // a CTA of the cluster gave up
     __device__ uint32_t other_issued() const { return tmem_slot() + 8; }  // 1 + the activation tiles that the pair's other CTA issued in all (0: not through yet)
 };
 static_assert(WdSmem<kActRows>::kActStage == kSlotBytes && 2 * WdSmem<kActRows>::kW8 == kSlotBytes, "one stage per slot");
@@ -1341,6 +1342,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         }
         mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps)); mbar_init(bar_sums, 1);
         *abort_flag = 0;
+        *reinterpret_cast<volatile int*>(sm + lay.gave_up()) = 0;
         if (ACT == kActExpanded) *reinterpret_cast<volatile uint32_t*>(sm + lay.other_issued()) = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1644,9 +1646,19 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     if (tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    if (*abort_flag) cluster_arrive();  // (signals to other CTAs that nobody waited for land first)
-    else cluster_arrive_relaxed();
+    if (*abort_flag) {
+        if (threadIdx.x < 2u * split) st_cluster_u32(map_to_cta(lay.gave_up(), threadIdx.x), 1u);
+        __syncwarp();
+        cluster_arrive();
+    } else cluster_arrive_relaxed();  // (in a run that succeeds every signal to another CTA has been waited for or fenced)
     cluster_wait();
+    if (*reinterpret_cast<volatile int*>(sm + lay.gave_up())) {
+        // A wait gave up in one of the CTAs (the same answer in all of them), so the others may have signalled to it and it to them
+        // what nobody waited for: the partial sums are waited for here, the rest is released by a second barrier.
+        if (split > 1 && threadIdx.x == 0) wait_landed(bar_sums, 0, 1);
+        __syncwarp();
+        cluster_sync_all();
+    }
     if (warp == kMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");

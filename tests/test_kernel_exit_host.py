@@ -56,3 +56,21 @@ def test_stores_to_another_block_land_before_the_relaxed_barrier():
     setup = text[:text.find("cluster_wait()")]
     zeroed = setup.rfind("lay.other_issued()) = 0u")
     assert "threadIdx.x == kTmaWarp * 32" in setup[:zeroed] and re.search(r"if \(warp == kTmaWarp\) cluster_arrive\(\);\s*else cluster_arrive_relaxed\(\);", setup[zeroed:])
+
+
+@pytest.mark.parametrize("kernel,word", [("hif8_gemm_weights_kernel", "lay.gave_up()"), ("bf16_gemm_pair_kernel", "SmemLayout2::gave_up")])
+def test_a_cta_that_gave_up_tells_the_cluster(kernel, word):
+    # the others' own waits may all have succeeded while their signals to that CTA are under way: every CTA learns of it at the first
+    # barrier of the end and passes a second one, with release, before it leaves
+    text = body(kernel)
+    end = text[text.rfind("tc_fence_before();\n    __syncthreads();"):]
+    told, first = end.find("st_cluster_u32(map_to_cta("), end.find("cluster_wait()")
+    first = end.find("cluster_sync_all()") if first < 0 else first
+    assert 0 <= told < first and word in end[told:first]
+    rest = end[first:]
+    asked = rest.find(word)
+    second = rest.find("cluster_sync_all()", asked)
+    assert 0 <= asked < second < rest.find("tcgen05.dealloc")
+    if kernel == "hif8_gemm_weights_kernel":
+        assert "*reinterpret_cast<volatile int*>(sm + lay.gave_up()) = 0;" in text[:text.find("cluster_arrive();")]
+        assert asked < rest.find("wait_landed(bar_sums, 0, 1)") < second
