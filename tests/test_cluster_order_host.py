@@ -8,13 +8,14 @@ import re
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2409_16626_b200", "csrc")
-REMOTE = ("st.shared::cluster", "st_cluster_v4(", "st_cluster_u32(", "mbar_arrive_remote(", "atom.shared::cluster", "red.shared::cluster", "ld.shared::cluster")
+REMOTE = ("st.shared::cluster", "st_cluster_v4(", "st_cluster_u32(", "mbar_arrive_remote(", "atom.shared::cluster", "red.shared::cluster", "ld.shared::cluster",
+          "st_async_v4(", "ld_cluster_f32(")
 WAIT = ("barrier.cluster.wait", "cluster_wait()", "cluster_sync_all()")
 
 
 def kernels():
     found = []
-    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
         text = re.sub(r"//[^\n]*", "", open(path).read())
         for piece in re.split(r"(?=__global__ void)", text)[1:]:
             body = piece[:piece.find("\n}\n")]
@@ -25,7 +26,17 @@ def kernels():
 
 
 def test_there_are_such_kernels():
-    assert len(kernels()) >= 4
+    names = [n for n, _ in kernels()]
+    assert {"hif8_gemm_warp_kernel", "hif8_gemm_narrow_kernel", "hif8_gemm_weights_kernel", "bf16_gemm_pair_kernel"} < set(names), names
+
+
+def test_every_remote_access_is_known_here():
+    # helpers that touch another block's shared memory are called from kernels by a name in the list above
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        for name, code in re.findall(r"__device__ __forceinline__ \w+ (\w+)\([^)]*\)\s*\{(.*?)\n\}", text, flags=re.S):
+            if re.search(r'"(st|ld|atom|red|st\.async\.weak|mbarrier\.arrive)\.shared::cluster', code):
+                assert name + "(" in REMOTE, (path, name)
 
 
 @pytest.mark.parametrize("name,body", [pytest.param(n, b, id=n) for n, b in kernels()])
