@@ -229,13 +229,18 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
 
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.cluster.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 // Arrival that publishes nothing: "this CTA is through with what others may now overwrite".  One with release waits for every store
 // the SM has in flight, results included (256 x 1536 x 768 split in two: the two such barriers of a call took 1700 and 1260 cycles,
 // now 1500 and 410).
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-// What this thread stored before it is there for everybody by the cluster's next barrier, also where the thread arrives on that relaxed.
-__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all()
 {
@@ -356,12 +361,6 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
 {
     uint32_t v;
     asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ uint32_t lds_volatile_u32(uint32_t addr)
-{
-    uint32_t v;
-    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ uint2 lds_v2(uint32_t addr)
@@ -1197,7 +1196,7 @@ struct WdSmem {
     __device__ uint32_t tmem_slot() const { return bars + n_bars * 8; }
     __device__ uint32_t abort_flag() const { return tmem_slot() + 4; }
     __device__ uint32_t gave_up() const { return tmem_slot() + 12; }  // a CTA of the cluster gave up
-    __device__ uint32_t other_issued() const { return tmem_slot() + 8; }  // 1 + the activation tiles that the pair's other CTA issued in all (0: not through yet)
+    __device__ uint32_t issued() const { return tmem_slot() + 8; }  // 1 + the activation tiles that this CTA issued in all (0: not through yet)
 };
 static_assert(WdSmem<kActRows>::kActStage == kSlotBytes && 2 * WdSmem<kActRows>::kW8 == kSlotBytes, "one stage per slot");
 static_assert((kWdMaxSplit - 1) * (BN / kWdMaxSplit) * BM * 4 <= 2 * kWdStages * kSlotBytes && (2 - 1) * (BN / 2) * BM * 4 <= 2 * kWdStages * kSlotBytes,
@@ -1341,9 +1340,11 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             mbar_init(bar_bf_full(s), 2 * kGroupWarps + (ACT == kActExpanded ? 1 : 0)); mbar_init(bar_bf_empty(s), 1);
         }
         mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps)); mbar_init(bar_sums, 1);
-        *abort_flag = 0;
+        // (The others touch these two words when a wait has given up, seconds later, and the block's barrier stands in front of the
+        // cluster's: no fence at cluster scope, which would make every call 0.8 us longer, 201 x 7168 x 4096 19.9 -> 20.6.)
         *reinterpret_cast<volatile int*>(sm + lay.gave_up()) = 0;
-        if (ACT == kActExpanded) *reinterpret_cast<volatile uint32_t*>(sm + lay.other_issued()) = 0u;
+        *reinterpret_cast<volatile uint32_t*>(sm + lay.issued()) = 0u;
+        *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         if (ACT == kActExpanded) copy_bytes(0, t0, kb0);
@@ -1356,10 +1357,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     }
     tc_fence_before();
     __syncthreads();
-    // Barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once.  (The barriers' initialisation has been
-    // released; the words beside them that other CTAs write were zeroed by the copying warp.)
-    if (warp == kTmaWarp) cluster_arrive();
-    else cluster_arrive_relaxed();
+    cluster_arrive_relaxed();  // (the barriers' initialisation has been released) barriers and tensor memory of this CTA are there; every warp waits for the other CTAs' once
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     if (ACT != kActExpanded) {
@@ -1397,13 +1395,14 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         if (lane == 0) {
             if (!tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            // A tile's barrier (in the pair's leader) counts the bytes of both CTAs' halves.  A thread that gives up tells the other CTA's
-            // how many tiles it has issued, and the one that is behind issues its halves of the tiles that the other one
-            // issued: their stages were free for both, and hold nothing that anybody still wants.
+            // A tile's barrier (in the pair's leader) counts the bytes of both CTAs' halves.  A thread that is through says how many tiles
+            // it has issued, and one that gives up reads that of the other CTA and issues its halves of the tiles that the other
+            // one issued: their stages were free for both, and hold nothing that anybody still wants.  (It is read from there, and not
+            // sent here by every run: a store that nobody waits for could arrive after this CTA has left.)
             constexpr int kNoLimit = 0x7FFFFFFF;
             int it = 0, limit = kNoLimit;
             bool ok = ACT == kActExpanded;
-            auto tell = [&]() { st_cluster_u32(map_to_cta(lay.other_issued(), rank ^ 1u), (uint32_t)it + 1u); };
+            auto tell = [&]() { *reinterpret_cast<volatile uint32_t*>(sm + lay.issued()) = (uint32_t)it + 1u; };
             for (int t = t0; t < t_end && ok; t += t_step) {
                 int slab, m0;
                 if (FORM == kOneGroup) m0 = t % tp.chunks * tp.bn;
@@ -1414,7 +1413,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                     if (limit == kNoLimit && ((it >= kWdStages && !mbar_wait(bar_bf_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 46)) || *abort_flag)) {
                         tell();
                         const unsigned long long c0 = global_ns();
-                        do limit = (int)lds_volatile_u32(lay.other_issued()) - 1;  // (the other CTA's waits are bounded as well)
+                        do limit = (int)ld_cluster_u32(map_to_cta(lay.issued(), rank ^ 1u)) - 1;  // (the other CTA's waits are bounded as well)
                         while (limit < 0 && global_ns() - c0 < 2 * kWaitLimitNs);
                     }
                     if (it >= limit) { ok = false; break; }
@@ -1426,7 +1425,6 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             }
             if (ACT == kActExpanded) {
                 if (limit == kNoLimit) tell();
-                fence_cluster();  // (the barrier at the end is relaxed, and nobody waits for this word in a run that succeeds)
                 if (leader && *abort_flag) {
                     for (int i = max(0, it - kWdStages); i < it; i++) wait_landed(bar_bf_full(i % kWdStages), i, kWdStages);
                 }
@@ -1646,13 +1644,15 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     if (tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    if (*abort_flag) {
+    // (unlikely: what follows a wait that gave up stands behind the rest of the code, whose last lines would otherwise be fetched
+    // later, 300 cycles a call)
+    if (__builtin_expect(*abort_flag != 0, 0)) {
         if (threadIdx.x < 2u * split) st_cluster_u32(map_to_cta(lay.gave_up(), threadIdx.x), 1u);
         __syncwarp();
         cluster_arrive();
-    } else cluster_arrive_relaxed();  // (in a run that succeeds every signal to another CTA has been waited for or fenced)
+    } else cluster_arrive_relaxed();  // (in a run that succeeds every signal to another CTA has been waited for)
     cluster_wait();
-    if (*reinterpret_cast<volatile int*>(sm + lay.gave_up())) {
+    if (__builtin_expect(*reinterpret_cast<volatile int*>(sm + lay.gave_up()) != 0, 0)) {
         // A wait gave up in one of the CTAs (the same answer in all of them), so the others may have signalled to it and it to them
         // what nobody waited for: the partial sums are waited for here, the rest is released by a second barrier.
         if (split > 1 && threadIdx.x == 0) wait_landed(bar_sums, 0, 1);
