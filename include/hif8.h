@@ -325,13 +325,23 @@ int hif8_encode_transpose(const void* src, int src_dtype, uint8_t* dst, int64_t 
 int hif8_gemm_status(const void* workspace, hif8_stream_t stream);
 
 /*
- * Which general kernel a large workspace selects.  HIF8_GEMM_PATH_AUTO (the default): with room for both operands W is
- * expanded too only when the product is large enough to win that pass back (from about 1500 rows of A with [K,N] weights,
- * about 4800 with [N,K] weights); below that A alone is expanded.  HIF8_GEMM_PATH_EXPAND_BOTH: both operands are expanded whenever the workspace has room (for
- * measurements and tests of that kernel on small products).  Process-wide; returns the previous setting (0 or 1), or
- * HIF8_ERR_FLAGS for an unknown one.  Results do not depend on it.
+ * Which kernel takes a product.  HIF8_GEMM_PATH_AUTO (the default): the one that is expected to be fastest, by the sizes, the
+ * layouts and what the workspace has room for; with room for both operands W is expanded too only when the product is large
+ * enough to win that pass back.  The other settings are for measurements and tests of one kernel on products that another
+ * one would take:
+ *   HIF8_GEMM_PATH_EXPAND_BOTH  both operands expanded whenever the workspace has room
+ *   HIF8_GEMM_PATH_EXPAND_A     A expanded whenever the workspace has room, W decoded in the kernel
+ *   HIF8_GEMM_PATH_NO_WARP      as AUTO, without the kernel for few rows and a small weight (nor do the two above take it)
+ *   HIF8_GEMM_PATH_WARP         that kernel; HIF8_ERR_SHAPE for a product that it cannot take (K too long for its registers, far
+ *                               too large a product, [K,N] weights with N no multiple of four)
+ * Up to 64 rows of A given as [M,K] take the weight-streaming kernel under the first three.  Process-wide; returns the
+ * previous setting, or HIF8_ERR_FLAGS (4, which is no setting) for an unknown one.  What it computes does not depend on it,
+ * only the order of the FP32 sums does.
  */
-enum { HIF8_GEMM_PATH_AUTO = 0, HIF8_GEMM_PATH_EXPAND_BOTH = 1 };
+enum {
+    HIF8_GEMM_PATH_AUTO = 0, HIF8_GEMM_PATH_EXPAND_BOTH = 1, HIF8_GEMM_PATH_NO_WARP = 2, HIF8_GEMM_PATH_EXPAND_A = 3,
+    HIF8_GEMM_PATH_WARP = 5
+};
 int hif8_gemm_path_policy(int policy);
 
 /*

@@ -208,11 +208,11 @@ def hif8_gemm_status(workspace, stream=None):
     return int(lib.hif8_gemm_status(_ptr(workspace), _stream(stream)))
 
 
-GEMM_PATH_AUTO, GEMM_PATH_EXPAND_BOTH = 0, 1
+GEMM_PATH_AUTO, GEMM_PATH_EXPAND_BOTH, GEMM_PATH_NO_WARP, GEMM_PATH_EXPAND_A, GEMM_PATH_WARP = 0, 1, 2, 3, 5
 
 
 def hif8_gemm_path_policy(policy):
-    """Sets which general kernel a large workspace selects; returns the previous setting, or 4 (HIF8_ERR_FLAGS) for an unknown one."""
+    """Sets which kernel takes a product (one of GEMM_PATH_*); returns the previous setting, or 4 (HIF8_ERR_FLAGS) for an unknown one."""
     return int(lib.hif8_gemm_path_policy(int(policy)))
 
 

@@ -2447,7 +2447,9 @@ struct WarpTiling {
     }
     void divide(int M, int N, int K, bool w_is_nk, int m, const int* clusters)
     {
-        const int blocks = (M + 8 * m - 1) / (8 * m), ut = w_is_nk ? 1 : 2, max_chunks = (w_is_nk ? 4 : 2) / (m == 4 ? 2 : 1), cols = 16 * ut;
+        const int blocks = (M + 8 * m - 1) / (8 * m);
+        if (blocks > 65535) return;  // the second dimension of a grid
+        const int ut = w_is_nk ? 1 : 2, max_chunks = (w_is_nk ? 4 : 2) / (m == 4 ? 2 : 1), cols = 16 * ut;
         const int units = (N + cols - 1) / cols, kb = (K + 63) / 64;
         const uint32_t deposit = (uint32_t)(cols * 8 * m * 4);
         for (int c = 1; c <= kWarpMaxCluster; c++) {
@@ -2511,7 +2513,9 @@ static std::atomic<int> g_path_policy{HIF8_GEMM_PATH_AUTO};
 
 extern "C" int hif8_gemm_path_policy(int policy)
 {
-    if (policy != HIF8_GEMM_PATH_AUTO && policy != HIF8_GEMM_PATH_EXPAND_BOTH) return HIF8_ERR_FLAGS;
+    if (policy != HIF8_GEMM_PATH_AUTO && policy != HIF8_GEMM_PATH_EXPAND_BOTH && policy != HIF8_GEMM_PATH_NO_WARP &&
+        policy != HIF8_GEMM_PATH_EXPAND_A && policy != HIF8_GEMM_PATH_WARP)
+        return HIF8_ERR_FLAGS;
     return g_path_policy.exchange(policy, std::memory_order_relaxed);
 }
 
@@ -2559,26 +2563,36 @@ struct GemmChoice {
 };
 static LruCache<GemmKey, GemmChoice, 64> g_choices;
 
+// false: the kernel that hif8_gemm_path_policy asks for has no division of this product
 static bool choose(const GemmKey& k, int sm_count, const int* wd_clusters, const int* nw_clusters, const int* wp_clusters, GemmChoice* out)
 {
-    const bool narrow = !k.a_is_km && k.M <= kNarrowMaxM;
-    out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters);
-    const WeightsTiling bytes(k.M, k.N, k.K, k.a_is_km ? kActColumns : kActRows, k.a_is_km, wd_clusters);
-    const WeightsTiling expanded(k.M, k.N, k.K, kActExpanded, k.a_is_km, wd_clusters);
-    out->weights = k.room && expanded.cycles < bytes.cycles ? expanded : bytes;
-    out->form = narrow ? kFormNarrow : kFormWeights;
-    // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element moved, at
-    // 3300 bytes a cycle, and a launch) by the cheaper k-blocks and tiles of the pair kernel: 545 cycles per
-    // 64 k and nothing between tiles, against the weights kernel's cost above.  Measured (us, both expanded / weights decoded in
-    // the kernel): 2048 x 7168 x 4096 105 / 98, 3072 rows 130 / 133, 4096 rows 172 / 176; 1536 x 8192 x 1024 28.5 / 33;
-    // 2048 x 16384 x 8192 381 / 357, 4096 rows 702 / 732.
-    const long long pair_rounds = ((long long)((k.M + 2 * BM - 1) / (2 * BM)) * ((k.N + BN - 1) / BN) + sm_count / 2 - 1) / (sm_count / 2);
-    const double expand_w = 6000.0 + 3.0 * (double)k.K * k.N / 3300.0, pair_cycles = (double)pair_rounds * ((k.K + BK - 1) / BK * 545.0 + 500.0);
-    if (!narrow && k.room == 2 && (k.policy == HIF8_GEMM_PATH_EXPAND_BOTH ||
-                                   expand_w + pair_cycles < 1.03 * expanded.cost.all(expanded.tiles))) {  // (equal at 1.03: the lookups also cost clock under the power limit)
-        out->form = kFormPair;
-        return true;
+    if (k.policy == HIF8_GEMM_PATH_WARP) {
+        out->form = kFormWarp;
+        out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters);
+        return out->warp.cycles < 1e30;
     }
+    const bool narrow = !k.a_is_km && k.M <= kNarrowMaxM;
+    out->form = narrow ? kFormNarrow : kFormWeights;
+    if (!narrow) {
+        const WeightsTiling bytes(k.M, k.N, k.K, k.a_is_km ? kActColumns : kActRows, k.a_is_km, wd_clusters);
+        const WeightsTiling expanded(k.M, k.N, k.K, kActExpanded, k.a_is_km, wd_clusters);
+        out->weights = k.room && (k.policy == HIF8_GEMM_PATH_EXPAND_A || expanded.cycles < bytes.cycles) ? expanded : bytes;
+        // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element moved, at
+        // 3300 bytes a cycle, and a launch) by the cheaper k-blocks and tiles of the pair kernel: 545 cycles per
+        // 64 k and nothing between tiles, against the weights kernel's cost above.  Measured (us, both expanded / weights decoded in
+        // the kernel): 2048 x 7168 x 4096 105 / 98, 3072 rows 130 / 133, 4096 rows 172 / 176; 1536 x 8192 x 1024 28.5 / 33;
+        // 2048 x 16384 x 8192 381 / 357, 4096 rows 702 / 732.
+        const long long pair_rounds = ((long long)((k.M + 2 * BM - 1) / (2 * BM)) * ((k.N + BN - 1) / BN) + sm_count / 2 - 1) / (sm_count / 2);
+        const double expand_w = 6000.0 + 3.0 * (double)k.K * k.N / 3300.0, pair_cycles = (double)pair_rounds * ((k.K + BK - 1) / BK * 545.0 + 500.0);
+        if (k.room == 2 && k.policy != HIF8_GEMM_PATH_EXPAND_A &&
+            (k.policy == HIF8_GEMM_PATH_EXPAND_BOTH ||
+             expand_w + pair_cycles < 1.03 * expanded.cost.all(expanded.tiles))) {  // (equal at 1.03: the lookups also cost clock under the power limit)
+            out->form = kFormPair;
+            return true;
+        }
+    }
+    if (k.policy != HIF8_GEMM_PATH_AUTO) return true;
+    out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters);
     // (1.2: the search takes the division whose time is underestimated most; 6000: the launch in front of the narrow kernel, its start and end)
     const double other = narrow ? NarrowTiling(k.M, k.N, k.K, sm_count, nw_clusters, k.room > 0).cycles + 6000.0 : out->weights.cycles;
     if (1.2 * out->warp.cycles < other) out->form = kFormWarp;

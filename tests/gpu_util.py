@@ -48,12 +48,23 @@ import contextlib
 
 
 @contextlib.contextmanager
-def both_operands_expanded(on):
-    """Within the block a workspace with room for both operands selects the kernel that expands both, whatever the size of
-    the product (hif8_gemm_path_policy); the previous setting is restored afterwards."""
-    import paper_2409_16626_b200 as H
-    before = H.hif8_gemm_path_policy(H.GEMM_PATH_EXPAND_BOTH if on else H.GEMM_PATH_AUTO)
+def gemm_path(policy):
+    """Within the block products are taken by the kernel that `policy` (one of GEMM_PATH_*) asks for, whatever their size; the
+    previous setting is restored afterwards."""
+    before = H.hif8_gemm_path_policy(policy)
+    assert before != 4, "no such setting"
     try:
         yield
     finally:
         H.hif8_gemm_path_policy(before)
+
+
+# What a test's workspace is for: True: room for both operands, the kernel that takes both expanded; "a": room for A alone, A expanded
+# and W decoded in the kernel; False: the status word only, both decoded in the kernel -- none of them the kernel for few rows, which
+# would take most small products by itself; "warp": that one, with the status word; "auto": room for both, the library's own choice.
+POLICY = {True: H.GEMM_PATH_EXPAND_BOTH, "a": H.GEMM_PATH_EXPAND_A, False: H.GEMM_PATH_NO_WARP, "warp": H.GEMM_PATH_WARP, "auto": H.GEMM_PATH_AUTO}
+
+
+def gemm_workspace_bytes(staged, M, N, K):
+    n = {True: M * K + K * N, "auto": M * K + K * N, "a": M * K, False: 0, "warp": 0}[staged]
+    return H.hif8_workspace_bytes(H.WS_GEMM, n)

@@ -100,3 +100,14 @@ def test_gemm_path_policy_setting_round_trips():
     assert H.hif8_gemm_path_policy(7) == 4                   # HIF8_ERR_FLAGS
     assert H.hif8_gemm_path_policy(H.GEMM_PATH_AUTO) == H.GEMM_PATH_EXPAND_BOTH
     assert H.hif8_gemm_path_policy(before) == H.GEMM_PATH_AUTO
+
+
+def test_gemm_path_policy_settings():
+    settings = (H.GEMM_PATH_EXPAND_BOTH, H.GEMM_PATH_NO_WARP, H.GEMM_PATH_EXPAND_A, H.GEMM_PATH_WARP, H.GEMM_PATH_AUTO)
+    assert 4 not in settings                                 # HIF8_ERR_FLAGS, the answer to an unknown one
+    before = H.hif8_gemm_path_policy(H.GEMM_PATH_AUTO)
+    last = H.GEMM_PATH_AUTO
+    for s in settings:
+        assert H.hif8_gemm_path_policy(s) == last and H.hif8_gemm_path_policy(4) == 4 and H.hif8_gemm_path_policy(-1) == 4
+        last = s
+    H.hif8_gemm_path_policy(before)

@@ -9,7 +9,7 @@ import paper_2409_16626_b200 as H
 import workloads as W
 from oracle import hif8_oracle as O
 
-from gpu_util import bf16_half_ulp, both_operands_expanded, dev_empty, to_dev
+from gpu_util import POLICY, bf16_half_ulp, dev_empty, gemm_path, gemm_workspace_bytes, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -94,7 +94,7 @@ def codes(shape, seed):
     return q
 
 
-@pytest.mark.parametrize("staged", [False, True, "a"])  # "a": workspace for A alone (A expanded once, W decoded in the kernel)
+@pytest.mark.parametrize("staged", [False, True, "a", "warp", "auto"])
 @pytest.mark.parametrize("a_is_km,w_is_nk", [(1, 0), (1, 1), (0, 1)])
 @pytest.mark.parametrize("c_dtype,accumulate", [(H.F32, 0), (H.F32, 1), (H.BF16, 1)])
 def test_gemm_ex_layouts_and_accumulate(c_dtype, accumulate, a_is_km, w_is_nk, staged):
@@ -108,9 +108,9 @@ def test_gemm_ex_layouts_and_accumulate(c_dtype, accumulate, a_is_km, w_is_nk, s
     c0 = (rng.standard_normal((M, ldc)) * 50).astype(np.float32)
     C = torch.from_numpy(c0).cuda().to(torch.float32 if c_dtype == H.F32 else torch.bfloat16)
     c0 = C.float().cpu().numpy().astype(np.float64)
-    wsb = H.hif8_workspace_bytes(H.WS_GEMM, (M * K if staged == "a" else M * K + K * N) if staged else 0)
+    wsb = gemm_workspace_bytes(staged, M, N, K)
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
-    with both_operands_expanded(staged is True):
+    with gemm_path(POLICY[staged]):
         H.hif8_gemm_ex(to_dev(Aq), Aq.shape[1], a_is_km, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
                        torch.tensor([sa], dtype=torch.int32, device="cuda"), torch.tensor([sw], dtype=torch.int32, device="cuda"),
                        None, accumulate, ws, wsb)
@@ -128,14 +128,16 @@ def test_gemm_ex_layouts_and_accumulate(c_dtype, accumulate, a_is_km, w_is_nk, s
     assert np.all(np.abs(out[:, :N] - Cs) <= tol)
 
 
-def test_gemm_ex_channel_exponents_with_transposed_a():
+@pytest.mark.parametrize("kernel", [False, "warp"])
+def test_gemm_ex_channel_exponents_with_transposed_a(kernel):
     M, N, K = 128, 256, 64
     Amk, Wkn = codes((M, K), 8), codes((K, N), 9)
     sw = np.random.default_rng(5).integers(-12, 12, size=N).astype(np.int32)
     C = torch.zeros(M, N, dtype=torch.float32, device="cuda")
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
-    H.hif8_gemm_ex(to_dev(np.ascontiguousarray(Amk.T)), M, 1, to_dev(Wkn), N, 0, C, N, H.F32, M, N, K, None,
-                   torch.tensor([99], dtype=torch.int32, device="cuda"), to_dev(sw.view(np.uint32)), 0, ws, 256)
+    with gemm_path(POLICY[kernel]):
+        H.hif8_gemm_ex(to_dev(np.ascontiguousarray(Amk.T)), M, 1, to_dev(Wkn), N, 0, C, N, H.F32, M, N, K, None,
+                       torch.tensor([99], dtype=torch.int32, device="cuda"), to_dev(sw.view(np.uint32)), 0, ws, 256)
     assert H.hif8_gemm_status(ws) == 0
     rows, cols = np.divmod(np.arange(M * N), N)
     P, S = O.gemm_entries_ex(np.ascontiguousarray(Amk.T), 1, Wkn, 0, 0, sw, rows, cols)  # the channel array wins over d_sw
@@ -195,9 +197,10 @@ def test_backward_pass_of_a_linear_layer():
 
 @pytest.mark.parametrize("shape", [(200, 72, 16), (56, 264, 80), (129, 8, 1040)])
 @pytest.mark.parametrize("w_is_nk", [0, 1])
-def test_gemm_ex_transposed_a_ragged_shapes_and_padded_leading_dimensions(shape, w_is_nk):
-    # A stored [K, M] with lda > M, M not a multiple of anything convenient, tiny K / N: the fused kernel (operands not
-    # contiguous), out-of-range parts of the TMA boxes must read as zero
+@pytest.mark.parametrize("kernel", [False, "warp"])
+def test_gemm_ex_transposed_a_ragged_shapes_and_padded_leading_dimensions(shape, w_is_nk, kernel):
+    # A stored [K, M] with lda > M, M not a multiple of anything convenient, tiny K / N: the kernel that decodes both operands (they
+    # are not contiguous), where out-of-range parts of the TMA boxes must read as zero, and the one for few rows
     M, N, K = shape
     lda = (M + 15) // 16 * 16 + 16
     ldw = ((K if w_is_nk else N) + 15) // 16 * 16 + 16
@@ -210,7 +213,8 @@ def test_gemm_ex_transposed_a_ragged_shapes_and_padded_leading_dimensions(shape,
     ldc = (N + 7) // 8 * 8
     C = torch.full((M, ldc), float("nan"), dtype=torch.float32, device="cuda")
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
-    H.hif8_gemm_ex(to_dev(Aq), lda, 1, to_dev(Wq), ldw, w_is_nk, C, ldc, H.F32, M, N, K, None, None, None, 0, ws, 256)
+    with gemm_path(POLICY[kernel]):
+        H.hif8_gemm_ex(to_dev(Aq), lda, 1, to_dev(Wq), ldw, w_is_nk, C, ldc, H.F32, M, N, K, None, None, None, 0, ws, 256)
     assert H.hif8_gemm_status(ws) == 0
     out = C.cpu().numpy().astype(np.float64)
     assert np.all(np.isnan(out[:, N:]))
@@ -233,8 +237,9 @@ def test_gemm_ex_argument_checks():
     assert H.hif8_gemm_ex(A, 64, 1, A, 64, 0, C, 64, H.F32, 0, 64, 64, **ok) == 0     # empty output
 
 
+@pytest.mark.parametrize("kernel", [False, "warp"])
 @pytest.mark.parametrize("c_dtype,accumulate", [(H.F32, 0), (H.F32, 1), (H.BF16, 0), (H.BF16, 1)])
-def test_gemm_ex_rows_of_c_more_than_4_gib_apart(c_dtype, accumulate):
+def test_gemm_ex_rows_of_c_more_than_4_gib_apart(c_dtype, accumulate, kernel):
     # few activation rows given as [K,M]: C may be a strided view of a large buffer, a row pitch needs 64 bits
     M, N, K, lda = 9, 24, 32, 16
     ldc = (2 ** 32 + 64) // (4 if c_dtype == H.F32 else 2)
@@ -249,7 +254,8 @@ def test_gemm_ex_rows_of_c_more_than_4_gib_apart(c_dtype, accumulate):
     C.copy_(torch.from_numpy((np.random.default_rng(1).standard_normal((M, N)) * 50).astype(np.float32)))
     c0 = C.float().cpu().numpy().astype(np.float64)
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
-    H.hif8_gemm_ex(to_dev(A), lda, 1, to_dev(Wq), N + 8, 0, buf, ldc, c_dtype, M, N, K, None, None, None, accumulate, ws, 256)
+    with gemm_path(POLICY[kernel]):
+        H.hif8_gemm_ex(to_dev(A), lda, 1, to_dev(Wq), N + 8, 0, buf, ldc, c_dtype, M, N, K, None, None, None, accumulate, ws, 256)
     assert H.hif8_gemm_status(ws) == 0
     out = C.float().cpu().numpy().astype(np.float64)
     del buf, C
@@ -283,7 +289,7 @@ def test_gemm_both_operands_expanded_many_tiles_per_pair(many_tiles, c_dtype, ac
     c0 = C.float().cpu().numpy().astype(np.float64)
     wsb = H.hif8_workspace_bytes(H.WS_GEMM, M * K + K * N)
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
-    with both_operands_expanded(True):
+    with gemm_path(POLICY[True]):
         H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wq), N, 0, C, ldc, c_dtype, M, N, K, torch.tensor([3], dtype=torch.int32, device="cuda"),
                        torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
     assert H.hif8_gemm_status(ws) == 0

@@ -12,7 +12,7 @@ import paper_2409_16626_b200 as H
 import workloads as W
 from oracle import hif8_oracle as O
 
-from gpu_util import bf16_half_ulp, to_dev
+from gpu_util import POLICY, bf16_half_ulp, gemm_path, gemm_workspace_bytes, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -24,19 +24,13 @@ def run_gemm(Aq, Wq, w_is_nk, c_dtype, sa=None, sw=None, M=None, N=None, K=None,
     dA, dW = to_dev(Aq), to_dev(Wq)
     ldc = (N + 7) // 8 * 8
     C = torch.full((M, ldc), float("nan"), dtype=torch.float32 if c_dtype == H.F32 else torch.bfloat16, device="cuda")
-    # staged = True: workspace with room for both operands in BF16 -> decode-once path; "a": room for A alone -> A expanded
-    # once, W decoded inside the tensor-core kernel; False: the fused kernel decodes both
-    wsb = H.hif8_workspace_bytes(H.WS_GEMM, M * K if staged == "a" else M * K + K * N) if staged else H.hif8_workspace_bytes(H.WS_GEMM, 0)
+    wsb = gemm_workspace_bytes(staged, M, N, K)
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
     dsa = torch.tensor([sa], dtype=torch.int32, device="cuda") if sa is not None else None
     dsw = torch.tensor([sw], dtype=torch.int32, device="cuda") if sw is not None else None
-    # (staged = True means the kernel that takes both operands expanded, whatever the size of the product)
-    before = H.hif8_gemm_path_policy(H.GEMM_PATH_EXPAND_BOTH if staged is True else H.GEMM_PATH_AUTO)
-    try:
+    with gemm_path(POLICY[staged]):
         H.hif8_gemm(dA, Aq.shape[1] if lda is None else lda, dW, Wq.shape[1] if ldw is None else ldw, int(w_is_nk), C, ldc,
                     c_dtype, M, N, K, dsa, dsw, ws, wsb)
-    finally:
-        H.hif8_gemm_path_policy(before)
     assert H.hif8_gemm_status(ws) == 0
     out = C.float().cpu().numpy().astype(np.float64)
     assert np.all(np.isnan(out[:, N:]))                      # padding columns untouched
@@ -52,7 +46,7 @@ def check(C, Cstar, S, c_dtype):
     assert not bad.any(), f"{bad.sum()} of {bad.size} outside tolerance; worst ratio {np.max(err / np.maximum(tol, 1e-300)):.3g}"
 
 
-@pytest.mark.parametrize("staged", [False, True, "a"])
+@pytest.mark.parametrize("staged", [False, True, "a", "warp", "auto"])
 @pytest.mark.parametrize("w_is_nk", [0, 1])
 @pytest.mark.parametrize("c_dtype", [H.F32, H.BF16])
 @pytest.mark.parametrize("shape", [(128, 256, 64), (128, 256, 256), (256, 512, 192), (130, 264, 208), (77, 40, 16),
@@ -70,7 +64,7 @@ def test_gemm_small_full_compare(shape, c_dtype, w_is_nk, staged):
     check(C, Cs, S, c_dtype)
 
 
-@pytest.mark.parametrize("staged", [False, True, "a"])
+@pytest.mark.parametrize("staged", [False, True, "a", "warp"])
 @pytest.mark.parametrize("w_is_nk", [0, 1])
 def test_gemm_one_hot_rows_pin_tile_and_k_indexing(w_is_nk, staged):
     # A picks one k per row (value 1.0): C[m, :] must equal row perm[m] of W exactly
@@ -115,7 +109,7 @@ def test_gemm_specials_propagate(M):
     Wq = np.full((K, N), 0x08, dtype=np.uint8)
     Aq[3, 5] = 0x80                                           # NaN
     Aq[7, 9] = 0x6F                                           # +Inf
-    for staged in (False, True, "a"):
+    for staged in (False, True, "a", "warp"):
         C = run_gemm(Aq, Wq, 0, H.F32, staged=staged)
         assert np.all(np.isnan(C[3])) and np.all(np.isposinf(C[7]))
         ok = np.ones(M, bool); ok[[3, 7]] = False
@@ -155,17 +149,17 @@ def _same_sign_operands(M, N, K, relu_only):
 
 
 @pytest.mark.parametrize("relu_only", [False, True])
-@pytest.mark.parametrize("path", ["fused", "staged", "a_expanded", "narrow"])
+@pytest.mark.parametrize("path", ["fused", "staged", "a_expanded", "narrow", "warp"])
 def test_gemm_same_sign_operands_k8192(path, relu_only):
     # Section 4.1: activations are GEMM inputs, and activations behind a ReLU are non-negative.  With operands of one
     # sign nothing cancels, S equals |C*|, and 512 sequential FP32 accumulator updates per output must stay inside
     # 1e-5 * S with no further allowance (FP32 output).
-    M, N, K = (16 if path == "narrow" else 256), 512, 8192
+    M, N, K = (16 if path in ("narrow", "warp") else 256), 512, 8192
     Aq, Wkn, sa, sw = _same_sign_operands(M, N, K, relu_only)
     Cs, S = O.gemm_full(Aq, Wkn, False, sa, sw)
     if not relu_only:
         assert np.allclose(Cs, S, rtol=1e-12)
-    C = run_gemm(Aq, Wkn, 0, H.F32, sa=sa, sw=sw, staged={"staged": True, "a_expanded": "a"}.get(path, False))
+    C = run_gemm(Aq, Wkn, 0, H.F32, sa=sa, sw=sw, staged={"staged": True, "a_expanded": "a", "warp": "warp"}.get(path, False))
     ratio = np.max(np.abs(C - Cs) / (1e-5 * S))
     print(f"same-sign K=8192 {path} relu_only={relu_only}: worst |err| / (1e-5 S) = {ratio:.3f}")
     assert ratio <= 1.0, ratio
@@ -188,7 +182,7 @@ def test_bounded_wait_gives_up_and_reports_without_disturbing_the_device():
 
 @pytest.mark.parametrize("w_is_nk", [0, 1])
 @pytest.mark.parametrize("c_dtype", [H.F32, H.BF16])
-@pytest.mark.parametrize("staged", [False, True])
+@pytest.mark.parametrize("staged", [False, True, "auto"])
 @pytest.mark.parametrize("shape", [(1, 256, 64), (16, 1008, 272), (17, 640, 1040), (33, 128, 16), (64, 400, 208), (48, 2064, 4096),
                                    (8, 304, 8192), (20, 912, 1472), (64, 1296, 2048), (16, 1168, 2432), (40, 1168, 2368)])
 def test_gemm_narrow_products(shape, c_dtype, w_is_nk, staged):
@@ -251,8 +245,9 @@ def test_gemm_narrow_channel_scales_and_accumulate(K):
     C = torch.from_numpy(c0.copy()).cuda()
     wsb = H.hif8_workspace_bytes(H.WS_GEMM, M * K + K * N) if K > 1000 else 256
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
-    H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wkn), N, 0, C, N, H.F32, M, N, K, torch.tensor([2], dtype=torch.int32, device="cuda"),
-                   None, to_dev(sw.view(np.uint32)), 1, ws, wsb)
+    with gemm_path(H.GEMM_PATH_NO_WARP):
+        H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wkn), N, 0, C, N, H.F32, M, N, K, torch.tensor([2], dtype=torch.int32, device="cuda"),
+                       None, to_dev(sw.view(np.uint32)), 1, ws, wsb)
     assert H.hif8_gemm_status(ws) == 0
     rows, cols = np.divmod(np.arange(M * N), N)
     P, S = O.gemm_entries_channel(Aq, Wkn, 0, 2, sw, rows, cols)
@@ -262,18 +257,24 @@ def test_gemm_narrow_channel_scales_and_accumulate(K):
 
 def test_gemm_calls_replay_from_a_cuda_graph():
     # the narrow call is two launches chained by programmatic stream serialization, the general one (nothing but the status word)
-    # a cluster launch that clears it: both are captured into one graph and replayed on new operand contents
+    # a cluster launch that clears it, the one for few rows a single launch: all are captured into one graph and replayed on new
+    # operand contents
     M, N, K = 16, 1168, 2432
     M2 = 256
     dA, dW = torch.empty(M2 * K, dtype=torch.uint8, device="cuda"), torch.empty(K * N, dtype=torch.uint8, device="cuda")
-    Cn = torch.zeros(M, N, dtype=torch.float32, device="cuda")
+    Cn, Cw = torch.zeros(M, N, dtype=torch.float32, device="cuda"), torch.zeros(M, N, dtype=torch.float32, device="cuda")
     Cg = torch.zeros(M2, N, dtype=torch.float32, device="cuda")
     wsb = H.hif8_workspace_bytes(H.WS_GEMM, M2 * K + K * N)
-    ws_n, ws_g = torch.empty(wsb, dtype=torch.uint8, device="cuda"), torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    ws_n, ws_g, ws_w = (torch.empty(wsb, dtype=torch.uint8, device="cuda") for _ in range(3))
 
     def calls():
-        H.hif8_gemm(dA, K, dW, N, 0, Cn, N, H.F32, M, N, K, None, None, ws_n, wsb)
-        H.hif8_gemm(dA, K, dW, N, 0, Cg, N, H.F32, M2, N, K, None, None, ws_g, 256)
+        before = H.hif8_launch_count()
+        with gemm_path(H.GEMM_PATH_NO_WARP):
+            H.hif8_gemm(dA, K, dW, N, 0, Cn, N, H.F32, M, N, K, None, None, ws_n, wsb)
+            H.hif8_gemm(dA, K, dW, N, 0, Cg, N, H.F32, M2, N, K, None, None, ws_g, 256)
+        with gemm_path(H.GEMM_PATH_WARP):
+            H.hif8_gemm(dA, K, dW, N, 0, Cw, N, H.F32, M, N, K, None, None, ws_w, 256)
+        assert H.hif8_launch_count() == before + 4
 
     def load(seed):
         Aq, Wq = W.random_codes((M2, K), seed=seed), W.random_codes((K, N), seed=seed + 1)
@@ -293,10 +294,11 @@ def test_gemm_calls_replay_from_a_cuda_graph():
         Aq, Wq = load(seed)
         g.replay()
         torch.cuda.synchronize()
-        assert H.hif8_gemm_status(ws_n) == 0 and H.hif8_gemm_status(ws_g) == 0
+        assert H.hif8_gemm_status(ws_n) == 0 and H.hif8_gemm_status(ws_g) == 0 and H.hif8_gemm_status(ws_w) == 0
         Cs, S = O.gemm_full(Aq, Wq, False, 0, 0)
         check(Cg.cpu().numpy().astype(np.float64), Cs, S, H.F32)
         check(Cn.cpu().numpy().astype(np.float64), Cs[:M], S[:M], H.F32)
+        check(Cw.cpu().numpy().astype(np.float64), Cs[:M], S[:M], H.F32)
 
 
 def test_tensor_map_cache_survives_eviction_and_pointer_reuse():
@@ -357,8 +359,8 @@ def test_gemm_repeated_runs_are_bit_identical(mode):
 @pytest.mark.parametrize("shape", [(65, 272, 128), (96, 512, 16), (208, 1008, 2064), (128, 512, 4096), (512, 1040, 1168), (304, 10000, 1040), (512, 20000, 144)])
 def test_gemm_weights_decoded_in_the_kernel(shape, form, w_is_nk, c_dtype, accumulate):
     # One tile per pair without and with a split along K (parts of unequal length, K that ends within a k-block), 80 tiles on
-    # 74 pairs (the last ones split, in a launch of their own) and 160 (several tiles per pair, fewer k-blocks than decode groups);
-    # activation rows in one and two pieces, ending within a piece of eight; activations as bytes and expanded, from both layouts.
+    # 74 pairs (the last ones in parts, in a launch of their own) and 158 (several tiles per pair, fewer k-blocks than decode groups);
+    # activation rows in one to six pieces, ending within a piece of eight; activations as bytes and expanded, from both layouts.
     M, N, K = shape
     columns, expanded = form.startswith("columns"), form.endswith("expanded")
     lda = (M + 15) // 16 * 16 if columns else K
@@ -382,8 +384,11 @@ def test_gemm_weights_decoded_in_the_kernel(shape, form, w_is_nk, c_dtype, accum
         c0 = C.float().cpu().numpy()
     wsb = 256 + (2 * M * K + 255) // 256 * 256 if expanded else 256
     ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")
-    H.hif8_gemm_ex(to_dev(A), lda, columns, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
-                   torch.tensor([3], dtype=torch.int32, device="cuda"), torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    before = H.hif8_launch_count()
+    with gemm_path(POLICY["a" if expanded else False]):
+        H.hif8_gemm_ex(to_dev(A), lda, columns, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
+                       torch.tensor([3], dtype=torch.int32, device="cuda"), torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    assert H.hif8_launch_count() - before in ((2, 3) if expanded else (1, 2))
     assert H.hif8_gemm_status(ws) == 0
     out = C.float().cpu().numpy().astype(np.float64)
     assert np.array_equal(out[:, N:], c0[:, N:].astype(np.float64))
@@ -421,8 +426,9 @@ def test_gemm_narrow_splits(shape, staged, w_is_nk, c_dtype, accumulate):
         c0 = C.float().cpu().numpy()
     wsb = H.hif8_workspace_bytes(H.WS_GEMM, M * K + K * N) if staged else 256
     ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")
-    H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
-                   torch.tensor([3], dtype=torch.int32, device="cuda"), torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    with gemm_path(POLICY[staged]):
+        H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
+                       torch.tensor([3], dtype=torch.int32, device="cuda"), torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
     assert H.hif8_gemm_status(ws) == 0
     out = C.float().cpu().numpy().astype(np.float64)
     assert np.array_equal(out[:, N:], c0[:, N:].astype(np.float64))

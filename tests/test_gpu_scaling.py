@@ -9,7 +9,7 @@ import paper_2409_16626_b200 as H
 import workloads as W
 from oracle import hif8_oracle as O
 
-from gpu_util import NP_OF, bf16_half_ulp, both_operands_expanded, dev_empty, to_dev
+from gpu_util import NP_OF, POLICY, bf16_half_ulp, dev_empty, gemm_path, gemm_workspace_bytes, to_dev
 
 pytestmark = pytest.mark.gpu
 MODES = [H.RND_TA, H.RND_HR, H.RND_SSR, H.RND_TE, H.RND_SR]
@@ -177,8 +177,7 @@ def test_channel_encode_degenerate_shapes():
     assert H.hif8_channel_amax_scale_encode(x, 7, out, 4, 4, 1, d_amax=d_amax, check=False) == 2
 
 
-@pytest.mark.parametrize("staged", [False, True, "a"])  # "a": workspace for A alone (with [N,K] weights: the swapped form,
-                                                        # one weight exponent per accumulator row)
+@pytest.mark.parametrize("staged", [False, True, "a", "warp", "auto"])
 @pytest.mark.parametrize("w_is_nk", [0, 1])
 @pytest.mark.parametrize("c_dtype", [H.F32, H.BF16])
 def test_gemm_channel_scaled(c_dtype, w_is_nk, staged):
@@ -192,9 +191,9 @@ def test_gemm_channel_scaled(c_dtype, w_is_nk, staged):
     sa = -7
     ldc = (N + 7) // 8 * 8
     C = torch.full((M, ldc), float("nan"), dtype=torch.float32 if c_dtype == H.F32 else torch.bfloat16, device="cuda")
-    wsb = H.hif8_workspace_bytes(H.WS_GEMM, (M * K if staged == "a" else M * K + K * N) if staged else 0)
+    wsb = gemm_workspace_bytes(staged, M, N, K)
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
-    with both_operands_expanded(staged is True):
+    with gemm_path(POLICY[staged]):
         H.hif8_gemm_channel_scaled(to_dev(Aq), K, to_dev(Wq), Wq.shape[1], w_is_nk, C, ldc, c_dtype, M, N, K,
                                    torch.tensor([sa], dtype=torch.int32, device="cuda"), to_dev(sw.view(np.uint32)), ws, wsb)
     assert H.hif8_gemm_status(ws) == 0
