@@ -2438,6 +2438,16 @@ struct WarpTiling {
     WarpPlan plan{};
     int mt = 0, row_blocks = 0;
     double cycles = 1e30;
+    struct Limits {
+        int cols, chunks;  // columns of a unit; 64-k blocks of a slice at most
+        uint32_t deposit;
+    };
+    template <bool W_IS_NK, int MT>
+    static Limits limits()
+    {
+        using S = WarpShape<W_IS_NK, MT>;
+        return Limits{S::kCols, S::CH, S::kDeposit};
+    }
     WarpTiling() = default;
     WarpTiling(int M, int N, int K, bool w_is_nk, bool a_is_km, const int* clusters)
     {
@@ -2449,17 +2459,17 @@ struct WarpTiling {
     {
         const int blocks = (M + 8 * m - 1) / (8 * m);
         if (blocks > 65535) return;  // the second dimension of a grid
-        const int ut = w_is_nk ? 1 : 2, max_chunks = (w_is_nk ? 4 : 2) / (m == 4 ? 2 : 1), cols = 16 * ut;
-        const int units = (N + cols - 1) / cols, kb = (K + 63) / 64;
-        const uint32_t deposit = (uint32_t)(cols * 8 * m * 4);
+        const Limits l = w_is_nk ? (m == 1 ? limits<true, 1>() : (m == 2 ? limits<true, 2>() : limits<true, 4>()))
+                                 : (m == 1 ? limits<false, 1>() : (m == 2 ? limits<false, 2>() : limits<false, 4>()));
+        const int units = (N + l.cols - 1) / l.cols, kb = (K + 63) / 64;
         for (int c = 1; c <= kWarpMaxCluster; c++) {
             if (clusters[c] <= 0) continue;
             const int fit = clusters[c] / blocks, n = fit < 1 ? 1 : (fit < units ? fit : units), nu = (units + n - 1) / n;
             const int rounds = fit < 1 ? (blocks + clusters[c] - 1) / clusters[c] : 1;
-            if ((uint32_t)(units / n + 1) * deposit > kWarpSumBytes) continue;
+            if ((uint32_t)(units / n + 1) * l.deposit > kWarpSumBytes) continue;
             for (int s = 1; s <= kWarpWarps; s++) {
                 const int chunks = (kb + c * s - 1) / (c * s), lanes = kWarpWarps / s;
-                if (chunks > max_chunks || (kb + chunks - 1) / chunks <= (c - 1) * s) continue;  // (the latter: a block of the cluster without work)
+                if (chunks > l.chunks || (kb + chunks - 1) / chunks <= (c - 1) * s) continue;  // (the latter: a block of the cluster without work)
                 const int turns = (nu + lanes - 1) / lanes, active = s * (lanes < nu ? lanes : nu);
                 const double t = rounds * (w_is_nk ? 3500.0 + 40.0 * active * chunks * m + 46.0 * nu * s * m + 450.0 * turns + 890.0 * turns * chunks + (c > 1 ? 4100.0 : 0.0)
                                                    : 3300.0 + 24.0 * active * chunks * m + 122.0 * nu * s * chunks + 34.0 * nu * s * m + 970.0 * turns +
@@ -2472,7 +2482,7 @@ struct WarpTiling {
             }
         }
     }
-    int clusters_used() const { return plan.q > 0 ? (plan.units - plan.rem) / plan.q : plan.rem; }
+    int clusters_used() const { return (plan.units - plan.rem) / plan.q; }  // (no more clusters than units: q > 0)
 };
 
 template <int MT>
