@@ -2351,8 +2351,10 @@ struct WeightsTiling {
         const long long slabs = (N + 2 * BM - 1) / (2 * BM);
         // (the launch that expands, its passing over to the kernel, and 1 / 430 or, transposed, 1 / 260 of a cycle per element)
         const double before = act == kActExpanded ? 11000.0 + (double)M * K * (a_is_km ? 0.0039 : 0.0023) : 7500.0;
-        for (int pieces = least; pieces == least || (slabs * pieces <= clusters[1] && (pieces - 1) * unit < M); pieces++) {
+        int next;  // (the fewest pieces with fewer rows each: many numbers of pieces round up to the same rows)
+        for (int pieces = least; pieces == least || slabs * pieces <= clusters[1]; pieces = next) {
             const int rows = ((M + pieces - 1) / pieces + unit - 1) / unit * unit, n = (M + rows - 1) / rows;
+            next = rows > unit ? (M + rows - unit - 1) / (rows - unit) : 0x7FFFFFFF;
             const WeightsCost c{(K + kb - 1) / kb, rows, unit, act == kActExpanded, clusters};
             const double t = before + c.all(slabs * n);
             if (t < cycles) { cycles = t; chunks = n; bn = rows; tiles = slabs * n; cost = c; }
@@ -2449,7 +2451,8 @@ struct WarpTiling {
         return Limits{S::kCols, S::CH, S::kDeposit};
     }
     WarpTiling() = default;
-    WarpTiling(int M, int N, int K, bool w_is_nk, bool a_is_km, const int* clusters)
+    // the division that takes the fewest cycles, if it takes fewer than `below` (otherwise mt = 0)
+    WarpTiling(int M, int N, int K, bool w_is_nk, bool a_is_km, const int* clusters, double below) : cycles(below)
     {
         if ((double)M * N * K > 4e9 || K > 4096 * kWarpMaxCluster || (!w_is_nk && (N & 3))) return;  // (far beyond what it is good for; a thread loads four columns of [K,N] in one piece)
         for (int m = a_is_km ? 4 : 1; m <= 4; m *= 2)
@@ -2467,7 +2470,10 @@ struct WarpTiling {
             const int fit = clusters[c] / blocks, n = fit < 1 ? 1 : (fit < units ? fit : units), nu = (units + n - 1) / n;
             const int rounds = fit < 1 ? (blocks + clusters[c] - 1) / clusters[c] : 1;
             if ((uint32_t)(units / n + 1) * l.deposit > kWarpSumBytes) continue;
-            for (int s = 1; s <= kWarpWarps; s++) {
+            const int least = (kb + c * l.chunks - 1) / (c * l.chunks);  // (with fewer slices a slice is longer than a warp can hold)
+            // (what no division into this many blocks goes below: most are not looked at)
+            if (rounds * (w_is_nk ? 4840.0 + 46.0 * nu * least * m : 5510.0 + 122.0 * nu * (kb / c) + 34.0 * nu * least * m) >= cycles) continue;
+            for (int s = least; s <= kWarpWarps; s++) {
                 const int chunks = (kb + c * s - 1) / (c * s), lanes = kWarpWarps / s;
                 if (chunks > l.chunks || (kb + chunks - 1) / chunks <= (c - 1) * s) continue;  // (the latter: a block of the cluster without work)
                 const int turns = (nu + lanes - 1) / lanes, active = s * (lanes < nu ? lanes : nu);
@@ -2561,7 +2567,8 @@ struct NarrowTiling {
 };
 
 // Which kernel takes a product, and how it divides it: a function of the sizes, the layouts and what the workspace has room for, so
-// it is worked out once for each (the search over divisions takes a few microseconds).
+// it is kept for the 64 used last.  (The search over divisions takes 0.5 us on the host, 2 us at most: products of 1 to 8192 rows, N and K 16
+// to 28672.  It runs outside the lock, so that threads with new sizes do not wait for one another.)
 enum GemmForm { kFormWarp, kFormNarrow, kFormWeights, kFormPair };
 struct GemmKey {
     int M, N, K, dev, w_is_nk, a_is_km, room, policy;
@@ -2578,8 +2585,8 @@ static bool choose(const GemmKey& k, int sm_count, const int* wd_clusters, const
 {
     if (k.policy == HIF8_GEMM_PATH_WARP) {
         out->form = kFormWarp;
-        out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters);
-        return out->warp.cycles < 1e30;
+        out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters, 1e30);
+        return out->warp.mt > 0;
     }
     const bool narrow = !k.a_is_km && k.M <= kNarrowMaxM;
     out->form = narrow ? kFormNarrow : kFormWeights;
@@ -2602,10 +2609,10 @@ static bool choose(const GemmKey& k, int sm_count, const int* wd_clusters, const
         }
     }
     if (k.policy != HIF8_GEMM_PATH_AUTO) return true;
-    out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters);
     // (1.2: the search takes the division whose time is underestimated most; 6000: the launch in front of the narrow kernel, its start and end)
     const double other = narrow ? NarrowTiling(k.M, k.N, k.K, sm_count, nw_clusters, k.room > 0).cycles + 6000.0 : out->weights.cycles;
-    if (1.2 * out->warp.cycles < other) out->form = kFormWarp;
+    out->warp = WarpTiling(k.M, k.N, k.K, k.w_is_nk, k.a_is_km, wp_clusters, other / 1.2);
+    if (out->warp.mt > 0) out->form = kFormWarp;
     return true;
 }
 
@@ -2643,7 +2650,6 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     const int *wd_clusters = nullptr, *nw_clusters = nullptr, *wp_clusters = nullptr;
     if (!gemm_kernels_ready(dev, &sm_count, &wd_clusters, &nw_clusters, &wp_clusters)) return HIF8_ERR_CUDA;
 
-
     // Operands as BF16 in the workspace: none, the activations, both.
     const size_t bytes_a = (((size_t)M * K * 2) + 255) & ~(size_t)255, bytes_w = (((size_t)K * N * 2) + 255) & ~(size_t)255;
     const bool a_contiguous = lda == (a_is_km ? M : K), w_contiguous = ldw == (w_is_nk ? K : N), ws_aligned = !(reinterpret_cast<uintptr_t>(workspace) & 255);
@@ -2655,8 +2661,10 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
     key.w_is_nk = w_is_nk != 0; key.a_is_km = a_is_km != 0; key.room = room_w ? 2 : (room_a ? 1 : 0);
     key.policy = g_path_policy.load(std::memory_order_relaxed);
     GemmChoice choice;
-    if (!g_choices.lookup_or_make(key, &choice, [&](const GemmKey& k, GemmChoice* out) { return choose(k, sm_count, wd_clusters, nw_clusters, wp_clusters, out); }))
-        return HIF8_ERR_SHAPE;
+    if (!g_choices.find(key, &choice)) {
+        if (!choose(key, sm_count, wd_clusters, nw_clusters, wp_clusters, &choice)) return HIF8_ERR_SHAPE;
+        g_choices.put(key, choice);
+    }
     if (choice.form == kFormWarp) return launch_warp_gemm(Aq, lda, a_is_km, Wq, ldw, w_is_nk, p, choice.warp, st);
     // the status word is cleared on the stream before the kernels; the narrow path clears its tickets in the same operation
     size_t clear_bytes = 4;
