@@ -258,7 +258,7 @@ int hif8_fake_quant(const void* src, void* dst, int dtype, size_t n, int use_ama
  * multiple of 16 (HIF8_ERR_SHAPE).  NaN / Inf codes propagate as in IEEE arithmetic.
  * workspace: at least hif8_workspace_bytes(HIF8_WS_GEMM, 0) = 256 bytes, 16-byte aligned; its first int is a device
  * status word that the call clears and the kernel sets if one of its bounded waits ever gives up (see
- * hif8_gemm_status).  With only that, the tensor-core kernel decodes both byte operands itself.
+ * hif8_gemm_status).  With only that, the kernels decode both byte operands themselves.
  * With hif8_workspace_bytes(HIF8_WS_GEMM, M*K + K*N) bytes, 256-byte aligned, and contiguous operands (lda = K,
  * ldw = row length of Wq), each operand byte is instead decoded once into the workspace (BF16, exact) and the
  * tensor-core kernel streams BF16 tiles: several times faster for compute-bound shapes, same results.
@@ -266,10 +266,10 @@ int hif8_fake_quant(const void* src, void* dst, int dtype, size_t n, int use_ama
  * expanded into the workspace and the kernel decodes only the W tiles (any ldw): for when the weight's BF16 copy does
  * not fit but the activation's does; same results.  A workspace with room for both operands takes this form too while
  * the product is too small to win the pass over W back (see hif8_gemm_path_policy).
- * Products with at most 64 rows of A (and A given as [M,K]) take a weight-streaming kernel whatever the workspace;
- * with the workspace size above it first expands the few rows of A to BF16 there (one small launch more, A contiguous).
- * Products of few rows and a small weight, and those of few tiles, take A as bytes in one launch even when the workspace
- * has room for it, where that is faster.
+ * Products of few rows and a small weight take one launch in which every warp decodes its share of both operands, whatever
+ * the workspace.  Others with at most 64 rows of A (and A given as [M,K]) take a weight-streaming kernel; with the workspace
+ * size above it first expands the few rows of A to BF16 there (one small launch more, A contiguous).  Products of few tiles
+ * take A as bytes even when the workspace has room for it, where that is faster.
  * Where several SMs share the sum of an output (K split among them), the parts are added in a fixed order: results are
  * reproducible run to run; how K is split depends on the sizes, the device and the workspace.
  */

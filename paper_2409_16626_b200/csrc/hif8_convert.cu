@@ -594,9 +594,9 @@ __global__ void clear_accum_kernel(uint32_t* accum)
 // block) measured 2 us faster on a 64 MiB tensor than the four of the converting kernels.
 constexpr int kUnrollAmax = 8;
 // The pass that follows walks the tensor from its end, so the last 64 MiB are read with the default L2 policy and what comes before
-// them streams through: with the default policy for all of it the end was partly displaced again (8192 x 8192 BF16 fake-quant 63.6 ->
-// 61.8 us, 250 M elements 229 -> 221; 32 MiB 62.2, 48 MiB 61.6, 80 MiB 62.2, 96 MiB 62.6; evict-last for the end 62.6).  STREAM: there
-// is something before them.
+// them streams through: with the default policy for all of it the end was partly displaced again (BF16 fake-quant, four tensors in turn,
+// us: 8192 x 8192 63.4, now 61.8, 250 M elements 232 and 224; 32 MiB 62.2, 48 MiB 61.6, 80 MiB 62.2, 96 MiB 62.6; evict-last for the end
+// 62.6).  STREAM: there is something before them.
 constexpr unsigned long long kKeepVecs = (64ull << 20) / 16;
 template <int SRC, bool STREAM>
 __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__ srcv, unsigned long long n,
@@ -695,9 +695,9 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const uint8_t* __restr
 }
 
 // The same for 16-bit results of large tensors, with a table that has a copy per lane: the conflicts of one table for all lanes, 3.5
-// wavefronts per 32 lookups, took longer than the transfer (BF16, us, one table / a copy per lane: 3001 x 4099 codes 7.8 / 7.2, 8 M
-// 5.8 / 5.2, 100 M 49.1 / 46.0).  Filling it takes a block as long as half of its lookups, so a block of 512 threads has 16384 codes
-// (8192: 7.9, 32768: 7.6 us); below two million codes that leaves too few blocks (1 M: 2.1 / 2.2).  FP32 results store twice the
+// wavefronts per 32 lookups, took longer than the transfer (BF16, us, one table / a copy per lane, four pairs of buffers in turn:
+// 3001 x 4099 codes 8.3 / 7.3, 8 M 6.0 / 4.7, 100 M 48.9 / 45.5).  Filling it takes a block as long as half of its lookups, so a block of 512 threads has 16384 codes
+// (3001 x 4099 codes 7.2 us; 8192: 7.9, 32768: 7.6); below two million codes that leaves too few blocks (1 M: 2.1 / 2.2).  FP32 results store twice the
 // bytes a code and gain nothing (100 M: 75.3 / 76.4).
 constexpr int kDecodeThreads = 512, kDecodeCodes = 32;  // codes per thread
 constexpr size_t kDecodeStreamFrom = (size_t)1 << 21;

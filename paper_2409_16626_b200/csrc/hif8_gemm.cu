@@ -238,8 +238,8 @@ __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr)
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 // Arrival that publishes nothing: "this CTA is through with what others may now overwrite".  One with release waits for every store
-// the SM has in flight, results included (256 x 1536 x 768 split in two: the two such barriers of a call took 1700 and 1260 cycles,
-// now 1500 and 410).
+// the SM has in flight, results included (256 x 1536 x 768 split in two: the two such barriers of a call take 1500 and 410 cycles, with
+// release 1700 and 1260).  At the end of a kernel it needs that no signal to another CTA is under way that nobody has waited for.
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all()
@@ -1264,8 +1264,8 @@ __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, i
 // Instantiations by tile order and row pitch.  (With the choice of the order made in the kernel, the divisions of the other one in
 // the way of the first copies, 128 x 512 x 512 took 10.0 us instead of 9.8.)
 // kParts is the last, incomplete round of a large product in tiles of fewer activation rows: divided along K alone, two tiles of
-// 2048 x 7168 x 4096 kept 8 pairs of 74 busy (with it 104 -> 101.5 us, with activations as bytes 144 -> 140; that launch waits for
-// nothing of the one in front of it, see TilePlan::follows, which is 1 us of it).
+// 2048 x 7168 x 4096 kept 8 pairs of 74 busy (103.7 us, with it 101.5; with activations as bytes 138.4 and 135.8; that launch waits
+// for nothing of the one in front of it, see TilePlan::follows, which is 1 us of it).
 enum WeightsForm { kOneGroup, kGroups, kFarRows, kParts };  // up to eight pieces; more; the rows of C 4 GiB apart or more (any number of pieces); parts of tiles
 constexpr int kGroupPieces = 8;
 
@@ -1644,8 +1644,8 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     if (tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    // (unlikely: what follows a wait that gave up stands behind the rest of the code, whose last lines would otherwise be fetched
-    // later, 300 cycles a call)
+    // (unlikely, so that what follows a wait that gave up stands behind the rest of the code.  The question itself costs a small product
+    // 0.1 us; asked by one warp a CTA alone it costs the same.)
     if (__builtin_expect(*abort_flag != 0, 0)) {
         if (threadIdx.x < 2u * split) st_cluster_u32(map_to_cta(lay.gave_up(), threadIdx.x), 1u);
         __syncwarp();
@@ -2284,9 +2284,10 @@ int launch_bf16_pair_gemm(const void* a_bf, const void* w_bf, int w_is_nk, GemmP
 using namespace hif8;
 
 // Time of the weights kernel in cycles, from measurements: a k-block (128 k with expanded activations; 64 k with bytes, where the
-// activations' lookups count too) and a tile's drain; what the exchange of a split tile costs beyond that (two cluster barriers,
-// the sums at 20 bytes a cycle, less what the shared epilogue saves) at bn = 256, about half of it at 128; a launch of its own for
-// the last round (set-up, first copies).
+// activations' lookups count too) and a tile's drain; what the exchange of a split tile costs beyond that (a cluster barrier, the
+// sums at 20 bytes a cycle and the wait for them, less what the shared epilogue saves); a launch of its own for the last round (set-up,
+// first copies).  The exchange's terms were measured when a second cluster barrier, both with release, stood in the place of that
+// wait, and are up to 1200 cycles too high now: some products that would gain from it are not split.
 struct WeightsCost {
     int num_kb, bn, unit;  // unit: the activation rows of a tile are a multiple of this
     bool expanded;

@@ -10,9 +10,9 @@
 //
 // What bounds it: for the small products it is chosen for, latency (loads, the activations' decoding, a unit's deposit and sum:
 // about 5000 cycles with one unit a warp), which is why it exists: the tensor-memory kernels spend 12000 on barriers, tensor memory,
-// descriptors, hand-overs between their roles and another launch that expands the activations.  us a call, [N,K] weights, before
-// and now: 4 x 512 x 512 7.2 / 2.9, 16 x 1024 x 1024 8.0 / 4.5, 16 x 2048 x 2048 9.4 / 6.4, 128 x 512 x 1024 11.5 / 4.8; [K,N]:
-// 16 x 512 x 512 7.4 / 5.0.  A stream of weights it does not sustain (16 x 28672 x 8192: 100 us against 60): all warps of a block
+// descriptors, hand-overs between their roles and another launch that expands the activations.  us a call in a graph, [N,K] weights,
+// the kernel that would take it otherwise / this: 4 x 512 x 512 6.7 / 2.7, 16 x 1024 x 1024 7.1 / 3.8, 16 x 2048 x 2048 8.4 / 5.2,
+// 128 x 512 x 1024 6.8 / 5.4; [K,N]: 16 x 512 x 512 7.0 / 3.9; too large for it: 256 x 768 x 1536 8.6 / 9.3.  A stream of weights it does not sustain (16 x 28672 x 8192: 100 us against 60): all warps of a block
 // wait for one another once per unit, and four warps a scheduler do not cover the lookups' latency with 64 registers of activations each.
 //
 // Column units.  [N,K] weights: 16 columns, the rows of one m16n8k16 operand.  A thread (g = lane / 4, t = lane % 4) loads 16
