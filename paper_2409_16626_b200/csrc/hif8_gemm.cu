@@ -2380,8 +2380,10 @@ struct WeightsTiling {
     {
         const int unit = act == kActColumns ? 128 : 32, kb = act == kActExpanded ? 2 * BK : BK, least = (M + BN - 1) / BN;
         const long long slabs = (N + 2 * BM - 1) / (2 * BM);
-        // (the launch that expands, its passing over to the kernel, and 1 / 430 or, transposed, 1 / 260 of a cycle per element)
-        const double before = act == kActExpanded ? 11000.0 + (double)M * K * (a_is_km ? 0.0039 : 0.0023) : 7500.0;
+        // (Expanded: the launch that does it, its passing over to the kernel, and so much of a cycle per element; transposed, the first
+        // three million cost more.)
+        const double elements = (double)M * K, transposed = 0.0039 * elements < 8000.0 + 0.0013 * elements ? 0.0039 * elements : 8000.0 + 0.0013 * elements;
+        const double before = act == kActExpanded ? 11000.0 + (a_is_km ? transposed : 0.0009 * elements) : 7500.0;
         int next;  // (the fewest pieces with fewer rows each: many numbers of pieces round up to the same rows)
         for (int pieces = least; pieces == least || slabs * pieces <= clusters[1]; pieces = next) {
             const int rows = ((M + pieces - 1) / pieces + unit - 1) / unit * unit, n = (M + rows - 1) / rows;
@@ -2624,7 +2626,9 @@ static bool choose(const GemmKey& k, int sm_count, const int* wd_clusters, const
     if (!narrow) {
         const WeightsTiling bytes(k.M, k.N, k.K, k.a_is_km ? kActColumns : kActRows, k.a_is_km, wd_clusters);
         const WeightsTiling expanded(k.M, k.N, k.K, kActExpanded, k.a_is_km, wd_clusters);
-        out->weights = k.room && (k.policy == HIF8_GEMM_PATH_EXPAND_A || expanded.cycles < bytes.cycles) ? expanded : bytes;
+        // (3000: bytes [K,M] of 16 rows, of which every pair copies the same few lines)
+        const double crowded = k.a_is_km && k.M < 32 ? 3000.0 * (bytes.tiles < wd_clusters[1] ? (double)bytes.tiles / wd_clusters[1] : 1.0) : 0.0;
+        out->weights = k.room && (k.policy == HIF8_GEMM_PATH_EXPAND_A || expanded.cycles < bytes.cycles + crowded) ? expanded : bytes;
         // Expanding W as well only pays when the product is large enough to win back the pass over W (3 bytes per element moved, at
         // 3300 bytes a cycle, and a launch) by the cheaper k-blocks and tiles of the pair kernel: 545 cycles per
         // 64 k and nothing between tiles, against the weights kernel's cost above.  Measured (us, both expanded / weights decoded in
