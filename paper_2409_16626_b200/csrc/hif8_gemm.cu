@@ -2315,12 +2315,13 @@ using namespace hif8;
 
 // Time of the weights kernel in cycles, from measurements: a k-block (128 k with expanded activations; 64 k with bytes, where the
 // activations' lookups count too) and a tile's drain; what the exchange of a split tile costs beyond that (a cluster barrier, the
-// sums at 20 bytes a cycle and the wait for them, less what the shared epilogue saves); a launch of its own for the last round (set-up,
-// first copies).  The exchange's terms were measured when a second cluster barrier, both with release, stood in the place of that
-// wait, and are up to 1200 cycles too high now: some products that would gain from it are not split.
+// sums at 20 bytes a cycle and the wait for them, less what the shared epilogue saves).  A launch of its own for the last round:
+// from 90 products with and without one.  (With 4200 cycles for it and nothing in proportion 17 of them lost 3 to 16 % by it; behind a
+// transposing expansion 4200 it is.)  The exchange's terms were measured when a second cluster barrier, both with release, stood in
+// the place of that wait, and are up to 1200 cycles too high now: some products that would gain from it are not split.
 struct WeightsCost {
     int num_kb, bn, unit;  // unit: the activation rows of a tile are a multiple of this
-    bool expanded;
+    bool expanded, transposed;  // the activations are expanded by the launch in front, from [K,M]
     const int* clusters;  // clusters of s pairs that the device holds
     double tiles(long long n, int split) const
     {
@@ -2353,7 +2354,7 @@ struct WeightsCost {
             WeightsCost c = *this;
             c.bn = (bn + want * unit - 1) / (want * unit) * unit;
             const int parts = (bn + c.bn - 1) / c.bn, split = c.best_split(rem * parts);
-            const double t = c.tiles(rem * parts, split) + 4200.0;
+            const double t = transposed ? c.tiles(rem * parts, split) + 4200.0 : 1.08 * c.tiles(rem * parts, split) + 7000.0;
             if ((split > 1 || parts > 1) && rem * parts <= clusters[split] && t < r.cycles) r = Rest{rem, parts, c.bn, split, t};
         }
         return r;
@@ -2388,7 +2389,7 @@ struct WeightsTiling {
         for (int pieces = least; pieces == least || slabs * pieces <= clusters[1]; pieces = next) {
             const int rows = ((M + pieces - 1) / pieces + unit - 1) / unit * unit, n = (M + rows - 1) / rows;
             next = rows > unit ? (M + rows - unit - 1) / (rows - unit) : 0x7FFFFFFF;
-            const WeightsCost c{(K + kb - 1) / kb, rows, unit, act == kActExpanded, clusters};
+            const WeightsCost c{(K + kb - 1) / kb, rows, unit, act == kActExpanded, act == kActExpanded && a_is_km, clusters};
             const double t = before + c.all(slabs * n);
             if (t < cycles) { cycles = t; chunks = n; bn = rows; tiles = slabs * n; cost = c; }
         }

@@ -148,8 +148,8 @@ def test_gemm_pieces_of_activation_rows(shape, form):
 
 
 @pytest.mark.parametrize("accumulate", [0, 1])
-@pytest.mark.parametrize("shape,form", [((1216, 3904, 144), "rows"), ((1216, 3904, 144), "expanded"), ((1216, 3904, 528), "columns"), ((2400, 4096, 272), "rows")] +
-                         [(s, f) for s in ((1200, 3904, 1040), (512, 10000, 528), (2400, 4096, 1040)) for f in ("rows", "columns", "expanded")])
+@pytest.mark.parametrize("shape,form", [((1216, 3904, 1040), "rows"), ((1216, 3904, 1040), "columns"), ((304, 10000, 1552), "expanded"), ((2400, 4096, 1040), "rows")] +
+                         [(s, f) for s in ((1200, 3904, 1552), (512, 10000, 1552), (2400, 4096, 2064)) for f in ("rows", "columns", "expanded")])
 def test_gemm_last_round_in_parts(shape, form, accumulate):
     # 80 to 160 tiles of up to 256 activation rows on 74 pairs: the last ones in parts of fewer rows, some split along K, in a
     # launch of their own; the last part of a tile and the last piece of the matrix shorter than the others; more pieces than one
