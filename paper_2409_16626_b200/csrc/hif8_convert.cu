@@ -596,8 +596,10 @@ constexpr int kUnrollAmax = 8;
 // The pass that follows walks the tensor from its end, so the last 64 MiB are read with the default L2 policy and what comes before
 // them streams through: with the default policy for all of it the end was partly displaced again (BF16 fake-quant, four tensors in turn,
 // us: 8192 x 8192 63.4, now 61.8, 250 M elements 232 and 224; 32 MiB 62.2, 48 MiB 61.6, 80 MiB 62.2, 96 MiB 62.6; evict-last for the end
-// 62.6).  STREAM: there is something before them.
-constexpr unsigned long long kKeepVecs = (64ull << 20) / 16;
+// 62.6).  STREAM: there is something before them.  FP32 from 72 MiB on: with a little more than 64 MiB it loses (us, without
+// and with it: fake-quant of 16.8 M elements 29.3 / 29.5, scale and encode of 18 M 31.1 / 31.4; of 20 M 35.1 / 34.7 and 35.2 / 35.6, of
+// 22.5 M 39.4 / 39.0 and 38.9 / 38.7).
+constexpr unsigned long long kKeepVecs = (64ull << 20) / 16, kStreamVecsF32 = (72ull << 20) / 16;
 template <int SRC, bool STREAM>
 __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__ srcv, unsigned long long n,
                                                         unsigned long long n_vec, uint32_t* accum, float* d_amax_out)
@@ -901,7 +903,7 @@ int launch_amax(const void* src, int dtype, unsigned long long n, uint32_t* accu
     unsigned long long n_vec = vec_ok ? n / pv : 0;
     unsigned grid = grid_for(n_vec, n, sms, kUnrollAmax);
     switch (dtype) {
-        case HIF8_F32: launch_pdl(n_vec > kKeepVecs ? amax_kernel<HIF8_F32, true> : amax_kernel<HIF8_F32, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
+        case HIF8_F32: launch_pdl(n_vec > kStreamVecsF32 ? amax_kernel<HIF8_F32, true> : amax_kernel<HIF8_F32, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
         case HIF8_BF16: launch_pdl(n_vec > kKeepVecs ? amax_kernel<HIF8_BF16, true> : amax_kernel<HIF8_BF16, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
         default: launch_pdl(n_vec > kKeepVecs ? amax_kernel<HIF8_F16, true> : amax_kernel<HIF8_F16, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
     }
