@@ -1220,7 +1220,8 @@ struct TilePlan {
 
 // Eight results that are there already, `pitch` bytes apart.  All loads go out before the first is used: left to the compiler, an
 // instantiation that is short of registers waited for each of them (3872 x 3200 x 1680, [K,N] weights, operands as bytes, added
-// to FP32: 87.5 us a call, so 77.8).
+// to FP32: 87.5 us a call, so 77.8; BF16 86 and 75.7).  BATCH: where that matters, in the instantiations for more than eight pieces of
+// activation rows; with it in the one for up to eight, 2048 x 7168 x 4096 that adds to nothing took 134.7 us instead of 134.0.
 __device__ __forceinline__ void load_column_f32(const unsigned char* at, unsigned long long pitch, float (&v)[8])
 {
     asm volatile("{\n\t.reg .u64 a;\n\t"
@@ -1244,12 +1245,12 @@ __device__ __forceinline__ void load_column_bf16(const unsigned char* at, unsign
 // instructions a store.  So the pitch has 32 bits, one multiply-add per row, unless rows lie 4 GiB apart or more (a few rows of
 // a large buffer): that is an instantiation of its own, since 64-bit products for all cost 1 % (4096 x 28672 x 8192 with
 // expanded activations: 1320 -> 1352 us).
-template <typename Pitch>
+template <bool BATCH, typename Pitch>
 __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, int is_f32, int accumulate, int rows, float (&v)[8])
 {
     auto at = [&](int i) { return out + (unsigned long long)pitch * (uint32_t)i; };
     if (accumulate) {
-        if (is_f32 && rows >= 8) {
+        if (BATCH && is_f32 && rows >= 8) {
             float old[8];
             load_column_f32(out, (unsigned long long)pitch, old);
 #pragma unroll
@@ -1257,7 +1258,7 @@ __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, i
         } else if (is_f32) {
 #pragma unroll
             for (int i = 0; i < 8; i++) v[i] += i < rows ? __ldcs(reinterpret_cast<const float*>(at(i))) : 0.f;
-        } else if (rows >= 8) {
+        } else if (BATCH && rows >= 8) {
             unsigned short old[8];
             load_column_bf16(out, (unsigned long long)pitch, old);
 #pragma unroll
@@ -1656,7 +1657,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
 #pragma unroll
                     for (int i = 0; i < 8; i++) v[i] *= f2;
                 }
-                if (n < p.N) store_columns(out + j * 8 * pitch, (std::conditional_t<FORM == kFarRows, unsigned long long, uint32_t>)pitch, p.c_is_f32, p.accumulate, cols - j * 8, v);
+                if (n < p.N) store_columns<FORM != kOneGroup>(out + j * 8 * pitch, (std::conditional_t<FORM == kFarRows, unsigned long long, uint32_t>)pitch, p.c_is_f32, p.accumulate, cols - j * 8, v);
             }
             tc_fence_before();
             __syncwarp();
