@@ -93,37 +93,17 @@ constexpr TaTable make_trunc_table()
 }
 __device__ const TaTable g_trunc_table = make_trunc_table();
 
-// Hybrid / simplified stochastic rounding (Section 3.2, Eq. 3): both neighbours of a scaled magnitude in one word.  Index =
-// (biased exponent, top three mantissa bits) of the magnitude, no sign: 2^-23 .. 2^16 are the binades that differ.
-//   bits 0-4   left shift that puts the discarded field of this binade at the top of a word (9 + mantissa width)
-//   bits 8-15  the neighbour below (truncation), bits 16-23 the neighbour above; bit 7 of either byte says "takes the
-//              sign" (clear for the single zero; the NaN pattern 0x80 reads as a zero magnitude that takes a sign which
-//              the caller arranges to be set)
-//   bits 30-31 are filled in at set-up (stochastic or round-half-away binade)
-// The binade of 2^-23 stands for everything below 2^-22 (see pair32_lookup): neighbours 0 and 2^-22, no mantissa bit kept.
-__host__ __device__ constexpr uint32_t pair_entry(uint32_t idx)
+// Truncated magnitudes for the roundings that add before they look up (hybrid / simplified stochastic rounding): index = (biased exponent,
+// top three mantissa bits), no sign, four codes per word.  Anything below 2^-22 is the single zero.
+struct MagnitudeTable { uint32_t v[512]; };
+constexpr MagnitudeTable make_magnitude_table()
 {
-    int e = (int)(idx >> 3);
-    uint32_t m3 = idx & 7u;
-    if (e == 255) return m3 ? 0x00808009u : 0x00EFEF09u;  // NaN / Inf
-    int E = e - 127;
-    if (E >= 16) return 0x00EFEF09u;
-    if (E < -23) return 0u;
-    if (E == -23) return 0x00810009u;
-    int w = mant_width(E);
-    uint32_t M = m3 >> (3 - w);
-    uint32_t down = pack_magnitude(E, M);  // E = 15, M = 1 is the Inf pattern by construction
-    uint32_t up = (M + 1u == (1u << w)) ? (E + 1 >= 16 ? 0x6Fu : pack_magnitude(E + 1, 0u)) : pack_magnitude(E, M + 1u);
-    return (uint32_t)(9 + w) | ((down | 0x80u) << 8) | ((up | 0x80u) << 16);
-}
-struct PairTable { uint32_t v[2048]; };
-constexpr PairTable make_pair_table()
-{
-    PairTable t{};
-    for (uint32_t i = 0; i < 2048; i++) t.v[i] = pair_entry(i);
+    MagnitudeTable t{};
+    for (uint32_t i = 0; i < 2048; i++)
+        if ((i >> 3) >= 105u) t.v[i >> 2] |= (uint32_t)trunc_entry(((i >> 3) << 4) | ((i & 7u) << 1)) << (8 * (i & 3u));
     return t;
 }
-__device__ const PairTable g_pair_table = make_pair_table();
+__device__ const MagnitudeTable g_magnitude_table = make_magnitude_table();
 
 // value of one byte as binary32 bits (Eq. 1 / Eq. 2 / specials)
 __device__ __forceinline__ uint32_t decode_bits_f32(uint32_t c)
@@ -258,11 +238,7 @@ template <int DT> __device__ __forceinline__ uint32_t to_bits(float v)
 //  * SR: thr[e] = sh, the number of discarded mantissa bits (23 - width; 0: nothing to round).
 //  * TE: thr[e] = half - 1 (bits 0-22; half itself where no mantissa bit is kept: the implicit one is odd), bit 26 "add
 //    the kept LSB", sh in bits 27-31; the binade of 2^-23 adds 2^23 - 1 (anything above the tie carries into 2^-22).
-//  * Hybrid / simplified stochastic rounding, FP32 sources: thr[] is not used.  One word per (exponent, top three
-//    mantissa bits) holds both neighbours and the binade's shift (pair_entry); the discarded field, left-aligned, is
-//    compared with the threshold (SR14: the source's low 14 bits; one half in the round-half-away binades of Eq. 3) and
-//    the comparison picks the byte: one 4-byte lookup per element.  (The same form measured slower than the one below
-//    for 16-bit sources: 54.7 against 41.7 us per 2^26 BF16 elements.)
+//  * Hybrid / simplified stochastic rounding, FP32 sources: sixteen bits per exponent (see code_sum32).
 //  * Hybrid / simplified stochastic rounding, 16-bit sources (T2 = 2 LSB + 1, complement 3 - 2 LSB): an increment is added
 //    to the bit pattern so that the carry out of the discarded field rounds up (also across binade and width boundaries),
 //    the old binade's discarded bits are cleared (~0 << sh) and the code is read from the truncating table.
@@ -270,23 +246,26 @@ template <int DT> __device__ __forceinline__ uint32_t to_bits(float v)
 //    (result 0 or 2^-22, F = |y| / 2^-22) only the binades of 2^-23 and 2^-24 can reach the threshold; their entries add
 //    the complement at the top of the pattern and step the exponent down by one / two, which leaves 2^-23 or 2^-22 when
 //    the threshold is reached and something below 2^-23 when not.
-// FP32 sources, hybrid / simplified stochastic rounding: the neighbour-pair word of the scaled value y and whether the
-// upper neighbour is taken
+
+// FP32 sources, hybrid / simplified stochastic rounding: magnitude code of an element.  SR14 rounds up iff F14 >= max(T14, 1), i.e. iff
+// |y| + (1 - max(T14, 1) / 2^14) ulp, truncated, reaches the upper neighbour; in a round-half-away binade of Eq. 3 half an ulp is added
+// instead.  Both sums truncate (rz), so neither can reach a neighbour that the exact one does not, and what is left of the discarded bits
+// is dropped by the truncating table (past a binade's end the leftover is below one unit of the next one).  Below 2^-22 the unit is 2^-22.
+// units[e], by the exponent of |y|: bits 0-7 the biased exponent of the ulp (0 in a round-half-away binade), bits 8-15 that of half
+// an ulp there (0 elsewhere).  Shifted into the exponent field the one that is not wanted leaves a zero or something below 2^-126, which the
+// truncation drops.  The 60 exponents of a wide gradient lie in 30 words, one per bank.
+// What bounded this was the integer pipe, which takes an instruction every other cycle: as a lookup of both neighbours, a shift of the
+// discarded field and a comparison an element took about 14 of them, so five, with the rest in the floating-point pipe (2^28 log-uniform
+// elements, us: HR 228 -> 204, SSR 217 -> 201; round half away takes 202).
 template <int MODE>
-__device__ __forceinline__ bool pair32_lookup(float y, uint32_t raw, const uint32_t* tab, uint32_t& ent)
+__device__ __forceinline__ uint32_t code_sum32(float x, uint32_t raw, float scale, const uint8_t* code8, const uint16_t* units)
 {
-    const float a = fabsf(y);
-    // below 2^-22 the result is 0 or 2^-22 with F = |y| / 2^-22: |y| / 2 + 2^-23 with truncation puts floor(F 2^23)
-    // into the mantissa of a value in the binade of 2^-23, and exceeds |y| exactly when |y| < 2^-22
-    const uint32_t w = __float_as_uint(fmaxf(a, __fmaf_rz(a, 0.5f, 1.1920928955078125e-07f)));
-    ent = tab[w >> 20];
-    const uint32_t u = __funnelshift_l(0u, w, ent);  // discarded field, left-aligned (shift = low five bits of ent)
-    uint32_t thr = max(raw << 18, 0x40000u);         // SR14: round up iff F14 >= max(T14, 1), T14 = low 14 source bits
-    if (MODE == HIF8_RND_HR) {                       // round-half-away binades of Eq. 3 (bit 31): the top discarded bit decides
-        const uint32_t m = (uint32_t)((int32_t)ent >> 31);
-        thr = (thr & ~m) | (m & 0x80000000u);
-    }
-    return u >= thr;
+    const float y = fabsf(x) * scale;
+    const uint32_t v = units[__float_as_uint(y) >> 23];
+    const float ulp = __uint_as_float(v << 23);
+    const float g = fmaxf(__uint_as_float(((raw << 9) & 0x7FFE00u) | 0x3F800000u), 1.00006103515625f);  // 1 + max(T14, 1) / 2^14
+    const float z = MODE == HIF8_RND_HR ? __fadd_rz(y, __uint_as_float(v << 15)) : y;
+    return code8[__float_as_uint(__fmaf_rz(ulp, 2.f - g, z)) >> 20];
 }
 
 // Round half away with the code table read sign-free.  The table's negative half lies 4096 bytes (a multiple of the
@@ -358,20 +337,14 @@ template <int MODE, int SRC>
 __device__ __forceinline__ uint32_t encode_one(float x, uint32_t raw, float scale, const uint8_t* s_ta,
                                                const uint32_t* s_thr, uint32_t word)
 {
-    constexpr bool kPair = (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && SRC == HIF8_F32;
-    const float y = kPair ? x * -scale : x * scale;
-    uint32_t t = __float_as_uint(y);
+    if ((MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && SRC == HIF8_F32) {
+        const uint32_t c = code_sum32<MODE>(x, raw, scale, s_ta, reinterpret_cast<const uint16_t*>(s_thr));
+        return c | ((c + 0x7Fu) & (raw >> 24) & 0x80u);  // (no sign on the single zero; NaN is 0x80 whatever its sign)
+    }
+    const float y = x * scale;
+    const uint32_t t = __float_as_uint(y);
     if (MODE == HIF8_RND_TA) return s_ta[t >> 19];
 
-    if ((MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && SRC == HIF8_F32) {
-        // s_ta holds the neighbour-pair words here (see pair_entry).  The scale was negated above: every sign is then
-        // inverted except that of the canonical NaN the multiply produces, so "bit 7 of the code AND NOT the sign" gives
-        // the sign of every finite / infinite result, a set bit for NaN and nothing for the single zero.
-        uint32_t ent;
-        const bool up = pair32_lookup<MODE>(y, raw, reinterpret_cast<const uint32_t*>(s_ta), ent);
-        const uint32_t c = __byte_perm(ent, 0u, up ? 0x4442u : 0x4441u);
-        return c & (~(t >> 24) | 0x7Fu);
-    }
     if (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) {  // 16-bit sources; s_ta is the truncating table here
         // two entries per exponent, chosen by the source LSB, with sh in bits 0-4 (a widened 16-bit pattern has zeros
         // there, so they cannot carry)
@@ -402,8 +375,8 @@ __device__ __forceinline__ uint32_t encode_one(float x, uint32_t raw, float scal
         const uint32_t f24 = __float2uint_rz(fabsf(y) * 70368744177664.f);
         return f24 >= max(word >> 8, 1u) ? (sign7 | 0x01u) : 0u;
     }
-    t = sub ? (tz | (t & 0x80000000u)) : t;
-    const uint32_t sh = s_thr[(t >> 23) & 0xFFu];  // discarded mantissa bits (23 - width); 0: nothing to round
+    const uint32_t ts = sub ? (tz | (t & 0x80000000u)) : t;
+    const uint32_t sh = s_thr[(ts >> 23) & 0xFFu];  // discarded mantissa bits (23 - width); 0: nothing to round
     const uint32_t s = sh ? sh : 23u;
     // threshold T of Section 3.2, compared as max(T,1) so that a zero fraction never rounds up
     const uint32_t T = max(word >> (32 - kSrBits), 1u);
@@ -413,7 +386,7 @@ __device__ __forceinline__ uint32_t encode_one(float x, uint32_t raw, float scal
         inc = (1u << s) - ((T + (1u << k) - 1u) >> k);
     } else inc = (0x10000u - T) << (s - 16);
     if (sh == 0) inc = 0;
-    const uint32_t tr = (t + inc) & (0xFFFFFFFFu << sh);
+    const uint32_t tr = (ts + inc) & (0xFFFFFFFFu << sh);
     uint32_t code = s_ta[tr >> 19];
     if (sub) code = ((code & 0x7Fu) == 0x02u) ? (sign7 | 0x01u) : 0u;  // 2^-21 -> 2^-22, 2^-22 -> the single zero
     return code;
@@ -429,25 +402,37 @@ __device__ __forceinline__ uint32_t encode_one(float x, uint32_t raw, float scal
 //   LSB term: the source's LSB as the BF16 pattern 0x0001 (2^-133) times 2^64, times the high half
 //   Below 2^-22 (result 0 or 2^-22, F = |y| / 2^-22): the binades of 2^-23 and 2^-24 add 3 * 2^-24 - LSB * 2 * 2^-24 and
 //   reach 2^-22 exactly when floor(4 F) >= T2; smaller values add nothing.  Anything that ends below 2^-22 reads zero.
-//   code8[(e, top three mantissa bits)] is the truncated magnitude with bit 7 = "takes the sign" (see pair_entry).
+//   code8[(e, top three mantissa bits)] is the truncated magnitude with bit 7 = "takes the sign".
 // ------------------------------------------------------------------------------------------------
+// Fills the 2 KiB table of truncated magnitudes.  SIGN: bit 7 of a code says "takes the sign" (clear for the single zero).
+template <bool SIGN, int NT>
+__device__ __forceinline__ void setup_magnitudes(uint8_t* code8, uint32_t flags)
+{
+    for (int i = threadIdx.x; i < 512; i += NT) {
+        const int e = i >> 1;
+        uint32_t w = 0u;
+        if (e >= 105 && e <= 142) w = g_magnitude_table.v[i];
+        else if (e > 142) w = e < 255 ? 0x6F6F6F6Fu : ((i & 1) ? 0x80808080u : 0x8080806Fu);
+        if (flags) {  // Section 3 options: patch the Inf / NaN bytes
+            uint32_t o = 0;
+#pragma unroll
+            for (int b = 0; b < 4; b++) {
+                uint32_t c = (w >> (8 * b)) & 0xFFu;
+                if ((flags & HIF8_FLAG_SATURATE) && c == 0x6Fu) c = 0x6Eu;
+                if ((flags & HIF8_FLAG_NAN_TO_ZERO) && c == 0x80u) c = 0u;
+                o |= c << (8 * b);
+            }
+            w = o;
+        }
+        if (SIGN) w |= (w + 0x7F7F7F7Fu) & 0x80808080u;
+        reinterpret_cast<uint32_t*>(code8)[i] = w;
+    }
+}
+
 template <int MODE, int NT = kThreads>
 __device__ __forceinline__ void setup_sum16(uint8_t* code8, uint32_t* inck, unsigned flags)
 {
-    for (int i = threadIdx.x; i < 512; i += NT) {  // four codes per word
-        uint32_t word = 0;
-#pragma unroll
-        for (int b = 0; b < 4; b++) {
-            const int idx = 4 * i + b, e = idx >> 3;
-            uint32_t c = 0;
-            if (e >= 105 && e <= 142) c = (g_pair_table.v[idx] >> 8) & 0xFFu;
-            else if (e > 142) c = (e == 255 && (idx & 7)) ? 0x80u : 0xEFu;
-            if ((flags & HIF8_FLAG_SATURATE) && (c & 0x7Fu) == 0x6Fu) c &= 0xFEu;
-            if ((flags & HIF8_FLAG_NAN_TO_ZERO) && c == 0x80u) c = 0u;
-            word |= c << (8 * b);
-        }
-        reinterpret_cast<uint32_t*>(code8)[i] = word;
-    }
+    setup_magnitudes<true, NT>(code8, flags);
     if (NT == kThreads || threadIdx.x < kThreads) {
         const int e = threadIdx.x, E = e - 127;  // kThreads == 256 biased exponents
         uint32_t v = 0u;
@@ -499,34 +484,21 @@ struct __align__(16) SmemTables {
 template <bool NEED_TA, bool NEED_SH, bool NEED_DEC, int MODE = HIF8_RND_TA, int SRC = HIF8_F32, int NT = kThreads>
 __device__ __forceinline__ void setup_tables(SmemTables& s, unsigned flags)
 {
-    constexpr bool kPair = (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && SRC == HIF8_F32;  // neighbour-pair words instead of code bytes
-    if (NEED_TA && kPair) {
-        // 2048 words indexed by (exponent, top three mantissa bits).  The magnitudes that reach the lookup lie in
-        // 2^-23 .. Inf / NaN; 2^-23 .. 2^15 come from the compile-time table, everything above is Inf.
-        uint32_t* d = reinterpret_cast<uint32_t*>(s.ta);
-        for (int i = threadIdx.x; i < 2048; i += NT) {
-            const int e = i >> 3, E = e - 127;
-            uint32_t v = 0u;
-            if (e >= 104 && e <= 142) v = g_pair_table.v[i];
-            else if (e > 142) v = (e == 255 && (i & 7)) ? 0x00808009u : 0x00EFEF09u;
-            if (flags) {  // Section 3 options: patch the Inf / NaN bytes
-                uint32_t lo = (v >> 8) & 0xFFu, hi = (v >> 16) & 0xFFu;
-                if (flags & HIF8_FLAG_SATURATE) {
-                    if ((lo & 0x7Fu) == 0x6Fu) lo &= 0xFEu;
-                    if ((hi & 0x7Fu) == 0x6Fu) hi &= 0xFEu;
-                }
-                if (flags & HIF8_FLAG_NAN_TO_ZERO) {
-                    if (lo == 0x80u) lo = 0u;
-                    if (hi == 0x80u) hi = 0u;
-                }
-                v = (v & 0xFF0000FFu) | (lo << 8) | (hi << 16);
+    constexpr bool kSum32 = (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && SRC == HIF8_F32;  // see code_sum32
+    if (NEED_TA && kSum32) {
+        setup_magnitudes<false, NT>(s.ta, flags);
+        if (NT == kThreads || threadIdx.x < kThreads) {
+            const int e = threadIdx.x, E = e - 127;  // kThreads == 256 biased exponents
+            uint32_t v = 105u;                       // 2^-22
+            if (E >= 16) v = 0u;                     // Inf or NaN as it is
+            else if (E >= -22) {
+                const uint32_t u = (uint32_t)(e - mant_width(E));
+                v = MODE == HIF8_RND_HR && E > -4 && E < 4 ? (u - 1u) << 8 : u;
             }
-            // Eq. 3: round half away for |E| < 4 under hybrid rounding (bits 31-30 = 10), stochastic elsewhere (01)
-            v |= (MODE == HIF8_RND_HR && E > -4 && E < 4) ? 0x80000000u : 0x40000000u;
-            d[i] = v;
+            reinterpret_cast<uint16_t*>(s.thr)[e] = (uint16_t)v;
         }
     }
-    if (NEED_TA && !kPair) {
+    if (NEED_TA && !kSum32) {
         // Only binades 2^-24 .. 2^16 differ from their neighbours: those 41 x 16 entries per sign come from the
         // compile-time table (1.3 KiB of global reads per block); everything below is zero, everything above is
         // Inf (or NaN in the all-ones exponent), written straight into shared memory.
@@ -560,7 +532,7 @@ __device__ __forceinline__ void setup_tables(SmemTables& s, unsigned flags)
             d[i] = v;
         }
     }
-    if (NEED_SH && !kPair && (NT == kThreads || threadIdx.x < kThreads)) {
+    if (NEED_SH && !kSum32 && (NT == kThreads || threadIdx.x < kThreads)) {
         const int e = threadIdx.x, E = e - 127;  // kThreads == 256 biased exponents
         constexpr bool kThreshold = MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR;
         // TE / SR: thr[e] = e0.  Threshold modes (16-bit sources): thr[2e] = e0 (source LSB 0), thr[2e + 1] = e1 (LSB 1).

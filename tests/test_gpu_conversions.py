@@ -112,6 +112,20 @@ def test_encode_f32_subnormal_sources_with_large_scale():
             assert_same(gpu_encode(bits, H.F32, scale_exp=se, rnd=mode, seed=3), want, bits)
 
 
+@pytest.mark.parametrize("mode", [H.RND_HR, H.RND_SSR])
+@pytest.mark.parametrize("scale_exp", [-126, -40, 0, 3, 60, 126])
+def test_encode_f32_thresholds_at_the_edges_of_every_binade(mode, scale_exp):
+    # the first and last values of every binade of the scaled magnitude (carries into the next one, the binades below the format's
+    # range, overflow), with the source bits that are the threshold at 0, 1, 2, the middle and their largest value
+    e = np.arange(1, 255, dtype=np.uint32)[:, None, None]
+    top = np.array([0, 1, 2, 255, 256, 257, 509, 510, 511], dtype=np.uint32)[None, :, None] << 14
+    low = np.array([0, 1, 2, 3, 8191, 8192, 8193, 16381, 16382, 16383], dtype=np.uint32)[None, None, :]
+    bits = ((e << 23) | top | low).reshape(-1)
+    bits = np.concatenate([bits, bits | np.uint32(0x80000000)]).astype(np.uint32)
+    want = O.encode(bits, O.F32, scale_exp, mode, 0, quick=True)
+    assert_same(gpu_encode(bits, H.F32, scale_exp=scale_exp, rnd=mode), want, bits)
+
+
 @pytest.mark.parametrize("mode", [H.RND_TA, H.RND_SR, H.RND_HR, H.RND_SSR])
 def test_encode_ragged_sizes_and_misaligned_pointers(mode):
     base = W.loguniform_f32(5000, seed=5, lo_exp=-26, hi_exp=17).view(np.uint32)
