@@ -29,6 +29,7 @@
 
 #include "hif8.h"
 #include "hif8_device.cuh"
+#include "hif8_host_cache.h"
 #include "hif8_internal.cuh"
 
 namespace hif8 {
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const ConvParams p, u
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (p.d_scale_exp_out) *p.d_scale_exp_out = se;
         if (p.d_scale_out) *p.d_scale_out = scale;
-        if (!AMAX && p.d_amax_out && p.d_amax_bits) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
+        if (!AMAX && p.d_amax_out && p.d_amax_bits && !p.amax_slots) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
     }
     if (AMAX) {
         block_amax_commit(amax, p.amax_accum);
@@ -247,17 +248,16 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const ConvParams p, u
 }
 
 // ------------------------------------------------------------------------------------------------
-// Just-in-time scaling of a small tensor in one launch: a cluster of up to eight blocks holds the source in shared memory,
+// Just-in-time scaling of a small tensor in one launch: a cluster of up to sixteen blocks holds the source in shared memory,
 // reduces its amax (each block tells the others its own through distributed shared memory, between two cluster barriers, the
 // first of which completes under the loads and the table set-up), and converts from there.  No accumulator in the workspace,
-// so nothing to clear.  Latency and launches bound it: the three launches of the general path (clear, amax, convert) take 3.3 us
-// on the device and 8 us from the host, this 2.3 us and 4 us (512 BF16 elements, round half away); 3.9 against 3.1 us on the device
-// at 131072.  To bytes it takes what eight blocks hold without an opt-in to more than 48 KiB of shared memory each: 256 KiB of
-// source, where it is still the faster one.  Dequantized results carry more arithmetic, and at that size eight blocks are the
-// slower form (131072 BF16 elements under hybrid rounding: 4.5 us by three launches, 5.0 us by one): half of it.
+// so nothing to clear.  Latency and launches bound it: from the host one launch takes 3.5 us, two (amax, convert) 5.3 and three 8.  It ends
+// where sixteen SMs take longer than the launches over all of them, which depends on the arithmetic an element carries (one_launch_limit).
+// All copies of a block are asynchronous and in flight together, up to 128 KiB.
 // ------------------------------------------------------------------------------------------------
-constexpr int kOneThreads = 512, kOneVecs = 4, kOneBlocks = 8;  // 32 KiB of source per block
-constexpr unsigned long long kOneMaxVecs = (unsigned long long)kOneThreads * kOneVecs * kOneBlocks, kOneMaxVecsFq = kOneMaxVecs / 2;
+constexpr int kOneThreads = 512, kOneBlocks = 16, kOneBlocksPortable = 8;
+constexpr unsigned kOneSmem = 128 * 1024, kOneSmemDefault = 32 * 1024;  // source bytes per block: with the opt-in, and without
+static_assert(sizeof(SmemTables) + kOneSmemDefault + 256 <= 48 * 1024, "no opt-in to more shared memory for the smaller form");
 
 template <int SRC, int MODE, bool FQ>
 __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParams p, unsigned n_vec)
@@ -272,9 +272,10 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     const unsigned first = blockIdx.x * kOneThreads + threadIdx.x, step = gridDim.x * kOneThreads;  // vectors first, first + step, ..
     pdl_wait_prior_grid();
     const uint4* src = reinterpret_cast<const uint4*>(p.src);
-    uint4 v[kOneVecs];
-#pragma unroll
-    for (int j = 0; j < kOneVecs; j++) v[j] = first + j * step < n_vec ? __ldcs(src + first + j * step) : make_uint4(0, 0, 0, 0);
+    const uint32_t s_mine = (uint32_t)__cvta_generic_to_shared(s_src + threadIdx.x);
+#pragma unroll 4
+    for (unsigned u = first, at = s_mine; u < n_vec; u += step, at += kOneThreads * 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at), "l"(src + u) : "memory");
     // what whole vectors do not cover: at most PV - 1 elements, one per thread of the first block
     const unsigned long long i_tail = (unsigned long long)n_vec * PV + threadIdx.x;
     const bool tail = blockIdx.x == 0 && i_tail < p.n;
@@ -285,11 +286,9 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     if (kPair16) setup_sum16<MODE, kOneThreads>(sm.ta, sm.thr, p.flags);
     else setup_tables<true, MODE != HIF8_RND_TA, FQ, MODE, SRC, kOneThreads>(sm, p.flags);
     uint32_t acc = 0u;
-#pragma unroll
-    for (int j = 0; j < kOneVecs; j++) {
-        if (first + j * step < n_vec) s_src[j * kOneThreads + threadIdx.x] = v[j];
-        acc = amax_vector<SRC>(acc, v[j]);
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");  // (a thread reads what it copied itself)
+#pragma unroll 4
+    for (unsigned u = first, j = threadIdx.x; u < n_vec; u += step, j += kOneThreads) acc = amax_vector<SRC>(acc, s_src[j]);
     const float amax = amax_step(amax_value<SRC>(acc), x_tail);
     uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));  // non-negative floats order as integers
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = m;
@@ -573,7 +572,7 @@ __global__ void __launch_bounds__(kThreads) fq_ta_kernel(const ConvParams p, uns
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (p.d_scale_exp_out) *p.d_scale_exp_out = se;
         if (p.d_scale_out) *p.d_scale_out = pow2f(se);
-        if (p.d_amax_out && p.d_amax_bits) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
+        if (p.d_amax_out && p.d_amax_bits && !p.amax_slots) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
     }
 }
 
@@ -596,6 +595,64 @@ constexpr int kUnrollAmax = 8;
 // and with it: fake-quant of 16.8 M elements 29.3 / 29.5, scale and encode of 18 M 31.1 / 31.4; of 20 M 35.1 / 34.7 and 35.2 / 35.6, of
 // 22.5 M 39.4 / 39.0 and 38.9 / 38.7).
 constexpr unsigned long long kKeepVecs = (64ull << 20) / 16, kStreamVecsF32 = (72ull << 20) / 16;
+// The same pass for tensors of the middle sizes, in one launch where the one below takes two (it adds to an accumulator that has to be cleared
+// first): blocks in clusters of eight, whose amax goes to the cluster's own word of the workspace, all of them written.  The
+// pass that follows takes the largest of the words, which costs it the same one trip to L2.
+// Launches bound these sizes: a call on 512 K FP32 elements 8.8 us from the host, so 5.8; 1 M 8.7 / 6.1, 4 M 9.7 / 8.9; on the device alone 5.2 / 4.9, 6.5 / 5.7,
+// 8.7 / 8.3.  Up to 24 MiB of source: its one wave of blocks takes equal shares, and for larger tensors blocks that are handed out as SMs become free
+// are faster (FP32, 24 MiB 10.8 / 10.5, 28 MiB 12.1 / 13.1; BF16, 16 MiB 9.6 / 9.3, 24 MiB 12.3 / 12.1).  Standard stochastic rounding stays with the launches
+// below: with the next call's blocks resident early, its few blocks in the second pass share SMs (512 K FP32 elements 7.8 / 9.9).
+constexpr int kSlotThreads = 512, kSlotCluster = 8;
+constexpr unsigned kSlotVecs = kSlotThreads * kSlotCluster * kUnrollAmax;  // of a cluster
+constexpr unsigned kMaxSlots = 64;                                        // words of the workspace
+constexpr unsigned kSlotMaxVecs = (24u << 20) / 16;
+static_assert(kSlotMaxVecs <= kMaxSlots * kSlotVecs, "a word per cluster");
+template <int SRC>
+__global__ void __launch_bounds__(kSlotThreads) amax_slots_kernel(const void* __restrict__ srcv, unsigned long long n, unsigned n_vec, uint32_t* slots)
+{
+    constexpr int PV = SrcTraits<SRC>::kPerVec;
+    __shared__ uint32_t s_part[kSlotThreads / 32], s_block[kSlotCluster];
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this block has started (waited for before the first remote store)
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
+    const uint4* src = reinterpret_cast<const uint4*>(srcv);
+    uint32_t acc = 0u;
+    uint4 v[kUnrollAmax];
+#pragma unroll
+    for (int j = 0; j < kUnrollAmax; j++) {
+        const unsigned u = (j * gridDim.x + blockIdx.x) * kSlotThreads + threadIdx.x;
+        v[j] = u < n_vec ? __ldg(src + u) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int j = 0; j < kUnrollAmax; j++) acc = amax_vector<SRC>(acc, v[j]);
+    float amax = amax_value<SRC>(acc);
+    const unsigned long long i = (unsigned long long)n_vec * PV + threadIdx.x;  // at most PV - 1 elements are left
+    if (blockIdx.x == 0 && i < n) {
+        float x; uint32_t raw;
+        load_scalar<SRC>(srcv, i, x, raw);
+        amax = amax_step(amax, x);
+    }
+    uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));  // non-negative floats order as integers
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = m;
+    __syncthreads();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    const unsigned rank = blockIdx.x % kSlotCluster;
+    if (threadIdx.x < 32) {
+        m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kSlotThreads / 32 ? s_part[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) {
+            uint32_t to;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(s_block + rank)), "r"(0));
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to), "r"(m) : "memory");
+        }
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank == 0 && threadIdx.x < 32) {
+        m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kSlotCluster ? s_block[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) slots[blockIdx.x / kSlotCluster] = m;
+    }
+}
+
 template <int SRC, bool STREAM>
 __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__ srcv, unsigned long long n,
                                                         unsigned long long n_vec, uint32_t* accum, float* d_amax_out)
@@ -749,7 +806,7 @@ __global__ void __launch_bounds__(kDecodeThreads) decode_stream_kernel(const uin
 int g_sm_count[64];
 int g_cc[64];
 
-int device_info(int* sms)
+int device_info(int* sms, int* device = nullptr)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return HIF8_ERR_CUDA;
@@ -763,6 +820,7 @@ int device_info(int* sms)
     }
     if (g_cc[dev] != 100) return HIF8_ERR_CUDA;
     *sms = g_sm_count[dev];
+    if (device) *device = dev;
     return HIF8_OK;
 }
 
@@ -828,50 +886,82 @@ int dispatch_convert(int dtype, int rnd, const ConvParams& p, bool vec_ok, int s
     }
 }
 
-template <int SRC, int MODE, bool FQ>
-int launch_one(const ConvParams& p, cudaStream_t st)
+// Elements up to which one_launch_kernel is the faster form, by what an element costs.  On the device alone, us, one launch / amax_slots_kernel
+// and a conversion / the three launches: round half away to bytes, FP32 2^18.5 elements 4.2 / 4.1 / 4.2, 2^19 4.9 / 4.2 / 4.3, BF16 2^19 4.0 / 4.1 / 4.4;
+// hybrid rounding to bytes, FP32 2^18 4.4 / 4.3 / 4.8, 2^18.5 5.7 / 4.4 / 4.5, BF16 2^18 3.6 / 4.2 / 4.4; to dequantized values, round half away,
+// FP32 2^17.5 4.2 / 4.2 / 4.5, 2^18 4.8 / 4.3 / 4.5, hybrid, BF16 2^17.5 4.2 / 4.5 / 4.8, 2^18 4.8 / 4.3 / 4.5; standard stochastic rounding, FP32 2^17
+// 5.0 / 5.3 / 5.6, 2^17.5 6.6 / 5.6 / 5.7.
+constexpr unsigned one_launch_limit(int src, int mode, bool fq)
 {
-    static_assert(sizeof(SmemTables) + kOneThreads * kOneVecs * 16 + 256 <= 48 * 1024, "no opt-in to more shared memory");
+    if (mode == HIF8_RND_SR) return 1u << 17;
+    if (fq || mode == HIF8_RND_TE) return 3u << 16;
+    if (mode == HIF8_RND_TA) return src == HIF8_F32 ? 11u << 15 : 1u << 19;
+    return 1u << 18;
+}
+static_assert(one_launch_limit(HIF8_F32, HIF8_RND_TA, false) / 4 <= kOneBlocks * kOneSmem / 16 && one_launch_limit(HIF8_BF16, HIF8_RND_TA, false) / 8 <= kOneBlocks * kOneSmem / 16,
+              "sixteen blocks hold it");
+constexpr int kNotTaken = -1;
+
+template <int SRC, int MODE, bool FQ>
+int launch_one(const ConvParams& p, int dev, cudaStream_t st)
+{
+    if (p.n > one_launch_limit(SRC, MODE, FQ)) return kNotTaken;
     const unsigned n_vec = (unsigned)(p.n / SrcTraits<SRC>::kPerVec);
-    // two vectors per thread while there are blocks to add
-    unsigned blocks = 1;
-    while (blocks < (unsigned)kOneBlocks && blocks * kOneThreads * 2 < n_vec) blocks *= 2;
+    struct Setup { unsigned blocks, smem; };
+    static PerDevice<Setup> setup;
+    auto* kernel = one_launch_kernel<SRC, MODE, FQ>;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kOneThreads);
-    cfg.dynamicSmemBytes = (size_t)((n_vec + blocks * kOneThreads - 1) / (blocks * kOneThreads)) * kOneThreads * 16;
-    cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = blocks; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const cudaError_t lrc = cudaLaunchKernelEx(&cfg, one_launch_kernel<SRC, MODE, FQ>, p, n_vec);
+    // sixteen blocks of up to 128 KiB where the device can hold such a cluster, else eight of 32 KiB, which every device can
+    const Setup* s = setup.get(dev, [&](int, Setup* out) {
+        *out = Setup{kOneBlocksPortable, kOneSmemDefault};
+        int clusters = 0;
+        cfg.gridDim = dim3(kOneBlocks); cfg.dynamicSmemBytes = kOneSmem;
+        attr[1].val.clusterDim.x = kOneBlocks;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOneSmem) == cudaSuccess &&
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0) *out = Setup{kOneBlocks, kOneSmem};
+        else cudaGetLastError();
+    });
+    if (!s || n_vec > s->blocks * s->smem / 16) return kNotTaken;
+    // two vectors per thread while there are blocks to add
+    unsigned blocks = 1;
+    while (blocks < s->blocks && blocks * kOneThreads * 2 < n_vec) blocks *= 2;
+    cfg.gridDim = dim3(blocks);
+    attr[1].val.clusterDim.x = blocks;
+    cfg.dynamicSmemBytes = (size_t)((n_vec + blocks * kOneThreads - 1) / (blocks * kOneThreads)) * kOneThreads * 16;
+    cfg.stream = st;
+    const cudaError_t lrc = cudaLaunchKernelEx(&cfg, kernel, p, n_vec);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return lrc == cudaSuccess && cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
 }
 
 template <int SRC, bool FQ>
-int dispatch_one_mode(int rnd, const ConvParams& p, cudaStream_t st)
+int dispatch_one_mode(int rnd, const ConvParams& p, int dev, cudaStream_t st)
 {
     switch (rnd) {
-        case HIF8_RND_TA: return launch_one<SRC, HIF8_RND_TA, FQ>(p, st);
-        case HIF8_RND_HR: return launch_one<SRC, HIF8_RND_HR, FQ>(p, st);
-        case HIF8_RND_SSR: return launch_one<SRC, HIF8_RND_SSR, FQ>(p, st);
-        case HIF8_RND_TE: return launch_one<SRC, HIF8_RND_TE, FQ>(p, st);
-        default: return launch_one<SRC, HIF8_RND_SR, FQ>(p, st);
+        case HIF8_RND_TA: return launch_one<SRC, HIF8_RND_TA, FQ>(p, dev, st);
+        case HIF8_RND_HR: return launch_one<SRC, HIF8_RND_HR, FQ>(p, dev, st);
+        case HIF8_RND_SSR: return launch_one<SRC, HIF8_RND_SSR, FQ>(p, dev, st);
+        case HIF8_RND_TE: return launch_one<SRC, HIF8_RND_TE, FQ>(p, dev, st);
+        default: return launch_one<SRC, HIF8_RND_SR, FQ>(p, dev, st);
     }
 }
 
 template <bool FQ>
-int dispatch_one(int dtype, int rnd, const ConvParams& p, cudaStream_t st)
+int dispatch_one(int dtype, int rnd, const ConvParams& p, int dev, cudaStream_t st)
 {
     switch (dtype) {
-        case HIF8_F32: return dispatch_one_mode<HIF8_F32, FQ>(rnd, p, st);
-        case HIF8_BF16: return dispatch_one_mode<HIF8_BF16, FQ>(rnd, p, st);
-        default: return dispatch_one_mode<HIF8_F16, FQ>(rnd, p, st);
+        case HIF8_F32: return dispatch_one_mode<HIF8_F32, FQ>(rnd, p, dev, st);
+        case HIF8_BF16: return dispatch_one_mode<HIF8_BF16, FQ>(rnd, p, dev, st);
+        default: return dispatch_one_mode<HIF8_F16, FQ>(rnd, p, dev, st);
     }
 }
 
@@ -905,6 +995,29 @@ int launch_amax(const void* src, int dtype, unsigned long long n, uint32_t* accu
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
+}
+
+// amax of a tensor of whole vectors (and less than one more) to `slots`; the number of words written, 0 on failure
+unsigned launch_amax_slots(const void* src, int dtype, unsigned long long n, unsigned n_vec, uint32_t* slots, cudaStream_t st)
+{
+    // eight vectors per thread, four while that leaves SMs without a block
+    unsigned clusters = n_vec ? (n_vec + kSlotVecs - 1) / kSlotVecs : 1;
+    if (clusters < 19) clusters *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(clusters * kSlotCluster);
+    cfg.blockDim = dim3(kSlotThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kSlotCluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    auto* kernel = dtype == HIF8_F32 ? amax_slots_kernel<HIF8_F32> : dtype == HIF8_BF16 ? amax_slots_kernel<HIF8_BF16> : amax_slots_kernel<HIF8_F16>;
+    if (cudaLaunchKernelEx(&cfg, kernel, src, n, n_vec, slots) != cudaSuccess) return 0;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return clusters;
 }
 
 int check_common(int dtype, int rnd, unsigned flags)
@@ -1013,7 +1126,7 @@ static int scaled_convert(bool fq, const void* src, void* dst, int dtype, size_t
                           float* d_amax_out, int* d_scale_exp_out, float* d_scale_out, void* workspace,
                           size_t workspace_bytes, bool want_amax, cudaStream_t st, void* scale_state = nullptr)
 {
-    int sms; int rc = device_info(&sms);
+    int sms, dev; int rc = device_info(&sms, &dev);
     if (rc) return rc;
     uint32_t* ws = reinterpret_cast<uint32_t*>(workspace);
     ConvParams p{};
@@ -1024,11 +1137,18 @@ static int scaled_convert(bool fq, const void* src, void* dst, int dtype, size_t
     bool vec_ok = aligned16(src) && (reinterpret_cast<uintptr_t>(dst) % out_align) == 0;
     if (jit || want_amax) {
         if (!ws || workspace_bytes < kConvWorkspaceBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return HIF8_ERR_WORKSPACE;
-        // a tensor that one cluster holds: one launch (what is not 16-byte aligned: the general path)
-        if (jit && vec_ok && n / (dtype == HIF8_F32 ? 4 : 8) <= (fq ? kOneMaxVecsFq : kOneMaxVecs))
-            return fq ? dispatch_one<true>(dtype, rnd, p, st) : dispatch_one<false>(dtype, rnd, p, st);
+        // a small tensor: one launch; one of the middle sizes: two (what is not 16-byte aligned: the general path)
+        if (jit && vec_ok) {
+            rc = fq ? dispatch_one<true>(dtype, rnd, p, dev, st) : dispatch_one<false>(dtype, rnd, p, dev, st);
+            if (rc != kNotTaken) return rc;
+        }
+        const unsigned long long n_vec = n / (dtype == HIF8_F32 ? 4 : 8);
+        if (jit && rnd != HIF8_RND_SR && aligned16(src) && n_vec <= kSlotMaxVecs) {
+            p.amax_slots = launch_amax_slots(src, dtype, n, (unsigned)n_vec, ws, st);
+            if (!p.amax_slots) return HIF8_ERR_CUDA;
+        }
         // (a delayed-scaling state keeps its two words at zero between passes itself)
-        if (!scale_state) {
+        else if (!scale_state) {
             if (launch_pdl(clear_accum_kernel, 1u, st, ws) != cudaSuccess) return HIF8_ERR_CUDA;
             g_launches.fetch_add(1, std::memory_order_relaxed);
         }
@@ -1037,8 +1157,10 @@ static int scaled_convert(bool fq, const void* src, void* dst, int dtype, size_t
     const bool inplace_fq = fq && !want_amax && ((rnd == HIF8_RND_TA && (dtype == HIF8_F32 || dtype == HIF8_BF16)) ||
                                                 ((rnd == HIF8_RND_HR || rnd == HIF8_RND_SSR || rnd == HIF8_RND_TE || rnd == HIF8_RND_SR) && dtype == HIF8_BF16));
     if (jit) {
-        rc = launch_amax(src, dtype, n, ws, nullptr, sms, st);
-        if (rc) return rc;
+        if (!p.amax_slots) {
+            rc = launch_amax(src, dtype, n, ws, nullptr, sms, st);
+            if (rc) return rc;
+        }
         p.d_amax_bits = ws;
         p.reverse = 1;  // the amax pass has just read the tensor front to back
         if (inplace_fq) return launch_fq_ta(dtype, rnd, p, vec_ok, sms, st);

@@ -175,6 +175,7 @@ struct ConvParams {
     int scale_exp;                // used when neither pointer below is set
     const int* d_scale_exp;       // delayed scaling: exponent read from the device
     const uint32_t* d_amax_bits;  // just-in-time scaling: exponent derived from this amax
+    unsigned amax_slots;          // nonzero: amax is the largest of that many words there, up to 64
     int target_exp;
     unsigned flags;
     unsigned long long seed;
@@ -583,8 +584,16 @@ __device__ __forceinline__ void scale_state_push(ScaleState* st, uint32_t amax_b
     st->scale_exp = scale_exp_from_amax(m, target_exp);
 }
 
+// (all threads of a warp together)
 __device__ __forceinline__ int resolve_scale_exp(const ConvParams& p)
 {
+    if (p.amax_slots) {
+        const unsigned lane = threadIdx.x & 31u;
+        const uint32_t a = lane < p.amax_slots ? p.d_amax_bits[lane] : 0u, b = lane + 32u < p.amax_slots ? p.d_amax_bits[lane + 32u] : 0u;
+        const uint32_t ab = __reduce_max_sync(0xFFFFFFFFu, max(a, b));
+        if (blockIdx.x == 0 && threadIdx.x == 0 && p.d_amax_out) *p.d_amax_out = __uint_as_float(ab);
+        return scale_exp_from_amax(ab, p.target_exp);
+    }
     if (p.d_amax_bits) return scale_exp_from_amax(*p.d_amax_bits, p.target_exp);
     if (p.d_scale_exp) return clamp_exp(*p.d_scale_exp);
     return p.scale_exp;

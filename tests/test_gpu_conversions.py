@@ -255,6 +255,41 @@ def test_scaled_conversions_of_small_tensors(dtype, mode):
         assert_same(buf.cpu().numpy().view(NP_OF[dtype]), want_fq, src)
 
 
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
+@pytest.mark.parametrize("fq,mode", [(0, H.RND_TA), (0, H.RND_HR), (0, H.RND_SR), (1, H.RND_TA), (1, H.RND_HR)])
+def test_scaled_conversions_at_the_limits_of_the_launch_forms(dtype, fq, mode):
+    """The last size of the one-launch form and the first above it, one cluster of the two-launch form and a little more, its last
+    size with fewer and more clusters, its limit and the first size above; the largest element first, last, in the middle and in the tail."""
+    pv = 4 if dtype == H.F32 else 8
+    one = (1 << 17) if mode == H.RND_SR else (3 << 16) if fq else (1 << 18) if mode != H.RND_TA else (11 << 15) if dtype == H.F32 else (1 << 19)
+    two = (24 << 20) // (4 if dtype == H.F32 else 2)
+    cluster = 32768 * pv
+    sizes = [one, one + 1, 9 * cluster + pv - 1, 18 * cluster, 18 * cluster + 1, two + pv - 1, two + pv]
+    ws, wsb = workspace()
+    outs = torch.zeros(4, dtype=torch.int32, device="cuda")
+    np_t = {H.F32: np.float32, H.BF16: np.uint16, H.F16: np.float16}[dtype]
+    for i, n in enumerate(sizes):
+        base = W.normal_bf16(n, seed=i) if dtype == H.BF16 else W.normal_f32(n, seed=i).astype(np_t)
+        src = base.view(np.uint32 if dtype == H.F32 else np.uint16).copy()
+        at = [0, n - 1, n // 2, (n // pv) * pv - 1][i % 4]
+        src[at] = {H.F32: 0x42F00000, H.BF16: 0x42F0, H.F16: 0x5780}[dtype]  # 120
+        amax, se = O.amax_scale(src, dtype, 14)
+        assert amax == 120.0
+        d_src = to_dev(src)
+        if fq:
+            out = torch.empty(n, dtype=torch.int32 if dtype == H.F32 else torch.int16, device="cuda")
+            assert H.hif8_fake_quant(d_src, out, dtype, n, 1, 14, mode, 0, 9, outs[0:1], outs[1:2], ws, wsb) == 0
+            torch.cuda.synchronize()
+            assert_same(out.cpu().numpy().view(src.dtype), O.fake_quant(src, dtype, se, mode, 0, seed=9, quick=True), src)
+        else:
+            _, dptr, rb = dev_empty(n, np.uint8)
+            assert H.hif8_amax_scale_encode(d_src, dtype, dptr, n, 14, mode, 0, 9, None, outs[0:1], outs[1:2], outs[2:3], ws, wsb) == 0
+            torch.cuda.synchronize()
+            assert_same(rb(), O.encode(src, dtype, se, mode, 0, seed=9, quick=True), src)
+        o = outs.cpu().numpy()
+        assert o[0:1].view(np.float32)[0] == 120.0 and o[1] == se
+
+
 def test_amax_alone():
     ws, wsb = workspace()
     out = torch.zeros(1, dtype=torch.float32, device="cuda")
