@@ -112,6 +112,23 @@ __device__ __forceinline__ uint32_t group_max(uint32_t v, uint32_t* s_part, int 
     for (int w = 0; w < gs / 32; w++) v = max(v, s_part[w0 + w]);
     return v;
 }
+// The same with one barrier, of the group's threads alone (number g + 1; 0 is the block's): `s_part` is one of two sets of words, used in turn, so nobody
+// still reads it from the use before the last one, which the barrier of the last one stands behind.
+__device__ __forceinline__ uint32_t group_max_in_turn(uint32_t v, uint32_t* s_part, int lg, int g)
+{
+    v = __reduce_max_sync(0xFFFFFFFFu, v);
+    if (lg == 5) return v;
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
+    asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(1 << lg) : "memory");
+    const int w0 = g << (lg - 5);
+    v = s_part[w0];
+    if (lg == 6) return max(v, s_part[w0 + 1]);
+    const uint4 q = *reinterpret_cast<const uint4*>(s_part + w0);
+    v = max(max(q.x, q.y), max(q.z, q.w));
+    if (lg == 7) return v;
+    const uint4 r = *reinterpret_cast<const uint4*>(s_part + w0 + 4);
+    return max(v, max(max(r.x, r.y), max(r.z, r.w)));
+}
 
 // When the next launch may start.  Its blocks, which only wait, take the places that are free, and when they are few and long
 // they sit unevenly for all of their run: 512 rows of 65536 BF16 values 24.7 -> 28.8 us in a sequence of such calls, 1000 rows of
@@ -126,66 +143,60 @@ template <int SRC, int MODE, int NV, bool APART = false>
 __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanParams p, int gs, int iters)
 {
     __shared__ SmemTables sm;
-    __shared__ uint32_t s_part[kThreads / 32];
+    __shared__ __align__(16) uint32_t s_part[2][kThreads / 32];
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     if (MODE != HIF8_RND_SR) pdl_launch_dependents();
     setup_tables<true, MODE != HIF8_RND_TA, false, MODE, SRC>(sm, p.flags);
     pdl_wait_prior_grid();
-    const unsigned long long nv = (unsigned long long)p.cols / PV;  // vectors per row (cols is a multiple of PV here)
+    const unsigned nv = (unsigned)(p.cols / PV);  // vectors per row (cols is a multiple of PV here, and a row at most NV vectors per thread)
     const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
-    const int groups = kThreads / gs, g = threadIdx.x / gs, t = threadIdx.x % gs;
-    const uint4* base = reinterpret_cast<const uint4*>(p.src);
+    // Issue slots bound this kernel, at four blocks an SM (two sets of registers; five blocks with 48 registers are slower, 18.4).  Offsets within a row
+    // have 32 bits and a row's place is worked out once a set, a row of NV vectors per thread is not tested vector by vector, and a group waits for itself alone, once a
+    // set: 16 -> 13.5 instructions an element, 7168 x 4096 BF16 19.1 -> 16.7 us, 8192 x 2048 12.4 -> 10.6, FP32 28.3 -> 27.1.  (gs is a power of two.)
+    const int lg = 31 - __clz(gs), groups = kThreads >> lg, g = threadIdx.x >> lg, t = threadIdx.x & (gs - 1);
     const long long step = APART ? (long long)gridDim.x * groups : groups, first = (long long)blockIdx.x * (APART ? 1 : iters) * groups + g;
+    const uint4* src = reinterpret_cast<const uint4*>(p.src) + (unsigned long long)first * nv + t;
+    const unsigned long long src_step = (unsigned long long)step * nv;
+    const bool full = nv == (unsigned)(NV * gs);  // every thread has NV vectors of a row
+    auto load = [&](uint4 (&v)[NV], const uint4* at, bool live) {
+        if (full && live) {
+#pragma unroll
+            for (int j = 0; j < NV; j++) v[j] = __ldcs(at + j * gs);
+        } else {
+#pragma unroll
+            for (int j = 0; j < NV; j++) v[j] = live && (unsigned)(j * gs + t) < nv ? __ldcs(at + j * gs) : make_uint4(0, 0, 0, 0);
+        }
+    };
 
     // NV <= kUnroll: two register sets, the next row is in flight while this one is processed; larger rows use one set
     constexpr bool kPrefetch = NV <= kUnroll;
     uint4 cur[NV], nxt[kPrefetch ? NV : 1];
-    if (kPrefetch) {
-#pragma unroll
-        for (int j = 0; j < NV; j++) {
-            const unsigned long long u = (unsigned long long)j * gs + t;
-            nxt[j] = (first < p.rows && u < nv) ? __ldcs(base + (unsigned long long)first * nv + u) : make_uint4(0, 0, 0, 0);
-        }
-    }
-    for (int it = 0; it < iters; it++) {
-        const long long row = first + (long long)it * step, row_next = row + step;
+    if constexpr (kPrefetch) load(nxt, src, first < p.rows);
+    long long row = first;
+    for (int it = 0; it < iters; it++, row += step, src += src_step) {
         const bool live = row < p.rows;  // a group past the last row only takes part in the barriers
-        if (kPrefetch) {
+        if constexpr (kPrefetch) {
 #pragma unroll
             for (int j = 0; j < NV; j++) cur[j] = nxt[j];
-            if (it + 1 < iters) {
-#pragma unroll
-                for (int j = 0; j < NV; j++) {
-                    const unsigned long long u = (unsigned long long)j * gs + t;
-                    nxt[j] = (row_next < p.rows && u < nv) ? __ldcs(base + (unsigned long long)row_next * nv + u) : make_uint4(0, 0, 0, 0);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < NV; j++) {
-                const unsigned long long u = (unsigned long long)j * gs + t;
-                cur[j] = (live && u < nv) ? __ldcs(base + (unsigned long long)row * nv + u) : make_uint4(0, 0, 0, 0);
-            }
-        }
+            if (it + 1 < iters) load(nxt, src + src_step, row + step < p.rows);
+        } else load(cur, src, live);
         int se = 0;
         if (p.d_se_in) se = live ? clamp_exp(p.d_se_in[row]) : 0;
         else {
             uint32_t m = 0u;
 #pragma unroll
             for (int j = 0; j < NV; j++) m = amax_vector<SRC>(m, cur[j]);
-            const uint32_t b = group_max(__float_as_uint(amax_value<SRC>(m)), s_part, gs);
+            const uint32_t b = group_max_in_turn(__float_as_uint(amax_value<SRC>(m)), s_part[it & 1], lg, g);
             if (t == 0 && live) p.amax_bits[row] = b;
             se = scale_exp_from_amax(b, p.target_exp);
         }
         if (t == 0 && live && p.d_se_out) p.d_se_out[row] = se;
         const float scale = pow2f(se);
         if (live) {
+            const unsigned long long flat = (unsigned long long)row * nv + t;
 #pragma unroll
-            for (int j = 0; j < NV; j++) {
-                const unsigned long long u = (unsigned long long)j * gs + t;
-                if (u >= nv) continue;
-                encode_row_vector<SRC, MODE>(p, sm, cur[j], (unsigned long long)row * nv + u, scale, k0, k1);
-            }
+            for (int j = 0; j < NV; j++)
+                if (full || (unsigned)(j * gs + t) < nv) encode_row_vector<SRC, MODE>(p, sm, cur[j], flat + j * gs, scale, k0, k1);
         }
     }
     if (MODE == HIF8_RND_SR) pdl_launch_dependents();
@@ -430,8 +441,8 @@ int launch_encode(const ChanParams& p, const Plan& pl, cudaStream_t st)
             int iters = nv <= (long long)kUnroll * gs ? 8 : 1;
             while (iters > 1 && (sets + iters - 1) / iters < (long long)pl.sms * 8) iters >>= 1;
             // Few sets, with two register sets: as many blocks as are resident (four per SM) and their sets one grid apart, since blocks
-            // of consecutive sets then end in a round that is nearly empty (7168 x 4096 BF16, 6 sets a block: 19.55 us, apart 18.7;
-            // 8192 x 64 4.5 and 4.1).  With more than eight a block consecutive sets are faster (12288 x 4096 BF16, 10 a block: 27.7,
+            // of consecutive sets then end in a round that is nearly empty (7168 x 4096 BF16, 6 sets a block: 19.55 us, apart 18.7 (before a set's work was cut,
+            // now 16.7); 8192 x 64 4.5 and 4.1).  With more than eight a block consecutive sets are faster (12288 x 4096 BF16, 10 a block: 27.7,
             // apart 28.7; 28672 x 8192, 48 a block, under hybrid rounding with given exponents 158 and 168).  (An instantiation: a stride that is
             // an argument cost the other calls 2 to 10 %.)
             const long long resident = (long long)pl.sms * 4;

@@ -602,19 +602,19 @@ __device__ __forceinline__ int resolve_scale_exp(const ConvParams& p)
 // amax contribution of a value: |x| for finite x, ignored (NaN) otherwise; fmaxf drops NaN operands
 __device__ __forceinline__ float amax_step(float acc, float x) { return fmaxf(acc, fmaf(x, 0.0f, fabsf(x))); }
 
-// The same over whole source words.  16-bit sources stay packed, two running maxima in a word: |x| + 0 * |x| is |x| for finite
-// x and NaN otherwise, and the maximum drops NaN operands; 1.5 instructions an element where widening each took 3.5.
+// The same over whole source words.  16-bit sources stay packed, two running maxima in a word: x + 0 * x is x for finite x and NaN
+// otherwise, and the maximum of magnitudes drops NaN operands; one instruction an element where widening each took 3.5.  (The signs of
+// the running maxima mean nothing.  With the magnitude taken first it was 1.5: one scale per row, 7168 x 4096 BF16 17.1 -> 16.7 us.)
 template <int SRC> __device__ __forceinline__ uint32_t amax_word(uint32_t acc, uint32_t w)
 {
     if (SRC == HIF8_F32) return __float_as_uint(amax_step(__uint_as_float(acc), __uint_as_float(w)));
-    const uint32_t a = w & 0x7FFF7FFFu;
     uint32_t t, d;
     if (SRC == HIF8_BF16) {
-        asm("fma.rn.bf16x2 %0, %1, %2, %1;" : "=r"(t) : "r"(a), "r"(0u));
-        asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(acc), "r"(t));
+        asm("fma.rn.bf16x2 %0, %1, %2, %1;" : "=r"(t) : "r"(w), "r"(0u));
+        asm("max.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(acc), "r"(t));
     } else {
-        asm("fma.rn.f16x2 %0, %1, %2, %1;" : "=r"(t) : "r"(a), "r"(0u));
-        asm("max.f16x2 %0, %1, %2;" : "=r"(d) : "r"(acc), "r"(t));
+        asm("fma.rn.f16x2 %0, %1, %2, %1;" : "=r"(t) : "r"(w), "r"(0u));
+        asm("max.xorsign.abs.f16x2 %0, %1, %2;" : "=r"(d) : "r"(acc), "r"(t));
     }
     return d;
 }
@@ -626,8 +626,8 @@ template <int SRC> __device__ __forceinline__ uint32_t amax_vector(uint32_t acc,
 template <int SRC> __device__ __forceinline__ float amax_value(uint32_t acc)
 {
     if (SRC == HIF8_F32) return __uint_as_float(acc);
-    if (SRC == HIF8_BF16) return fmaxf(__uint_as_float(acc << 16), __uint_as_float(acc & 0xFFFF0000u));
-    return fmaxf(__half2float(__ushort_as_half((unsigned short)(acc & 0xFFFFu))), __half2float(__ushort_as_half((unsigned short)(acc >> 16))));
+    if (SRC == HIF8_BF16) return fmaxf(fabsf(__uint_as_float(acc << 16)), fabsf(__uint_as_float(acc & 0xFFFF0000u)));
+    return fmaxf(fabsf(__half2float(__ushort_as_half((unsigned short)(acc & 0xFFFFu)))), fabsf(__half2float(__ushort_as_half((unsigned short)(acc >> 16)))));
 }
 
 __device__ __forceinline__ void block_amax_commit(float acc, uint32_t* accum)
