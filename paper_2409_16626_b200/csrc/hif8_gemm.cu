@@ -80,6 +80,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// A warp that issues copies or MMAs runs its loop as a whole, waits included, and one elected lane (the same one every time) issues:
+// the compiler then keeps descriptors and addresses in uniform registers, which these instructions want.  In a branch of one lane
+// four MMAs and their commit took that thread 555 cycles, so 246 (back to back, waits that do not wait; in the narrow kernel it took 1000, and its decode warps
+// spent 43 of 101 thousand cycles waiting for MMAs), and a tile copy took 200.  us, a branch of lane 0 / elected: 16 x 28672 x 8192 59.5 / 48.5, 96 x 4096 x 4096 19.3 / 16.7,
+// 256 x 1536 x 768 7.9 / 7.0, 201 x 7168 x 4096 19.9 / 18.8, 2048 x 7168 x 4096 101.4 / 96.0, without a workspace 127.8 / 125.5; 48 products in the mean 8 %.
+// Whatever ends a loop is agreed on by the warp, since a lane of its own would be waited for at the next election.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+__device__ __forceinline__ bool warp_all(bool x) { return __all_sync(0xFFFFFFFFu, x); }
+__device__ __forceinline__ bool warp_any(bool x) { return __any_sync(0xFFFFFFFFu, x); }
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }
 __device__ __forceinline__ unsigned long long global_ns()
 {
     unsigned long long t;
@@ -521,8 +536,7 @@ __device__ __forceinline__ void apply_channel_scale(const GemmParams& p, int col
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kNarrowMaxM = 64;
 constexpr uint32_t kNwW8 = BM * BK;  // weight bytes of a k-block: 8 KiB
-// A copy brings two k-blocks (a "pair block": 128 bytes of k) of weights and of activations: issuing a tile copy costs
-// its thread a few hundred cycles whatever the size, and with one copy of each kind per k-block that thread set the pace.
+// A copy brings two k-blocks (a "pair block": 128 bytes of k) of weights and of activations: a tile copy costs the same whatever its size.
 constexpr int BK2 = 2 * BK;
 // Byte stages (one pair block of weights each, and of activations when they are bytes).  The weight stream needs about
 // 64 KiB per SM in flight for the rate of HBM, so six stages of 16 KiB where they fit: with four, and with the
@@ -578,9 +592,8 @@ struct NarrowSmem {
 };
 // Tensor memory: the accumulators (two per issuer: the epilogue of one segment overlaps the next segment's MMAs), then
 // one weight stage (128 rows x 64 BF16 = 32 columns) per operand stage.
-// MMA issuers.  One thread that waits for a stage, issues its four MMAs and commits spends about a thousand cycles per
-// k-block, more than the decode groups or the copies need; so up to four threads (one per warp) share the k-blocks,
-// issuer q taking the k-blocks it = q (mod issuers) into accumulators of its own, which the epilogue adds.  Up to 32
+// MMA issuers: four warps share the k-blocks, issuer q taking the k-blocks it = q (mod issuers) into accumulators of its own, which the
+// epilogue adds (one lane that waited, issued and committed was busy 1000 cycles per k-block; see elect_one).  Up to 32
 // activation rows every issuer has two accumulators, above that one: issuers x buffers x rows stays within 256 columns.
 constexpr int kNwMaxIssuers = 4;
 constexpr int kNwMaxSplit = 8;
@@ -698,7 +711,7 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             return;
         }
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     constexpr int S = kNwTmemStages;  // operand ring: the it-th k-block uses stage it % S
     static_assert(S % kDecodeGroups == 0, "an operand stage is always written by the same group");
     const int S8 = lay.stages8;         // byte ring: the i-th pair block of this CTA lands in stage i % S8
@@ -737,30 +750,34 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     const int bufs = mp <= 32 ? 2 : 1;
     auto acc_col = [&](int q, int buf) { return (uint32_t)((q * bufs + buf) * mp); };  // accumulator of issuer q, buffer buf
 
-    // copies of the range's next unit: its weight bytes (and, as bytes, its activations) into stage s
+    // (the whole copying warp) copies of the range's next unit: its weight bytes (and, as bytes, its activations) into stage s
     int cp_slab = slab0, cp_pb = pb0;
     auto copy_bytes = [&](int s) {
         const uint32_t dst_w = lay.u8(s), dst_a = dst_w + kU8Act;
         const uint64_t w_policy = l2_policy_evict_first();
-        mbar_arrive_expect_tx(bar_u8_full(s), 2 * kNwW8 + (ACT_BF16 ? 0u : act_bytes));
-        // (the weight is read once: its lines are the first to leave L2 again, so that the expanded activations, which
-        // every CTA reads, and the slices of the slabs that two CTAs share stay there)
-        if (W_IS_NK) tma_load_2d_hint(dst_w, &map_w, cp_pb * BK2, cp_slab * BM, bar_u8_full(s), w_policy);
-        else tma_load_2d_hint(dst_w, &map_w, cp_slab * BM, cp_pb * BK2, bar_u8_full(s), w_policy);
-        if (!ACT_BF16) tma_load_2d(dst_a, &map_act, cp_pb * BK2, 0, bar_u8_full(s));
+        if (elect_one()) {
+            mbar_arrive_expect_tx(bar_u8_full(s), 2 * kNwW8 + (ACT_BF16 ? 0u : act_bytes));
+            // (the weight is read once: its lines are the first to leave L2 again, so that the expanded activations, which
+            // every CTA reads, and the slices of the slabs that two CTAs share stay there)
+            if (W_IS_NK) tma_load_2d_hint(dst_w, &map_w, cp_pb * BK2, cp_slab * BM, bar_u8_full(s), w_policy);
+            else tma_load_2d_hint(dst_w, &map_w, cp_slab * BM, cp_pb * BK2, bar_u8_full(s), w_policy);
+            if (!ACT_BF16) tma_load_2d(dst_a, &map_act, cp_pb * BK2, 0, bar_u8_full(s));
+        }
         if (++cp_pb == num_pb) { cp_pb = 0; cp_slab++; }
     };
     const int n_early = min(2, n_pairs);
-    if (threadIdx.x == kTmaWarp * 32) {
-        for (int s = 0; s < S8; s++) { mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), 2 * kGroupWarps); }  // both halves' groups
-        // operands ready: the group's warps, plus (ACT_BF16) the announcement of the activation tile's bytes
-        for (int s = 0; s < S; s++) { mbar_init(bar_bf_full(s), kGroupWarps + (ACT_BF16 ? 1 : 0)); mbar_init(bar_bf_empty(s), 1); }
-        for (int b = 0; b < 2; b++) { mbar_init(bar_acc_full(b), issuers); mbar_init(bar_acc_empty(b), kEpiWarps); }
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        // The first byte copies start here, under the table set-up (two of them: each takes this thread a few hundred cycles,
-        // and the block waits for it): nothing in front of this kernel writes the
+    if (warp == kTmaWarp) {
+        if (elect_one()) {
+            for (int s = 0; s < S8; s++) { mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), 2 * kGroupWarps); }  // both halves' groups
+            // operands ready: the group's warps, plus (ACT_BF16) the announcement of the activation tile's bytes
+            for (int s = 0; s < S; s++) { mbar_init(bar_bf_full(s), kGroupWarps + (ACT_BF16 ? 1 : 0)); mbar_init(bar_bf_empty(s), 1); }
+            for (int b = 0; b < 2; b++) { mbar_init(bar_acc_full(b), issuers); mbar_init(bar_acc_empty(b), kEpiWarps); }
+            *abort_flag = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        __syncwarp();
+        // The first byte copies start here, under the table set-up (two of them: the block waits for this warp): nothing in front of this kernel writes the
         // operands (the launch before it writes the expanded activations and the cleared words only, and that launch itself
         // waits for everything before it).
         for (int i = 0; i < n_early; i++) copy_bytes(i);
@@ -781,31 +798,32 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
     if (ACT_BF16 && warp != kTmaWarp) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp == kTmaWarp) {
-        if (lane == 0) {
-            int issued = n_early, s = n_early;
-            uint32_t ph = 1;  // parity of the round before the one that fills stage s next
-            for (int it = n_early; it < n_pairs; it++) {
-                if (it >= S8 && !mbar_wait(bar_u8_empty(s), ph, abort_flag, p.status, 31)) break;
-                if (*abort_flag) break;
-                copy_bytes(s);
-                issued = it + 1;
-                if (++s == S8) { s = 0; ph ^= 1u; }
-            }
-            if (*abort_flag)
-                for (int it = max(0, issued - S8); it < issued; it++) wait_landed(bar_u8_full(it % S8), it, S8);
+        int issued = n_early, s = n_early;
+        uint32_t ph = 1;  // parity of the round before the one that fills stage s next
+        for (int it = n_early; it < n_pairs; it++) {
+            if (it >= S8 && !warp_all(mbar_wait(bar_u8_empty(s), ph, abort_flag, p.status, 31))) break;
+            if (warp_any(*abort_flag)) break;
+            copy_bytes(s);
+            issued = it + 1;
+            if (++s == S8) { s = 0; ph ^= 1u; }
         }
+        if (*abort_flag)
+            for (int it = max(0, issued - S8); it < issued; it++) wait_landed(bar_u8_full(it % S8), it, S8);
     } else if (warp == kNwActWarp) {
         // Activations expanded to BF16 beforehand (map_act is then the map of that copy): the tile of every k-block goes
         // straight into its operand stage, in the 128-byte-swizzled layout the MMA reads, once the MMAs of the stage's
         // previous use have read it.
-        if (ACT_BF16 && lane == 0) {
+        if (ACT_BF16) {
             int issued = 0, kb = 2 * pb0;
             for (int it = 0; it < n_it; it++) {
                 const int sb = it % S, rb = it / S;
-                if (rb > 0 && !mbar_wait(bar_bf_empty(sb), (rb - 1) & 1, abort_flag, p.status, 37)) break;
-                if (*abort_flag) break;
-                mbar_arrive_expect_tx(bar_bf_full(sb), (uint32_t)mp * BK * 2u);
-                tma_load_2d(lay.bf(sb), &map_act, kb * BK, 0, bar_bf_full(sb));
+                if (rb > 0 && !warp_all(mbar_wait(bar_bf_empty(sb), (rb - 1) & 1, abort_flag, p.status, 37))) break;
+                if (warp_any(*abort_flag)) break;
+                const uint32_t dst = lay.bf(sb);
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(bar_bf_full(sb), (uint32_t)mp * BK * 2u);
+                    tma_load_2d(dst, &map_act, kb * BK, 0, bar_bf_full(sb));
+                }
                 issued = it + 1;
                 if (++kb == num_kb) kb = 0;
             }
@@ -814,7 +832,7 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
         }
     } else if (warp == kMmaWarp || warp >= kFirstDecodeWarp + kDecodeWarps) {
         const int q = warp == kMmaWarp ? 0 : warp - (kFirstDecodeWarp + kDecodeWarps) + 1;  // issuer number
-        if (lane == 0 && q < issuers) {
+        if (q < issuers) {
             // FP32 accumulator, BF16 operands; A = weight slab (K-major for [N,K] weights, MN-major for [K,N]), B = activations
             // (K-major), N = mp, M = 128
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(mp >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
@@ -827,27 +845,27 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                 if ((it & (issuers - 1)) == q) {
                     const int s = it % S, round = it / S;
                     // a segment's first MMA overwrites the accumulator: the epilogue must have read its previous contents
-                    if (first && use >= 1) ok = mbar_wait(bar_acc_empty(buf), (use - 1) & 1, abort_flag, p.status, 36);
-                    if (ok) ok = mbar_wait(bar_bf_full(s), round & 1, abort_flag, p.status, 32);
+                    if (first && use >= 1) ok = warp_all(mbar_wait(bar_acc_empty(buf), (use - 1) & 1, abort_flag, p.status, 36));
+                    if (ok) ok = warp_all(mbar_wait(bar_bf_full(s), round & 1, abort_flag, p.status, 32));
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + acc_col(q, buf);
+                    const uint32_t d_tmem = tmem_base + acc_col(q, buf), a_tmem = tmem_base + kTmemAccN + (uint32_t)(s * (BK / 2));
+                    const uint64_t db = da0 + (uint64_t)((lay.bf(s) - lay.bf(0)) >> 4);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; kk++) {
-                        // weights from tensor memory: operand stage s, 16 k = 8 columns
-                        tc_mma_bf16_cta_a_tmem(d_tmem, tmem_base + kTmemAccN + (uint32_t)(s * (BK / 2) + kk * 8),
-                                               da0 + (uint64_t)((lay.bf(s) - lay.bf(0) + kk * 32) >> 4), idesc, (!first || kk > 0) ? 1u : 0u);
+                        for (int kk = 0; kk < BK / 16; kk++)  // weights from tensor memory: operand stage s, 16 k = 8 columns
+                            tc_mma_bf16_cta_a_tmem(d_tmem, a_tmem + kk * 8, db + (uint64_t)(kk * 2), idesc, (!first || kk > 0) ? 1u : 0u);
+                        tc_commit_cta(bar_bf_empty(s));
                     }
-                    tc_commit_cta(bar_bf_empty(s));
                     first = false;
                 }
                 if (++kb == num_kb || it == n_it - 1) {  // the segment ends with its slab or with this CTA's range
                     // An issuer without a k-block in the segment only arrives.  With one buffer that arrival must not fall
                     // into the barrier's previous phase (the other issuers' commits of the last segment may still be on
                     // their way): it waits until the epilogue has read the last segment, as a first MMA would have.
-                    if (first && bufs == 1 && use >= 1) ok = mbar_wait(bar_acc_empty(buf), (use - 1) & 1, abort_flag, p.status, 36);
+                    if (first && bufs == 1 && use >= 1) ok = warp_all(mbar_wait(bar_acc_empty(buf), (use - 1) & 1, abort_flag, p.status, 36));
                     if (!ok) break;
-                    tc_commit_cta(bar_acc_full(buf));
+                    if (elect_one()) tc_commit_cta(bar_acc_full(buf));
                     kb = 0; seg++; first = true;
                 }
             }
@@ -1319,7 +1337,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
             return;
         }
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank(), half = rank & 1u, lead = rank & ~1u;  // half 0: leader of its pair (issues the MMAs)
     const bool leader = half == 0;
     const uint32_t bars = lay.bars;
@@ -1350,34 +1368,37 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         } else tile_coords(FORM == kParts ? t / tp.parts : t, tp.chunks, tp.slabs, piece, slab);
         m0 = FORM == kParts ? piece * tp.tile_rows + t % tp.parts * tp.bn : piece * tp.bn;
     };
-    auto copy_bytes = [&](int it, int t, int kb) {  // tile t's bytes of k-block kb into stage it % kWdStages, which is free
+    auto copy_bytes = [&](int it, int t, int kb) {  // (the whole copying warp) tile t's bytes of k-block kb into stage it % kWdStages, which is free
         int slab, m0;
         place(t, slab, m0);
         const int s = it % kWdStages, n0 = slab * 2 * BM + (int)half * BM;
         const uint32_t dst = lay.u8(s), bar = bar_u8_full(s);
-        mbar_arrive_expect_tx(bar, Smem::kW8 + (ACT == kActExpanded ? 0u : (uint32_t)(tp.bn / 2) * KB));
-        if (W_IS_NK) tma_load_2d(dst, &map_w, kb * KB, n0, bar);
-        else tma_load_2d(dst, &map_w, n0, kb * KB, bar);
-        if (ACT != kActExpanded) {
-            m0 += (int)half * (tp.bn / 2);
+        m0 += (int)half * (tp.bn / 2);
+        if (elect_one()) {
+            mbar_arrive_expect_tx(bar, Smem::kW8 + (ACT == kActExpanded ? 0u : (uint32_t)(tp.bn / 2) * KB));
+            if (W_IS_NK) tma_load_2d(dst, &map_w, kb * KB, n0, bar);
+            else tma_load_2d(dst, &map_w, n0, kb * KB, bar);
             if (ACT == kActRows) tma_load_2d(dst + Smem::kW8, &map_act, kb * KB, m0, bar);
-            else tma_load_2d(dst + Smem::kW8, &map_act, m0, kb * KB, bar);
+            else if (ACT == kActColumns) tma_load_2d(dst + Smem::kW8, &map_act, m0, kb * KB, bar);
         }
     };
-    if (threadIdx.x == kTmaWarp * 32) {
-        for (int s = 0; s < kWdStages; s++) {
-            mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps);
-            // operands ready: both CTAs' groups, plus (expanded activations) the leader's announcement of the tile bytes
-            mbar_init(bar_bf_full(s), 2 * kGroupWarps + (ACT == kActExpanded ? 1 : 0)); mbar_init(bar_bf_empty(s), 1);
+    if (warp == kTmaWarp) {
+        if (elect_one()) {
+            for (int s = 0; s < kWdStages; s++) {
+                mbar_init(bar_u8_full(s), 1); mbar_init(bar_u8_empty(s), kGroupWarps);
+                // operands ready: both CTAs' groups, plus (expanded activations) the leader's announcement of the tile bytes
+                mbar_init(bar_bf_full(s), 2 * kGroupWarps + (ACT == kActExpanded ? 1 : 0)); mbar_init(bar_bf_empty(s), 1);
+            }
+            mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps)); mbar_init(bar_sums, 1);
+            // (The others touch these two words when a wait has given up, seconds later, and the block's barrier stands in front of the
+            // cluster's: no fence at cluster scope, which would make every call 0.8 us longer, 201 x 7168 x 4096 19.9 -> 20.6.)
+            *reinterpret_cast<volatile int*>(sm + lay.gave_up()) = 0;
+            *reinterpret_cast<volatile uint32_t*>(sm + lay.issued()) = 0u;
+            *abort_flag = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
-        mbar_init(bar_acc_full, 1); mbar_init(bar_acc_empty, 2 * (kEpiWarps + kDecodeWarps)); mbar_init(bar_sums, 1);
-        // (The others touch these two words when a wait has given up, seconds later, and the block's barrier stands in front of the
-        // cluster's: no fence at cluster scope, which would make every call 0.8 us longer, 201 x 7168 x 4096 19.9 -> 20.6.)
-        *reinterpret_cast<volatile int*>(sm + lay.gave_up()) = 0;
-        *reinterpret_cast<volatile uint32_t*>(sm + lay.issued()) = 0u;
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
         if (ACT == kActExpanded) copy_bytes(0, t0, kb0);
     }
     fill_decode_table<(1 << (kLutShift - 2))>(reinterpret_cast<uint32_t*>(sm + lay.lut), warp, lane, kThreadsWd / 32);
@@ -1401,29 +1422,26 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         // ------------------------------------------------------------------ bytes (each CTA feeds itself).  Beside expanded
         // activations nothing is read here that the launch in front of this one writes, and what came before that is complete.
         const int n_early = min(kWdStages, kb1 - kb0);  // of the first tile, without waiting for anybody
-        if (lane == 0)
-            for (int i = ACT == kActExpanded ? 1 : 0; i < n_early; i++) copy_bytes(i, t0, kb0 + i);
+        for (int i = ACT == kActExpanded ? 1 : 0; i < n_early; i++) copy_bytes(i, t0, kb0 + i);
         __syncwarp();
         cluster_wait();
-        if (lane == 0) {
-            int it = 0;
-            bool ok = true;
-            for (int t = t0; t < t_end && ok; t += t_step) {
-                for (int kb = kb0; kb < kb1; kb++, it++) {
-                    if (it < n_early) continue;
-                    if (it >= kWdStages) ok = mbar_wait(bar_u8_empty(it % kWdStages), (it / kWdStages - 1) & 1, abort_flag, p.status, 41);
-                    if (!ok || *abort_flag) { ok = false; break; }
-                    copy_bytes(it, t, kb);
-                }
+        int it = 0;
+        bool ok = true;
+        for (int t = t0; t < t_end && ok; t += t_step) {
+            for (int kb = kb0; kb < kb1; kb++, it++) {
+                if (it < n_early) continue;
+                if (it >= kWdStages) ok = warp_all(mbar_wait(bar_u8_empty(it % kWdStages), (it / kWdStages - 1) & 1, abort_flag, p.status, 41));
+                if (!ok || warp_any(*abort_flag)) { ok = false; break; }
+                copy_bytes(it, t, kb);
             }
-            if (*abort_flag)
-                for (int i = max(0, it - kWdStages); i < it; i++) wait_landed(bar_u8_full(i % kWdStages), i, kWdStages);
         }
+        if (*abort_flag)
+            for (int i = max(0, it - kWdStages); i < it; i++) wait_landed(bar_u8_full(i % kWdStages), i, kWdStages);
     } else if (warp == kWdActWarp) {
         // ------------------------------------------------------------------ expanded activations: this CTA's bn / 2 rows, two boxes of
         // 64 k (the swizzle span); both CTAs' copies complete on the leader's "operands ready" barrier
         cluster_wait();
-        if (lane == 0) {
+        {
             if (!tp.follows) asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch in front expands them
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             // A tile's barrier (in the pair's leader) counts the bytes of both CTAs' halves.  A thread that is through says how many tiles
@@ -1441,17 +1459,20 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
                 m0 += (int)half * (tp.bn / 2);
                 for (int kb = kb0; kb < kb1; kb++, it++) {
                     const int s = it % kWdStages;
-                    if (limit == kNoLimit && ((it >= kWdStages && !mbar_wait(bar_bf_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 46)) || *abort_flag)) {
+                    if (limit == kNoLimit && ((it >= kWdStages && !warp_all(mbar_wait(bar_bf_empty(s), (it / kWdStages - 1) & 1, abort_flag, p.status, 46))) || warp_any(*abort_flag))) {
                         tell();
                         const unsigned long long c0 = global_ns();
                         do limit = (int)ld_cluster_u32(map_to_cta(lay.issued(), rank ^ 1u)) - 1;  // (the other CTA's waits are bounded as well)
                         while (limit < 0 && global_ns() - c0 < 2 * kWaitLimitNs);
+                        limit = __shfl_sync(0xFFFFFFFFu, limit, 0);
                     }
                     if (it >= limit) { ok = false; break; }
-                    if (leader) mbar_arrive_expect_tx(bar_bf_full(s), (uint32_t)tp.bn * KB * 2u);
                     const uint32_t full = map_to_cta(bar_bf_full(s), lead);
-                    tma_load_3d_pair(lay.act(s), &map_act, kb * KB, m0, 0, full);
-                    tma_load_3d_pair(lay.act(s) + Smem::kActStage / 2, &map_act, kb * KB + BK, m0, 0, full);
+                    if (elect_one()) {
+                        if (leader) mbar_arrive_expect_tx(bar_bf_full(s), (uint32_t)tp.bn * KB * 2u);
+                        tma_load_3d_pair(lay.act(s), &map_act, kb * KB, m0, 0, full);
+                        tma_load_3d_pair(lay.act(s) + Smem::kActStage / 2, &map_act, kb * KB + BK, m0, 0, full);
+                    }
                 }
             }
             if (ACT == kActExpanded) {
@@ -1464,30 +1485,34 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
         cluster_wait();
-        if (lane == 0 && leader) {
+        if (leader) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((ACT == kActColumns ? 1u : 0u) << 16) | ((uint32_t)(tp.bn >> 3) << 17) |
                                    ((uint32_t)((2 * BM) >> 4) << 24);
             int it = 0, local = 0;
             bool ok = true;
             for (int t = t0; t < t_end && ok; t += t_step, local++) {
                 if (local > 0) ok = mbar_wait(bar_acc_empty, (local - 1) & 1, abort_flag, p.status, 45);
+                ok = warp_all(ok);
                 for (int kb = kb0; kb < kb1 && ok; kb++, it++) {
                     const int s = it % kWdStages;
-                    ok = mbar_wait(bar_bf_full(s), (it / kWdStages) & 1, abort_flag, p.status, 42);
+                    ok = warp_all(mbar_wait(bar_bf_full(s), (it / kWdStages) & 1, abort_flag, p.status, 42));
                     if (!ok) break;
                     tc_fence_after();
                     // [M,K]: 16 k = 32 bytes inside the 128-byte rows (the second 64 k of an expanded block are the stage's second
                     // half); [K,M]: 16 k = two 1024-byte atoms
                     const uint64_t db = ACT == kActColumns ? make_smem_desc(lay.act(s), 8192, 1024) : make_smem_desc(lay.act(s), 16, 1024);
+                    const uint32_t a_tmem = tmem_base + kTmemColsAcc + (uint32_t)(s * (KB / 2));
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < KB / 16; kk++) {
-                        const uint32_t off = ACT == kActColumns ? kk * 2048 : (kk >> 2) * (Smem::kActStage / 2) + (kk & 3) * 32;
-                        tc_mma_bf16_pair_a_tmem(tmem_base, tmem_base + kTmemColsAcc + (uint32_t)(s * (KB / 2) + kk * 8), db + (uint64_t)(off >> 4), idesc,
-                                                (kb > kb0 || kk > 0) ? 1u : 0u);
+                        for (int kk = 0; kk < KB / 16; kk++) {
+                            const uint32_t off = ACT == kActColumns ? kk * 2048 : (kk >> 2) * (Smem::kActStage / 2) + (kk & 3) * 32;
+                            tc_mma_bf16_pair_a_tmem(tmem_base, a_tmem + kk * 8, db + (uint64_t)(off >> 4), idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
+                        }
+                        tc_commit_pair(bar_bf_empty(s), lead);
                     }
-                    tc_commit_pair(bar_bf_empty(s), lead);
                 }
-                if (ok) tc_commit_pair(bar_acc_full, lead);
+                if (ok && elect_one()) tc_commit_pair(bar_acc_full, lead);
+                __syncwarp();
             }
             if (!ok && it > 0) wait_landed(bar_bf_empty((it - 1) % kWdStages), it - 1, kWdStages);
         }
@@ -1706,8 +1731,7 @@ hif8_gemm_weights_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
 //   warps 0-3  epilogue (TMEM -> global), overlapped with the next tile through two TMEM accumulators
 //   warp  4    TMA producer of the A tiles: BF16 tiles land directly in the 128-byte-swizzled operand layout
 //   warp  5    MMA issuer
-//   warp  6    TMA producer of the W tiles (issuing a tile copy costs its thread about 200 cycles; one thread issuing the
-//              two or three copies of a k-block, with its waits, took longer than the 512 cycles of the k-block's MMAs)
+//   warp  6    TMA producer of the W tiles
 // A cluster of two CTAs on two SMs computes one 256 x 256 tile: each CTA stages its own 128 rows of A and its own 128
 // columns of W (so the tensor core reads half as many operand bytes per SM and flop as with one CTA per tile, which is
 // what bounds a one-CTA kernel), both accumulate their 128 rows in their own TMEM.  The even CTA of the pair (the
@@ -1745,7 +1769,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char* sm = smem_raw + (base - smem_u32(smem_raw));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();          // 0: leader (issues the MMAs), 1: peer
     const bool leader = rank == 0;
     const uint32_t bars = base + SmemLayout2::bars;
@@ -1799,7 +1823,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         }
     };
     if (warp == kTmaWarp || warp == kTmaWarpW) {
-        if (lane == 0) {
+        {
             int s = 0;            // stage of the next k-block
             uint32_t ph = 0;      // parity of the round the ring is in
             bool ok = true, wrapped = false;
@@ -1809,17 +1833,18 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                 tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n);
                 const int m0 = tile_m * 2 * BM + (int)rank * BM, n0 = tile_n * BN + (int)rank * (BN / 2);
                 for (int kb = 0; kb < num_kb; kb++) {
-                    if (wrapped) ok = mbar_wait(bar_empty(s), ph ^ 1u, abort_flag, p.status, 21);  // the previous round's use of the stage
-                    if (!ok || *abort_flag) { ok = false; break; }
-                    copy_block(m0, n0, ia, iw, kb, s);
+                    if (wrapped) ok = warp_all(mbar_wait(bar_empty(s), ph ^ 1u, abort_flag, p.status, 21));  // the previous round's use of the stage
+                    if (!ok || warp_any(*abort_flag)) { ok = false; break; }
+                    if (elect_one()) copy_block(m0, n0, ia, iw, kb, s);
                     progress++;
                     if (++s == kStages2) { s = 0; ph ^= 1u; wrapped = true; }
                 }
             }
-            for (uint32_t r = 0; r < 2; r++) st_cluster_u32(map_to_cta(base + SmemLayout2::issued + 4u * (2u * rank + (loads_a ? 0u : 1u)), r), (uint32_t)progress);
+            if (lane == 0)
+                for (uint32_t r = 0; r < 2; r++) st_cluster_u32(map_to_cta(base + SmemLayout2::issued + 4u * (2u * rank + (loads_a ? 0u : 1u)), r), (uint32_t)progress);
         }
     } else if (warp == kMmaWarp) {
-        if (lane == 0 && leader) {
+        if (leader) {
             // M = 256 over the pair, N = 256
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((W_IS_NK ? 0u : 1u) << 16) |
                                    ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
@@ -1828,27 +1853,27 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
             bool ok = true;
             for (int t = pair_id; t < tiles && ok; t += pairs, local++) {
                 const int acc = local & 1, use = local >> 1;
-                if (use > 0) ok = mbar_wait(bar_acc_empty(acc), (uint32_t)((use - 1) & 1), abort_flag, p.status, 22);
+                if (use > 0) ok = warp_all(mbar_wait(bar_acc_empty(acc), (uint32_t)((use - 1) & 1), abort_flag, p.status, 22));
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * 256;
                 for (int kb = 0; kb < num_kb; kb++) {
-                    ok = mbar_wait(bar_full(s), ph, abort_flag, p.status, 23);
+                    ok = warp_all(mbar_wait(bar_full(s), ph, abort_flag, p.status, 23));
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t a_addr = base + s * kStageBytes2, b_addr = a_addr + kABfBytes;
+                    const uint64_t da = make_smem_desc(a_addr, 16, 1024), db = W_IS_NK ? make_smem_desc(b_addr, 16, 1024) : make_smem_desc(b_addr, 8192, 1024);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; kk++) {
-                        const uint64_t da = make_smem_desc(a_addr + kk * 32, 16, 1024);
-                        const uint64_t db = W_IS_NK ? make_smem_desc(b_addr + kk * 32, 16, 1024)
-                                                    : make_smem_desc(b_addr + kk * 2048, 8192, 1024);
-                        tc_mma_bf16_pair(d_tmem, da, db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                        for (int kk = 0; kk < BK / 16; kk++)
+                            tc_mma_bf16_pair(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * (W_IS_NK ? 2 : 128)), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                        tc_commit_pair(bar_empty(s));
                     }
-                    tc_commit_pair(bar_empty(s));
                     progress++;
                     if (++s == kStages2) { s = 0; ph ^= 1u; }
                 }
-                if (ok) tc_commit_pair(bar_acc_full(acc));
+                if (ok && elect_one()) tc_commit_pair(bar_acc_full(acc));
+                __syncwarp();
             }
         }
     } else if (warp < kEpiWarps) {
