@@ -2112,7 +2112,8 @@ struct MapKey {
     uint64_t inner, rows, count, ld;  // ld: row pitch in elements (2-D) or distance between stacked matrices (3-D)
     uint32_t box_inner, box_rows;
     uint32_t kind;                    // 0: bytes, 2-D; 1: BF16, 2-D, 128-byte swizzle; 2: BF16, 3-D stack, 128-byte swizzle;
-                                      // 3: bytes, 2-D, 64-byte swizzle; 4: bytes, 2-D, 128-byte swizzle; 5: FP32, 2-D, 128-byte swizzle
+                                      // 3: bytes, 2-D, 64-byte swizzle; 4: bytes, 2-D, 128-byte swizzle; 5: FP32, 2-D, 128-byte swizzle;
+                                      // 6: as 4, lines of 128 bytes brought to L2
     uint32_t pad;
 };
 LruCache<MapKey, CUtensorMap, 64> g_map_cache;
@@ -2145,20 +2146,20 @@ bool encode_map(const MapKey& k, CUtensorMap* map)
     cuuint32_t estr[2] = {1, 1};
     return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(k.ptr), dims,
               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              (bf16 || k.kind == 4) ? CU_TENSOR_MAP_SWIZZLE_128B : (k.kind == 3 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE),
-              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+              (bf16 || k.kind == 4 || k.kind == 6) ? CU_TENSOR_MAP_SWIZZLE_128B : (k.kind == 3 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE),
+              k.kind == 6 ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // 2-D tensor [rows][ld elements] with a box of box_inner x box_rows elements, zero fill out of bounds.
 // bf16 = false: bytes, with no swizzle or the 64- or 128-byte one (box_inner at most that many bytes).  bf16 = true: 16-bit
-// elements, 128-byte swizzle (box_inner must be 64).
+// elements, 128-byte swizzle (box_inner must be 64).  lines_128: a copy brings lines of 128 bytes to L2 and not of 256.
 bool make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t rows, uint64_t ld, uint32_t box_inner, uint32_t box_rows,
-              bool bf16 = false, uint32_t bytes_swizzle = 0)
+              bool bf16 = false, uint32_t bytes_swizzle = 0, bool lines_128 = false)
 {
     MapKey k;
     std::memset(&k, 0, sizeof k);
     k.ptr = ptr; k.inner = inner; k.rows = rows; k.count = 1; k.ld = ld; k.box_inner = box_inner; k.box_rows = box_rows;
-    k.kind = bf16 ? 1u : (bytes_swizzle == 64 ? 3u : (bytes_swizzle == 128 ? 4u : 0u));
+    k.kind = bf16 ? 1u : (bytes_swizzle == 64 ? 3u : (bytes_swizzle == 128 ? (lines_128 ? 6u : 4u) : 0u));
     return g_map_cache.lookup_or_make(k, map, encode_map);
 }
 
@@ -2740,9 +2741,10 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         const int mp = (M + 15) & ~15;
         CUtensorMap map_act, map_ws;
         if (!make_map(&map_act, Aq, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK2, (uint32_t)mp)) return HIF8_ERR_CUDA;
-        // (weight tiles: 128-byte rows with the 128-byte swizzle, of 128 k or of 128 columns)
+        // (Weight tiles: 128-byte rows with the 128-byte swizzle, of 128 k or of 128 columns.  Columns: the other half of a line of 256 bytes is
+        // another slab's, which another CTA reads at another time, and is not brought along: 16 x 28672 x 8192 58.0 -> 48.8 us a call, 64 rows 68.2 -> 64.4.)
         const bool okn = w_is_nk ? make_map(&map_ws, Wq, (uint64_t)K, (uint64_t)N, (uint64_t)ldw, BK2, BM, false, 128)
-                                 : make_map(&map_ws, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, BK2, false, 128);
+                                 : make_map(&map_ws, Wq, (uint64_t)N, (uint64_t)K, (uint64_t)ldw, BM, BK2, false, 128, true);
         if (!okn) return HIF8_ERR_CUDA;
         const long long slabs = (N + BM - 1) / BM, num_pb = (K + BK2 - 1) / BK2;  // pair blocks: two k-blocks
         NarrowPlan plan{};
