@@ -547,10 +547,13 @@ constexpr int kNwMaxByteStages = 6, kNwMinByteStages = 4;
 // that a group starts its next k-block without waiting for the MMAs of its previous one
 constexpr int kNwTmemStages = 2 * kDecodeGroups;
 constexpr uint32_t kNwBars = 2 * kNwMaxByteStages + 2 * kNwTmemStages + 4;
-// Where the narrow kernel keeps what (mp activation rows).  WIDE (activations expanded beforehand):
+// Where the narrow kernel keeps what (mp activation rows).  WIDE:
 // the decode table has rows of 256 bytes and starts on a 64 KiB boundary of the shared window, so that one byte permute makes
 // a lookup's address (see decode8); operand stages and then byte stages as they fit in front of it, the rest behind it.
-// Otherwise: operand stages, byte stages and the 32 KiB table in a row.
+// Otherwise: operand stages, byte stages and the 32 KiB table in a row, for more than 48 rows of activations given as bytes, beside which
+// the larger table does not fit.  (With rows of 128 bytes a lookup's address takes three instructions: 16 x 28672 x 8192 with
+// activations as bytes 75.9 us a call, with the larger table 68.2, and with their decode as a loop in front of the weights 61.7.)
+constexpr int kNwWideBytesM = 48;
 template <bool WIDE, bool ACT_BF16>
 struct NarrowSmem {
     uint32_t base, lut, bars, end;  // shared-window addresses; base is 1024-byte aligned
@@ -578,7 +581,7 @@ struct NarrowSmem {
             act_front = kNwTmemStages;
             while ((uint32_t)act_front * act_bytes > front) act_front--;
             front_u8 = base + (uint32_t)act_front * act_bytes;
-            u8_front = (int)min((lut - front_u8) / (2 * kNwW8), (uint32_t)stages8);  // (WIDE: weights only)
+            u8_front = (int)min((lut - front_u8) / u8_bytes, (uint32_t)stages8);
             behind_act = lut + kLutBytesWide;
             behind_u8 = behind_act + (uint32_t)(kNwTmemStages - act_front) * act_bytes;
             bars = behind_u8 + (uint32_t)(stages8 - u8_front) * u8_bytes;
@@ -689,20 +692,18 @@ __global__ void __launch_bounds__(kExpandThreads) expand_activations_stream_kern
     }
 }
 
-template <bool W_IS_NK, bool ACT_BF16, bool CLUSTER>
+template <bool W_IS_NK, bool ACT_BF16, bool CLUSTER, bool WIDE>
 __global__ void __launch_bounds__(kThreadsN, 1)
 hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_constant__ CUtensorMap map_w, const GemmParams p, int mp,
                         const NarrowPlan plan)
 {
     extern __shared__ unsigned char smem_raw[];
-    // the 64 KiB table fits once no activations are decoded here (76 against 85 us at 16 x 28672 x 8192, [N,K])
-    constexpr bool kWideN = ACT_BF16;
-    constexpr int kLutShiftN = kWideN ? 8 : 7;
+    constexpr int kLutShiftN = WIDE ? 8 : 7;
     uint32_t dyn_bytes;
     asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
     // (a wait that gives up does so two seconds into the kernel, long after this; a separate launch cost 2 us)
     if (!ACT_BF16 && plan.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile int*>(p.status) = 0;
-    const NarrowSmem<kWideN, ACT_BF16> lay(smem_u32(smem_raw), smem_u32(smem_raw) + dyn_bytes, mp);
+    const NarrowSmem<WIDE, ACT_BF16> lay(smem_u32(smem_raw), smem_u32(smem_raw) + dyn_bytes, mp);
     unsigned char* sm = smem_raw - smem_u32(smem_raw);  // generic pointer of shared-window address 0
     {
         if (lay.end > smem_u32(smem_raw) + dyn_bytes) {  // the layout does not fit (the same answer in every thread)
@@ -895,7 +896,14 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
             }
             const uint32_t w8 = lay.u8(s8), a8 = w8 + kU8Act + (uint32_t)h * BK;
             const uint32_t abf = lay.bf(s);
-            uint2 va[kNarrowMaxM * (BK / 8) / kGroupThreads];
+            if (!ACT_BF16) {
+                // (the tile's 8-byte chunks, up to four per thread; a loop, so that what a smaller tile does not have is not fetched either)
+#pragma unroll 1
+                for (int q = dt; q < act_chunks; q += kGroupThreads) {
+                    const int row = q >> 3, jc = q & 7;
+                    sts_v4(abf + (row >> 3) * 1024 + (row & 7) * 128 + ((jc ^ (row & 7)) << 4), decode8<kLutShiftN>(lds_v2(a8 + row * BK2 + jc * 8), lut));
+                }
+            }
             uint4 vr[BK / 16];
             // this warp's 32 weight columns (operand rows, tensor-memory lanes): quarter * 32 ..
             const int quarter = warp & 3;
@@ -917,13 +925,6 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
 #pragma unroll
                     for (int c = 0; c < 2; c++)
                         vr[2 * i + c] = ldmatrix_trans_bytes_x2(w8 + (uint32_t)(k + 32 * i) * BM + ((uint32_t)((2 * quarter + c) ^ (lane & 7)) << 4));
-            }
-            if (!ACT_BF16) {
-#pragma unroll
-                for (int i = 0; i < kNarrowMaxM * (BK / 8) / kGroupThreads; i++) {
-                    const int q = i * kGroupThreads + dt;
-                    if (q < act_chunks) va[i] = lds_v2(a8 + (q >> 3) * BK2 + (q & 7) * 8);
-                }
             }
             __syncwarp();  // the byte stage has been read: the producer may refill it during the decode
             if (lane == 0) mbar_arrive(bar_u8_empty(s8));
@@ -948,13 +949,6 @@ hif8_gemm_narrow_kernel(const __grid_constant__ CUtensorMap map_act, const __gri
                         d[0] = lo.x; d[1] = lo.y; d[2] = lo.z; d[3] = lo.w; d[4] = hi.x; d[5] = hi.y; d[6] = hi.z; d[7] = hi.w;
                     }
                     tmem_st_16x256b_x4(st_base + ((uint32_t)(16 * c) << 16), o + 16 * c);
-                }
-            }
-            if (!ACT_BF16) {
-#pragma unroll
-                for (int i = 0; i < kNarrowMaxM * (BK / 8) / kGroupThreads; i++) {
-                    const int q = i * kGroupThreads + dt, row = q >> 3, jc = q & 7;
-                    if (q < act_chunks) sts_v4(abf + (row >> 3) * 1024 + (row & 7) * 128 + ((jc ^ (row & 7)) << 4), decode8<7>(va[i], lut));
                 }
             }
             tmem_st_wait();  // the weight column is in tensor memory
@@ -2194,6 +2188,12 @@ struct GemmDeviceSetup {
 };
 PerDevice<GemmDeviceSetup> g_gemm_setup;
 
+template <bool ACT_BF16, bool WIDE>
+void narrow_kernels(const void** k)
+{
+    k[0] = (const void*)hif8_gemm_narrow_kernel<false, ACT_BF16, false, WIDE>; k[1] = (const void*)hif8_gemm_narrow_kernel<true, ACT_BF16, false, WIDE>;
+    k[2] = (const void*)hif8_gemm_narrow_kernel<false, ACT_BF16, true, WIDE>; k[3] = (const void*)hif8_gemm_narrow_kernel<true, ACT_BF16, true, WIDE>;
+}
 template <int FORM>
 void weights_kernels(const void** k)
 {
@@ -2231,11 +2231,9 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
             cfg.attrs = attr; cfg.numAttrs = 1;
             out->rc = cudaOccupancyMaxActiveClusters(&out->wd_clusters[s], wd[1], &cfg);
         }
-        const void* narrow[8] = {(const void*)hif8_gemm_narrow_kernel<false, false, false>, (const void*)hif8_gemm_narrow_kernel<false, true, false>,
-                                 (const void*)hif8_gemm_narrow_kernel<true, false, false>, (const void*)hif8_gemm_narrow_kernel<true, true, false>,
-                                 (const void*)hif8_gemm_narrow_kernel<false, false, true>, (const void*)hif8_gemm_narrow_kernel<false, true, true>,
-                                 (const void*)hif8_gemm_narrow_kernel<true, false, true>, (const void*)hif8_gemm_narrow_kernel<true, true, true>};
-        for (int i = 0; i < 8 && out->rc == cudaSuccess; i++)
+        const void* narrow[12];
+        narrow_kernels<false, true>(narrow); narrow_kernels<true, true>(narrow + 4); narrow_kernels<false, false>(narrow + 8);
+        for (int i = 0; i < 12 && out->rc == cudaSuccess; i++)
             out->rc = cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesMax);
         for (int s = 1; s <= kNwMaxSplit && out->rc == cudaSuccess; s *= 2) {
             cudaLaunchConfig_t cfg{};
@@ -2244,7 +2242,7 @@ bool gemm_kernels_ready(int dev, int* sm_count_out, const int** wd_clusters = nu
             attr[0].val.clusterDim.x = s; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
             cfg.gridDim = dim3(s); cfg.blockDim = dim3(kThreadsN); cfg.dynamicSmemBytes = kSmemBytesMax;
             cfg.attrs = attr; cfg.numAttrs = 1;
-            out->rc = cudaOccupancyMaxActiveClusters(&out->nw_clusters[s], narrow[7], &cfg);
+            out->rc = cudaOccupancyMaxActiveClusters(&out->nw_clusters[s], narrow[7], &cfg);  // (all of them take the same)
         }
         std::memset(out->wp_clusters, 0, sizeof out->wp_clusters);
         const void* wp[8];
@@ -2490,12 +2488,20 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
 }
 
-template <bool W_IS_NK, bool ACT_BF16>
-static cudaError_t launch_narrow_kernel(const cudaLaunchConfig_t& cfg, bool cluster, const CUtensorMap& map_act, const CUtensorMap& map_w, const GemmParams& p,
-                                        int mp, const NarrowPlan& plan)
+template <bool W_IS_NK, bool ACT_BF16, bool WIDE>
+static cudaError_t launch_narrow_form(const cudaLaunchConfig_t& cfg, bool cluster, const CUtensorMap& map_act, const CUtensorMap& map_w, const GemmParams& p,
+                                      int mp, const NarrowPlan& plan)
 {
-    return cluster ? cudaLaunchKernelEx(&cfg, hif8_gemm_narrow_kernel<W_IS_NK, ACT_BF16, true>, map_act, map_w, p, mp, plan)
-                   : cudaLaunchKernelEx(&cfg, hif8_gemm_narrow_kernel<W_IS_NK, ACT_BF16, false>, map_act, map_w, p, mp, plan);
+    return cluster ? cudaLaunchKernelEx(&cfg, hif8_gemm_narrow_kernel<W_IS_NK, ACT_BF16, true, WIDE>, map_act, map_w, p, mp, plan)
+                   : cudaLaunchKernelEx(&cfg, hif8_gemm_narrow_kernel<W_IS_NK, ACT_BF16, false, WIDE>, map_act, map_w, p, mp, plan);
+}
+template <bool W_IS_NK>
+static cudaError_t launch_narrow_kernel(const cudaLaunchConfig_t& cfg, bool cluster, bool act_bf16, const CUtensorMap& map_act, const CUtensorMap& map_w,
+                                        const GemmParams& p, int mp, const NarrowPlan& plan)
+{
+    if (act_bf16) return launch_narrow_form<W_IS_NK, true, true>(cfg, cluster, map_act, map_w, p, mp, plan);
+    return mp <= kNwWideBytesM ? launch_narrow_form<W_IS_NK, false, true>(cfg, cluster, map_act, map_w, p, mp, plan)
+                               : launch_narrow_form<W_IS_NK, false, false>(cfg, cluster, map_act, map_w, p, mp, plan);
 }
 
 // How the warp kernel divides a product, and what that takes in cycles from call to results.  The terms are fitted to 670 measured
@@ -2600,7 +2606,8 @@ extern "C" int hif8_gemm_path_policy(int policy)
     return g_path_policy.exchange(policy, std::memory_order_relaxed);
 }
 
-// How the narrow kernel divides a product.  Cycles: a k-block takes about 500 (mp = 16) to 590 (64); a cluster's exchange 4000, and
+// How the narrow kernel divides a product.  Cycles: a k-block was taken to cost 500 (mp = 16) to 590 (64); it is 390 to 423 now, 530 to 828 with activations as
+// bytes, but with those figures in its place 250 products came out no faster in the mean and some 10 to 25 % slower.  A cluster's exchange 4000, and
 // clusters of eight start later; ranges of slabs end in a reduction of 2500 + 290 mp.  A cluster per slab (or one CTA: split 1), or,
 // when the workspace holds the partial sums of the slabs that a range boundary cuts, one CTA per SM with equal ranges: for many
 // slabs that do not divide among the SMs, and few rows.
@@ -2804,10 +2811,8 @@ static int gemm_entry(const uint8_t* Aq, int64_t lda, int a_is_km, const uint8_t
         cn.attrs = an; cn.numAttrs = (unsigned)n_an;
         cudaError_t nrc;
         const bool cluster = plan.split > 1;
-        if (w_is_nk) nrc = act_bf16 ? launch_narrow_kernel<true, true>(cn, cluster, map_act, map_ws, p, mp, plan)
-                                    : launch_narrow_kernel<true, false>(cn, cluster, map_act, map_ws, p, mp, plan);
-        else nrc = act_bf16 ? launch_narrow_kernel<false, true>(cn, cluster, map_act, map_ws, p, mp, plan)
-                            : launch_narrow_kernel<false, false>(cn, cluster, map_act, map_ws, p, mp, plan);
+        nrc = w_is_nk ? launch_narrow_kernel<true>(cn, cluster, act_bf16, map_act, map_ws, p, mp, plan)
+                      : launch_narrow_kernel<false>(cn, cluster, act_bf16, map_act, map_ws, p, mp, plan);
         if (nrc != cudaSuccess) return HIF8_ERR_CUDA;
         g_launches.fetch_add(1, std::memory_order_relaxed);
         return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
