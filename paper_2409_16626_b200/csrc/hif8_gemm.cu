@@ -428,12 +428,12 @@ __device__ __forceinline__ uint4 decode8(uint2 v, uint32_t lut_lane)
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-__device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int& tile_m, int& tile_n)
+// Groups of `group` tile-rows sweep N together: their W tiles stay in L2 (8: kGroupPieces is the same number).
+__device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int& tile_m, int& tile_n, int group = 8)
 {
-    constexpr int kGroupM = 8;  // groups of 8 tile-rows sweep N together: their W tiles stay in L2 (kGroupPieces is the same number)
-    const int per_group = kGroupM * tiles_n;
-    const int g = t / per_group, first_m = g * kGroupM;
-    const int rows_in_group = min(kGroupM, tiles_m - first_m);
+    const int per_group = group * tiles_n;
+    const int g = t / per_group, first_m = g * group;
+    const int rows_in_group = min(group, tiles_m - first_m);
     tile_m = first_m + (t % per_group) % rows_in_group;
     tile_n = (t % per_group) / rows_in_group;
 }
@@ -1775,6 +1775,9 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + SmemLayout2::abort_flag);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + SmemLayout2::tmem_slot);
     const int num_kb = (p.K + BK - 1) / BK;
+    // Up to K = 4096 the A tiles of sixteen tile-rows (32 MiB) stay in L2 beside the W tiles, and W is read half as often; beyond, those of eight (8192 x 28672
+    // x 8192 in a sequence of calls 2600 us, with sixteen 2655, with four 2676; x 4096 1255 and with sixteen 1240; 3000 x 11008 x 4096 203.5 and 197.9).
+    const int group = p.K <= 4096 ? 16 : 8;
     const int tiles_m2 = (p.M + 2 * BM - 1) / (2 * BM), tiles_n2 = p.tiles_n;
     // a batch of n x n products (A variant ia, W variant iw) is one list of tiles: product b = ia * n + iw owns tiles
     // [b * tiles_one, (b + 1) * tiles_one)
@@ -1824,7 +1827,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
             for (int t = pair_id; t < tiles && ok; t += pairs) {
                 int tile_m, tile_n;
                 const int b = t / tiles_one, ia = b / nb, iw = b - ia * nb;
-                tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n);
+                tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n, group);
                 const int m0 = tile_m * 2 * BM + (int)rank * BM, n0 = tile_n * BN + (int)rank * (BN / 2);
                 for (int kb = 0; kb < num_kb; kb++) {
                     if (wrapped) ok = warp_all(mbar_wait(bar_empty(s), ph ^ 1u, abort_flag, p.status, 21));  // the previous round's use of the stage
@@ -1886,7 +1889,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
             const int acc = local & 1, use = local >> 1;
             int tile_m, tile_n;
             const int b = t / tiles_one, ia = b / nb, iw = b - ia * nb;
-            tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n);
+            tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n, group);
             const int row0 = tile_m * 2 * BM + (int)rank * BM + warp * 32, row = row0 + lane, n0 = tile_n * BN;
             const int pieces = p.c_by_tma && row0 < p.M ? (min(BN, p.N - n0) + piece_cols - 1) / piece_cols : 0;
             auto fetch_old = [&](int i) {  // lane 0; the staging piece is free
@@ -2024,7 +2027,7 @@ bf16_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                 for (int i = progress; i < top; i++) {
                     int tile_m, tile_n;
                     const int t = pair_id + i / num_kb * pairs, b = t / tiles_one, ia = b / nb;
-                    tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n);
+                    tile_coords(t - b * tiles_one, tiles_m2, tiles_n2, tile_m, tile_n, group);
                     copy_block(tile_m * 2 * BM + (int)rank * BM, tile_n * BN + (int)rank * (BN / 2), ia, b - ia * nb, i % num_kb, i % kStages2);
                 }
                 if (leader && loads_a)
