@@ -1309,7 +1309,7 @@ __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, i
 // kParts is the last, incomplete round of a large product in tiles of fewer activation rows: divided along K alone, two tiles of
 // 2048 x 7168 x 4096 kept 8 pairs of 74 busy (103.7 us, with it 101.5; with activations as bytes 138.4 and 135.8; that launch waits
 // for nothing of the one in front of it, see TilePlan::follows, which is 1 us of it).
-enum WeightsForm { kOneGroup, kGroups, kFarRows, kParts };  // up to eight pieces; more; the rows of C 4 GiB apart or more (any number of pieces); parts of tiles
+enum WeightsForm { kOneGroup, kGroups, kFarRows, kParts };  // up to eight pieces (or sixteen, see launch_weights_kernel); more; the rows of C 4 GiB apart or more (any number of pieces); parts of tiles
 constexpr int kGroupPieces = 8;
 
 template <bool W_IS_NK, int ACT, int FORM>
@@ -2442,8 +2442,11 @@ static cudaError_t launch_weights_kernel(const cudaLaunchConfig_t& cfg, int w_is
 {
     if ((p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) return launch_weights_form<ACT, kFarRows>(cfg, w_is_nk, map_w, map_act, p, tp);
     if (tp.parts > 1) return launch_weights_form<ACT, kParts>(cfg, w_is_nk, map_w, map_act, p, tp);
-    return tp.chunks > kGroupPieces ? launch_weights_form<ACT, kGroups>(cfg, w_is_nk, map_w, map_act, p, tp)
-                                    : launch_weights_form<ACT, kOneGroup>(cfg, w_is_nk, map_w, map_act, p, tp);
+    // Sixteen pieces of K up to 4096 stay in L2 as eight of more do, and the instantiation for one group has the cheaper tiles; the other has the
+    // cheaper sums.  2400 x 7168 x 4096 115.5 us, as one group 113.1; 3000 x 1024 x 1024 12.9 and 12.4; 4096 cubed added to FP32 169.0 and 170.3.
+    const int one_group = p.K <= 4096 && !p.accumulate ? 2 * kGroupPieces : kGroupPieces;
+    return tp.chunks > one_group ? launch_weights_form<ACT, kGroups>(cfg, w_is_nk, map_w, map_act, p, tp)
+                                 : launch_weights_form<ACT, kOneGroup>(cfg, w_is_nk, map_w, map_act, p, tp);
 }
 
 // C = A W with the weights decoded inside the kernel.  act = kActExpanded: `a` is BF16 [M,K], written by the launch in front of

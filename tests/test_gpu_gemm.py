@@ -402,6 +402,24 @@ def test_gemm_weights_decoded_in_the_kernel(shape, form, w_is_nk, c_dtype, accum
     assert np.all(np.abs(out[rows, cols] - want) <= tol)
 
 
+@pytest.mark.parametrize("w_is_nk", [0, 1])
+@pytest.mark.parametrize("staged", ["a", False])
+@pytest.mark.parametrize("shape", [(2320, 1300, 144), (2064, 4100, 304), (4096, 1300, 4096), (4112, 1300, 144), (2320, 1300, 4112)])
+def test_gemm_rows_in_more_than_eight_pieces(shape, staged, w_is_nk):
+    # Nine to sixteen pieces of activation rows as one group, seventeen and a K above 4096 in groups of eight.
+    M, N, K = shape
+    N = (N + 15) // 16 * 16 if not w_is_nk else N
+    Aq, Wkn = W.random_codes((M, K), seed=M + K), W.random_codes((K, N), seed=N + K + 1)
+    for t in (Aq, Wkn):
+        t[(t == 0x80) | ((t & 0x7F) == 0x6F)] = 0x33
+    out = run_gemm(Aq, np.ascontiguousarray(Wkn.T) if w_is_nk else Wkn, w_is_nk, H.F32, sa=3, sw=-4, staged=staged)
+    rng = np.random.default_rng(M)
+    rows = np.concatenate([rng.integers(0, M, 20000), np.arange(M), np.full(N, M - 1)])
+    cols = np.concatenate([rng.integers(0, N, 20000), np.arange(M) % N, np.arange(N)])
+    P, S = O.gemm_entries(Aq, Wkn, False, 3, -4, rows, cols)
+    assert np.all(np.abs(out[rows, cols] - P) <= 1e-5 * S + 2.0 ** -24 * np.abs(P))
+
+
 @pytest.mark.parametrize("accumulate", [0, 1])
 @pytest.mark.parametrize("c_dtype", [H.F32, H.BF16])
 @pytest.mark.parametrize("w_is_nk", [0, 1])
