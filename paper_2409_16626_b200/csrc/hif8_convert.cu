@@ -23,6 +23,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <type_traits>
@@ -826,9 +827,7 @@ int device_info(int* sms, int* device = nullptr)
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-constexpr int kGroupsConvert = 4;  // encode / fake-quant kernels: groups per block on large tensors
-
-unsigned grid_for(unsigned long long n_vec, unsigned long long n, int sms, int unroll = kUnroll, int max_groups = 1)
+unsigned grid_for(unsigned long long n_vec, unsigned long long n, int sms, int unroll = kUnroll)
 {
     // Many more blocks than the SMs can hold, no persistent loop: blocks are handed to SMs as they free up, which
     // balances the load between SMs near to and far from a memory partition (measured 10-20 % faster than a static
@@ -837,12 +836,6 @@ unsigned grid_for(unsigned long long n_vec, unsigned long long n, int sms, int u
     unsigned long long need;
     if (n_vec) {
         need = (n_vec + per_block - 1) / per_block;
-        // Large tensors: up to max_groups groups per block (grid-stride), as long as at least one full wave of resident
-        // blocks remains for the scheduler to balance.  The per-block prologue (table set-up, scale) is then paid
-        // once per 64 KiB instead of once per 16 KiB, which the arithmetic-bound rounding modes feel most.
-        const unsigned long long wave = (unsigned long long)sms * kBlocksPerSM;
-        const unsigned long long groups = need / wave < (unsigned long long)max_groups ? need / wave : (unsigned long long)max_groups;
-        if (groups > 1) need = (need + groups - 1) / groups;
     } else {
         need = (n + kThreads - 1) / kThreads;
         unsigned long long cap = (unsigned long long)sms * kBlocksPerSM * 4;
@@ -853,12 +846,47 @@ unsigned grid_for(unsigned long long n_vec, unsigned long long n, int sms, int u
     return (unsigned)need;
 }
 
+// Blocks of a conversion.  A tensor is `need` groups of kUnroll vectors a thread, and `wave` blocks are resident at a time.  What a block pays once
+// (tables, the exponent) weighs more the fewer groups it takes; but with several groups each, a last wave that is half empty costs as much as a full
+// one.  So arithmetic-bound conversions take whole waves of blocks, each with an equal share of the groups, and the ones bound
+// by memory take a group per block, which balances SMs near to and far from a memory partition.  (Up to four groups per block at all sizes / here, us:
+// FP32 to bytes, hybrid rounding 10.2 M elements 13.3 / 11.3, 22.5 M 24.6 / 20.7, 60 M 52.7 / 50.0, round half away 22.5 M 19.5 / 18.3; BF16, hybrid 33 M
+// 21.8 / 19.5, half to even 33 M 31.4 / 28.7, stochastic 33 M 70.3 / 65.9; FP32 to dequantized values, hybrid 22.5 M 33.3 / 29.7; BF16 in place, hybrid 66 M
+// 43.5 / 41.5; bytes and amax, FP32, hybrid 10 M 15.3 / 13.1.)  The lines between the numbers of waves are where they met in sweeps of 4 to 268 M
+// elements; near a line its two sides differ by 2 %.  just_read: the source has just been read for its amax and lies partly in L2; memory binds all of
+// these more loosely, and from ten waves on four groups per block are as good as any (FP32 to bytes, round half away 16.8 M 22.9 / 22.1, BF16, stochastic 33 M 82.9 / 78.3).
+unsigned convert_grid(unsigned long long n_vec, unsigned long long n, int sms, int src, int mode, bool fq, bool amax, bool in_place, bool just_read)
+{
+    constexpr unsigned long long kGroupVecs = (unsigned long long)kThreads * kUnroll;
+    const unsigned long long need = (n_vec + kGroupVecs - 1) / kGroupVecs, wave = (unsigned long long)sms * kBlocksPerSM, whole = need / wave;
+    if (!n_vec || need <= wave) return grid_for(n_vec, n, sms);
+    const bool wide = src == HIF8_F32, away = mode == HIF8_RND_TA, thresholds = (mode == HIF8_RND_HR || mode == HIF8_RND_SSR) && src != HIF8_F16;
+    const unsigned long long shared = (need + std::min(whole, 4ull) - 1) / std::min(whole, 4ull);  // blocks with up to four groups each
+    unsigned long long blocks = need;
+    if (amax) {  // (a block's share of the maximum is two atomics on one address)
+        if (whole < 2 || (wide ? whole < 5 : thresholds && whole < 3)) blocks = wave;
+        else blocks = away || whole < 3 ? shared : 2 * wave;
+    } else if (just_read) {
+        if (!fq && (away || thresholds) && whole >= 2 && whole < 5) blocks = wave;
+        else if (whole >= (away ? 9 : 10)) blocks = in_place && away ? need : shared;
+        else if (whole >= 2) blocks = whole < 3 ? shared : 2 * wave;
+    } else if (in_place ? away || mode == HIF8_RND_TE : away && !fq) {
+        if (!in_place && whole < 4 && (whole > 1 || 4 * need < (wide ? 6 : 5) * wave)) blocks = whole * wave;
+    } else if (fq && mode != HIF8_RND_SR && src != HIF8_F16) {  // as many bytes out as in
+        if (whole >= 2) blocks = std::min((need + 2 * wave - 1) / (2 * wave), std::max(12ull, whole / 4)) * wave;
+        else if (in_place) blocks = wave;
+    } else if (thresholds) {
+        if (wide || whole > 1 || 4 * need < 5 * wave) blocks = whole < 9 ? wave : whole < 20 ? 2 * wave : shared;
+    } else if (whole >= 2) blocks = !wide && mode == HIF8_RND_SR && whole < 3 ? shared : (whole < 14 ? 2 : 4) * wave;
+    return (unsigned)std::min(blocks, 0x7FFFFFFFull);
+}
+
 template <int SRC, int MODE, bool FQ, bool AMAX>
 int launch_convert(const ConvParams& p, bool vec_ok, int sms, cudaStream_t st)
 {
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     unsigned long long n_vec = vec_ok ? p.n / PV : 0;
-    unsigned grid = grid_for(n_vec, p.n, sms, kUnroll, kGroupsConvert);
+    const unsigned grid = convert_grid(n_vec, p.n, sms, SRC, MODE, FQ, AMAX, false, p.reverse != 0);
     launch_pdl(convert_kernel<SRC, MODE, FQ, AMAX>, grid, st, p, n_vec);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
@@ -969,9 +997,7 @@ int launch_fq_ta(int dtype, int rnd, const ConvParams& p, bool vec_ok, int sms, 
 {
     const unsigned long long pv = dtype == HIF8_F32 ? 4 : 8;
     const unsigned long long n_vec = vec_ok ? p.n / pv : 0;
-    // round half away is bound by memory here and runs best with one group per block (42.3 against 43.6 us per 2^26
-    // BF16 elements); the threshold modes carry more arithmetic per element and gain from sharing the prologue
-    const unsigned grid = grid_for(n_vec, p.n, sms, kUnroll, rnd == HIF8_RND_TA ? 1 : kGroupsConvert);
+    const unsigned grid = convert_grid(n_vec, p.n, sms, dtype, rnd, true, false, true, p.reverse != 0);
     if (dtype == HIF8_F32) launch_pdl(fq_ta_kernel<HIF8_F32, HIF8_RND_TA>, grid, st, p, n_vec);
     else if (rnd == HIF8_RND_TA) launch_pdl(fq_ta_kernel<HIF8_BF16, HIF8_RND_TA>, grid, st, p, n_vec);
     else if (rnd == HIF8_RND_HR) launch_pdl(fq_ta_kernel<HIF8_BF16, HIF8_RND_HR>, grid, st, p, n_vec);
@@ -988,6 +1014,10 @@ int launch_amax(const void* src, int dtype, unsigned long long n, uint32_t* accu
     unsigned long long pv = dtype == HIF8_F32 ? 4 : 8;
     unsigned long long n_vec = vec_ok ? n / pv : 0;
     unsigned grid = grid_for(n_vec, n, sms, kUnrollAmax);
+    // On its own the last block publishes the result, and a block's ticket is an atomic on one address with a fence: two waves of blocks (us, a block for
+    // every 32 KiB / here: FP32 34.6 M elements 26.9 / 23.7, 57.7 M 44.6 / 35.5, 268 M 227.9 / 148.8; BF16 268 M 113.5 / 75.6).  In front of a conversion
+    // there is no ticket, and a block for every 32 KiB is 2 to 4 % faster.
+    if (d_amax_out) grid = std::min(grid, 2u * sms * kBlocksPerSM);
     switch (dtype) {
         case HIF8_F32: launch_pdl(n_vec > kStreamVecsF32 ? amax_kernel<HIF8_F32, true> : amax_kernel<HIF8_F32, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
         case HIF8_BF16: launch_pdl(n_vec > kKeepVecs ? amax_kernel<HIF8_BF16, true> : amax_kernel<HIF8_BF16, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
@@ -1097,7 +1127,7 @@ int hif8_encode_f32_patterns(uint32_t first_pattern, uint8_t* dst, size_t n, int
     ConvParams p{};
     p.dst = dst; p.n = n; p.scale_exp = scale_exp; p.flags = flags; p.seed = seed; p.pattern_first = first_pattern;
     const unsigned long long n_vec = (reinterpret_cast<uintptr_t>(dst) & 3u) ? 0 : n / 4;
-    const unsigned grid = grid_for(n_vec, n, sms, kUnroll, kGroupsConvert);
+    const unsigned grid = convert_grid(n_vec, n, sms, HIF8_F32, rnd, false, false, false, false);
     cudaStream_t st = (cudaStream_t)stream;
     switch (rnd) {
         case HIF8_RND_TA: launch_pdl(convert_kernel<HIF8_F32, HIF8_RND_TA, false, false, true>, grid, st, p, n_vec); break;

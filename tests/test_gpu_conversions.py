@@ -472,3 +472,51 @@ def test_generated_f32_patterns_sweep_with_both_options(mode):
     torch.cuda.synchronize()
     assert np.array_equal(readback(), ref.cpu().numpy())
     assert np.array_equal(readback(), O.encode(bits, O.F32, 5, omode, 0, seed=7, quick=True))
+
+
+@pytest.mark.parametrize("rnd", [H.RND_TA, H.RND_HR, H.RND_TE])
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
+@pytest.mark.parametrize("groups", [1184, 1185, 1184 * 5 // 4 + 1, 2 * 1184 - 1, 2 * 1184, 5 * 1184 + 3, 10 * 1184 - 5, 14 * 1184])
+def test_conversions_whatever_the_number_of_blocks(groups, dtype, rnd):
+    # Blocks of a launch come from how often the groups of a tensor fill the device: on both sides of those lines, every code and value is the one
+    # that the tensor's pieces, which are one group a block, have; nothing in front of or behind the results is written.
+    pv = 4 if dtype == H.F32 else 8
+    n = groups * 1024 * pv - 3
+    t = {H.F32: torch.float32, H.BF16: torch.bfloat16, H.F16: torch.float16}[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(groups)
+    x = (torch.randn(n, generator=gen, device="cuda") * 3).to(t)
+    x[12345] = 77.0
+    exp, amax = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(1, device="cuda")
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    guard, piece = 256, 1000 * 1024 * pv
+
+    def fresh(like):
+        return torch.full((n + 2 * guard,), 0x5A, dtype=torch.uint8, device="cuda") if like is None else torch.full((n + 2 * guard,), 9.0, dtype=t, device="cuda")
+
+    def check(out, want):
+        assert torch.equal(out[guard:guard + n].view(torch.uint8), want.view(torch.uint8))
+        assert bool((out[:guard] == (0x5A if out.dtype == torch.uint8 else 9.0)).all()) and bool((out[guard + n:] == (0x5A if out.dtype == torch.uint8 else 9.0)).all())
+
+    H.hif8_amax(x, dtype, n, amax, ws, 256)
+    assert float(amax) == 77.0
+    codes, values = torch.empty(n, dtype=torch.uint8, device="cuda"), torch.empty(n, dtype=t, device="cuda")
+    for scale_exp in (8, None):  # 14 - floor(log2 77) = 8: a given exponent, and the one worked out from the amax
+        for a in range(0, n, piece):
+            m = min(piece, n - a)
+            H.hif8_encode(x[a:], dtype, codes[a:], m, 8, rnd)
+            H.hif8_fake_quant(x[a:], values[a:], dtype, m, 0, 8, rnd)
+        out, back = fresh(None), fresh(t)
+        if scale_exp is None:
+            H.hif8_amax_scale_encode(x, dtype, out[guard:], n, 14, rnd, 0, 0, None, amax, exp, None, ws, 256)
+            H.hif8_fake_quant(x, back[guard:], dtype, n, 1, 14, rnd, 0, 0, None, None, ws, 256)
+            assert int(exp) == 8
+        else:
+            H.hif8_encode(x, dtype, out[guard:], n, scale_exp, rnd)
+            H.hif8_fake_quant(x, back[guard:], dtype, n, 0, scale_exp, rnd)
+        check(out, codes)
+        check(back, values)
+    out = fresh(None)
+    amax.zero_()
+    H.hif8_amax_scale_encode(x, dtype, out[guard:], n, 14, rnd, 0, 0, exp, amax, None, None, ws, 256)  # encodes with the exponent and measures
+    check(out, codes)
+    assert float(amax) == 77.0
