@@ -1309,7 +1309,7 @@ __device__ __forceinline__ void store_columns(unsigned char* out, Pitch pitch, i
 // kParts is the last, incomplete round of a large product in tiles of fewer activation rows: divided along K alone, two tiles of
 // 2048 x 7168 x 4096 kept 8 pairs of 74 busy (103.7 us, with it 101.5; with activations as bytes 138.4 and 135.8; that launch waits
 // for nothing of the one in front of it, see TilePlan::follows, which is 1 us of it).
-enum WeightsForm { kOneGroup, kGroups, kFarRows, kParts };  // up to eight pieces (or sixteen, see launch_weights_kernel); more; the rows of C 4 GiB apart or more (any number of pieces); parts of tiles
+enum WeightsForm { kOneGroup, kGroups, kFarRows, kParts };  // up to eight pieces (or sixteen, see launch_weights_gemm); more; the rows of C 4 GiB apart or more (any number of pieces); parts of tiles
 constexpr int kGroupPieces = 8;
 
 template <bool W_IS_NK, int ACT, int FORM>
@@ -2438,15 +2438,12 @@ static cudaError_t launch_weights_form(const cudaLaunchConfig_t& cfg, int w_is_n
 
 template <int ACT>
 static cudaError_t launch_weights_kernel(const cudaLaunchConfig_t& cfg, int w_is_nk, const CUtensorMap& map_w, const CUtensorMap& map_act, const GemmParams& p,
-                                         const TilePlan& tp)
+                                         const TilePlan& tp, bool one_group)
 {
     if ((p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) return launch_weights_form<ACT, kFarRows>(cfg, w_is_nk, map_w, map_act, p, tp);
     if (tp.parts > 1) return launch_weights_form<ACT, kParts>(cfg, w_is_nk, map_w, map_act, p, tp);
-    // Sixteen pieces of K up to 4096 stay in L2 as eight of more do, and the instantiation for one group has the cheaper tiles; the other has the
-    // cheaper sums.  2400 x 7168 x 4096 115.5 us, as one group 113.1; 3000 x 1024 x 1024 12.9 and 12.4; 4096 cubed added to FP32 169.0 and 170.3.
-    const int one_group = p.K <= 4096 && !p.accumulate ? 2 * kGroupPieces : kGroupPieces;
-    return tp.chunks > one_group ? launch_weights_form<ACT, kGroups>(cfg, w_is_nk, map_w, map_act, p, tp)
-                                 : launch_weights_form<ACT, kOneGroup>(cfg, w_is_nk, map_w, map_act, p, tp);
+    return one_group ? launch_weights_form<ACT, kOneGroup>(cfg, w_is_nk, map_w, map_act, p, tp)
+                     : launch_weights_form<ACT, kGroups>(cfg, w_is_nk, map_w, map_act, p, tp);
 }
 
 // C = A W with the weights decoded inside the kernel.  act = kActExpanded: `a` is BF16 [M,K], written by the launch in front of
@@ -2464,6 +2461,10 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
     WeightsCost::Rest rest = tl.cost.rest(tiles);
     if (rest.parts > 1 && (p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) rest = WeightsCost::Rest{};  // (rows of C 4 GiB apart have an instantiation for whole tiles)
     const int rem = (int)rest.tiles, clear = act != kActExpanded, slabs = tiles / tl.chunks;
+    // Sixteen pieces of K up to 4096 stay in L2 as eight of more do, and the instantiation for one group has the cheaper tiles; the other has the
+    // cheaper sums.  2400 x 7168 x 4096 115.5 us, as one group 113.1; 3000 x 1024 x 1024 12.9 and 12.4; 4096 cubed added to FP32 169.0 and 170.3.
+    // (Not where a launch of parts follows: it and the tiles in front of it number them in the same order, and parts are numbered in groups.)
+    const bool one_group = tl.chunks <= (K <= 4096 && !p.accumulate && rest.parts == 1 ? 2 * kGroupPieces : kGroupPieces);
     TilePlan launch[2];
     launch[0] = TilePlan{0, tiles - rem, tl.chunks, tl.bn, slabs, tiles <= pairs ? tl.cost.best_split(tiles) : 1, clear, 0, 1, tl.bn};
     launch[1] = TilePlan{(tiles - rem) * rest.parts, rem * rest.parts, tl.chunks, rest.rows, slabs, rest.split, 0, 1, rest.parts, tl.bn};
@@ -2485,9 +2486,9 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = 2;
-        const cudaError_t rc = act == kActExpanded ? launch_weights_kernel<kActExpanded>(cfg, w_is_nk, map_w, map_act, p, tp)
-                               : act == kActRows   ? launch_weights_kernel<kActRows>(cfg, w_is_nk, map_w, map_act, p, tp)
-                                                   : launch_weights_kernel<kActColumns>(cfg, w_is_nk, map_w, map_act, p, tp);
+        const cudaError_t rc = act == kActExpanded ? launch_weights_kernel<kActExpanded>(cfg, w_is_nk, map_w, map_act, p, tp, one_group)
+                               : act == kActRows   ? launch_weights_kernel<kActRows>(cfg, w_is_nk, map_w, map_act, p, tp, one_group)
+                                                   : launch_weights_kernel<kActColumns>(cfg, w_is_nk, map_w, map_act, p, tp, one_group);
         if (rc != cudaSuccess) return HIF8_ERR_CUDA;
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
