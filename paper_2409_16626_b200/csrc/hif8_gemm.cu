@@ -2463,8 +2463,9 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
     const int rem = (int)rest.tiles, clear = act != kActExpanded, slabs = tiles / tl.chunks;
     // Sixteen pieces of K up to 4096 stay in L2 as eight of more do, and the instantiation for one group has the cheaper tiles; the other has the
     // cheaper sums.  2400 x 7168 x 4096 115.5 us, as one group 113.1; 3000 x 1024 x 1024 12.9 and 12.4; 4096 cubed added to FP32 169.0 and 170.3.
-    // (Not where a launch of parts follows: it and the tiles in front of it number them in the same order, and parts are numbered in groups.)
-    const bool one_group = tl.chunks <= (K <= 4096 && !p.accumulate && rest.parts == 1 ? 2 * kGroupPieces : kGroupPieces);
+    // (Not where a launch for the last round follows: both number the tiles in the same order, parts of tiles are numbered in groups, and which tiles
+    // are divided along K, so how their sums are rounded, is as it is in groups.)
+    const bool one_group = tl.chunks <= (K <= 4096 && !p.accumulate && rem == 0 ? 2 * kGroupPieces : kGroupPieces);
     TilePlan launch[2];
     launch[0] = TilePlan{0, tiles - rem, tl.chunks, tl.bn, slabs, tiles <= pairs ? tl.cost.best_split(tiles) : 1, clear, 0, 1, tl.bn};
     launch[1] = TilePlan{(tiles - rem) * rest.parts, rem * rest.parts, tl.chunks, rest.rows, slabs, rest.split, 0, 1, rest.parts, tl.bn};
