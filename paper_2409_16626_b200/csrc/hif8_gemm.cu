@@ -2462,7 +2462,7 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
     if (rest.parts > 1 && (p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) rest = WeightsCost::Rest{};  // (rows of C 4 GiB apart have an instantiation for whole tiles)
     const int rem = (int)rest.tiles, clear = act != kActExpanded, slabs = tiles / tl.chunks;
     // Sixteen pieces of K up to 4096 stay in L2 as eight of more do, and the instantiation for one group has the cheaper tiles; the other has the
-    // cheaper sums.  2400 x 7168 x 4096 115.5 us, as one group 113.1; 3000 x 1024 x 1024 12.9 and 12.4; 4096 cubed added to FP32 169.0 and 170.3.
+    // cheaper sums.  4000 x 11008 x 1024 119.3 us, as one group 117.4; 3000 x 1024 x 1024 12.9 and 12.4; 2400 x 7168 x 4096 added to FP32 169.0 and 170.3.
     // (Not where a launch for the last round follows: both number the tiles in the same order, parts of tiles are numbered in groups, and which tiles
     // are divided along K, so how their sums are rounded, is as it is in groups.)
     const bool one_group = tl.chunks <= (K <= 4096 && !p.accumulate && rem == 0 ? 2 * kGroupPieces : kGroupPieces);
