@@ -181,10 +181,13 @@ __device__ __forceinline__ void convert_group(const ConvParams& p, const SmemTab
 // Encode / fake-quant kernel.  FQ = false: bytes out.  FQ = true: dequantized values in the source format.
 // AMAX = true: also reduce amax of the source into p.amax_accum[0]; the last block publishes it.
 // ------------------------------------------------------------------------------------------------
-// (Left to the compiler, round half away that measures amax takes 39 registers on BF16 and 16-bit fake-quant 40, two blocks a SM fewer: 40.3 us
-// a measuring encode of 2^26 BF16 elements, with 32 registers 36.6.)
-template <int SRC, int MODE, bool FQ, bool AMAX, bool PATTERN = false>
-__global__ void __launch_bounds__(kThreads, (AMAX && MODE == HIF8_RND_TA) || (FQ && SRC != HIF8_F32 && MODE != HIF8_RND_SR) ? kBlocksPerSM : 0) convert_kernel(const ConvParams p, unsigned long long n_vec)
+// SLOTS: the amax comes in several words (see resolve_scale_exp).
+// Blocks per SM: left to the compiler, encode takes 32 registers (stochastic rounding excepted), which is eight blocks.  Two kinds of fake-quant are faster
+// with the bound (us, without / with it): half to even of FP32, 34 registers so, 9.8 M elements 16.7 / 15.4, 68 M 91.0 / 86.1 (3 M 6.2 / 6.7), half away of FP16 11 M
+// 11.8 / 11.1, 82 M 60.8 / 59.8; other FP16 modes 0 to 0.6 % slower.
+template <int SRC, int MODE, bool FQ, bool AMAX, bool PATTERN = false, bool SLOTS = false>
+__global__ void __launch_bounds__(kThreads, FQ && !SLOTS && ((SRC == HIF8_F32 && MODE == HIF8_RND_TE) || (SRC == HIF8_F16 && MODE == HIF8_RND_TA)) ? kBlocksPerSM : 0)
+convert_kernel(const ConvParams p, unsigned long long n_vec)
 {
     static_assert(!PATTERN || (SRC == HIF8_F32 && !FQ && !AMAX), "generated sources are FP32 patterns, encode only");
     __shared__ SmemTables sm;
@@ -193,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, (AMAX && MODE == HIF8_RND_TA) || (FQ
     if (kPair16) setup_sum16<MODE>(sm.ta, sm.thr, p.flags);
     else setup_tables<true, MODE != HIF8_RND_TA, FQ, MODE, SRC>(sm, p.flags);  // reads only the constant table
     pdl_wait_prior_grid();
-    const int se = resolve_scale_exp(p);
+    const int se = resolve_scale_exp<SLOTS>(p);
     const float scale = pow2f(se);
     const int da = (-se) / 2, db = -se - da;  // descale in two exact steps (the first cannot leave the normal range)
     const float d1 = pow2f(da), d2 = pow2f(db);
@@ -227,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, (AMAX && MODE == HIF8_RND_TA) || (FQ
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (p.d_scale_exp_out) *p.d_scale_exp_out = se;
         if (p.d_scale_out) *p.d_scale_out = scale;
-        if (!AMAX && p.d_amax_out && p.d_amax_bits && !p.amax_slots) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
+        if (!AMAX && !SLOTS && p.d_amax_out && p.d_amax_bits) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
     }
     if (AMAX) {
         block_amax_commit(amax, p.amax_accum);
@@ -401,8 +404,10 @@ __device__ __noinline__ uint32_t fq_rare(uint32_t raw, int se, unsigned flags, u
 // the element's own power of two and the element's sign.  The sum lies in the binade of C, whose spacing is the HiF8
 // spacing of the element's binade (2^-22 over the scale below the format's range), so the hardware's round-to-nearest-even
 // does the rounding, ties to the even kept significand (the implicit one counts), and x - x = +0 gives the single zero.
-template <int SRC, int MODE>
-__global__ void __launch_bounds__(kThreads) fq_ta_kernel(const ConvParams p, unsigned long long n_vec)
+// (Five blocks an SM for FP32 after amax_slots_kernel: with the 40 registers that the compiler takes there, six, a call on 1.4 M elements takes 7.2 us and on
+// 2 M 7.9, so 6.8 and 7.5.)
+template <int SRC, int MODE, bool SLOTS>
+__global__ void __launch_bounds__(kThreads, SLOTS && SRC == HIF8_F32 ? 5 : 0) fq_ta_kernel(const ConvParams p, unsigned long long n_vec)
 {
     static_assert(MODE == HIF8_RND_TA || SRC == HIF8_BF16, "threshold modes and round half to even are done in place for BF16 only");
     constexpr int MB = SRC == HIF8_F32 ? 23 : 7;      // mantissa bits of the source format
@@ -412,7 +417,7 @@ __global__ void __launch_bounds__(kThreads) fq_ta_kernel(const ConvParams p, uns
     __shared__ uint32_t s_mask[(SRC == HIF8_F32 || kThr) ? 256 : 1];  // threshold modes: the LSB term's factor
     pdl_launch_dependents();
     pdl_wait_prior_grid();  // the scale may come from the previous kernel
-    const int se = resolve_scale_exp(p);
+    const int se = resolve_scale_exp<SLOTS>(p);
     {
         const int e = threadIdx.x, E = e - 127 + se;
         uint32_t inc = 0, mask = 0, kfac = 0;
@@ -575,7 +580,7 @@ __global__ void __launch_bounds__(kThreads) fq_ta_kernel(const ConvParams p, uns
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (p.d_scale_exp_out) *p.d_scale_exp_out = se;
         if (p.d_scale_out) *p.d_scale_out = pow2f(se);
-        if (p.d_amax_out && p.d_amax_bits && !p.amax_slots) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
+        if (!SLOTS && p.d_amax_out && p.d_amax_bits) *p.d_amax_out = __uint_as_float(*p.d_amax_bits);
     }
 }
 
@@ -889,7 +894,10 @@ int launch_convert(const ConvParams& p, bool vec_ok, int sms, cudaStream_t st)
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     unsigned long long n_vec = vec_ok ? p.n / PV : 0;
     const unsigned grid = convert_grid(n_vec, p.n, sms, SRC, MODE, FQ, AMAX, false, p.reverse != 0);
-    launch_pdl(convert_kernel<SRC, MODE, FQ, AMAX>, grid, st, p, n_vec);
+    if constexpr (!AMAX && MODE != HIF8_RND_SR) {
+        if (p.amax_slots) launch_pdl(convert_kernel<SRC, MODE, FQ, AMAX, false, true>, grid, st, p, n_vec);
+        else launch_pdl(convert_kernel<SRC, MODE, FQ, AMAX>, grid, st, p, n_vec);
+    } else launch_pdl(convert_kernel<SRC, MODE, FQ, AMAX>, grid, st, p, n_vec);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
 }
@@ -995,17 +1003,26 @@ int dispatch_one(int dtype, int rnd, const ConvParams& p, int dev, cudaStream_t 
     }
 }
 
+template <int SRC, int MODE>
+void launch_fq_ta_form(unsigned grid, const ConvParams& p, unsigned long long n_vec, cudaStream_t st)
+{
+    if constexpr (MODE != HIF8_RND_SR) {
+        if (p.amax_slots) { launch_pdl(fq_ta_kernel<SRC, MODE, true>, grid, st, p, n_vec); return; }
+    }
+    launch_pdl(fq_ta_kernel<SRC, MODE, false>, grid, st, p, n_vec);
+}
+
 int launch_fq_ta(int dtype, int rnd, const ConvParams& p, bool vec_ok, int sms, cudaStream_t st)
 {
     const unsigned long long pv = dtype == HIF8_F32 ? 4 : 8;
     const unsigned long long n_vec = vec_ok ? p.n / pv : 0;
     const unsigned grid = convert_grid(n_vec, p.n, sms, dtype, rnd, true, false, true, p.reverse != 0);
-    if (dtype == HIF8_F32) launch_pdl(fq_ta_kernel<HIF8_F32, HIF8_RND_TA>, grid, st, p, n_vec);
-    else if (rnd == HIF8_RND_TA) launch_pdl(fq_ta_kernel<HIF8_BF16, HIF8_RND_TA>, grid, st, p, n_vec);
-    else if (rnd == HIF8_RND_HR) launch_pdl(fq_ta_kernel<HIF8_BF16, HIF8_RND_HR>, grid, st, p, n_vec);
-    else if (rnd == HIF8_RND_TE) launch_pdl(fq_ta_kernel<HIF8_BF16, HIF8_RND_TE>, grid, st, p, n_vec);
-    else if (rnd == HIF8_RND_SR) launch_pdl(fq_ta_kernel<HIF8_BF16, HIF8_RND_SR>, grid, st, p, n_vec);
-    else launch_pdl(fq_ta_kernel<HIF8_BF16, HIF8_RND_SSR>, grid, st, p, n_vec);
+    if (dtype == HIF8_F32) launch_fq_ta_form<HIF8_F32, HIF8_RND_TA>(grid, p, n_vec, st);
+    else if (rnd == HIF8_RND_TA) launch_fq_ta_form<HIF8_BF16, HIF8_RND_TA>(grid, p, n_vec, st);
+    else if (rnd == HIF8_RND_HR) launch_fq_ta_form<HIF8_BF16, HIF8_RND_HR>(grid, p, n_vec, st);
+    else if (rnd == HIF8_RND_TE) launch_fq_ta_form<HIF8_BF16, HIF8_RND_TE>(grid, p, n_vec, st);
+    else if (rnd == HIF8_RND_SR) launch_fq_ta_form<HIF8_BF16, HIF8_RND_SR>(grid, p, n_vec, st);
+    else launch_fq_ta_form<HIF8_BF16, HIF8_RND_SSR>(grid, p, n_vec, st);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
 }
