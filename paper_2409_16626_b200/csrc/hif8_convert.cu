@@ -191,11 +191,13 @@ convert_kernel(const ConvParams p, unsigned long long n_vec)
 {
     static_assert(!PATTERN || (SRC == HIF8_F32 && !FQ && !AMAX), "generated sources are FP32 patterns, encode only");
     __shared__ SmemTables sm;
-    pdl_launch_dependents();
+    constexpr unsigned kFewBlocks = MODE == HIF8_RND_TA && !FQ ? 64 : 16;  // (see pdl_launch_dependents)
+    if (AMAX || gridDim.x <= kFewBlocks) pdl_launch_dependents();
     constexpr bool kPair16 = SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ;
     if (kPair16) setup_sum16<MODE>(sm.ta, sm.thr, p.flags);
     else setup_tables<true, MODE != HIF8_RND_TA, FQ, MODE, SRC>(sm, p.flags);  // reads only the constant table
     pdl_wait_prior_grid();
+    pdl_launch_dependents();  // (a second time: nothing)
     const int se = resolve_scale_exp<SLOTS>(p);
     const float scale = pow2f(se);
     const int da = (-se) / 2, db = -se - da;  // descale in two exact steps (the first cannot leave the normal range)
@@ -274,9 +276,9 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     constexpr bool kPair16 = SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ;
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this block has started (waited for before the first remote store)
-    pdl_launch_dependents();
     const unsigned first = blockIdx.x * kOneThreads + threadIdx.x, step = gridDim.x * kOneThreads;  // vectors first, first + step, ..
     pdl_wait_prior_grid();
+    pdl_launch_dependents();
     const uint4* src = reinterpret_cast<const uint4*>(p.src);
     const uint32_t s_mine = (uint32_t)__cvta_generic_to_shared(s_src + threadIdx.x);
 #pragma unroll 4
@@ -415,8 +417,8 @@ __global__ void __launch_bounds__(kThreads, SLOTS && SRC == HIF8_F32 ? 5 : 0) fq
     constexpr bool kThr = MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR;  // packed BF16 arithmetic with an LSB term
     __shared__ uint32_t s_inc[256];                   // BF16: mask16 | inc16 << 16 (threshold modes: mask16 | addend << 16)
     __shared__ uint32_t s_mask[(SRC == HIF8_F32 || kThr) ? 256 : 1];  // threshold modes: the LSB term's factor
-    pdl_launch_dependents();
     pdl_wait_prior_grid();  // the scale may come from the previous kernel
+    pdl_launch_dependents();
     const int se = resolve_scale_exp<SLOTS>(p);
     {
         const int e = threadIdx.x, E = e - 127 + se;
@@ -621,8 +623,8 @@ __global__ void __launch_bounds__(kSlotThreads) amax_slots_kernel(const void* __
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     __shared__ uint32_t s_part[kSlotThreads / 32], s_block[kSlotCluster];
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this block has started (waited for before the first remote store)
-    pdl_launch_dependents();
     pdl_wait_prior_grid();
+    pdl_launch_dependents();
     const uint4* src = reinterpret_cast<const uint4*>(srcv);
     uint32_t acc = 0u;
     uint4 v[kUnrollAmax];
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(kSlotThreads) amax_slots_kernel(const void* __
     }
 }
 
-template <int SRC, bool STREAM>
+template <int SRC, bool STREAM, bool ALONE>
 __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__ srcv, unsigned long long n,
                                                         unsigned long long n_vec, uint32_t* accum, float* d_amax_out)
 {
@@ -669,8 +671,9 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__
     const uint4* src = reinterpret_cast<const uint4*>(srcv);
     float amax = 0.f;
     uint32_t acc = 0u;
-    pdl_launch_dependents();
+    if (ALONE) pdl_launch_dependents();
     pdl_wait_prior_grid();
+    if (!ALONE) pdl_launch_dependents();
     const unsigned long long stride = (unsigned long long)gridDim.x * kThreads * kUnrollAmax;
     for (unsigned long long base = (unsigned long long)blockIdx.x * kThreads * kUnrollAmax; base < n_vec; base += stride) {
         uint4 v[kUnrollAmax];
@@ -691,7 +694,7 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__
         amax = amax_step(amax, x);
     }
     block_amax_commit(amax, accum);
-    if (d_amax_out && threadIdx.x == 0) {  // stand-alone amax: the last block to finish publishes the result
+    if (ALONE && threadIdx.x == 0) {  // the last block to finish publishes the result
         __threadfence();
         if (atomicAdd(accum + 1, 1u) == gridDim.x - 1) {
             __threadfence();
@@ -1027,6 +1030,13 @@ int launch_fq_ta(int dtype, int rnd, const ConvParams& p, bool vec_ok, int sms, 
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;
 }
 
+template <int SRC>
+void launch_amax_form(bool stream, unsigned grid, cudaStream_t st, const void* src, unsigned long long n, unsigned long long n_vec, uint32_t* accum, float* d_amax_out)
+{
+    if (d_amax_out) launch_pdl(stream ? amax_kernel<SRC, true, true> : amax_kernel<SRC, false, true>, grid, st, src, n, n_vec, accum, d_amax_out);
+    else launch_pdl(stream ? amax_kernel<SRC, true, false> : amax_kernel<SRC, false, false>, grid, st, src, n, n_vec, accum, d_amax_out);
+}
+
 int launch_amax(const void* src, int dtype, unsigned long long n, uint32_t* accum, float* d_amax_out, int sms, cudaStream_t st)
 {
     bool vec_ok = aligned16(src);
@@ -1038,9 +1048,9 @@ int launch_amax(const void* src, int dtype, unsigned long long n, uint32_t* accu
     // there is no ticket, and a block for every 32 KiB is 2 to 4 % faster.
     if (d_amax_out) grid = std::min(grid, 2u * sms * kBlocksPerSM);
     switch (dtype) {
-        case HIF8_F32: launch_pdl(n_vec > kStreamVecsF32 ? amax_kernel<HIF8_F32, true> : amax_kernel<HIF8_F32, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
-        case HIF8_BF16: launch_pdl(n_vec > kKeepVecs ? amax_kernel<HIF8_BF16, true> : amax_kernel<HIF8_BF16, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
-        default: launch_pdl(n_vec > kKeepVecs ? amax_kernel<HIF8_F16, true> : amax_kernel<HIF8_F16, false>, grid, st, src, n, n_vec, accum, d_amax_out); break;
+        case HIF8_F32: launch_amax_form<HIF8_F32>(n_vec > kStreamVecsF32, grid, st, src, n, n_vec, accum, d_amax_out); break;
+        case HIF8_BF16: launch_amax_form<HIF8_BF16>(n_vec > kKeepVecs, grid, st, src, n, n_vec, accum, d_amax_out); break;
+        default: launch_amax_form<HIF8_F16>(n_vec > kKeepVecs, grid, st, src, n, n_vec, accum, d_amax_out); break;
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HIF8_OK : HIF8_ERR_CUDA;

@@ -520,3 +520,45 @@ def test_conversions_whatever_the_number_of_blocks(groups, dtype, rnd):
     H.hif8_amax_scale_encode(x, dtype, out[guard:], n, 14, rnd, 0, 0, exp, amax, None, None, ws, 256)  # encodes with the exponent and measures
     check(out, codes)
     assert float(amax) == 77.0
+
+
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
+def test_scaled_conversions_in_flight_together_share_a_workspace(dtype):
+    # Calls of all launch forms one behind the other in a stream, with one workspace and no wait in between: every result is the one the
+    # call gives by itself.
+    t = {H.F32: torch.float32, H.BF16: torch.bfloat16, H.F16: torch.float16}[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(int(dtype) + 1)
+    ws, wsb = workspace()
+    calls = []
+    for i, n in enumerate([700, 9000, 1_300_001, 150_000, 2_100_000, 2_100_000, 500_003, 40_000, 4_000_000, 1_000_000, 6_500_000, 80_000, 3_000_003, 1_700_000]):
+        x = (torch.randn(n + 1, generator=gen, device="cuda") * 2.0 ** (i % 7 - 3)).to(t)
+        x[n // 2] = 3.0 * 2.0 ** (i % 9)  # every call has another scale
+        src = x[1:] if i == 4 else x[:n]  # (off its alignment: the general path)
+        rnd = [H.RND_TA, H.RND_HR, H.RND_SSR, H.RND_TE, H.RND_SR][i % 5]
+        calls.append((src, n, rnd, i % 3 == 2, torch.empty(n, dtype=t, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda"),
+                      torch.zeros(1, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")))
+
+    def run(c):
+        src, n, rnd, fq, values, codes, amax, exp = c
+        if fq:
+            assert H.hif8_fake_quant(src, values, dtype, n, 1, 14, rnd, 0, 5, amax, exp, ws, wsb) == 0
+        else:
+            assert H.hif8_amax_scale_encode(src, dtype, codes, n, 14, rnd, 0, 5, None, amax, exp, None, ws, wsb) == 0
+        return (values if fq else codes), amax, exp
+
+    alone = []
+    for c in calls:
+        out = run(c)
+        torch.cuda.synchronize()
+        alone.append([o.view(torch.uint8).clone() for o in out])
+    for order in (range(len(calls)), reversed(range(len(calls)))):
+        for c in calls:
+            for o in c[4:]:
+                o.zero_()
+        torch.cuda.synchronize()
+        order = list(order)
+        outs = {i: run(calls[i]) for i in order}
+        torch.cuda.synchronize()
+        for i in order:
+            for got, want in zip(outs[i], alone[i]):
+                assert torch.equal(got.view(torch.uint8), want), (i, calls[i][1:4])
