@@ -287,8 +287,8 @@ __global__ void __launch_bounds__(kThreads) col_amax_kernel(const ChanParams p, 
             }
 #pragma unroll
             for (int j = 0; j < kUnroll; j++) {
-                m[0] = amax_word<SRC>(m[0], v[j].x); m[1] = amax_word<SRC>(m[1], v[j].y);
-                m[2] = amax_word<SRC>(m[2], v[j].z); m[3] = amax_word<SRC>(m[3], v[j].w);
+                m[0] = amax_word<SRC, true>(m[0], v[j].x); m[1] = amax_word<SRC, true>(m[1], v[j].y);
+                m[2] = amax_word<SRC, true>(m[2], v[j].z); m[3] = amax_word<SRC, true>(m[3], v[j].w);
             }
         }
     }

@@ -284,3 +284,27 @@ def test_delayed_scale_argument_checks():
     assert H.hif8_delayed_scale_encode(x, H.F32, out, 8, H.RND_TA, 0, 0, None, 1, check=False) == 1
     assert H.hif8_delayed_scale_encode(x, H.F32, out, 8, H.RND_TA, 0, 0, aligned, 1, target_exp=16, check=False) == 5
     assert H.hif8_delayed_scale_encode(x, H.F32, out, 0, H.RND_TA, 0, 0, aligned, 1) == 0
+
+
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("shape", [(33, 40), (300, 1032), (1025, 264)])
+def test_channel_amax_of_negative_values_beside_infinities_and_nan(shape, axis, dtype):
+    # 16-bit maxima run in packed words, two elements each, with or without their signs: every channel's largest magnitude is a
+    # negative value, neighbours in a word have Inf, NaN of either sign, or nothing but zeros.
+    f = np.random.default_rng(5).uniform(-1, 1, size=shape).astype(np.float32)
+    x = f.view(np.uint32) if dtype == H.F32 else W.f32_to_bf16_bits(f) if dtype == H.BF16 else f.astype(np.float16).view(np.uint16)
+    one, inf, sign = {H.F32: (0x3F800000, 0x7F800000, 1 << 31), H.BF16: (0x3F80, 0x7F80, 1 << 15), H.F16: (0x3C00, 0x7C00, 1 << 15)}[dtype]
+    step = {H.F32: 1 << 23, H.BF16: 1 << 7, H.F16: 1 << 10}[dtype]
+    v = (x if axis == 0 else x.T)
+    for c in range(v.shape[0]):
+        v[c, c % v.shape[1]] = sign | (one + (3 + c % 8) * step)  # -8 .. -1024
+        v[c, (c + 5) % v.shape[1]] = (inf, sign | inf, inf + 1, sign | (inf + 1))[c % 4]
+        if c % 16 == 7:
+            v[c] = (0, sign, inf, sign | inf)[c // 16 % 4]
+    x = x.view(np.float32) if dtype == H.F32 else x
+    q, amax, se = run_channel(x, dtype, axis)
+    amax_o, se_o = O.channel_amax_scale(x, dtype, axis, 14)
+    assert np.array_equal(amax, amax_o) and np.array_equal(se, se_o)
+    assert amax[1] == 16.0 and amax[7] == 0.0
+    assert np.array_equal(q, O.channel_encode(x, dtype, axis, se_o, quick=True))
