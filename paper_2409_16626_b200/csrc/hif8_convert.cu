@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     constexpr bool kPair16 = SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ;
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this block has started (waited for before the first remote store)
+    if (gridDim.x == 1) pdl_launch_dependents();  // (see there: few blocks; up to 8 K BF16 elements 2.38 us, behind the wait 2.48)
     const unsigned first = blockIdx.x * kOneThreads + threadIdx.x, step = gridDim.x * kOneThreads;  // vectors first, first + step, ..
     pdl_wait_prior_grid();
     pdl_launch_dependents();
