@@ -261,10 +261,12 @@ convert_kernel(const ConvParams p, unsigned long long n_vec)
 // first of which completes under the loads and the table set-up), and converts from there.  No accumulator in the workspace,
 // so nothing to clear.  Latency and launches bound it: from the host one launch takes 3.5 us, two (amax, convert) 5.3 and three 8.  It ends
 // where sixteen SMs take longer than the launches over all of them, which depends on the arithmetic an element carries (one_launch_limit).
-// All copies of a block are asynchronous and in flight together, up to 128 KiB.
+// All copies of a block are asynchronous and in flight together, up to 88 KiB.
+// A cluster of sixteen wants sixteen SMs of one GPC with room at the same time.  Beside another stream's work it still is the faster form (us a call, three launches / this, in
+// the time that stream was busy: 300 K BF16 elements beside products of 4096 x 8192 x 8192, whose blocks fill their SMs, 51 / 31, beside fake-quant of 2^26 elements 60 / 44).
 // ------------------------------------------------------------------------------------------------
 constexpr int kOneThreads = 512, kOneBlocks = 16, kOneBlocksPortable = 8;
-constexpr unsigned kOneSmem = 128 * 1024, kOneSmemDefault = 32 * 1024;  // source bytes per block: with the opt-in, and without
+constexpr unsigned kOneSmem = 88 * 1024, kOneSmemDefault = 32 * 1024;  // source bytes per block: with the opt-in (what one_launch_limit needs), and without
 static_assert(sizeof(SmemTables) + kOneSmemDefault + 256 <= 48 * 1024, "no opt-in to more shared memory for the smaller form");
 
 template <int SRC, int MODE, bool FQ>
@@ -940,8 +942,8 @@ constexpr unsigned one_launch_limit(int src, int mode, bool fq)
     if (mode == HIF8_RND_TA) return src == HIF8_F32 ? 11u << 15 : 1u << 19;
     return 1u << 18;
 }
-static_assert(one_launch_limit(HIF8_F32, HIF8_RND_TA, false) / 4 <= kOneBlocks * kOneSmem / 16 && one_launch_limit(HIF8_BF16, HIF8_RND_TA, false) / 8 <= kOneBlocks * kOneSmem / 16,
-              "sixteen blocks hold it");
+static_assert(one_launch_limit(HIF8_F32, HIF8_RND_TA, false) * 4 == kOneBlocks * kOneSmem && one_launch_limit(HIF8_BF16, HIF8_RND_TA, false) * 2 <= kOneBlocks * kOneSmem,
+              "sixteen blocks hold the largest, with nothing to spare");
 constexpr int kNotTaken = -1;
 
 template <int SRC, int MODE, bool FQ>
@@ -961,7 +963,7 @@ int launch_one(const ConvParams& p, int dev, cudaStream_t st)
     attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    // sixteen blocks of up to 128 KiB where the device can hold such a cluster, else eight of 32 KiB, which every device can
+    // sixteen blocks of up to 88 KiB where the device can hold such a cluster, else eight of 32 KiB, which every device can
     const Setup* s = setup.get(dev, [&](int, Setup* out) {
         *out = Setup{kOneBlocksPortable, kOneSmemDefault};
         int clusters = 0;

@@ -562,3 +562,28 @@ def test_scaled_conversions_in_flight_together_share_a_workspace(dtype):
         for i in order:
             for got, want in zip(outs[i], alone[i]):
                 assert torch.equal(got.view(torch.uint8), want), (i, calls[i][1:4])
+
+
+def test_one_launch_form_beside_the_work_of_another_stream():
+    # The cluster of a just-in-time call waits for room of its own: it gets it, and its results, while another stream keeps the device busy.
+    n = 11 << 15  # the largest the form takes: sixteen blocks of all the shared memory it asks for
+    x = torch.randn(n, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+    x[n - 2] = -96.0
+    big = torch.randn(1 << 25, device="cuda")
+    junk = torch.empty_like(big)
+    ws, wsb = workspace()
+    codes = torch.empty(n, dtype=torch.uint8, device="cuda")
+    outs = [(torch.empty(n, dtype=torch.uint8, device="cuda"), torch.zeros(1, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")) for _ in range(20)]
+    H.hif8_encode(x, H.F32, codes, n, 14 - 6)
+    busy = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    before = H.hif8_launch_count()
+    for _ in range(40):
+        H.hif8_fake_quant(big, junk, H.F32, big.numel(), 0, 3, H.RND_HR, stream=busy)
+    between = H.hif8_launch_count()
+    for out, amax, exp in outs:
+        H.hif8_amax_scale_encode(x, H.F32, out, n, 14, H.RND_TA, 0, 0, None, amax, exp, None, ws, wsb)
+    assert between - before == 40 and H.hif8_launch_count() - between == 20  # one launch a call
+    torch.cuda.synchronize()
+    for out, amax, exp in outs:
+        assert torch.equal(out, codes) and float(amax) == 96.0 and int(exp) == 8
