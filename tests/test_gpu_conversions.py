@@ -264,7 +264,7 @@ def test_scaled_conversions_at_the_limits_of_the_launch_forms(dtype, fq, mode):
     one = (1 << 17) if mode == H.RND_SR else (3 << 16) if fq else (1 << 18) if mode != H.RND_TA else (11 << 15) if dtype == H.F32 else (1 << 19)
     two = (24 << 20) // (4 if dtype == H.F32 else 2)
     cluster = 32768 * pv
-    sizes = [one, one + 1, 9 * cluster + pv - 1, 18 * cluster, 18 * cluster + 1, two + pv - 1, two + pv]
+    sizes = [one, one + 1, 9 * cluster + pv - 1, 18 * cluster, 18 * cluster + pv, two + pv - 1, two + pv]  # (from 19 clusters on they are not doubled)
     ws, wsb = workspace()
     outs = torch.zeros(4, dtype=torch.int32, device="cuda")
     np_t = {H.F32: np.float32, H.BF16: np.uint16, H.F16: np.float16}[dtype]
@@ -587,3 +587,73 @@ def test_one_launch_form_beside_the_work_of_another_stream():
     torch.cuda.synchronize()
     for out, amax, exp in outs:
         assert torch.equal(out, codes) and float(amax) == 96.0 and int(exp) == 8
+
+
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
+@pytest.mark.parametrize("n", [600_003, 2_600_005])
+def test_scaled_conversions_of_middle_sizes_with_specials_in_place_and_misaligned(n, dtype):
+    # The two-launch form: the largest magnitude is negative, beside Inf and NaN of either sign, which do not count; fake-quant into its own source;
+    # and a destination off its alignment, where a conversion element by element reads the words that the amax launch left.
+    sign, inf = {H.F32: (1 << 31, 0x7F800000), H.BF16: (1 << 15, 0x7F80), H.F16: (1 << 15, 0x7C00)}[dtype]
+    np_t = {H.F32: np.float32, H.F16: np.float16}.get(dtype)
+    src = W.normal_bf16(n, seed=4) if dtype == H.BF16 else W.normal_f32(n, seed=4).astype(np_t).view(NP_OF[dtype])
+    src = src.view(NP_OF[dtype]).copy()
+    src[n // 3] = sign | {H.F32: 0x42F00000, H.BF16: 0x42F0, H.F16: 0x5780}[dtype]  # -120
+    src[[5, n // 2, n - 1, 77]] = inf, sign | inf, inf + 1, sign | (inf + 1)
+    amax, se = O.amax_scale(src, dtype, 14)
+    assert amax == 120.0
+    ws, wsb = workspace()
+    outs = torch.zeros(4, dtype=torch.int32, device="cuda")
+    for rnd in (H.RND_TA, H.RND_HR):
+        for offset in (0, 1):
+            outs.zero_()
+            _, dptr, rb = dev_empty(n, np.uint8, offset)
+            assert H.hif8_amax_scale_encode(to_dev(src), dtype, dptr, n, 14, rnd, 0, 0, None, outs[0:1], outs[1:2], outs[2:3], ws, wsb) == 0
+            torch.cuda.synchronize()
+            assert_same(rb(), O.encode(src, dtype, se, rnd, 0, quick=True), src)
+            assert outs[0:1].view(torch.float32).item() == 120.0 and outs[1].item() == se
+        buf = to_dev(src)
+        assert H.hif8_fake_quant(buf, buf, dtype, n, 1, 14, rnd, 0, 0, outs[0:1], outs[1:2], ws, wsb) == 0
+        torch.cuda.synchronize()
+        assert_same(buf.cpu().numpy().view(NP_OF[dtype]), O.fake_quant(src, dtype, se, rnd, 0, quick=True), src)
+
+
+@pytest.mark.parametrize("rnd", [H.RND_SSR, H.RND_SR])
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
+@pytest.mark.parametrize("groups", [1184, 1185, 2 * 1184 + 7, 3 * 1184 + 1, 10 * 1184 - 5, 14 * 1184])
+def test_stochastic_conversions_whatever_the_number_of_blocks(groups, dtype, rnd):
+    # Random words belong to elements, whichever block converts them: all codes and values are those of the element-by-element path, which a source
+    # and destination off their alignment take.
+    pv = 4 if dtype == H.F32 else 8
+    n = groups * 1024 * pv - 3
+    t = {H.F32: torch.float32, H.BF16: torch.bfloat16, H.F16: torch.float16}[dtype]
+    shifted = torch.empty(n + 1, dtype=t, device="cuda")
+    x = (torch.randn(n, generator=torch.Generator(device="cuda").manual_seed(groups), device="cuda") * 3).to(t)
+    x[54321] = -77.0
+    shifted[1:] = x
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    amax, exp = torch.zeros(1, device="cuda"), torch.full((1,), 8, dtype=torch.int32, device="cuda")
+    state = torch.empty(H.SCALE_STATE_BYTES, dtype=torch.uint8, device="cuda")
+    want_codes, want = torch.empty(n + 1, dtype=torch.uint8, device="cuda"), torch.empty(n + 1, dtype=t, device="cuda")
+    H.hif8_encode(shifted[1:], dtype, want_codes[1:], n, 8, rnd, 0, 11)
+    H.hif8_fake_quant(shifted[1:], want[1:], dtype, n, 0, 8, rnd, 0, 11)
+    for call in ("encode", "jit", "measure", "delayed"):
+        codes = torch.zeros(n, dtype=torch.uint8, device="cuda")
+        amax.zero_()
+        if call == "encode":
+            H.hif8_encode(x, dtype, codes, n, 8, rnd, 0, 11)
+        elif call == "jit":
+            H.hif8_amax_scale_encode(x, dtype, codes, n, 14, rnd, 0, 11, None, amax, None, None, ws, 256)
+        elif call == "measure":
+            H.hif8_amax_scale_encode(x, dtype, codes, n, 14, rnd, 0, 11, exp, amax, None, None, ws, 256)
+        else:
+            H.hif8_scale_state_init(state, 1)
+            H.hif8_delayed_scale_encode(x, dtype, codes, n, rnd, 0, 11, state, 1)  # measures: exponent 8 from the next call on
+            H.hif8_delayed_scale_encode(x, dtype, codes, n, rnd, 0, 11, state, 0)
+            assert int(state[:4].view(torch.int32)) == 8
+        assert torch.equal(codes, want_codes[1:])
+        assert call in ("encode", "delayed") or float(amax) == 77.0
+    for use_amax in (0, 1):
+        back = torch.zeros(n, dtype=t, device="cuda")
+        H.hif8_fake_quant(x, back, dtype, n, use_amax, 14 if use_amax else 8, rnd, 0, 11, None, None, ws, 256)
+        assert torch.equal(back.view(torch.uint8), want[1:].clone().view(torch.uint8))
