@@ -406,7 +406,7 @@ def test_gemm_weights_decoded_in_the_kernel(shape, form, w_is_nk, c_dtype, accum
 @pytest.mark.parametrize("staged", ["a", False])
 @pytest.mark.parametrize("shape", [(2320, 1300, 144), (2064, 4100, 304), (4096, 1300, 4096), (4112, 1300, 144), (2320, 1300, 4112)])
 def test_gemm_rows_in_more_than_eight_pieces(shape, staged, w_is_nk):
-    # Nine to sixteen pieces of activation rows as one group, seventeen and a K above 4096 in groups of eight.
+    # Nine and eleven pieces of activation rows as one group; sixteen with a launch for the last round, seventeen, and a K above 4096 in groups of eight.
     M, N, K = shape
     N = (N + 15) // 16 * 16 if not w_is_nk else N
     Aq, Wkn = W.random_codes((M, K), seed=M + K), W.random_codes((K, N), seed=N + K + 1)
@@ -458,3 +458,43 @@ def test_gemm_narrow_splits(shape, staged, w_is_nk, c_dtype, accumulate):
     if c_dtype == H.BF16:
         tol = tol + bf16_half_ulp(np.abs(want) + tol)
     assert np.all(np.abs(out[rows, cols] - want) <= tol)
+
+
+@pytest.mark.parametrize("accumulate", [0, 1])
+@pytest.mark.parametrize("w_is_nk", [0, 1])
+@pytest.mark.parametrize("staged", ["a", False])
+def test_gemm_sixteen_pieces_of_rows_in_a_single_launch(staged, w_is_nk, accumulate):
+    # Sixteen pieces at K = 4096 on 64 of 74 pairs, no launch for a last round: as one group, and in groups of eight where C is added to.
+    M, N, K = 4090, 1024, 4096
+    Aq, Wkn = W.random_codes((M, K), seed=1), W.random_codes((K, N), seed=2)
+    for t in (Aq, Wkn):
+        t[(t == 0x80) | ((t & 0x7F) == 0x6F)] = 0x33
+    Wq = np.ascontiguousarray(Wkn.T) if w_is_nk else Wkn
+    rng = np.random.default_rng(M)
+    c0 = (rng.standard_normal((M, N)) * 50).astype(np.float32)
+    C = torch.from_numpy(c0.copy()).cuda()
+    wsb = gemm_workspace_bytes(staged, M, N, K)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    before = H.hif8_launch_count()
+    with gemm_path(POLICY[staged]):
+        H.hif8_gemm_ex(to_dev(Aq), K, 0, to_dev(Wq), Wq.shape[1], w_is_nk, C, N, H.F32, M, N, K, torch.tensor([3], dtype=torch.int32, device="cuda"),
+                       torch.tensor([-4], dtype=torch.int32, device="cuda"), None, accumulate, ws, wsb)
+    assert H.hif8_gemm_status(ws) == 0 and H.hif8_launch_count() - before == (2 if staged == "a" else 1)
+    rows = np.concatenate([rng.integers(0, M, 20000), np.arange(M), np.full(N, M - 1)])
+    cols = np.concatenate([rng.integers(0, N, 20000), np.arange(M) % N, np.arange(N)])
+    P, S = O.gemm_entries(Aq, Wkn, False, 3, -4, rows, cols)
+    want = P + c0[rows, cols] if accumulate else P
+    assert np.all(np.abs(C.cpu().numpy().astype(np.float64)[rows, cols] - want) <= 1e-5 * S + 2.0 ** -24 * np.abs(want))
+
+
+@pytest.mark.parametrize("w_is_nk", [0, 1])
+@pytest.mark.parametrize("shape", [(4370, 528, 80), (8200, 272, 16)])
+def test_gemm_pair_kernel_more_than_sixteen_tile_rows(shape, w_is_nk):
+    # Tile-rows of the pair kernel go in groups of sixteen up to K = 4096: two and three groups, the last one short.
+    M, N, K = shape
+    Aq, Wkn = W.random_codes((M, K), seed=M), W.random_codes((K, N), seed=N)
+    for t in (Aq, Wkn):
+        t[(t == 0x80) | ((t & 0x7F) == 0x6F)] = 0x33
+    out = run_gemm(Aq, np.ascontiguousarray(Wkn.T) if w_is_nk else Wkn, w_is_nk, H.F32, sa=3, sw=-4, staged=True)
+    P, S = O.gemm_entries(Aq, Wkn, False, 3, -4, np.repeat(np.arange(M), N), np.tile(np.arange(N), M))
+    assert np.all(np.abs(out.reshape(-1) - P) <= 1e-5 * S + 2.0 ** -24 * np.abs(P))
