@@ -190,6 +190,7 @@ __global__ void __launch_bounds__(kThreads, FQ && !SLOTS && ((SRC == HIF8_F32 &&
 convert_kernel(const ConvParams p, unsigned long long n_vec)
 {
     static_assert(!PATTERN || (SRC == HIF8_F32 && !FQ && !AMAX), "generated sources are FP32 patterns, encode only");
+    static_assert(!(FQ && AMAX) && !(AMAX && SLOTS), "fake-quant measures in a launch of its own");
     __shared__ SmemTables sm;
     constexpr unsigned kFewBlocks = MODE == HIF8_RND_TA && !FQ ? 64 : 16;  // (see pdl_launch_dependents)
     if (AMAX || gridDim.x <= kFewBlocks) pdl_launch_dependents();
@@ -619,7 +620,6 @@ constexpr int kSlotThreads = 512, kSlotCluster = 8;
 constexpr unsigned kSlotVecs = kSlotThreads * kSlotCluster * kUnrollAmax;  // of a cluster
 constexpr unsigned kMaxSlots = 64;                                        // words of the workspace
 constexpr unsigned kSlotMaxVecs = (24u << 20) / 16;
-static_assert(kSlotMaxVecs <= kMaxSlots * kSlotVecs, "a word per cluster");
 template <int SRC>
 __global__ void __launch_bounds__(kSlotThreads) amax_slots_kernel(const void* __restrict__ srcv, unsigned long long n, unsigned n_vec, uint32_t* slots)
 {
@@ -859,7 +859,8 @@ unsigned grid_for(unsigned long long n_vec, unsigned long long n, int sms, int u
     return (unsigned)need;
 }
 
-// Blocks of a conversion.  A tensor is `need` groups of kUnroll vectors a thread, and `wave` blocks are resident at a time.  What a block pays once
+// Blocks of a conversion.  A tensor is `need` groups of kUnroll vectors a thread; `wave` is eight blocks an SM, what is resident of kernels of up to 32 registers
+// (fewer of others: in place 44 to 60 registers, five or four an SM, stochastic 37 to 53, six to four; the lines below are measured with them as they are).  What a block pays once
 // (tables, the exponent) weighs more the fewer groups it takes; but with several groups each, a last wave that is half empty costs as much as a full
 // one.  So arithmetic-bound conversions take whole waves of blocks, each with an equal share of the groups, and the ones bound
 // by memory take a group per block, which balances SMs near to and far from a memory partition.  (Up to four groups per block at all sizes / here, us:
@@ -912,7 +913,9 @@ template <int SRC, bool FQ, bool AMAX>
 int dispatch_mode(int rnd, const ConvParams& p, bool vec_ok, int sms, cudaStream_t st)
 {
     switch (rnd) {
-        case HIF8_RND_TA: return launch_convert<SRC, HIF8_RND_TA, FQ, AMAX>(p, vec_ok, sms, st);
+        case HIF8_RND_TA:
+            if constexpr (FQ && SRC == HIF8_F32) return HIF8_ERR_ROUND;  // (launch_fq_ta)
+            else return launch_convert<SRC, HIF8_RND_TA, FQ, AMAX>(p, vec_ok, sms, st);
         case HIF8_RND_HR: return launch_convert<SRC, HIF8_RND_HR, FQ, AMAX>(p, vec_ok, sms, st);
         case HIF8_RND_SSR: return launch_convert<SRC, HIF8_RND_SSR, FQ, AMAX>(p, vec_ok, sms, st);
         case HIF8_RND_TE: return launch_convert<SRC, HIF8_RND_TE, FQ, AMAX>(p, vec_ok, sms, st);
@@ -925,7 +928,9 @@ int dispatch_convert(int dtype, int rnd, const ConvParams& p, bool vec_ok, int s
 {
     switch (dtype) {
         case HIF8_F32: return dispatch_mode<HIF8_F32, FQ, AMAX>(rnd, p, vec_ok, sms, st);
-        case HIF8_BF16: return dispatch_mode<HIF8_BF16, FQ, AMAX>(rnd, p, vec_ok, sms, st);
+        case HIF8_BF16:
+            if constexpr (FQ) return HIF8_ERR_DTYPE;  // (launch_fq_ta)
+            else return dispatch_mode<HIF8_BF16, FQ, AMAX>(rnd, p, vec_ok, sms, st);
         default: return dispatch_mode<HIF8_F16, FQ, AMAX>(rnd, p, vec_ok, sms, st);
     }
 }
@@ -1091,6 +1096,7 @@ int check_common(int dtype, int rnd, unsigned flags)
 }
 
 constexpr size_t kConvWorkspaceBytes = 256;
+static_assert(kMaxSlots * sizeof(uint32_t) <= kConvWorkspaceBytes && kSlotMaxVecs <= kMaxSlots * kSlotVecs, "a word per cluster of the amax launch");
 
 }  // namespace
 
@@ -1183,7 +1189,7 @@ int hif8_decode(const uint8_t* src, void* dst, int dst_dtype, size_t n, int scal
     return decode_codes(src, dst, dst_dtype, n, scale_exp, kDecodeStreamFrom, (cudaStream_t)stream);
 }
 
-// shared by hif8_amax_scale_encode and hif8_fake_quant
+// shared by hif8_amax_scale_encode, hif8_delayed_scale_encode and hif8_fake_quant (which does not measure in passing: want_amax is false)
 static int scaled_convert(bool fq, const void* src, void* dst, int dtype, size_t n, bool jit, int target_exp,
                           const int* d_scale_exp_in, int scale_exp, int rnd, unsigned flags, uint64_t seed,
                           float* d_amax_out, int* d_scale_exp_out, float* d_scale_out, void* workspace,
@@ -1217,8 +1223,7 @@ static int scaled_convert(bool fq, const void* src, void* dst, int dtype, size_t
         }
     }
     p.scale_state = scale_state;
-    const bool inplace_fq = fq && !want_amax && ((rnd == HIF8_RND_TA && (dtype == HIF8_F32 || dtype == HIF8_BF16)) ||
-                                                ((rnd == HIF8_RND_HR || rnd == HIF8_RND_SSR || rnd == HIF8_RND_TE || rnd == HIF8_RND_SR) && dtype == HIF8_BF16));
+    const bool inplace_fq = fq && (dtype == HIF8_BF16 || (dtype == HIF8_F32 && rnd == HIF8_RND_TA));
     if (jit) {
         if (!p.amax_slots) {
             rc = launch_amax(src, dtype, n, ws, nullptr, sms, st);
@@ -1233,8 +1238,7 @@ static int scaled_convert(bool fq, const void* src, void* dst, int dtype, size_t
     if (inplace_fq) return launch_fq_ta(dtype, rnd, p, vec_ok, sms, st);
     if (want_amax) {
         p.amax_accum = ws;
-        return fq ? dispatch_convert<true, true>(dtype, rnd, p, vec_ok, sms, st)
-                  : dispatch_convert<false, true>(dtype, rnd, p, vec_ok, sms, st);
+        return dispatch_convert<false, true>(dtype, rnd, p, vec_ok, sms, st);
     }
     return fq ? dispatch_convert<true, false>(dtype, rnd, p, vec_ok, sms, st)
               : dispatch_convert<false, false>(dtype, rnd, p, vec_ok, sms, st);
@@ -1348,8 +1352,8 @@ uint64_t hif8_launch_count(void) { return g_launches.load(std::memory_order_rela
 
 // ------------------------------------------------------------------------------------------------
 // Variant of hif8_amax_scale_encode for callers that have no workspace to give.
-// The 8 bytes the amax reduction needs (running maximum + block ticket) live in a file-scope device array
-// that every device loading this library carries until the process exits.
+// What the amax reduction needs (a maximum and a ticket, or a word per cluster of the amax launch; nothing for small tensors) lives in a file-scope
+// device array that every device loading this library carries until the process exits.
 // ------------------------------------------------------------------------------------------------
 namespace {
 constexpr size_t kStaticScratchBytes = 256;
@@ -1389,7 +1393,7 @@ extern "C" int hif8_amax_scale_encode_static(const void* src, int src_dtype, uin
     rc = static_scratch(&scratch);
     if (rc) return rc;
     bool jit = d_scale_exp_in == nullptr;
-    // scaled_convert clears the two words that must start at zero before the first kernel reads them
+    // scaled_convert writes or clears every word before a kernel reads it
     return scaled_convert(false, src, dst, src_dtype, n, jit, target_exp, d_scale_exp_in, 0, rnd, flags, seed,
                           d_amax_out, d_scale_exp_out, d_scale_out, scratch, kStaticScratchBytes, !jit,
                           (cudaStream_t)stream);
