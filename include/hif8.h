@@ -107,7 +107,7 @@ int hif8_decode(const uint8_t* src, void* dst, int dst_dtype, size_t n, int scal
  *   d_scale_exp_in == NULL  (just-in-time):  amax = max |src[i]| over finite elements;
  *        scale_exp = clamp(target_exp - floor(log2 amax), -126, 126)  (0 if amax is 0), so that
  *        amax * 2^scale_exp lies in [2^target_exp, 2^(target_exp+1)); then dst = To_HiF8(src * 2^scale_exp).
- *        Two kernels, the scale never leaves the device.
+ *        One to three kernels, by size and alignment; the scale never leaves the device.
  *   d_scale_exp_in != NULL  (delayed scaling: Section 5.1 measures amax once per ten iterations): the scale exponent
  *        is read from that device int; amax of this tensor is still produced for the next update.  One pass.
  * Outputs (device scalars, each may be NULL): d_amax_out (float, exact), d_scale_exp_out (int, the exponent
@@ -159,8 +159,8 @@ int hif8_encode_from_amax(const void* src, int src_dtype, uint8_t* dst, size_t n
  *   - No cudaMalloc / cudaFree / allocating library routine is called, now or later.
  *   - The first call on each device looks up the array's device address (cudaGetSymbolAddress); make that
  *     first call outside any stream capture.
- *   - All calls on a device share the one array.  Each call clears the words it needs on `stream` before
- *     using them, so back-to-back calls on one stream are safe; two calls that can overlap on the GPU
+ *   - All calls on a device share the one array.  A call may overwrite all of it and writes what it reads there
+ *     itself first, on `stream`, so back-to-back calls on one stream are safe; two calls that can overlap on the GPU
  *     (different streams, no dependency) race on it and give wrong scales -- serialise them, or use
  *     hif8_amax_scale_encode with separate workspaces.
  */
@@ -239,7 +239,7 @@ int hif8_check_finite(const void* src, int dtype, size_t n, int* d_found_inf, hi
  * value with its nearest HiF8-representable one):   dst[i] = value( To_HiF8_<rnd>(src[i] * 2^e) ) * 2^(-e)   in `dtype`.
  *   use_amax == 0: e = scale_or_target_exp.  No workspace needed (may be NULL).
  *   use_amax == 1: e derived from the tensor's amax with target exponent scale_or_target_exp, as in
- *                  hif8_amax_scale_encode (two kernels); workspace as for HIF8_WS_FAKE_QUANT.
+ *                  hif8_amax_scale_encode (one to three kernels, by size); workspace as for HIF8_WS_FAKE_QUANT.
  * dst may be the same pointer as src (in place); any other overlap is rejected with HIF8_ERR_OVERLAP.
  * d_amax_out / d_scale_exp_out: optional device scalars as above.
  */

@@ -428,7 +428,7 @@ __device__ __forceinline__ uint4 decode8(uint2 v, uint32_t lut_lane)
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// Groups of `group` tile-rows sweep N together: their W tiles stay in L2 (8: kGroupPieces is the same number).
+// Groups of `group` tile-rows sweep N together: their W tiles stay in L2 (8 in the weights kernel, whose kGroupPieces is the same number; the pair kernel says its own).
 __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int& tile_m, int& tile_n, int group = 8)
 {
     const int per_group = group * tiles_n;
@@ -2462,7 +2462,8 @@ static int launch_weights_gemm(const uint8_t* Wq, int64_t ldw, int w_is_nk, cons
     if (rest.parts > 1 && (p.ldc * (p.c_is_f32 ? 4 : 2)) >> 32) rest = WeightsCost::Rest{};  // (rows of C 4 GiB apart have an instantiation for whole tiles)
     const int rem = (int)rest.tiles, clear = act != kActExpanded, slabs = tiles / tl.chunks;
     // Sixteen pieces of K up to 4096 stay in L2 as eight of more do, and the instantiation for one group has the cheaper tiles; the other has the
-    // cheaper sums.  4000 x 11008 x 1024 119.3 us, as one group 117.4; 3000 x 1024 x 1024 12.9 and 12.4; 2400 x 7168 x 4096 added to FP32 169.0 and 170.3.
+    // cheaper sums (us in groups / as one group, activations as bytes: 4000 x 11008 x 1024 119.9 / 118.4, 3072 x 1024 x 4096 36.0 / 34.4, 3000 x 1024 x 1024 13.3 / 13.0;
+    // added to FP32 171.1 / 172.4, 38.2 / 37.0 and 15.2 / 15.4, to BF16 162.1 / 190.8, 37.8 / 37.3 and 15.0 / 15.8).
     // (Not where a launch for the last round follows: both number the tiles in the same order, parts of tiles are numbered in groups, and which tiles
     // are divided along K, so how their sums are rounded, is as it is in groups.)
     const bool one_group = tl.chunks <= (K <= 4096 && !p.accumulate && rem == 0 ? 2 * kGroupPieces : kGroupPieces);
