@@ -220,7 +220,7 @@ def test_amax_scale_encode_jit_and_delayed(dtype):
 @pytest.mark.parametrize("dtype", [H.F32, H.BF16, H.F16])
 @pytest.mark.parametrize("mode", MODES)
 def test_scaled_conversions_of_small_tensors(dtype, mode):
-    """The one-launch form: no, one and several vectors per thread, 1 to 8 blocks, tails; its limit and the first size above;
+    """The one-launch form: no, one and several vectors per thread, tails, 1 to 16 blocks and the sizes where their number doubles;
     a source that is not 16-byte aligned takes the general path and gives the same."""
     pv = 4 if dtype == H.F32 else 8
     ws, wsb = workspace()
