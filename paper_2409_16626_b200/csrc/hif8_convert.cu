@@ -193,12 +193,13 @@ convert_kernel(const ConvParams p, unsigned long long n_vec)
     static_assert(!(FQ && AMAX) && !(AMAX && SLOTS), "fake-quant measures in a launch of its own");
     __shared__ SmemTables sm;
     constexpr unsigned kFewBlocks = MODE == HIF8_RND_TA && !FQ ? 64 : 16;  // (see pdl_launch_dependents)
-    if (AMAX || gridDim.x <= kFewBlocks) pdl_launch_dependents();
+    const bool early = AMAX || PATTERN || n_vec == 0 || gridDim.x <= kFewBlocks;
+    if (early) pdl_launch_dependents();
     constexpr bool kPair16 = SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ;
     if (kPair16) setup_sum16<MODE>(sm.ta, sm.thr, p.flags);
     else setup_tables<true, MODE != HIF8_RND_TA, FQ, MODE, SRC>(sm, p.flags);  // reads only the constant table
     pdl_wait_prior_grid();
-    pdl_launch_dependents();  // (a second time: nothing)
+    if (!early) pdl_launch_dependents();
     const int se = resolve_scale_exp<SLOTS>(p);
     const float scale = pow2f(se);
     const int da = (-se) / 2, db = -se - da;  // descale in two exact steps (the first cannot leave the normal range)
@@ -421,8 +422,9 @@ __global__ void __launch_bounds__(kThreads, SLOTS && SRC == HIF8_F32 ? 5 : 0) fq
     constexpr bool kThr = MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR;  // packed BF16 arithmetic with an LSB term
     __shared__ uint32_t s_inc[256];                   // BF16: mask16 | inc16 << 16 (threshold modes: mask16 | addend << 16)
     __shared__ uint32_t s_mask[(SRC == HIF8_F32 || kThr) ? 256 : 1];  // threshold modes: the LSB term's factor
+    if (n_vec == 0) pdl_launch_dependents();
     pdl_wait_prior_grid();  // the scale may come from the previous kernel
-    pdl_launch_dependents();
+    if (n_vec != 0) pdl_launch_dependents();
     const int se = resolve_scale_exp<SLOTS>(p);
     {
         const int e = threadIdx.x, E = e - 127 + se;
@@ -674,9 +676,9 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const void* __restrict__
     const uint4* src = reinterpret_cast<const uint4*>(srcv);
     float amax = 0.f;
     uint32_t acc = 0u;
-    if (ALONE) pdl_launch_dependents();
+    if (ALONE || n_vec == 0) pdl_launch_dependents();
     pdl_wait_prior_grid();
-    if (!ALONE) pdl_launch_dependents();
+    if (!ALONE && n_vec != 0) pdl_launch_dependents();
     const unsigned long long stride = (unsigned long long)gridDim.x * kThreads * kUnrollAmax;
     for (unsigned long long base = (unsigned long long)blockIdx.x * kThreads * kUnrollAmax; base < n_vec; base += stride) {
         uint4 v[kUnrollAmax];

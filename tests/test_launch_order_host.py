@@ -14,6 +14,7 @@ def test_the_next_launch_starts_behind_the_wait(kernel):
     text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "hif8_convert.cu")).read())
     body = next(p for p in re.split(r"(?=__global__ void)", text)[1:] if re.search(r"\b" + kernel + r"\(const", p))
     body = body[:body.find("\n}\n")]
-    # (measuring and stand-alone instantiations and launches of few blocks: named by the condition in front)
-    general = [m.start() for m in re.finditer(r"pdl_launch_dependents\(\)", body) if not re.search(r"if \((AMAX|ALONE|gridDim\.x)[^()]*\) $", body[:m.start()])]
+    # (measuring and stand-alone instantiations, launches of few blocks and element-by-element ones let it start in front: named by the condition)
+    in_front = r"if \((early|ALONE \|\| n_vec == 0|n_vec == 0|gridDim\.x == 1)\) $"
+    general = [m.start() for m in re.finditer(r"pdl_launch_dependents\(\)", body) if not re.search(in_front, body[:m.start()])]
     assert general and min(general) > body.index("pdl_wait_prior_grid()")
