@@ -98,19 +98,21 @@ template <int SRC, int MODE> __device__ __forceinline__ void encode_row_vector(c
 // ------------------------------------------------------------------------------------------------
 constexpr int kRowCache = 8;  // vectors per thread a row may occupy to be held in registers: 32 KiB per row
 
-// maximum of non-negative bit patterns over the block; every thread gets the result
-__device__ __forceinline__ uint32_t block_max(uint32_t v, uint32_t* s_part)
+// maximum of non-negative bit patterns over the group of `gs` threads (a power of two, 32 .. kThreads, aligned in the
+// block) that shares a row; every thread of the group gets the result.  Called by all threads of the block.
+__device__ __forceinline__ uint32_t group_max(uint32_t v, uint32_t* s_part, int gs)
 {
     v = __reduce_max_sync(0xFFFFFFFFu, v);
+    if (gs == 32) return v;
     __syncthreads();  // the previous use of s_part is over
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
     __syncthreads();
+    const int w0 = (threadIdx.x / gs) * (gs / 32);
     v = 0;
-    for (int w = 0; w < kThreads / 32; w++) v = max(v, s_part[w]);
+    for (int w = 0; w < gs / 32; w++) v = max(v, s_part[w0 + w]);
     return v;
 }
-// The same over a group of 1 << lg threads (32 .. kThreads, aligned in the block) that shares a row, called by all threads of the block: one barrier, of the
-// group's threads alone (number g + 1; 0 is the block's).  `s_part` is one of two sets of words, used in turn, so nobody
+// The same with one barrier, of the group's threads alone (number g + 1; 0 is the block's): `s_part` is one of two sets of words, used in turn, so nobody
 // still reads it from the use before the last one, which the barrier of the last one stands behind.
 __device__ __forceinline__ uint32_t group_max_in_turn(uint32_t v, uint32_t* s_part, int lg, int g)
 {
@@ -228,7 +230,7 @@ __global__ void __launch_bounds__(kThreads) long_row_channel_kernel(const ChanPa
 #pragma unroll
                 for (int j = 0; j < kUnroll; j++) m = amax_vector<SRC>(m, v[j]);
             }
-            const uint32_t b = block_max(__float_as_uint(amax_value<SRC>(m)), s_part);
+            const uint32_t b = group_max(__float_as_uint(amax_value<SRC>(m)), s_part, kThreads);
             if (threadIdx.x == 0) p.amax_bits[row] = b;
             se = scale_exp_from_amax(b, p.target_exp);
         }
