@@ -308,3 +308,14 @@ def test_channel_amax_of_negative_values_beside_infinities_and_nan(shape, axis, 
     assert np.array_equal(amax, amax_o) and np.array_equal(se, se_o)
     assert amax[1] == 16.0 and amax[7] == 0.0
     assert np.array_equal(q, O.channel_encode(x, dtype, axis, se_o, quick=True))
+
+
+@pytest.mark.parametrize("dtype", [H.F32, H.BF16])
+@pytest.mark.parametrize("vectors", [1028, 1500, 2047, 2048])
+def test_channel_encode_stochastic_rows_of_eight_vectors_a_thread(vectors, dtype):
+    # rows held in registers, five to eight vectors a thread, full and ended within one: every element's own random word
+    x = weight(5, vectors * (4 if dtype == H.F32 else 8), seed=vectors, dtype=dtype)
+    q, amax, se = run_channel(x, dtype, 0, rnd=H.RND_SR, seed=0x123456789)
+    amax_o, se_o = O.channel_amax_scale(x, dtype, 0, 14)
+    assert np.array_equal(amax, amax_o) and np.array_equal(se, se_o)
+    assert np.array_equal(q, O.channel_encode(x, dtype, 0, se_o, rnd=H.RND_SR, seed=0x123456789, quick=True))
