@@ -265,7 +265,9 @@ convert_kernel(const ConvParams p, unsigned long long n_vec)
 // where sixteen SMs take longer than the launches over all of them, which depends on the arithmetic an element carries (one_launch_limit).
 // All copies of a block are asynchronous and in flight together, up to 88 KiB.
 // A cluster of sixteen wants sixteen SMs of one GPC with room at the same time.  Beside another stream's work it still is the faster form (us a call, three launches / this, in
-// the time that stream was busy: 300 K BF16 elements beside products of 4096 x 8192 x 8192, whose blocks fill their SMs, 51 / 31, beside fake-quant of 2^26 elements 60 / 44).
+// the time that stream was busy: 300 K BF16 elements beside products of 4096 x 8192 x 8192, whose blocks fill their SMs, 50 / 31 to 40, beside fake-quant of 2^26 elements 60 / 44).
+// It lets the next launch start at once: behind its wait, where other conversions do, calls on 12 K to 70 K elements in a graph took 2.2 us instead of 2.4, 1 K to 8 K 2.48 instead
+// of 2.38, and beside those products 52.
 // ------------------------------------------------------------------------------------------------
 constexpr int kOneThreads = 512, kOneBlocks = 16, kOneBlocksPortable = 8;
 constexpr unsigned kOneSmem = 88 * 1024, kOneSmemDefault = 32 * 1024;  // source bytes per block: with the opt-in (what one_launch_limit needs), and without
@@ -280,10 +282,9 @@ __global__ void __launch_bounds__(kOneThreads) one_launch_kernel(const ConvParam
     constexpr int PV = SrcTraits<SRC>::kPerVec;
     constexpr bool kPair16 = SRC == HIF8_BF16 && (MODE == HIF8_RND_HR || MODE == HIF8_RND_SSR) && !FQ;
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this block has started (waited for before the first remote store)
-    if (gridDim.x == 1) pdl_launch_dependents();  // (see there: few blocks; up to 8 K BF16 elements 2.38 us, behind the wait 2.48)
+    pdl_launch_dependents();
     const unsigned first = blockIdx.x * kOneThreads + threadIdx.x, step = gridDim.x * kOneThreads;  // vectors first, first + step, ..
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     const uint4* src = reinterpret_cast<const uint4*>(p.src);
     const uint32_t s_mine = (uint32_t)__cvta_generic_to_shared(s_src + threadIdx.x);
 #pragma unroll 4

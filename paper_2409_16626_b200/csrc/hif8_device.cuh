@@ -153,9 +153,9 @@ __device__ __forceinline__ uint32_t philox_word(const uint4& r, unsigned lane)
 // was let in as well: its blocks only waited, in the places that the next one's blocks then lacked, so that these sat unevenly, the more so the fewer
 // registers a kernel takes (us, in front / behind: FP32 fake-quant under simplified stochastic rounding 1.7 M elements 6.2 / 4.5; scale and encode, BF16
 // hybrid 1.2 M 7.5 / 5.5; FP16 half-to-even fake-quant 2 M 8.9 / 4.5; BF16 stochastic encode 0.9 M 8.9 / 4.4; FP32 half-away encode 2 M 3.5 / 2.9; from 5 M on the same).
-// In front of it still: launches of few blocks, which leave places for all (600 FP16 elements 1.14 / 1.29, 150 K BF16 1.41 / 1.50; hybrid 150 K the same), or of short ones (element by
-// element: 360 K FP32 2.24 / 2.76; generated sources), what
-// clears or measures for the next launch, a conversion that measures amax (small ones were up to 12 % slower behind it in some processes), an amax on its own (3 M 5.3 / 5.7), decode.
+// In front of it still: launches of few blocks, which leave places for all (600 FP16 elements 1.14 / 1.29, 150 K BF16 1.41 / 1.50; hybrid 150 K the same), or of
+// short ones (element by element: 360 K FP32 2.24 / 2.76; generated sources), the one-launch form of small tensors (see there), what clears or measures for the next
+// launch, a conversion that measures amax (small ones were up to 12 % slower behind it in some processes), an amax on its own (3 M 5.3 / 5.7), decode.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
