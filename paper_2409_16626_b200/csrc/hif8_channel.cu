@@ -197,11 +197,13 @@ __global__ void __launch_bounds__(kThreads, 4) row_channel_kernel(const ChanPara
             const unsigned long long flat = (unsigned long long)row * nv + t;
 #pragma unroll
             for (int j = 0; j < NV; j++) {
-                unsigned long long u = flat + j * gs;
-                // (A vector's counter is hidden from the compiler until its turn: the first rounds of all eight, worked out in front, cost 120 bytes of spills.  FP32,
-                // standard stochastic rounding, 500 x 8192 16.8 us, so 14.6, 2000 x 6000 37.7 and 31.8.)
-                if (MODE == HIF8_RND_SR && SRC == HIF8_F32 && NV > kUnroll) asm volatile("" : "+l"(u));
-                if (full || (unsigned)(j * gs + t) < nv) encode_row_vector<SRC, MODE>(p, sm, cur[j], u, scale, k0, k1);
+                if constexpr (MODE == HIF8_RND_SR && SRC == HIF8_F32 && NV > kUnroll) {
+                    // A vector's counter is hidden from the compiler until its turn: the first rounds of all eight, worked out in front, cost 120 bytes of spills (500 x 8192
+                    // 16.8 us, so 14.6, 2000 x 6000 37.7 and 31.8).
+                    unsigned long long u = flat + j * gs;
+                    asm volatile("" : "+l"(u));
+                    if (full || (unsigned)(j * gs + t) < nv) encode_row_vector<SRC, MODE>(p, sm, cur[j], u, scale, k0, k1);
+                } else if (full || (unsigned)(j * gs + t) < nv) encode_row_vector<SRC, MODE>(p, sm, cur[j], flat + j * gs, scale, k0, k1);
             }
         }
     }
