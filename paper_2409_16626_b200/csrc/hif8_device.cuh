@@ -193,6 +193,7 @@ struct ConvParams {
     uint32_t pattern_first;       // PATTERN kernels only: element i is the FP32 value whose encoding is pattern_first + i
     int reverse;                  // walk the tensor from its end: set for the second pass of just-in-time scaling, so that
                                   // the lines the amax pass read last (still in L2) are the ones re-read first
+    int next_at_end;              // convert_kernel: its dependents start when its blocks end
 };
 
 template <int SRC> struct SrcTraits;
