@@ -184,10 +184,16 @@ __device__ __forceinline__ void convert_group(const ConvParams& p, const SmemTab
 // SLOTS: the amax comes in several words (see resolve_scale_exp).
 // Blocks per SM: left to the compiler, encode takes 32 registers (stochastic rounding excepted), which is eight blocks.  Two kinds of fake-quant are faster
 // with the bound (us, without / with it): half to even of FP32, 34 registers so, 9.8 M elements 16.7 / 15.4, 68 M 91.0 / 86.1 (3 M 6.2 / 6.7), half away of FP16 11 M
-// 11.8 / 11.1, 82 M 60.8 / 59.8; other FP16 modes 0 to 0.6 % slower.
+// 11.8 / 11.1, 82 M 60.8 / 59.8; other FP16 modes 0 to 0.6 % slower.  FP16 encode behind amax_slots_kernel finds its source in L2 and is faster with six blocks of 40 registers
+// under hybrid and simplified stochastic rounding (scale and encode of 2 M elements 8.4 / 7.0, 5.3 M 10.9 / 9.6).
+constexpr int blocks_per_sm(int src, int mode, bool fq, bool slots)
+{
+    if (fq && !slots && ((src == HIF8_F32 && mode == HIF8_RND_TE) || (src == HIF8_F16 && mode == HIF8_RND_TA))) return kBlocksPerSM;
+    if (!fq && slots && src == HIF8_F16 && (mode == HIF8_RND_HR || mode == HIF8_RND_SSR)) return 6;
+    return 0;
+}
 template <int SRC, int MODE, bool FQ, bool AMAX, bool PATTERN = false, bool SLOTS = false>
-__global__ void __launch_bounds__(kThreads, FQ && !SLOTS && ((SRC == HIF8_F32 && MODE == HIF8_RND_TE) || (SRC == HIF8_F16 && MODE == HIF8_RND_TA)) ? kBlocksPerSM : 0)
-convert_kernel(const ConvParams p, unsigned long long n_vec)
+__global__ void __launch_bounds__(kThreads, blocks_per_sm(SRC, MODE, FQ, SLOTS)) convert_kernel(const ConvParams p, unsigned long long n_vec)
 {
     static_assert(!PATTERN || (SRC == HIF8_F32 && !FQ && !AMAX), "generated sources are FP32 patterns, encode only");
     static_assert(!(FQ && AMAX) && !(AMAX && SLOTS), "fake-quant measures in a launch of its own");

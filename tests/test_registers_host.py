@@ -15,8 +15,9 @@ def report_of(source, tmp_path):
 
 def test_encode_kernels_leave_room_for_eight_blocks_an_sm(tmp_path):
     report = report_of("hif8_convert.cu", tmp_path)
-    kernels = re.findall(r"Compiling entry function '\w*?convert_kernelILi(\d)ELi(\d)ELb(\d)ELb(\d)E\w*'.*?(\d+) bytes spill stores.*?Used (\d+) registers", report, re.S)
-    encode = [(int(src), int(mode), int(spill), int(regs)) for src, mode, fq, amax, spill, regs in kernels if fq == "0" and amax == "0" and int(mode) != SR]
+    kernels = re.findall(r"Compiling entry function '\w*?convert_kernelILi(\d)ELi(\d)ELb(\d)ELb(\d)ELb\dELb(\d)E\w*'.*?(\d+) bytes spill stores.*?Used (\d+) registers", report, re.S)
+    encode = [(int(src), int(mode), int(spill), int(regs)) for src, mode, fq, amax, slots, spill, regs in kernels
+              if fq == "0" and amax == "0" and slots == "0" and int(mode) != SR]
     assert len(encode) >= 3 * 4  # source formats, rounding methods
     assert [k for k in encode if k[2] or k[3] > 32] == []
 
