@@ -186,9 +186,12 @@ __device__ __forceinline__ void convert_group(const ConvParams& p, const SmemTab
 // with the bound (us, without / with it): half to even of FP32, 34 registers so, 9.8 M elements 16.7 / 15.4, 68 M 91.0 / 86.1 (3 M 6.2 / 6.7), half away of FP16 11 M
 // 11.8 / 11.1, 82 M 60.8 / 59.8; other FP16 modes 0 to 0.6 % slower.  FP16 encode behind amax_slots_kernel finds its source in L2 and is faster with six blocks of 40 registers
 // under hybrid and simplified stochastic rounding (scale and encode of 2 M elements 8.4 / 7.0, 5.3 M 10.9 / 9.6).
+// FP16 fake-quant under stochastic rounding, whose random words are long chains, with four of 64 (40 registers by themselves: with its amax 1.9 M elements 19.5 / 14.2, without it 5.2 M 17.0 / 14.9, 2.6 M 9.6 / 11.6; from 8 M
+// on the same).
 constexpr int blocks_per_sm(int src, int mode, bool fq, bool slots)
 {
     if (fq && !slots && ((src == HIF8_F32 && mode == HIF8_RND_TE) || (src == HIF8_F16 && mode == HIF8_RND_TA))) return kBlocksPerSM;
+    if (fq && src == HIF8_F16 && mode == HIF8_RND_SR) return 4;
     if (!fq && slots && src == HIF8_F16 && (mode == HIF8_RND_HR || mode == HIF8_RND_SSR)) return 6;
     return 0;
 }
